@@ -686,6 +686,7 @@ wc_status wc_destroy_lattice(wc_lattice lat)
     free_clover(lat->cinv);
     free_clover(lat->ceo);
     cudaFree(lat->staging);
+    cudaFree(lat->eom_ws);
     for (cudaStream_t cs : {lat->copy_stream, lat->copy_out_stream})
         if (cs) {
             cudaStreamSynchronize(cs);
@@ -942,17 +943,17 @@ wc_status wc_apply_schur(wc_lattice lat, wc_field out, wc_field in, int dagger)
     wc_lattice h = nullptr;
     st = half_lattice(lat, &h);
     if (st != WC_OK) return st;
-    wc_field e = nullptr, o = nullptr, r = nullptr;
-    st = wc_field_create(h, in->prec, &e);
-    if (st == WC_OK) st = wc_field_create(h, in->prec, &o);
-    if (st == WC_OK) st = wc_field_create(h, in->prec, &r);
-    if (st == WC_OK) st = check_cuda(lat, launch_split(lat, in, e, o, lat->stream), "split");
-    if (st == WC_OK) st = check_cuda(lat, launch_schur(h, r, e, dagger ? 1 : 0, lat->stream), "schur");
-    if (st == WC_OK) st = check_cuda(lat, launch_merge(lat, r, nullptr, out, lat->stream), "merge");
+    // the half fields are kept between calls (creating and freeing three per
+    // call had cost 0.4 ms, the FP64 operator itself takes 0.3 ms at
+    // 16^3x32); the lock is held until the stream has finished
+    std::lock_guard<std::mutex> lk(lat->eom_mutex);
+    wc_field *io = lat->schur_io[in->prec];
+    for (int k = 0; k < 2 && st == WC_OK; ++k)
+        if (!io[k]) st = wc_field_create(h, in->prec, &io[k]);
+    if (st == WC_OK) st = check_cuda(lat, launch_split(lat, in, io[0], nullptr, lat->stream), "split");
+    if (st == WC_OK) st = check_cuda(lat, launch_schur(h, io[1], io[0], dagger ? 1 : 0, lat->stream), "schur");
+    if (st == WC_OK) st = check_cuda(lat, launch_merge(lat, io[1], nullptr, out, lat->stream), "merge");
     if (st == WC_OK) st = check_cuda(lat, cudaStreamSynchronize(lat->stream), "sync");
-    wc_field_destroy(e);
-    wc_field_destroy(o);
-    wc_field_destroy(r);
     return st;
 }
 wc_status wc_apply_Mdag(wc_lattice lat, wc_field out, wc_field in) { return apply_common(lat, out, in, 1); }

@@ -17,9 +17,9 @@
 // right-hand side) is otherwise that of the single-field pass (spin
 // projection, the block product, beta = -kappa^2 on the even pass).  Per-field device flags (the
 // skip word of a lockstep batch's solver scalars) may skip fields.
+#include <mutex>
 #include <string>
 #include <type_traits>
-#include <vector>
 
 #include "wc_internal.cuh"
 #include "wc_stencil.cuh"
@@ -165,17 +165,19 @@ __device__ __forceinline__ void eom_link(const typename EoMStage<P>::W (*st)[kEo
     }
 }
 
-template <class P, int MU, int SF, int SB>
+// (FIN: `in` is a full-lattice field, read at the full index)
+template <class P, int MU, int SF, int SB, bool FIN>
 __device__ __forceinline__ void eom_hops(const Geom &g, const typename EoMStage<P>::W (*st)[kEoMSites],
                                         const float2 (*r3)[3][kEoMSites], int s, const void *in,
                                         const float *in_nrm, int Vh, int x, const int c[4], cx<float> acc[12])
 {
+    const int Vin = FIN ? g.V : Vh;
     const int L = g.L[MU], stride = g.stride[MU];
     {
         const bool wrap = c[MU] == L - 1;
         const int xf = wc_idx(wrap ? x - (L - 1) * stride : x + stride, g.V);
         cx<float> p[12], h[6], u[6], r2[3], w[6];
-        const float scale = P::load_spinor_raw(in, in_nrm, Vh, xf >> 1, p);
+        const float scale = P::load_spinor_raw(in, in_nrm, Vin, FIN ? xf : xf >> 1, p);
         const float coef = ((MU == 3 && wrap) ? (float)g.tbc : 1.f) * scale;
         project<MU, SF>(p, h);
         eom_link<P>(st, r3, s, MU, u, r2);
@@ -186,7 +188,7 @@ __device__ __forceinline__ void eom_hops(const Geom &g, const typename EoMStage<
         const bool wrap = c[MU] == 0;
         const int xb = wc_idx(wrap ? x + (L - 1) * stride : x - stride, g.V);
         cx<float> p[12], h[6], u[6], r2[3], w[6];
-        const float scale = P::load_spinor_raw(in, in_nrm, Vh, xb >> 1, p);
+        const float scale = P::load_spinor_raw(in, in_nrm, Vin, FIN ? xb : xb >> 1, p);
         const float coef = ((MU == 3 && wrap) ? (float)g.tbc : 1.f) * scale;
         project<MU, SB>(p, h);
         eom_link<P>(st, r3, s, 4 + MU, u, r2);
@@ -207,7 +209,13 @@ __device__ __forceinline__ int eom_full_site(const Geom &g, int i, int p, int c[
 
 // MODE 0 (odd pass): out_r = Blk H hin_r      (Blk = A^-1)
 // MODE 1 (even pass): out_r = Blk vin_r + beta H hin_r   (Blk = A)
-template <class P, int DAG, int MODE>
+// FULL: the operator's input (hin of the odd pass, vin of the even pass) and
+// output are full-lattice fields, the odd-site intermediate stays a half
+// field: the even pass writes its site and the zero of the odd site beside
+// it, so wc_apply_schur_multi needs no split and merge passes (at
+// 16^3x32 with 12 FP32 fields two launches instead of 26: 48 of them, 264
+// us, in an M^+ M^ pair before).
+template <class P, int DAG, int MODE, bool FULL>
 __global__ void __maxnreg__(80) k_eo_multi(Geom g, int p, GaugeStore U, CloverStore Blk,
                                                                    const __grid_constant__ EoMultiArgs a,
                                                                    double beta)
@@ -253,17 +261,17 @@ __global__ void __maxnreg__(80) k_eo_multi(Geom g, int p, GaugeStore U, CloverSt
     cx<float> h[12];
 #pragma unroll
     for (int k = 0; k < 12; ++k) h[k] = mkc(0.f, 0.f);
-    eom_hops<P, 0, SF, SB>(g, st, r3, s, a.hin[r], a.hin_nrm[r], Vh, x, c, h);
-    eom_hops<P, 1, SF, SB>(g, st, r3, s, a.hin[r], a.hin_nrm[r], Vh, x, c, h);
-    eom_hops<P, 2, SF, SB>(g, st, r3, s, a.hin[r], a.hin_nrm[r], Vh, x, c, h);
-    eom_hops<P, 3, SF, SB>(g, st, r3, s, a.hin[r], a.hin_nrm[r], Vh, x, c, h);
+    eom_hops<P, 0, SF, SB, FULL && MODE == 0>(g, st, r3, s, a.hin[r], a.hin_nrm[r], Vh, x, c, h);
+    eom_hops<P, 1, SF, SB, FULL && MODE == 0>(g, st, r3, s, a.hin[r], a.hin_nrm[r], Vh, x, c, h);
+    eom_hops<P, 2, SF, SB, FULL && MODE == 0>(g, st, r3, s, a.hin[r], a.hin_nrm[r], Vh, x, c, h);
+    eom_hops<P, 3, SF, SB, FULL && MODE == 0>(g, st, r3, s, a.hin[r], a.hin_nrm[r], Vh, x, c, h);
     cx<float> v[12], o[12];
     const float bt = (float)beta;
     if (MODE == 0) {
 #pragma unroll
         for (int k = 0; k < 12; ++k) v[k] = h[k];
     } else {
-        P::load_spinor(a.vin[r], a.vin_nrm[r], Vh, i, v);
+        P::load_spinor(a.vin[r], a.vin_nrm[r], FULL ? g.V : Vh, FULL ? x : i, v);
     }
 #pragma unroll
     for (int b = 0; b < 2; ++b) {
@@ -274,7 +282,15 @@ __global__ void __maxnreg__(80) k_eo_multi(Geom g, int p, GaugeStore U, CloverSt
     if (MODE == 1)
 #pragma unroll
         for (int k = 0; k < 12; ++k) o[k] = o[k] + bt * h[k];
-    P::store_spinor(a.out[r], a.out_nrm[r], Vh, i, o);
+    if constexpr (FULL && MODE == 1) {
+        P::store_spinor(a.out[r], a.out_nrm[r], g.V, x, o);
+        cx<float> z[12];
+#pragma unroll
+        for (int k = 0; k < 12; ++k) z[k] = mkc(0.f, 0.f);
+        P::store_spinor(a.out[r], a.out_nrm[r], g.V, wc_idx(x ^ 1, g.V), z);   // the row's odd site beside x
+    } else {
+        P::store_spinor(a.out[r], a.out_nrm[r], Vh, i, o);
+    }
     if (MODE == 1 && a.red == 1) {
         cx<float> d[12];
         P32::load_spinor(a.dot[r], nullptr, Vh, i, d);
@@ -305,9 +321,9 @@ __global__ void __maxnreg__(80) k_eo_multi(Geom g, int p, GaugeStore U, CloverSt
     }
 }
 
-template <class P, int DAG>
-cudaError_t launch_eom(const wc_lattice_s *full, int n, wc_field const *outs, wc_field const *ins,
-                       wc_field const *tmps, const int *const *skip, int red, wc_field const *dots, double *part,
+template <class P, int DAG, bool FULL>
+cudaError_t launch_eom(const wc_lattice_s *full, int n, wc_field_s *const *outs, wc_field_s *const *ins,
+                       wc_field_s *const *tmps, const int *const *skip, int red, wc_field const *dots, double *part,
                        cudaStream_t stream)
 {
     const int Vh = full->g.V >> 1;
@@ -322,7 +338,7 @@ cudaError_t launch_eom(const wc_lattice_s *full, int n, wc_field const *outs, wc
         a.out_nrm[r] = tmps[r]->nrm;
     }
     // odd sites: tmp = A_oo^-1 H_oe in
-    k_eo_multi<P, DAG, 0><<<grid, block, 0, stream>>>(full->g, 1, full->gauge, full->cinv, a, 0.0);
+    k_eo_multi<P, DAG, 0, FULL><<<grid, block, 0, stream>>>(full->g, 1, full->gauge, full->cinv, a, 0.0);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     // even sites: out = A_ee in - kappa^2 H_eo tmp
@@ -337,7 +353,7 @@ cudaError_t launch_eom(const wc_lattice_s *full, int n, wc_field const *outs, wc
     a.red = red;
     a.part = part;
     for (int r = 0; r < n && red == 1; ++r) a.dot[r] = dots[r]->data;
-    k_eo_multi<P, DAG, 1><<<grid, block, 0, stream>>>(full->g, 0, full->gauge, full->ceo, a,
+    k_eo_multi<P, DAG, 1, FULL><<<grid, block, 0, stream>>>(full->g, 0, full->gauge, full->ceo, a,
                                                       -full->kappa * full->kappa);
     return cudaGetLastError();
 }
@@ -353,11 +369,11 @@ cudaError_t launch_schur_multi(wc_lattice half, int n, wc_field const *outs, wc_
     const wc_prec pr = ins[0]->prec;
     if (red != 0 && (pr != WC_F32 || !part || (red == 1 && !dots))) return cudaErrorInvalidValue;
     if (pr == WC_F32)
-        return dagger ? launch_eom<P32, 1>(full, n, outs, ins, tmps, skip, red, dots, part, stream)
-                      : launch_eom<P32, 0>(full, n, outs, ins, tmps, skip, red, dots, part, stream);
+        return dagger ? launch_eom<P32, 1, false>(full, n, outs, ins, tmps, skip, red, dots, part, stream)
+                      : launch_eom<P32, 0, false>(full, n, outs, ins, tmps, skip, red, dots, part, stream);
     if (pr == WC_F16)
-        return dagger ? launch_eom<P16, 1>(full, n, outs, ins, tmps, skip, 0, nullptr, nullptr, stream)
-                      : launch_eom<P16, 0>(full, n, outs, ins, tmps, skip, 0, nullptr, nullptr, stream);
+        return dagger ? launch_eom<P16, 1, false>(full, n, outs, ins, tmps, skip, 0, nullptr, nullptr, stream)
+                      : launch_eom<P16, 0, false>(full, n, outs, ins, tmps, skip, 0, nullptr, nullptr, stream);
     return cudaErrorInvalidValue;
 }
 
@@ -389,24 +405,41 @@ extern "C" wc_status wc_apply_schur_multi(wc_lattice lat, int n, wc_field *outs,
     st = half_lattice(lat, &h);
     if (st != WC_OK) return st;
     const wc_prec pr = ins[0]->prec;
-    std::vector<wc_field> e(n, nullptr), r(n, nullptr), t(n, nullptr);
-    for (int k = 0; k < n && st == WC_OK; ++k) {
-        st = wc_field_create(h, pr, &e[k]);
-        if (st == WC_OK) st = wc_field_create(h, pr, &r[k]);
-        if (st == WC_OK) st = wc_field_create(h, pr, &t[k]);
+    const int Vh = h->g.V;
+    // n odd-site intermediates in the lattice's workspace, kept between
+    // calls (allocating three half fields per right-hand side on every call
+    // cost 2.7 ms of a
+    // 2.9 ms call at 12 right-hand sides and 16^3x32); one call at a time uses it:
+    // the lock is held until the stream has finished
+    const size_t data_bytes = (spinor_bytes(pr, Vh) + 255) / 256 * 256;
+    const size_t nrm_bytes = pr == WC_F16 ? ((size_t)Vh * sizeof(float) + 255) / 256 * 256 : 0;
+    std::lock_guard<std::mutex> lk(lat->eom_mutex);
+    if (lat->eom_ws_bytes < (data_bytes + nrm_bytes) * n) {
+        cudaFree(lat->eom_ws);
+        lat->eom_ws = nullptr;
+        lat->eom_ws_bytes = 0;
+        st = check_cuda(lat, cudaMalloc(&lat->eom_ws, (data_bytes + nrm_bytes) * n), "cudaMalloc(schur_multi)");
+        if (st != WC_OK) return st;
+        lat->eom_ws_bytes = (data_bytes + nrm_bytes) * n;
     }
-    for (int k = 0; k < n && st == WC_OK; ++k)
-        st = check_cuda(lat, launch_split(lat, ins[k], e[k], nullptr, lat->stream), "split");
-    if (st == WC_OK)
-        st = check_cuda(lat, launch_schur_multi(h, n, r.data(), e.data(), t.data(), dagger ? 1 : 0, nullptr, lat->stream),
-                        "schur_multi");
-    for (int k = 0; k < n && st == WC_OK; ++k)
-        st = check_cuda(lat, launch_merge(lat, r[k], nullptr, outs[k], lat->stream), "merge");
+    wc_field_s tmp[kMrhsMax];
+    wc_field_s *tmps[kMrhsMax];
+    char *ws = static_cast<char *>(lat->eom_ws);
+    for (int k = 0; k < n; ++k, ws += data_bytes + nrm_bytes) {
+        tmp[k].lat = h;
+        tmp[k].prec = pr;
+        tmp[k].data = ws;
+        tmp[k].nrm = nrm_bytes ? reinterpret_cast<float *>(ws + data_bytes) : nullptr;
+        tmps[k] = &tmp[k];
+    }
+    cudaError_t e;
+    if (pr == WC_F32)
+        e = dagger ? launch_eom<P32, 1, true>(lat, n, outs, ins, tmps, nullptr, 0, nullptr, nullptr, lat->stream)
+                   : launch_eom<P32, 0, true>(lat, n, outs, ins, tmps, nullptr, 0, nullptr, nullptr, lat->stream);
+    else
+        e = dagger ? launch_eom<P16, 1, true>(lat, n, outs, ins, tmps, nullptr, 0, nullptr, nullptr, lat->stream)
+                   : launch_eom<P16, 0, true>(lat, n, outs, ins, tmps, nullptr, 0, nullptr, nullptr, lat->stream);
+    st = check_cuda(lat, e, "schur_multi");
     if (st == WC_OK) st = check_cuda(lat, cudaStreamSynchronize(lat->stream), "sync");
-    for (int k = 0; k < n; ++k) {
-        wc_field_destroy(e[k]);
-        wc_field_destroy(r[k]);
-        wc_field_destroy(t[k]);
-    }
     return st;
 }

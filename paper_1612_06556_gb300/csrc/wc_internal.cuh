@@ -5,6 +5,7 @@
 
 #include <cuda_runtime.h>
 
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -109,6 +110,14 @@ struct wc_lattice_s {
     // wc_ras_schur: the even-site input and output on the half lattice, per
     // precision (created on first use)
     wc_field_s *ras_half[3][2] = {};
+    // wc_apply_schur_multi: odd-site intermediates of its right-hand sides
+    // (up to kMrhsMax half-lattice spinors), held until wc_destroy_lattice
+    void *eom_ws = nullptr;
+    size_t eom_ws_bytes = 0;
+    std::mutex eom_mutex;
+    // wc_apply_schur: the even-site input and output on the half lattice, per
+    // precision (created on first use)
+    wc_field_s *schur_io[3][2] = {};
     std::string err;
 };
 
