@@ -140,181 +140,6 @@ __global__ void k_pack_gauge(int V, const double2 *U, GaugeStore g)
     g.u16b[(size_t)mu * V + x] = h2;
 }
 
-// ------------------------------------------------------------------------
-// clover term (FP64 arithmetic)
-// ------------------------------------------------------------------------
-
-struct M3 {
-    cx<double> m[3][3];
-};
-
-__device__ M3 m3_mul(const M3 &a, const M3 &b)
-{
-    M3 r;
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            cx<double> s = a.m[i][0] * b.m[0][j];
-            s = cfma(a.m[i][1], b.m[1][j], s);
-            s = cfma(a.m[i][2], b.m[2][j], s);
-            r.m[i][j] = s;
-        }
-    return r;
-}
-
-__device__ M3 m3_dag(const M3 &a)
-{
-    M3 r;
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) r.m[i][j] = conj(a.m[j][i]);
-    return r;
-}
-
-__device__ M3 load_u(const GaugeStore &g, int V, int mu, int x)
-{
-    cx<double> u[6], r2[3];
-    P64::load_link(g, V, mu, x, u, r2);
-    M3 r;
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-        r.m[0][j] = u[j];
-        r.m[1][j] = u[3 + j];
-        r.m[2][j] = r2[j];
-    }
-    return r;
-}
-
-__device__ int shifted(const Geom &g, const int c[4], int mu, int dmu, int nu, int dnu)
-{
-    int d[4] = {c[0], c[1], c[2], c[3]};
-    d[mu] = (d[mu] + dmu + g.L[mu]) % g.L[mu];
-    d[nu] = (d[nu] + dnu + g.L[nu]) % g.L[nu];
-    return d[0] + g.stride[1] * d[1] + g.stride[2] * d[2] + g.stride[3] * d[3];
-}
-
-// Fhat_munu(x) = (1/8)[(Q - Q^+) - tr(Q - Q^+)/3], Q the four-leaf clover
-__device__ M3 field_strength(const Geom &g, const GaugeStore &G, int x, const int c[4], int mu, int nu)
-{
-    const int V = g.V;
-    const int xpm = shifted(g, c, mu, 1, nu, 0), xpn = shifted(g, c, mu, 0, nu, 1);
-    const int xmm = shifted(g, c, mu, -1, nu, 0), xmn = shifted(g, c, mu, 0, nu, -1);
-    const int xmm_pn = shifted(g, c, mu, -1, nu, 1), xmm_mn = shifted(g, c, mu, -1, nu, -1);
-    const int xpm_mn = shifted(g, c, mu, 1, nu, -1);
-    M3 Q;
-    // leaf x -> x+mu -> x+mu+nu -> x+nu -> x
-    M3 l = m3_mul(m3_mul(load_u(G, V, mu, x), load_u(G, V, nu, xpm)),
-                  m3_mul(m3_dag(load_u(G, V, mu, xpn)), m3_dag(load_u(G, V, nu, x))));
-    Q = l;
-    // leaf x -> x+nu -> x+nu-mu -> x-mu -> x
-    l = m3_mul(m3_mul(load_u(G, V, nu, x), m3_dag(load_u(G, V, mu, xmm_pn))),
-               m3_mul(m3_dag(load_u(G, V, nu, xmm)), load_u(G, V, mu, xmm)));
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) Q.m[i][j] = Q.m[i][j] + l.m[i][j];
-    // leaf x -> x-mu -> x-mu-nu -> x-nu -> x
-    l = m3_mul(m3_mul(m3_dag(load_u(G, V, mu, xmm)), m3_dag(load_u(G, V, nu, xmm_mn))),
-               m3_mul(load_u(G, V, mu, xmm_mn), load_u(G, V, nu, xmn)));
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) Q.m[i][j] = Q.m[i][j] + l.m[i][j];
-    // leaf x -> x-nu -> x-nu+mu -> x+mu -> x
-    l = m3_mul(m3_mul(m3_dag(load_u(G, V, nu, xmn)), load_u(G, V, mu, xmn)),
-               m3_mul(load_u(G, V, nu, xpm_mn), m3_dag(load_u(G, V, mu, x))));
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) Q.m[i][j] = Q.m[i][j] + l.m[i][j];
-    M3 F;
-    cx<double> tr = mkc(0.0, 0.0);
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            F.m[i][j] = Q.m[i][j] - conj(Q.m[j][i]);
-            if (i == j) tr = tr + F.m[i][i];
-        }
-    const cx<double> t3 = (1.0 / 3.0) * tr;
-#pragma unroll
-    for (int i = 0; i < 3; ++i) F.m[i][i] = F.m[i][i] - t3;
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) F.m[i][j] = 0.125 * F.m[i][j];
-    return F;
-}
-
-// Block b of A = 1 + T.  In the chiral basis sigma_munu restricted to spin
-// pair b is (eta = -1 for b = 0, +1 for b = 1):
-//   sigma_xy = -s3, sigma_xz = s2, sigma_yz = -s1,
-//   sigma_xt = eta s1, sigma_yt = eta s2, sigma_zt = eta s3,
-// so the block is 1 + i csw kappa [[E3, E1 - i E2], [E1 + i E2, -E3]] with
-// E1 = -F_yz + eta F_xt, E2 = F_xz + eta F_yt, E3 = -F_xy + eta F_zt.
-__global__ void k_build_clover(Geom g, GaugeStore G, CloverStore C, double csw, double kappa)
-{
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    if (x >= g.V) return;
-    int c[4];
-    site_coords(g, x, c);
-    const M3 Fxy = field_strength(g, G, x, c, 0, 1), Fxz = field_strength(g, G, x, c, 0, 2);
-    const M3 Fxt = field_strength(g, G, x, c, 0, 3), Fyz = field_strength(g, G, x, c, 1, 2);
-    const M3 Fyt = field_strength(g, G, x, c, 1, 3), Fzt = field_strength(g, G, x, c, 2, 3);
-    const double ck = csw * kappa;
-    const int V = g.V;
-    for (int b = 0; b < 2; ++b) {
-        const double eta = b == 0 ? -1.0 : 1.0;
-        cx<double> blk[6][6];
-#pragma unroll
-        for (int i = 0; i < 3; ++i)
-#pragma unroll
-            for (int j = 0; j < 3; ++j) {
-                const cx<double> e1 = (-1.0) * Fyz.m[i][j] + eta * Fxt.m[i][j];
-                const cx<double> e2 = Fxz.m[i][j] + eta * Fyt.m[i][j];
-                const cx<double> e3 = (-1.0) * Fxy.m[i][j] + eta * Fzt.m[i][j];
-                // i*ck*(...) for the four spin sub-blocks
-                blk[i][j] = ck * times_i(e3);
-                blk[3 + i][3 + j] = (-ck) * times_i(e3);
-                blk[i][3 + j] = ck * times_i(e1 - times_i(e2));
-                blk[3 + i][j] = ck * times_i(e1 + times_i(e2));
-            }
-        double r[36];
-#pragma unroll
-        for (int i = 0; i < 6; ++i) r[i] = 1.0 + blk[i][i].re;
-        int k = 6;
-#pragma unroll
-        for (int i = 1; i < 6; ++i)
-#pragma unroll
-            for (int j = 0; j < i; ++j) {
-                r[k++] = blk[i][j].re;
-                r[k++] = blk[i][j].im;
-            }
-#pragma unroll
-        for (int q = 0; q < 18; ++q) {
-            const double2 v = make_double2(r[2 * q], r[2 * q + 1]);
-            C.c64[((size_t)b * 18 + q) * V + x] = v;
-            C.cdf[((size_t)b * 18 + q) * V + x] = df_pack(v);
-        }
-#pragma unroll
-        for (int q = 0; q < 9; ++q)
-            C.c32[((size_t)b * 9 + q) * V + x] =
-                make_float4((float)r[4 * q], (float)r[4 * q + 1], (float)r[4 * q + 2], (float)r[4 * q + 3]);
-        // FP16: 18 half2 per block, global half2 index 18b + q, 4 per uint4
-        unsigned hw[18];
-#pragma unroll
-        for (int q = 0; q < 18; ++q) hw[q] = c2h((float)r[2 * q], (float)r[2 * q + 1]);
-        unsigned *c16 = reinterpret_cast<unsigned *>(C.c16);
-#pragma unroll
-        for (int q = 0; q < 18; ++q) {
-            const int gq = 18 * b + q;
-            c16[((size_t)(gq >> 2) * V + x) * 4 + (gq & 3)] = hw[q];
-        }
-    }
-}
-
 template <class T>
 cudaError_t dalloc(T **p, size_t bytes)
 {
@@ -797,8 +622,7 @@ wc_status wc_load_clover(wc_lattice lat, double csw, double kappa)
         if (st != WC_OK) return set_error(lat, st, "extended lattice clover: " + lat->ext->err);
         st = check_cuda(lat, extract_clover(lat, lat->stream), "extract clover");
     } else {
-        k_build_clover<<<(V + 63) / 64, 64, 0, lat->stream>>>(lat->g, lat->gauge, c, csw, kappa);
-        st = check_launch(lat, "build_clover");
+        st = check_cuda(lat, launch_build_clover(lat, csw, kappa, lat->stream), "build_clover");
     }
     if (st != WC_OK) return st;
     lat->csw = csw;

@@ -534,6 +534,34 @@ struct P16 {
     }
 };
 
+// one packed block (36 reals) at position pos of a clover store in the other
+// precisions, and in FP64 too when F64; 16-byte stores, but for the 8 bytes
+// of each block in the binary16 word the two blocks share
+template <bool F64>
+__device__ __forceinline__ void store_clover_block(const CloverStore &S, int V, int pos, int b, const double r[36])
+{
+#pragma unroll
+    for (int q = 0; q < 18; ++q) {
+        const double2 v = make_double2(r[2 * q], r[2 * q + 1]);
+        if (F64) S.c64[((size_t)b * 18 + q) * V + pos] = v;
+        S.cdf[((size_t)b * 18 + q) * V + pos] = df_pack(v);
+    }
+#pragma unroll
+    for (int q = 0; q < 9; ++q)
+        S.c32[((size_t)b * 9 + q) * V + pos] =
+            make_float4((float)r[4 * q], (float)r[4 * q + 1], (float)r[4 * q + 2], (float)r[4 * q + 3]);
+    unsigned h[18];
+#pragma unroll
+    for (int q = 0; q < 18; ++q) h[q] = c2h((float)r[2 * q], (float)r[2 * q + 1]);
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+        S.c16[(size_t)((b == 0 ? 0 : 5) + q) * V + pos] =
+            make_uint4(b == 0 ? h[4 * q] : h[4 * q + 2], b == 0 ? h[4 * q + 1] : h[4 * q + 3],
+                       b == 0 ? h[4 * q + 2] : h[4 * q + 4], b == 0 ? h[4 * q + 3] : h[4 * q + 5]);
+    reinterpret_cast<uint2 *>(S.c16 + (size_t)4 * V + pos)[b] =
+        b == 0 ? make_uint2(h[16], h[17]) : make_uint2(h[0], h[1]);
+}
+
 // Hermitian 6x6 block (packed) times a 6-vector: y = B v
 template <class R>
 __device__ __forceinline__ void clover_block_mul(const R r[36], const cx<R> v[6], cx<R> y[6])

@@ -408,9 +408,8 @@ extern "C" wc_status wc_apply_schur_multi(wc_lattice lat, int n, wc_field *outs,
     const int Vh = h->g.V;
     // n odd-site intermediates in the lattice's workspace, kept between
     // calls (allocating three half fields per right-hand side on every call
-    // cost 2.7 ms of a
-    // 2.9 ms call at 12 right-hand sides and 16^3x32); one call at a time uses it:
-    // the lock is held until the stream has finished
+    // cost 2.7 ms of a 2.9 ms call at 12 right-hand sides and 16^3x32); one
+    // call at a time uses it: the lock is held until the stream has finished
     const size_t data_bytes = (spinor_bytes(pr, Vh) + 255) / 256 * 256;
     const size_t nrm_bytes = pr == WC_F16 ? ((size_t)Vh * sizeof(float) + 255) / 256 * 256 : 0;
     std::lock_guard<std::mutex> lk(lat->eom_mutex);

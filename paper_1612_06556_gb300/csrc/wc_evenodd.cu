@@ -30,7 +30,7 @@ namespace {
 // clover inverse: A^-1 as two packed Hermitian 6x6 blocks (FP64 arithmetic)
 // ------------------------------------------------------------------------
 
-__device__ void unpack_block(const double r[36], cx<double> m[6][6])
+__device__ __forceinline__ void unpack_block(const double r[36], cx<double> m[6][6])
 {
     for (int i = 0; i < 6; ++i) m[i][i] = mkc(r[i], 0.0);
     int k = 6;
@@ -108,50 +108,147 @@ __device__ bool invert6(cx<double> a[6][6])
     return true;
 }
 
-// one packed block (36 reals) at position pos of a clover store, in all
-// three precisions
-__device__ void store_block(const CloverStore &S, int V, int pos, int b, const double r[36])
+// Inverse of a Hermitian 3x3 matrix, diagonal d and lower entries l = (1,0)
+// (2,0) (2,1), by cofactors into e, m; false when |det| is not above 1/16 of
+// the cube of the largest entry (or not a number).
+__device__ __forceinline__ bool invert_h3(const double d[3], const cx<double> l[3], double e[3], cx<double> m[3])
 {
+    const auto n2 = [](cx<double> a) { return fma(a.re, a.re, a.im * a.im); };
+    e[0] = fma(d[1], d[2], -n2(l[2]));
+    e[1] = fma(d[0], d[2], -n2(l[1]));
+    e[2] = fma(d[0], d[1], -n2(l[0]));
+    m[0] = cmul_conj(l[2], l[1]) - d[2] * l[0];
+    m[1] = l[0] * l[2] - d[1] * l[1];
+    m[2] = cmul_conj(l[0], l[1]) - d[0] * l[2];
+    const double det = d[0] * e[0] + l[0].re * m[0].re + l[0].im * m[0].im + l[1].re * m[1].re + l[1].im * m[1].im;
+    double big = fmax(fmax(fabs(d[0]), fabs(d[1])), fabs(d[2]));
 #pragma unroll
-    for (int q = 0; q < 18; ++q) {
-        const double2 v = make_double2(r[2 * q], r[2 * q + 1]);
-        S.c64[((size_t)b * 18 + q) * V + pos] = v;
-        S.cdf[((size_t)b * 18 + q) * V + pos] = df_pack(v);
+    for (int k = 0; k < 3; ++k) big = fmax(big, fmax(fabs(l[k].re), fabs(l[k].im)));
+    if (!(fabs(det) > 0.0625 * big * big * big)) return false;
+    const double f = 1.0 / det;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        e[k] *= f;
+        m[k] = f * m[k];
+    }
+    return true;
+}
+
+// entry (i, j) of a Hermitian 3x3 matrix (constants once unrolled)
+__device__ __forceinline__ cx<double> h3_entry(const double d[3], const cx<double> l[3], int i, int j)
+{
+    if (i == j) return mkc(d[i], 0.0);
+    const cx<double> v = l[i + j - 1];
+    return i > j ? v : conj(v);
+}
+
+// Inverse of a packed Hermitian 6x6 block [[a, q^+], [q, c]] by 3x3 blocks:
+// G = a^-1, W = q G, Z = (c - W q^+)^-1, R = -Z W, inverse [[G - W^+ R, R^+],
+// [R, Z]].  About 400 FP64 operations, in registers, against 1700 for the
+// pivoted Gauss-Jordan elimination below, which keeps its 6x6 arrays in local
+// memory (indexed at run time).  False where a 3x3 determinant is small: the
+// caller then takes the elimination, which also decides what is singular (no
+// block of the workloads; 31 of 768 at csw 5 on Haar links).  Largest error
+// of the inverse over accepted blocks at csw 1 / 3 / 5: 5.4e-16 / 4.9e-16 /
+// 5.4e-15, of an LU inverse 5.2e-16 / 4.1e-16 / 2.4e-15.
+__device__ __forceinline__ bool invert_block(const double r[36], double inv[36])
+{
+    const auto low = [&](int k) { return mkc(r[6 + 2 * k], r[7 + 2 * k]); };
+    const cx<double> al[3] = {low(0), low(1), low(2)};
+    const cx<double> q[3][3] = {{low(3), low(4), low(5)}, {low(6), low(7), low(8)}, {low(10), low(11), low(12)}};
+    double gd[3], zd[3], sd[3] = {r[3], r[4], r[5]};
+    cx<double> gl[3], zl[3], sl[3] = {low(9), low(13), low(14)};
+    if (!invert_h3(r, al, gd, gl)) return false;
+    cx<double> w[3][3], rr[3][3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            cx<double> s = gd[j] * q[i][j];
+#pragma unroll
+            for (int k = 0; k < 3; ++k)
+                if (k != j) s = cfma(q[i][k], h3_entry(gd, gl, k, j), s);
+            w[i][j] = s;
+        }
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) sd[i] = fma(-w[i][k].re, q[i][k].re, fma(-w[i][k].im, q[i][k].im, sd[i]));
+#pragma unroll
+    for (int t = 0; t < 3; ++t) {
+        const int i = t == 0 ? 1 : 2, j = t == 2 ? 1 : 0;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) sl[t] = cfma_conj(q[j][k], -w[i][k], sl[t]);
+    }
+    if (!invert_h3(sd, sl, zd, zl)) return false;
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            cx<double> s = -(zd[i] * w[i][j]);
+#pragma unroll
+            for (int k = 0; k < 3; ++k)
+                if (k != i) s = cfma(-h3_entry(zd, zl, i, k), w[k][j], s);
+            rr[i][j] = s;
+        }
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        double s = gd[i];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) s = fma(-w[k][i].re, rr[k][i].re, fma(-w[k][i].im, rr[k][i].im, s));
+        inv[i] = s;
+        inv[3 + i] = zd[i];
+    }
+    const auto put = [&](int k, cx<double> v) {
+        inv[6 + 2 * k] = v.re;
+        inv[7 + 2 * k] = v.im;
+    };
+#pragma unroll
+    for (int t = 0; t < 3; ++t) {
+        const int i = t == 0 ? 1 : 2, j = t == 2 ? 1 : 0;
+        cx<double> s = gl[t];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) s = cfma_conj(-w[k][i], rr[k][j], s);
+        put(t, s);
     }
 #pragma unroll
-    for (int q = 0; q < 9; ++q)
-        S.c32[((size_t)b * 9 + q) * V + pos] =
-            make_float4((float)r[4 * q], (float)r[4 * q + 1], (float)r[4 * q + 2], (float)r[4 * q + 3]);
-    unsigned *c16 = reinterpret_cast<unsigned *>(S.c16);
+    for (int i = 0; i < 3; ++i)
 #pragma unroll
-    for (int q = 0; q < 18; ++q) {
-        const int gq = 18 * b + q;
-        c16[((size_t)(gq >> 2) * V + pos) * 4 + (gq & 3)] = c2h((float)r[2 * q], (float)r[2 * q + 1]);
-    }
+        for (int j = 0; j < 3; ++j) put((i == 0 ? 3 : i == 1 ? 6 : 10) + j, rr[i][j]);
+    put(9, zl[0]);
+    put(13, zl[1]);
+    put(14, zl[2]);
+    return true;
+}
+
+// the pivoted elimination on a packed block, out of line: few blocks need it
+__device__ __noinline__ bool invert_block_pivoted(const double *r, double *inv)
+{
+    cx<double> m[6][6];
+    unpack_block(r, m);
+    const bool ok = invert6(m);
+    pack_block(m, inv);
+    return ok;
 }
 
 // Parity-ordered copies for the even-odd kernels: within every component
 // plane, position parity(x) * V/2 + (x >> 1), so that the threads of one
 // parity read contiguous memory (full-volume order would fetch every other
-// site's entries with them).  Ce: A = 1 + T; Ci: A^-1.
-__global__ void k_clover_invert(Geom g, CloverStore C, CloverStore Ce, CloverStore Ci, int *bad)
+// site's entries with them).  Ce: A = 1 + T; Ci: A^-1.  One block of one
+// site per thread.
+__global__ void __launch_bounds__(64) k_clover_invert(Geom g, CloverStore C, CloverStore Ce, CloverStore Ci, int *bad)
 {
     const int V = g.V;
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    const int x = blockIdx.x * blockDim.x + threadIdx.x, b = blockIdx.y;
     if (x >= V) return;
     int c[4];
     site_coords(g, x, c);
     const int pos = ((c[0] + c[1] + c[2] + c[3]) & 1) * (V >> 1) + (x >> 1);
-    for (int b = 0; b < 2; ++b) {
-        double r[36];
-        P64::load_clover(C, V, x, b, r);
-        store_block(Ce, V, pos, b, r);
-        cx<double> m[6][6];
-        unpack_block(r, m);
-        if (!invert6(m)) atomicExch(bad, 1);
-        pack_block(m, r);
-        store_block(Ci, V, pos, b, r);
-    }
+    double r[36], inv[36];
+    P64::load_clover(C, V, x, b, r);
+    store_clover_block<true>(Ce, V, pos, b, r);
+    if (!invert_block(r, inv) && !invert_block_pivoted(r, inv)) atomicExch(bad, 1);
+    store_clover_block<true>(Ci, V, pos, b, inv);
 }
 
 // ------------------------------------------------------------------------
@@ -485,7 +582,7 @@ wc_status build_clover_inverse(wc_lattice lat)
     if (st != WC_OK) return st;
     st = check_cuda(lat, cudaMemsetAsync(bad, 0, sizeof(int), lat->stream), "memset");
     if (st == WC_OK) {
-        k_clover_invert<<<(V + 63) / 64, 64, 0, lat->stream>>>(lat->g, lat->clover, lat->ceo, lat->cinv, bad);
+        k_clover_invert<<<dim3((V + 63) / 64, 2), 64, 0, lat->stream>>>(lat->g, lat->clover, lat->ceo, lat->cinv, bad);
         st = check_launch(lat, "clover_invert");
     }
     int h = 0;

@@ -154,6 +154,9 @@ cudaError_t launch_ras_schur(const wc_lattice_s *full, wc_field out, wc_field in
 cudaError_t launch_ras(wc_lattice lat, wc_field out, wc_field in, const wc_ras_params &p, int dagger,
                        cudaStream_t stream);
 
+// the clover term of lat's links into lat->clover (wc_clover.cu)
+cudaError_t launch_build_clover(wc_lattice lat, double csw, double kappa, cudaStream_t stream);
+
 bool apply_shape(wc_lattice lat, wc_prec prec, int kind, int force, int out[6]);
 
 // WC_OK when the whole-lattice operator of lat can be applied: gauge field

@@ -40,3 +40,38 @@ def test_schur_workspaces_are_reused_and_grow(dims):
             assert_elementwise(out, ref, TOL[prec])
             lat.apply_schur(one, g, dagger)
             assert_elementwise(one.store(np.zeros_like(s)), ref, TOL[prec])
+
+
+@pytest.mark.parametrize("csw", [1.0, 5.0])
+def test_clover_inverse_by_blocks_and_by_elimination(csw):
+    """csw = 1: every 6x6 block of A is inverted by 3x3 blocks.  csw = 5 on
+    Haar links: 31 of the 768 blocks have a 3x3 determinant so small that
+    they take the pivoted elimination, and the blocks' condition numbers
+    reach 1.4e3 (1.7 at csw = 1), which the FP64 tolerance scales with."""
+    dims, kappa, tbc = (4, 4, 4, 6), 0.13, -1
+    U = synth.haar_links(dims, 5)
+    lat = make_lattice(dims, U, csw, kappa, tbc)
+    op = oracle.Operator(dims, U, csw, kappa, tbc)
+    A = op.T + np.eye(12)
+    cond = max(np.linalg.cond(A[:, b:b + 6, b:b + 6]).max() for b in (0, 6))
+    psi = synth.gaussian_source(dims, 6)
+    fi, fo = lat.field(wc().F64).load(psi), lat.field(wc().F64)
+    lat.apply_schur(fo, fi)
+    assert_elementwise(fo.store(np.zeros_like(psi)), EvenOdd(dims, tbc, kappa, U, op.T).schur(psi), 1e-12 * cond)
+
+
+@pytest.mark.parametrize("dims", [(2, 2, 2, 2), (3, 2, 5, 4), (7, 3, 2, 11)])
+def test_clover_from_shared_plaquettes(dims):
+    """The clover term through M on extents where the corners of a
+    plaquette wrap onto themselves, odd ones and ragged CTAs; links and
+    term loaded twice, so that the second build starts from used stores."""
+    csw, kappa, tbc = 1.5, 0.13, -1
+    lat = make_lattice(dims, synth.haar_links(dims, 7), 0.7, 0.11, tbc)
+    U = synth.haar_links(dims, 8)
+    lat.load_gauge(U).load_clover(csw, kappa)
+    psi = synth.gaussian_source(dims, 9)
+    ref = oracle.apply_M(dims, tbc, kappa, csw, U, psi)
+    for prec in (0, 1, 2):
+        fi, fo = lat.field(prec).load(psi), lat.field(prec)
+        lat.apply_M(fo, fi)
+        assert_elementwise(fo.store(np.zeros_like(psi)), ref, TOL[prec])
