@@ -127,6 +127,44 @@ __global__ void __launch_bounds__(kApplyMaxThreads, MINB)
         apply_site<P, KIND>(g, tm, blk, U, C, in, in_nrm, out, out_nrm, kappa);
 }
 
+// The FP64 operator on four warps per 32 sites (hop_split64).  168 registers,
+// three CTAs per SM: three warps for each FP64 unit (four CTAs of 128
+// registers measured the same).
+template <int KIND>
+__global__ void __launch_bounds__(kSplit64 * kSplit64Sites, 3)
+    k_apply_split64(Geom g, GaugeStore U, CloverStore C, const void *in, void *out, double kappa)
+{
+    __shared__ Split64Mem sm;
+    const int s = threadIdx.x & (kSplit64Sites - 1), w = threadIdx.x / kSplit64Sites;
+    const int x = blockIdx.x * kSplit64Sites + s;
+    const bool valid = x < g.V;
+    if (valid) {
+        int c[4];
+        site_coords_fast(g, x, c);
+        hop_split64<KIND == 1 ? +1 : -1>(g, U, in, g.V, x, c, sm, w, s, [](int y) { return y; });
+    }
+    __syncthreads();
+    if (!valid) return;
+    cx<double> y[3];
+    if (KIND != 2) {
+        cx<double> v[6];
+        const double2 *p = static_cast<const double2 *>(in) + (size_t)(w >> 1) * 6 * g.V + x;
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+            const double2 a = __ldg(p + (size_t)k * g.V);
+            v[k] = mkc(a.x, a.y);
+        }
+        clover_rows64(C, g.V, x, w, v, y);
+    }
+    double2 *o = static_cast<double2 *>(out) + (size_t)3 * w * g.V + x;
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+        const cx<double> h = sum_split64(sm, 3 * w + r, s);
+        o[(size_t)r * g.V] = KIND == 2 ? make_double2(h.re, h.im)
+                                       : make_double2(fma(-kappa, h.re, y[r].re), fma(-kappa, h.im, y[r].im));
+    }
+}
+
 // ---- launch shapes and their autotuner ---------------------------------
 
 struct ApplyShape {
@@ -150,6 +188,12 @@ constexpr ApplyShape kShapes[] = {
     {32, {0, 0, 0, 0}, 0, 0}, {64, {0, 0, 0, 0}, 0, 0},
 };
 constexpr int kNumShapes = sizeof(kShapes) / sizeof(kShapes[0]);
+// What the FP64 operator takes unless a caller pins one of the shapes above:
+// it measured as fast as the best of them or faster on every lattice (4^4 13
+// against 39 us, 8^4 14 / 39, 12^4 49 / 60, 16^3x32 247 / 266, 24^3x32
+// 828 / 863, 17x19x21x23 299 / 331, 32^3x64 3960-4016 / 4014-4022), so
+// nothing is timed for it.
+constexpr int kShapeSplit64 = kNumShapes;
 
 // caps: bit c-1 set if register cap c is compiled for the operator (P::kCaps)
 bool shape_fits(const Geom &g, const ApplyShape &s, int caps)
@@ -173,10 +217,21 @@ int resident_ctas(K kernel, int threads)
     return n;
 }
 
-template <class P>
-cudaError_t launch_shape(wc_lattice lat, wc_field out, wc_field in, int kind, const ApplyShape &sh,
-                         cudaStream_t stream)
+cudaError_t launch_split64(wc_lattice lat, wc_field out, wc_field in, int kind, cudaStream_t stream)
 {
+    const Geom &g = lat->g;
+    const dim3 grid((g.V + kSplit64Sites - 1) / kSplit64Sites), block(kSplit64 * kSplit64Sites);
+    if (kind == 0) k_apply_split64<0><<<grid, block, 0, stream>>>(g, lat->gauge, lat->clover, in->data, out->data, lat->kappa);
+    else if (kind == 1) k_apply_split64<1><<<grid, block, 0, stream>>>(g, lat->gauge, lat->clover, in->data, out->data, lat->kappa);
+    else k_apply_split64<2><<<grid, block, 0, stream>>>(g, lat->gauge, lat->clover, in->data, out->data, lat->kappa);
+    return cudaGetLastError();
+}
+
+template <class P>
+cudaError_t launch_shape(wc_lattice lat, wc_field out, wc_field in, int kind, int index, cudaStream_t stream)
+{
+    if (index == kShapeSplit64) return launch_split64(lat, out, in, kind, stream);
+    const ApplyShape &sh = kShapes[index];
     const Geom &g = lat->g;
     TileMap tm{};
     int nlogical;
@@ -278,10 +333,10 @@ int tune_shape(wc_lattice lat, wc_field out, wc_field in, int kind, cudaStream_t
     for (int round = 0; round < 3; ++round) {
         for (int i = 0; i < kNumShapes; ++i) {
             if (!shape_fits(lat->g, kShapes[i], P::kCaps)) continue;
-            if (launch_shape<P>(lat, out, in, kind, kShapes[i], stream) != cudaSuccess) continue;
+            if (launch_shape<P>(lat, out, in, kind, i, stream) != cudaSuccess) continue;
             cudaEventRecord(e0, stream);
             for (int r = 0; r < 16; ++r)
-                launch_shape<P>(lat, outs[r % npair], ins[r % npair], kind, kShapes[i], stream);
+                launch_shape<P>(lat, outs[r % npair], ins[r % npair], kind, i, stream);
             cudaEventRecord(e1, stream);
             if (cudaEventSynchronize(e1) != cudaSuccess) continue;
             float ms = 0.f;
@@ -314,7 +369,11 @@ cudaError_t launch_apply_p(wc_lattice lat, wc_field out, wc_field in, int kind, 
         auto it = g_shape_choice.find(key);
         if (it != g_shape_choice.end()) choice = it->second;
     }
-    if (choice < 0) {
+    if (choice < 0 && std::is_same<P, P64>::value) {
+        choice = kShapeSplit64;
+        std::lock_guard<std::mutex> lk(g_shape_mutex);
+        g_shape_choice.emplace(key, choice);
+    } else if (choice < 0) {
         cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
         cudaStreamIsCapturing(stream, &cs);
         if (cs != cudaStreamCaptureStatusNone) {
@@ -325,7 +384,7 @@ cudaError_t launch_apply_p(wc_lattice lat, wc_field out, wc_field in, int kind, 
             g_shape_choice[key] = choice;
         }
     }
-    return launch_shape<P>(lat, out, in, kind, kShapes[choice], stream);
+    return launch_shape<P>(lat, out, in, kind, choice, stream);
 }
 
 // ------------------------------------------------------------------------
@@ -394,6 +453,12 @@ bool apply_shape(wc_lattice lat, wc_prec prec, int kind, int force, int out[6])
     }
     auto it = g_shape_choice.find(key);
     if (it == g_shape_choice.end()) return true;
+    if (it->second == kShapeSplit64) {
+        out[0] = kSplit64 * kSplit64Sites;
+        for (int m = 0; m < 4; ++m) out[1 + m] = 0;
+        out[5] = 64;
+        return true;
+    }
     const ApplyShape &s = kShapes[it->second];
     out[0] = s.threads;
     for (int m = 0; m < 4; ++m) out[1 + m] = s.tile[m];

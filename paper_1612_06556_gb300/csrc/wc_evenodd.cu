@@ -418,6 +418,96 @@ __global__ void __launch_bounds__(128, P::kEoMinBlocks) k_eo(Geom g, int p, Gaug
     }
 }
 
+// k_eo in FP64 on four warps per 32 sites (hop_split64): warp w finishes
+// components 3 w .. 3 w + 2; a product with A or A^-1 takes its vector from
+// shared memory.
+template <int DAG, int MODE>
+__global__ void __launch_bounds__(kSplit64 * kSplit64Sites, 3)
+    k_eo_split64(Geom g, int p, GaugeStore U, CloverStore C, CloverStore Ci, const void *hin, const double2 *vin,
+                 double2 *out, double2 *out2, double beta)
+{
+    __shared__ Split64Mem sm;
+    const int Vh = g.V >> 1;
+    const int s = threadIdx.x & (kSplit64Sites - 1), w = threadIdx.x / kSplit64Sites;
+    const int i = blockIdx.x * kSplit64Sites + s;
+    const bool valid = i < Vh;
+    if (MODE != 4 && valid) {
+        int c[4];
+        const int x = full_site(g, i, p, c);
+        hop_split64<DAG ? +1 : -1>(g, U, hin, Vh, x, c, sm, w, s, [](int y) { return y >> 1; });
+    }
+    __syncthreads();
+    cx<double> v[3], o[3], vb[6];
+    if (valid) {
+#pragma unroll
+        for (int r = 0; r < 3; ++r) {
+            const int k = 3 * w + r;
+            const cx<double> h = MODE == 4 ? mkc(0.0, 0.0) : sum_split64(sm, k, s);
+            if (MODE == 0) {
+                v[r] = h;
+            } else if (MODE == 1) {
+                v[r] = beta * h;
+            } else {
+                const double2 a = __ldg(vin + (size_t)k * Vh + i);
+                v[r] = MODE == 4 ? mkc(a.x, a.y) : mkc(fma(beta, h.re, a.x), fma(beta, h.im, a.y));
+            }
+        }
+    }
+    // every thread reads and writes column s, component k only in its own
+    // warp until the barrier
+    const auto share = [&](const cx<double> a[3]) {
+        if (valid)
+#pragma unroll
+            for (int r = 0; r < 3; ++r) sm[0][3 * w + r][s] = make_double2(a[r].re, a[r].im);
+        __syncthreads();
+        if (valid)
+#pragma unroll
+            for (int k = 0; k < 6; ++k) {
+                const double2 b = sm[0][(w >> 1) * 6 + k][s];
+                vb[k] = mkc(b.x, b.y);
+            }
+    };
+    const auto store = [&](double2 *f, const cx<double> a[3]) {
+#pragma unroll
+        for (int r = 0; r < 3; ++r) f[(size_t)(3 * w + r) * Vh + i] = make_double2(a[r].re, a[r].im);
+    };
+    if (MODE == 2) {
+        if (valid) store(out, v);
+        return;
+    }
+    const int pos = wc_idx(p * Vh + (valid ? i : 0), g.V);
+    if (MODE == 1) {
+        if (!valid) return;
+        const double2 *q = vin + (size_t)(w >> 1) * 6 * Vh + i;
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+            const double2 a = __ldg(q + (size_t)k * Vh);
+            vb[k] = mkc(a.x, a.y);
+        }
+        clover_rows64(C, g.V, pos, w, vb, o);
+#pragma unroll
+        for (int r = 0; r < 3; ++r) o[r] = o[r] + v[r];
+        store(out, o);
+        return;
+    }
+    share(v);
+    if (valid) {
+        clover_rows64(Ci, g.V, pos, w, vb, o);
+        store(out, o);
+    }
+    if (MODE == 5) {
+        __syncthreads();   // vb is read
+        share(o);
+        if (valid) {
+            cx<double> y[3];
+            clover_rows64(C, g.V, pos, w, vb, y);
+#pragma unroll
+            for (int r = 0; r < 3; ++r) y[r] = v[r] - y[r];
+            store(out2, y);
+        }
+    }
+}
+
 // full field <-> the two half fields (parity 0 = even, 1 = odd)
 template <class P>
 __global__ void k_split(Geom g, const void *full, const float *full_nrm, void *ev, float *ev_nrm, void *od,
@@ -455,6 +545,32 @@ __global__ void k_merge(Geom g, const void *ev, const float *ev_nrm, const void 
     P::store_spinor(full, full_nrm, g.V, full_site(g, i, 1, c), s);
 }
 
+template <int DAG>
+cudaError_t launch_eo_split64(const wc_lattice_s *full, int parity, int mode, const wc_field_s *hin,
+                              const wc_field_s *vin, wc_field_s *out, double beta, cudaStream_t stream,
+                              wc_field_s *out2)
+{
+    if (mode == 5 && (!out2 || out2->prec != WC_F64)) return cudaErrorInvalidValue;
+    const int Vh = full->g.V >> 1;
+    const dim3 grid((Vh + kSplit64Sites - 1) / kSplit64Sites), block(kSplit64 * kSplit64Sites);
+    const void *hd = hin ? hin->data : nullptr;
+    const double2 *vd = vin ? static_cast<const double2 *>(vin->data) : nullptr;
+    double2 *od = static_cast<double2 *>(out->data), *o2 = out2 ? static_cast<double2 *>(out2->data) : nullptr;
+#define WC_EO(M)                                                                                                 \
+    k_eo_split64<DAG, M><<<grid, block, 0, stream>>>(full->g, parity, full->gauge, full->ceo, full->cinv, hd, vd, \
+                                                     od, o2, beta)
+    switch (mode) {
+    case 0: WC_EO(0); break;
+    case 1: WC_EO(1); break;
+    case 2: WC_EO(2); break;
+    case 3: WC_EO(3); break;
+    case 4: WC_EO(4); break;
+    default: WC_EO(5);
+    }
+#undef WC_EO
+    return cudaGetLastError();
+}
+
 template <class P, int DAG>
 cudaError_t launch_eo_p(const wc_lattice_s *full, int parity, int mode, const wc_field_s *hin, const wc_field_s *vin,
                         wc_field_s *out, double beta, cudaStream_t stream, wc_field_s *out2)
@@ -479,7 +595,7 @@ cudaError_t launch_eo_p(const wc_lattice_s *full, int parity, int mode, const wc
     case 3: WC_EO(3); break;
     case 4: WC_EO(4); break;
     default:
-        if constexpr (std::is_same<P, P64>::value || std::is_same<P, PDF>::value) {
+        if constexpr (std::is_same<P, PDF>::value) {
             if (!out2 || out2->prec != WC_F64) return cudaErrorInvalidValue;
             WC_EO(5);
         } else {
@@ -501,8 +617,8 @@ cudaError_t launch_eo(const wc_lattice_s *full, int parity, int mode, int dagger
         return dagger ? launch_eo_p<PDF, 1>(full, parity, mode, hin, vin, out, beta, stream, out2)
                       : launch_eo_p<PDF, 0>(full, parity, mode, hin, vin, out, beta, stream, out2);
     if (pr == WC_F64)
-        return dagger ? launch_eo_p<P64, 1>(full, parity, mode, hin, vin, out, beta, stream, out2)
-                      : launch_eo_p<P64, 0>(full, parity, mode, hin, vin, out, beta, stream, out2);
+        return dagger ? launch_eo_split64<1>(full, parity, mode, hin, vin, out, beta, stream, out2)
+                      : launch_eo_split64<0>(full, parity, mode, hin, vin, out, beta, stream, out2);
     if (pr == WC_F32)
         return dagger ? launch_eo_p<P32, 1>(full, parity, mode, hin, vin, out, beta, stream, out2)
                       : launch_eo_p<P32, 0>(full, parity, mode, hin, vin, out, beta, stream, out2);

@@ -460,6 +460,177 @@ __device__ __forceinline__ void hop_dir_h16(const Geom &g, const GaugeStore &U, 
     }
 }
 
+// ---- FP64: the two hops of a direction together ------------------------
+// The FP64 pipe is what bounds the FP64 operators (each of its four units per
+// SM issues one warp instruction per 64 cycles), so what counts is the
+// number of FP64 instructions.  With w_f, w_b the link products of the
+// forward and the backward hop, the lower spins of both come from d = w_f -
+// w_b, whose sum runs on through both products, and the upper ones from
+// w_f + w_b = 2 w_f - d: 180 instructions a direction, the hopping
+// coefficient applied once to the sum of all four, against 236 for hops
+// taken one at a time with a coefficient each.
+
+// a with the sign bit flipped by mask (0 or 0x80000000): no FP64 instruction
+__device__ __forceinline__ double flip(double a, unsigned mask)
+{
+    return __hiloint2double((int)((unsigned)__double2hiint(a) ^ mask), __double2loint(a));
+}
+
+// i^Q a, the signs by flip: a negated value that is only stored would cost an
+// FP64 instruction
+template <int Q>
+__device__ __forceinline__ cx<double> times_iq(cx<double> a)
+{
+    constexpr unsigned m = 0x80000000u;
+    if (Q == 1) return mkc(flip(a.im, m), a.re);
+    if (Q == 2) return mkc(flip(a.re, m), flip(a.im, m));
+    if (Q == 3) return mkc(a.im, flip(a.re, m));
+    return a;
+}
+
+// t = the upper, lo = the lower spins (components 0..5 and 6..11) of
+// W_f (1 + SF g_MU) in(x+mu) + W_b (1 - SF g_MU) in(x-mu), the neighbour
+// spinors read at sidx(y) of a field of Vin sites
+template <int MU, int SF, class SiteIdx>
+__device__ __forceinline__ void hop_pair64(const Geom &g, const GaugeStore &U, const void *in, int Vin, int x,
+                                           const int c[4], cx<double> t[6], cx<double> lo[6], SiteIdx sidx)
+{
+    const int L = g.L[MU], st = g.stride[MU];
+    const bool wf = c[MU] == L - 1, wb = c[MU] == 0;
+    const int xf = wc_idx(wf ? x - (L - 1) * st : x + st, g.V), xb = wc_idx(wb ? x + (L - 1) * st : x - st, g.V);
+    cx<double> d[6];
+    {
+        cx<double> p[12], h[6], u[6], r2[3];
+        P64::load_spinor(in, nullptr, Vin, sidx(xf), p);
+        P64::load_link(U, g.V, MU, x, u, r2);
+        project<MU, SF>(p, h);
+        if (MU == 3) {
+            const unsigned m = wf && g.tbc < 0 ? 0x80000000u : 0u;
+#pragma unroll
+            for (int k = 0; k < 6; ++k) h[k] = mkc(flip(h[k].re, m), flip(h[k].im, m));
+        }
+#pragma unroll
+        for (int s = 0; s < 2; ++s)
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                const cx<double> *row = i == 2 ? r2 : u + 3 * i;
+                cx<double> y = row[0] * h[3 * s];
+                y = cfma(row[1], h[3 * s + 1], y);
+                t[3 * s + i] = cfma(row[2], h[3 * s + 2], y);
+            }
+    }
+    {
+        cx<double> p[12], h[6], u[6], r2[3];
+        P64::load_spinor(in, nullptr, Vin, sidx(xb), p);
+        P64::load_link(U, g.V, MU, xb, u, r2);
+        project<MU, -SF>(p, h);
+        if (MU == 3) {
+            const unsigned m = wb && g.tbc < 0 ? 0x80000000u : 0u;
+#pragma unroll
+            for (int k = 0; k < 6; ++k) h[k] = mkc(flip(h[k].re, m), flip(h[k].im, m));
+        }
+#pragma unroll
+        for (int s = 0; s < 2; ++s)
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                cx<double> y = cfma_conj(u[i], -h[3 * s], t[3 * s + i]);
+                y = cfma_conj(u[3 + i], -h[3 * s + 1], y);
+                d[3 * s + i] = cfma_conj(r2[i], -h[3 * s + 2], y);
+            }
+    }
+#pragma unroll
+    for (int k = 0; k < 6; ++k) t[k] = mkc(fma(2.0, t[k].re, -d[k].re), fma(2.0, t[k].im, -d[k].im));
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const cx<double> d0 = d[k], d1 = d[3 + k];
+        constexpr int P = SF > 0 ? 0 : 2, N = 2 - P;   // i^P = SF, i^N = -SF
+        if (MU == 0) {          // -SF i d1, -SF i d0
+            lo[k] = times_iq<(N + 1) & 3>(d1);
+            lo[3 + k] = times_iq<(N + 1) & 3>(d0);
+        } else if (MU == 1) {   // -SF d1, SF d0
+            lo[k] = times_iq<N>(d1);
+            lo[3 + k] = times_iq<P>(d0);
+        } else if (MU == 2) {   // -SF i d0, SF i d1
+            lo[k] = times_iq<(N + 1) & 3>(d0);
+            lo[3 + k] = times_iq<(P + 1) & 3>(d1);
+        } else {                // SF d0, SF d1
+            lo[k] = times_iq<P>(d0);
+            lo[3 + k] = times_iq<P>(d1);
+        }
+    }
+}
+
+// FP64 sites are split over the four warps of a CTA of 32 sites: warp w
+// takes direction w, puts its 12 components into shared memory and, after a
+// barrier, sums and finishes components 3 w .. 3 w + 2 (a warp lies on one of
+// the SM's four FP64 units: a site per thread left three of them idle on
+// lattices of a few thousand sites, and its last wave of CTAs a quarter
+// full at 16^3x32).
+constexpr int kSplit64 = 4;
+constexpr int kSplit64Sites = 32;
+using Split64Mem = double2[kSplit64][12][kSplit64Sites];
+
+template <int SF, class SiteIdx>
+__device__ __forceinline__ void hop_split64(const Geom &g, const GaugeStore &U, const void *in, int Vin, int x,
+                                            const int c[4], Split64Mem &sm, int w, int s, SiteIdx sidx)
+{
+    cx<double> t[6], lo[6];
+    if (w == 0) hop_pair64<0, SF>(g, U, in, Vin, x, c, t, lo, sidx);
+    else if (w == 1) hop_pair64<1, SF>(g, U, in, Vin, x, c, t, lo, sidx);
+    else if (w == 2) hop_pair64<2, SF>(g, U, in, Vin, x, c, t, lo, sidx);
+    else hop_pair64<3, SF>(g, U, in, Vin, x, c, t, lo, sidx);
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+        sm[w][k][s] = make_double2(t[k].re, t[k].im);
+        sm[w][6 + k][s] = make_double2(lo[k].re, lo[k].im);
+    }
+}
+
+// component k of the sum over the directions
+__device__ __forceinline__ cx<double> sum_split64(const Split64Mem &sm, int k, int s)
+{
+    const double2 a = sm[0][k][s], b = sm[1][k][s], c = sm[2][k][s], d = sm[3][k][s];
+    return mkc((a.x + b.x) + (c.x + d.x), (a.y + b.y) + (c.y + d.y));
+}
+
+// rows I0 .. I0 + 2 of y = B v, clover block b of the packed FP64 store at
+// position x
+template <int I0>
+__device__ __forceinline__ void clover_rows64_at(const CloverStore &C, int V, int x, int b, const cx<double> v[6],
+                                                 cx<double> y[3])
+{
+    const double2 *p = C.c64 + (size_t)b * 18 * V + x;
+    double d[3];
+    if (I0 == 0) {
+        const double2 a = __ldg(p), e = __ldg(p + (size_t)V);
+        d[0] = a.x, d[1] = a.y, d[2] = e.x;
+    } else {
+        const double2 a = __ldg(p + (size_t)V), e = __ldg(p + (size_t)2 * V);
+        d[0] = a.y, d[1] = e.x, d[2] = e.y;
+    }
+#pragma unroll
+    for (int r = 0; r < 3; ++r) y[r] = d[r] * v[I0 + r];
+#pragma unroll
+    for (int i = 1; i < 6; ++i)
+#pragma unroll
+        for (int j = 0; j < i; ++j) {
+            const bool row = i >= I0 && i < I0 + 3, col = j >= I0 && j < I0 + 3;
+            if (!row && !col) continue;
+            const double2 e = __ldg(p + (size_t)(3 + i * (i - 1) / 2 + j) * V);
+            const cx<double> l = mkc(e.x, e.y);
+            if (row) y[i - I0] = cfma(l, v[j], y[i - I0]);
+            if (col) y[j - I0] = cfma_conj(l, v[i], y[j - I0]);
+        }
+}
+
+// rows 3 w .. 3 w + 2 of the 12 (w uniform in the warp)
+__device__ __forceinline__ void clover_rows64(const CloverStore &C, int V, int x, int w, const cx<double> v[6],
+                                              cx<double> y[3])
+{
+    if (w & 1) clover_rows64_at<3>(C, V, x, w >> 1, v, y);
+    else clover_rows64_at<0>(C, V, x, w >> 1, v, y);
+}
+
 // One site: out(x) = M in, M^+ in or H in (KIND 0, 1, 2) for the site of
 // this thread in logical block blk.
 template <class P, int KIND>

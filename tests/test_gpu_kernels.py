@@ -75,3 +75,28 @@ def test_clover_from_shared_plaquettes(dims):
         fi, fo = lat.field(prec).load(psi), lat.field(prec)
         lat.apply_M(fo, fi)
         assert_elementwise(fo.store(np.zeros_like(psi)), ref, TOL[prec])
+
+
+@pytest.mark.parametrize("dims,tbc", [((2, 2, 2, 2), -1), ((3, 5, 2, 7), 1), ((5, 3, 7, 4), -1), ((8, 4, 4, 4), -1)])
+def test_fp64_operator_with_directions_on_four_warps(dims, tbc):
+    """M, M^+ and H in FP64 with no shape pinned: volumes of half a CTA of 32
+    sites, ragged ones and a whole number of CTAs, both time boundaries; and
+    the same as the shapes that take a site per thread."""
+    csw, kappa = 1.2, 0.13
+    U = synth.haar_links(dims, 60 + sum(dims))
+    lat = make_lattice(dims, U, csw, kappa, tbc)
+    op = oracle.Operator(dims, U, csw, kappa, tbc)
+    psi = synth.gaussian_source(dims, 61)
+    F64 = wc().F64
+    fi, fo = lat.field(F64).load(psi), lat.field(F64)
+    ref = {"M": op.M(psi), "Mdag": op.Mdag(psi), "hop": oracle.apply_hop(dims, tbc, U, psi)}
+    outs = {}
+    for kind, name in enumerate(ref):
+        getattr(lat, "apply_" + name)(fo, fi)
+        assert lat.apply_shape(F64, kind)[2] == 64
+        outs[name] = fo.store(np.zeros_like(psi))
+        assert_elementwise(outs[name], ref[name], 1e-12)
+    for kind, name in enumerate(ref):
+        lat.apply_shape(F64, kind, force=22)
+        getattr(lat, "apply_" + name)(fo, fi)
+        assert_elementwise(fo.store(np.zeros_like(psi)), outs[name], 1e-14)
