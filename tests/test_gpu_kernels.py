@@ -100,3 +100,36 @@ def test_fp64_operator_with_directions_on_four_warps(dims, tbc):
         lat.apply_shape(F64, kind, force=22)
         getattr(lat, "apply_" + name)(fo, fi)
         assert_elementwise(fo.store(np.zeros_like(psi)), outs[name], 1e-14)
+
+
+@pytest.mark.parametrize("dims", [(2, 2, 2, 2), (3, 3, 5, 2), (4, 4, 4, 2), (5, 3, 3, 3), (6, 7, 5, 9)])
+@pytest.mark.parametrize("prec", [0, 1, 2])
+@pytest.mark.parametrize("offset", [0, 1])
+def test_transfers_turn_rows_round_at_ragged_sizes(dims, prec, offset):
+    """Import and export of complex64 and complex128 tensors at volumes below,
+    at and above the 128 sites of a CTA; offset 1 starts the complex64 rows
+    8 bytes off a 16-byte boundary.  FP64 round trips are exact, FP32 ones
+    round once, binary16 components lie within 2^-11 of the site's largest."""
+    import torch
+    V = int(np.prod(dims))
+    lat = wc().Lattice(dims)
+    ref = torch.from_numpy(synth.gaussian_source(dims, 77))
+    for dtype in (torch.complex64, torch.complex128):
+        store = torch.zeros(V * 12 + 1 + 8, dtype=dtype, device="cuda")
+        src = store[offset:offset + V * 12].view(V, 4, 3)
+        src.copy_(ref)
+        f = lat.field(prec).load(src)
+        store2 = torch.full((V * 12 + 1 + 8,), 7.0, dtype=dtype, device="cuda")
+        f.store(store2[offset:offset + V * 12].view(V, 4, 3))
+        out = store2.cpu()
+        assert (out[:offset] == 7).all() and (out[offset + V * 12:] == 7).all()
+        got = out[offset:offset + V * 12].view(V, 4, 3)
+        want = ref.to(dtype)
+        if prec == 0 or (prec == 1 and dtype == torch.complex64):
+            assert torch.equal(got, want)
+        elif prec == 1:
+            assert torch.equal(got, ref.to(torch.complex64).to(dtype))
+        else:
+            r, w = torch.view_as_real(got.to(torch.complex128)), torch.view_as_real(want.to(torch.complex128))
+            big = w.abs().amax(dim=(1, 2, 3), keepdim=True)
+            assert ((r - w).abs() <= 2.0 ** -11 * big * (1 + 1e-5)).all()
