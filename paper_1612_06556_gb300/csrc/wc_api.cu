@@ -276,7 +276,11 @@ wc_status require_operator(wc_lattice lat, bool need_clover)
 
 wc_status state_init(wc_lattice lat, SolverState &s)
 {
-    const int max_blocks = 8 * sm_count();
+    // four blocks of 256 per SM: the last block adds one partial per block
+    // and sum, so more blocks lengthen its tail and fewer leave the loads of
+    // the vectors uncovered (lo_alpha at 16^3x32 10.0 / 7.7 / 8.1 / 8.2 us,
+    // lo_xr 12.1 / 11.5 / 12.9 / 13.2 us with 8 / 4 / 3 / 2 per SM)
+    const int max_blocks = 4 * sm_count();
     s.red.max_blocks = max_blocks;
     wc_status st = check_cuda(lat, dalloc(&s.red.partials, sizeof(double) * 8 * max_blocks), "cudaMalloc");
     if (st == WC_OK) st = check_cuda(lat, dalloc(&s.red.ticket, sizeof(unsigned)), "cudaMalloc");

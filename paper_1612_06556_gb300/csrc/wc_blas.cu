@@ -2,10 +2,21 @@
 // per-iteration vector updates of BiCGStab, each one pass over its fields.
 //
 // Reductions are deterministic: every block reduces its grid-stride share
-// (warp shuffles, then one warp over the block's warps), writes one partial,
-// and the last block to finish (completion ticket) adds the partials in
-// block order and runs the scalar update of the solver in one thread.  The
-// ticket resets itself, so no memset is needed between launches.
+// (warp shuffles, then one warp over the block's warps), writes one partial
+// per sum, and the last block to finish (completion ticket) adds the
+// partials in a fixed order and runs the scalar update of the solver in one
+// warp.  The ticket resets itself, so no memset is needed between launches.
+//
+// The tail of such a kernel -- from a block's own sums to the solver's scalar
+// -- is a chain of FP64 instructions, each of which occupies one of GB300's
+// FP64 units for 64 cycles per warp whatever the number of active lanes.  So
+// lanes share the work: N sums are reduced together (half of the lanes take
+// over half of the sums at each of the first shuffle steps: 6 adds for four
+// sums instead of 20), the final warps take one sum each, and the quotients
+// of a scalar update are formed in different lanes by the same instructions.
+// Against a shuffle tree per sum and one thread for the scalars: FP64 x, r
+// update at 8^4 13.9 -> 8.8 us, omega 10.3 -> 6.9, FP32 omega at 16^3x32 14.6
+// -> 8.4, |b|^2 at 24^3x32 61 -> 23 (no imaginary part).
 #include <math.h>
 
 #include <algorithm>
@@ -19,84 +30,104 @@ namespace {
 
 constexpr int kRedBlock = 256;
 
-__device__ __forceinline__ double warp_sum(double v)
+// Sums of v[0..N) over the lanes, N = 1, 2 or 4: lane l returns the sum of
+// v[l / (32 / N)].
+template <int N, class T>
+__device__ __forceinline__ T warp_sums(T (&v)[N])
 {
+    static_assert(N == 1 || N == 2 || N == 4, "one, two or four sums");
+    const int lane = threadIdx.x & 31;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    return v;
+    for (int half = N / 2, o = 16; half > 0; half /= 2, o /= 2) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int i = 0; i < half; ++i) {
+            const T give = up ? v[i] : v[half + i], keep = up ? v[half + i] : v[i];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+        }
+    }
+#pragma unroll
+    for (int o = 16 / N; o > 0; o /= 2) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+    return v[0];
 }
+
+constexpr int kRedWarps = kRedBlock / 32;
+
+// Sum i over w[.][k] where warp k of the block has put its sums (lane i * 8 +
+// k of the calling warp reads it): every lane of i * 8 .. i * 8 + 7.
+template <int N, class T>
+__device__ __forceinline__ T block_sums(const T (&w)[N][kRedWarps])
+{
+    static_assert(kRedWarps == 8, "eight warps");
+    const int lane = threadIdx.x & 31;
+    T u = lane < N * 8 ? w[lane >> 3][lane & 7] : T(0);
+#pragma unroll
+    for (int o = 4; o > 0; o /= 2) u += __shfl_xor_sync(0xffffffffu, u, o);
+    return u;
+}
+
+struct NoUpdate {
+    __device__ void operator()(double, const double *) const {}
+};
+struct NoAhead {
+    __device__ double operator()() const { return 0.0; }
+};
 
 }  // namespace
 
-// Last block of a grid reduction: every thread adds the partials of blocks
-// t, t + blockDim, ... (independent loads, unrolled), then the block sums
-// the thread totals by warp shuffles and one warp over the warp totals --
-// a fixed order, so the result is the same on every run.  (One warp
-// walking all partials serialises ~gridDim/32 L2 round trips per value,
-// 15-20 us per reduction kernel at 8 blocks per SM.)  sm: >= 32 * N
-// doubles of shared scratch.  Resets the ticket.
-template <int N>
-__device__ __forceinline__ void final_sum(const ReduceScratch &rs, double *out, double *sm)
+// Reduce v[0..M) over the grid (blocks of kRedBlock threads, one dimension x).
+// The last block to arrive leaves the grid sums in out[0..M), summed in a
+// fixed order, and its warp 0 calls post(t, extra) with sum i in lane i
+// (zero above).  ahead() runs meanwhile in the last warp of that block;
+// extra[l] is what lane l of it returned.
+template <int M, class T, class Post = NoUpdate, class Ahead = NoAhead>
+__device__ __forceinline__ void grid_reduce(T (&acc)[M], const ReduceScratch &rs, double *out, Post post = Post(),
+                                            Ahead ahead = Ahead())
 {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    double t[N];
-#pragma unroll
-    for (int i = 0; i < N; ++i) t[i] = 0.0;
-#pragma unroll 4
-    for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x)
-#pragma unroll
-        for (int i = 0; i < N; ++i) t[i] += __ldcg(rs.partials + (size_t)b * 8 + i);
-#pragma unroll
-    for (int i = 0; i < N; ++i) t[i] = warp_sum(t[i]);
-    __syncthreads();   // sm may still be read by the first stage
-    if (lane == 0)
-#pragma unroll
-        for (int i = 0; i < N; ++i) sm[wid * N + i] = t[i];
-    __syncthreads();
-    if (wid == 0) {
-#pragma unroll
-        for (int i = 0; i < N; ++i) {
-            double u = lane < nw ? sm[lane * N + i] : 0.0;
-            u = warp_sum(u);
-            if (lane == 0) out[i] = u;
-        }
-        if (lane == 0) *rs.ticket = 0u;
-    }
-    __syncthreads();   // out[] is read by thread 0 after return
-}
-
-// Reduce v[0..N) over the grid.  Returns true in thread 0 of the last block,
-// after out[0..N) holds the grid totals (summed in a fixed order).
-template <int N>
-__device__ __forceinline__ bool grid_reduce(double (&v)[N], const ReduceScratch &rs, double *out)
-{
-    __shared__ double sm[32][N];
+    constexpr int N = M == 3 ? 4 : M;
+    __shared__ T sm[N][kRedWarps];
+    __shared__ double fin[kRedWarps], extra[32];
     __shared__ bool last;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    T v[N];
 #pragma unroll
-    for (int i = 0; i < N; ++i) v[i] = warp_sum(v[i]);
-    if (lane == 0)
-#pragma unroll
-        for (int i = 0; i < N; ++i) sm[wid][i] = v[i];
+    for (int i = 0; i < N; ++i) v[i] = i < M ? acc[i] : T(0);
+    const T t = warp_sums(v);
+    if (lane % (32 / N) == 0) sm[lane / (32 / N)][wid] = t;
     __syncthreads();
     if (wid == 0) {
-#pragma unroll
-        for (int i = 0; i < N; ++i) {
-            double s = lane < nw ? sm[lane][i] : 0.0;
-            s = warp_sum(s);
-            if (lane == 0) rs.partials[(size_t)blockIdx.x * 8 + i] = s;
+        const T u = block_sums(sm);
+        if (lane < N * 8 && (lane & 7) == 0) {
+            rs.partials[(size_t)blockIdx.x * 8 + (lane >> 3)] = (double)u;
+            __threadfence();
         }
-    }
-    if (threadIdx.x == 0) {
-        __threadfence();
-        const unsigned t = atomicAdd(rs.ticket, 1u);
-        last = (t == gridDim.x - 1);
+        __syncwarp();
+        if (lane == 0) last = atomicAdd(rs.ticket, 1u) == gridDim.x - 1;
     }
     __syncthreads();
-    if (!last) return false;
+    if (!last) return;
     __threadfence();
-    final_sum<N>(rs, out, &sm[0][0]);
-    return threadIdx.x == 0;
+    // warp w adds the partials of sum w % N
+    double s = 0.0;
+    const int i = wid % N;
+    if (i < M) {
+#pragma unroll 4
+        for (int b = (wid / N) * 32 + lane; b < (int)gridDim.x; b += kRedBlock / N)
+            s += __ldcg(rs.partials + (size_t)b * 8 + i);
+        double one[1] = {s};
+        s = warp_sums(one);
+    }
+    if (lane == 0) fin[wid] = s;
+    if (wid == kRedWarps - 1) extra[lane] = ahead();
+    __syncthreads();
+    if (wid != 0) return;
+    double u = lane < kRedWarps ? fin[lane] : 0.0;
+#pragma unroll
+    for (int o = N; o < kRedWarps; o *= 2) u += __shfl_xor_sync(0xffffffffu, u, o);
+    if (lane >= M) u = 0.0;
+    if (lane < M) out[lane] = u;
+    if (lane == 0) *rs.ticket = 0u;
+    post(u, extra);
 }
 
 int reduce_grid(const ReduceScratch &rs, long long n)
@@ -112,6 +143,25 @@ namespace {
 // ------------------------------------------------------------------------
 // generic (any precision, per site) dot / norm / axpy for the C ABI
 // ------------------------------------------------------------------------
+
+// |a|^2: half of the products of <a, a>, and no imaginary part
+template <class P>
+__global__ void __launch_bounds__(kRedBlock) k_norm2(int V, const void *a, const float *an, ReduceScratch rs)
+{
+    double v[1] = {0.0};
+    for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < V; x += gridDim.x * blockDim.x) {
+        cx<typename P::real> s[12];
+        P::load_spinor(a, an, V, x, s);
+        double w = 0.0;
+#pragma unroll
+        for (int k = 0; k < 12; ++k) {
+            const double re = s[k].re, im = s[k].im;
+            w = fma(re, re, fma(im, im, w));
+        }
+        v[0] += w;
+    }
+    grid_reduce<1>(v, rs, rs.result);
+}
 
 template <class PA, class PB>
 __global__ void __launch_bounds__(kRedBlock) k_dot(int V, const void *a, const float *an, const void *b,
@@ -203,10 +253,13 @@ wc_status reduce_dot(wc_lattice lat, wc_field a, wc_field b, double out[2])
 
 wc_status reduce_norm2(wc_lattice lat, wc_field a, double *out)
 {
-    double d[2];
-    wc_status st = reduce_dot(lat, a, a, d);
-    if (st == WC_OK) *out = d[0];
-    return st;
+    const int V = lat->g.V;
+    const int grid = reduce_grid(lat->st.red, V);
+    if (a->prec == WC_F64) k_norm2<P64><<<grid, kRedBlock, 0, lat->stream>>>(V, a->data, a->nrm, lat->st.red);
+    else if (a->prec == WC_F32) k_norm2<P32><<<grid, kRedBlock, 0, lat->stream>>>(V, a->data, a->nrm, lat->st.red);
+    else k_norm2<P16><<<grid, kRedBlock, 0, lat->stream>>>(V, a->data, a->nrm, lat->st.red);
+    wc_status st = check_launch(lat, "norm2");
+    return st == WC_OK ? fetch_result(lat, 1, out) : st;
 }
 
 wc_status axpy_norm(wc_lattice lat, const double a[2], wc_field x, wc_field y, double *norm2)
@@ -247,13 +300,91 @@ __device__ __forceinline__ cx<double> ld(const double2 *p, long long i)
 }
 __device__ __forceinline__ void st(double2 *p, long long i, cx<double> a) { p[i] = make_double2(a.re, a.im); }
 __device__ __forceinline__ cx<double> c_of(double2 a) { return {a.x, a.y}; }
-__device__ __forceinline__ double2 d2_of(cx<double> a) { return make_double2(a.re, a.im); }
-__device__ __forceinline__ cx<double> cdiv(cx<double> a, cx<double> b)
+
+// ---- scalar updates, run by one warp -------------------------------------
+// t: sum i of the reduction in lane i.
+
+__device__ __forceinline__ double sum_of(double t, int i) { return __shfl_sync(0xffffffffu, t, i); }
+
+// a / b, the real part in even lanes, the imaginary part in odd ones
+__device__ __forceinline__ double cdiv_part(cx<double> a, cx<double> b)
 {
+    const bool im = threadIdx.x & 1;
     const double d = b.re * b.re + b.im * b.im;
-    return {(a.re * b.re + a.im * b.im) / d, (a.im * b.re - a.re * b.im) / d};
+    const double p = im ? a.im : a.re, q = im ? -a.re : a.im;
+    return (p * b.re + q * b.im) / d;
 }
-__device__ __forceinline__ bool finite2(cx<double> a) { return isfinite(a.re) && isfinite(a.im); }
+
+__device__ __forceinline__ void init_update(double t, SolverScalars *sc)
+{
+    if ((threadIdx.x & 31) != 0) return;
+    const double rr = t;
+    sc->rr = rr;
+    sc->rho = make_double2(rr, 0.0);   // <rhat, r> with rhat = r
+    sc->rho0 = make_double2(1.0, 0.0);
+    sc->alpha = make_double2(1.0, 0.0);
+    sc->omega = make_double2(1.0, 0.0);
+    sc->beta = make_double2(rr, 0.0);  // (rho/rho0)(alpha/omega)
+    sc->flags = isfinite(rr) ? 0 : FLAG_NAN;
+    if (rr == 0.0) sc->flags |= FLAG_BREAKDOWN;
+}
+
+// alpha = rho / <rhat, v>
+__device__ __forceinline__ void alpha_update(double t, SolverScalars *sc)
+{
+    const int lane = threadIdx.x & 31;
+    const cx<double> rv = mkc(sum_of(t, 0), sum_of(t, 1));
+    const double a = cdiv_part(c_of(sc->rho), rv);
+    const bool zero = rv.re == 0.0 && rv.im == 0.0;
+    if (lane < 2) (&sc->alpha.x)[lane] = zero ? 0.0 : a;
+    if (lane == 0) {
+        if (!isfinite(rv.re) || !isfinite(rv.im)) sc->flags |= FLAG_NAN;
+        if (zero) sc->flags |= FLAG_BREAKDOWN;
+    }
+}
+
+// omega = <t, s> / <t, t>
+__device__ __forceinline__ void omega_update(double t, SolverScalars *sc)
+{
+    const int lane = threadIdx.x & 31;
+    const double tt = sum_of(t, 2);
+    const bool bad = !isfinite(tt) || !isfinite(sum_of(t, 0)) || !isfinite(sum_of(t, 1));
+    const double om = t / tt;
+    if (lane < 2) (&sc->omega.x)[lane] = tt > 0.0 ? om : 0.0;
+    if (lane == 0) {
+        sc->tt = tt;
+        if (bad) sc->flags |= FLAG_NAN;
+    }
+}
+
+// alpha / omega in lanes 0, 1 and 1 / rho in lanes 2, 3, while the sums of
+// the x, r update are added
+__device__ __forceinline__ double xr_ahead(const SolverScalars *sc)
+{
+    const bool second = threadIdx.x & 2;
+    return cdiv_part(second ? mkc(1.0, 0.0) : c_of(sc->alpha), second ? c_of(sc->rho) : c_of(sc->omega));
+}
+
+// rho' = <rhat, r>, rr = |r|^2, beta = (rho'/rho)(alpha/omega), rho0 = rho,
+// rho = rho'; e: what xr_ahead returned
+__device__ __forceinline__ void xr_update(double t, const double *e, SolverScalars *sc)
+{
+    const cx<double> rho_new = mkc(sum_of(t, 0), sum_of(t, 1));
+    const double rr = sum_of(t, 2);
+    if ((threadIdx.x & 31) != 0) return;
+    const cx<double> rho = c_of(sc->rho), om = c_of(sc->omega);
+    sc->rr = rr;
+    if (!isfinite(rr) || !isfinite(rho_new.re) || !isfinite(rho_new.im)) sc->flags |= FLAG_NAN;
+    if ((om.re == 0.0 && om.im == 0.0) || (rho.re == 0.0 && rho.im == 0.0)) {
+        sc->flags |= FLAG_BREAKDOWN;
+    } else {
+        const cx<double> b = (rho_new * mkc(e[2], e[3])) * mkc(e[0], e[1]);
+        sc->beta = make_double2(b.re, b.im);
+    }
+    if (rho_new.re == 0.0 && rho_new.im == 0.0 && rr > 0.0) sc->flags |= FLAG_BREAKDOWN;
+    sc->rho0 = sc->rho;
+    sc->rho = make_double2(rho_new.re, rho_new.im);
+}
 
 // result[0] = |a|^2 (FP64 field as a flat array)
 __global__ void __launch_bounds__(kRedBlock) k_norm2_flat(long long n, const double2 *a, ReduceScratch rs)
@@ -282,20 +413,13 @@ __global__ void __launch_bounds__(kRedBlock) k_bicg_init(long long n, const doub
         v[i] = make_double2(0.0, 0.0);
         acc[0] += ri.re * ri.re + ri.im * ri.im;
     }
-    if (grid_reduce<1>(acc, rs, rs.result)) {
-        const double rr = rs.result[0];
-        sc->rr = rr;
-        sc->rho = make_double2(rr, 0.0);   // <rhat, r> with rhat = r
-        sc->rho0 = make_double2(1.0, 0.0);
-        sc->alpha = make_double2(1.0, 0.0);
-        sc->omega = make_double2(1.0, 0.0);
-        sc->beta = make_double2(rr, 0.0);  // (rho/rho0)(alpha/omega)
-        sc->flags = isfinite(rr) ? 0 : FLAG_NAN;
-        if (rr == 0.0) sc->flags |= FLAG_BREAKDOWN;
-    }
+    grid_reduce<1>(acc, rs, rs.result, [=](double t, const double *) { init_update(t, sc); });
 }
 
-// p = r + beta (p - omega v);  pp = |p|^2
+// p = r + beta (p - omega v);  with NORM pp = |p|^2 (the scale of the defect
+// correction; without a preconditioner nothing reads it, and a value that is
+// not finite shows in the sums of the next kernels)
+template <bool NORM>
 __global__ void __launch_bounds__(kRedBlock) k_bicg_p(long long n, const double2 *r, const double2 *v, double2 *p,
                                                       ReduceScratch rs, SolverScalars *sc)
 {
@@ -305,12 +429,14 @@ __global__ void __launch_bounds__(kRedBlock) k_bicg_p(long long n, const double2
          i += (long long)gridDim.x * blockDim.x) {
         const cx<double> pi = ld(r, i) + beta * (ld(p, i) - omega * ld(v, i));
         st(p, i, pi);
-        acc[0] += pi.re * pi.re + pi.im * pi.im;
+        if (NORM) acc[0] += pi.re * pi.re + pi.im * pi.im;
     }
-    if (grid_reduce<1>(acc, rs, rs.result)) {
-        sc->pp = rs.result[0];
-        if (!isfinite(sc->pp)) sc->flags |= FLAG_NAN;
-    }
+    if (NORM)
+        grid_reduce<1>(acc, rs, rs.result, [=](double t, const double *) {
+            if ((threadIdx.x & 31) != 0) return;
+            sc->pp = t;
+            if (!isfinite(t)) sc->flags |= FLAG_NAN;
+        });
 }
 
 // alpha = rho / <rhat, v>
@@ -324,19 +450,11 @@ __global__ void __launch_bounds__(kRedBlock) k_bicg_alpha(long long n, const dou
         acc[0] += a.re * b.re + a.im * b.im;
         acc[1] += a.re * b.im - a.im * b.re;
     }
-    if (grid_reduce<2>(acc, rs, rs.result)) {
-        const cx<double> rv = mkc(rs.result[0], rs.result[1]);
-        if (!finite2(rv)) sc->flags |= FLAG_NAN;
-        if (rv.re == 0.0 && rv.im == 0.0) {
-            sc->flags |= FLAG_BREAKDOWN;
-            sc->alpha = make_double2(0.0, 0.0);
-        } else {
-            sc->alpha = d2_of(cdiv(c_of(sc->rho), rv));
-        }
-    }
+    grid_reduce<2>(acc, rs, rs.result, [=](double t, const double *) { alpha_update(t, sc); });
 }
 
-// s = r - alpha v;  ss = |s|^2
+// s = r - alpha v;  with NORM ss = |s|^2 (as pp above)
+template <bool NORM>
 __global__ void __launch_bounds__(kRedBlock) k_bicg_s(long long n, const double2 *r, const double2 *v, double2 *s,
                                                       ReduceScratch rs, SolverScalars *sc)
 {
@@ -346,12 +464,14 @@ __global__ void __launch_bounds__(kRedBlock) k_bicg_s(long long n, const double2
          i += (long long)gridDim.x * blockDim.x) {
         const cx<double> si = ld(r, i) - alpha * ld(v, i);
         st(s, i, si);
-        acc[0] += si.re * si.re + si.im * si.im;
+        if (NORM) acc[0] += si.re * si.re + si.im * si.im;
     }
-    if (grid_reduce<1>(acc, rs, rs.result)) {
-        sc->ss = rs.result[0];
-        if (!isfinite(sc->ss)) sc->flags |= FLAG_NAN;
-    }
+    if (NORM)
+        grid_reduce<1>(acc, rs, rs.result, [=](double t, const double *) {
+            if ((threadIdx.x & 31) != 0) return;
+            sc->ss = t;
+            if (!isfinite(t)) sc->flags |= FLAG_NAN;
+        });
 }
 
 // omega = <t, s> / <t, t>
@@ -366,15 +486,7 @@ __global__ void __launch_bounds__(kRedBlock) k_bicg_omega(long long n, const dou
         acc[1] += a.re * b.im - a.im * b.re;
         acc[2] += a.re * a.re + a.im * a.im;
     }
-    if (grid_reduce<3>(acc, rs, rs.result)) {
-        const double tt = rs.result[2];
-        sc->tt = tt;
-        if (!isfinite(tt) || !isfinite(rs.result[0]) || !isfinite(rs.result[1])) sc->flags |= FLAG_NAN;
-        if (tt > 0.0)
-            sc->omega = make_double2(rs.result[0] / tt, rs.result[1] / tt);
-        else
-            sc->omega = make_double2(0.0, 0.0);
-    }
+    grid_reduce<3>(acc, rs, rs.result, [=](double t, const double *) { omega_update(t, sc); });
 }
 
 // x += alpha phat + omega shat;  r = s - omega t;  rho' = <rhat, r>, rr = |r|^2,
@@ -399,20 +511,8 @@ __global__ void __launch_bounds__(kRedBlock) k_bicg_xr(long long n, double2 *x, 
         acc[1] += h.re * ri.im - h.im * ri.re;
         acc[2] += ri.re * ri.re + ri.im * ri.im;
     }
-    if (grid_reduce<3>(acc, rs, rs.result)) {
-        const cx<double> rho_new = mkc(rs.result[0], rs.result[1]);
-        const cx<double> rho = c_of(sc->rho);
-        sc->rr = rs.result[2];
-        if (!isfinite(sc->rr) || !finite2(rho_new)) sc->flags |= FLAG_NAN;
-        if ((omega.re == 0.0 && omega.im == 0.0) || (rho.re == 0.0 && rho.im == 0.0)) {
-            sc->flags |= FLAG_BREAKDOWN;
-        } else {
-            sc->beta = d2_of(cdiv(rho_new, rho) * cdiv(alpha, omega));
-        }
-        if (rho_new.re == 0.0 && rho_new.im == 0.0 && sc->rr > 0.0) sc->flags |= FLAG_BREAKDOWN;
-        sc->rho0 = sc->rho;
-        sc->rho = d2_of(rho_new);
-    }
+    grid_reduce<3>(acc, rs, rs.result, [=](double t, const double *e) { xr_update(t, e, sc); },
+                   [=] { return xr_ahead(sc); });
 }
 
 // r = b - r (r holds M x);  rr = |r|^2  (true residual)
@@ -426,7 +526,9 @@ __global__ void __launch_bounds__(kRedBlock) k_residual(long long n, const doubl
         st(r, i, ri);
         acc[0] += ri.re * ri.re + ri.im * ri.im;
     }
-    if (grid_reduce<1>(acc, rs, rs.result)) sc->rr = rs.result[0];
+    grid_reduce<1>(acc, rs, rs.result, [=](double t, const double *) {
+        if ((threadIdx.x & 31) == 0) sc->rr = t;
+    });
 }
 
 }  // namespace
@@ -440,8 +542,6 @@ __global__ void __launch_bounds__(kRedBlock) k_residual(long long n, const doubl
 
 namespace {
 
-__device__ __forceinline__ cx<float> f2c(float2 a) { return {a.x, a.y}; }
-
 // Fields are flat arrays of n = 6 V float4 (two complex each).
 __device__ __forceinline__ void ld4(const float4 *p, long long i, cx<float> &a, cx<float> &b)
 {
@@ -454,124 +554,47 @@ __device__ __forceinline__ void st4(float4 *p, long long i, cx<float> a, cx<floa
     p[i] = make_float4(a.re, a.im, b.re, b.im);
 }
 
-// Grid sum of per-thread FP32 partials: lanes and warps in FP32, the block
-// partials (one per block) in FP64 by the last block, in block order.
-// Returns true in thread 0 of the last block once out[0..N) is final.
-template <int N>
-__device__ __forceinline__ bool grid_reduce_f(float (&v)[N], const ReduceScratch &rs, double *out)
-{
-    __shared__ float sm[32][N];
-    __shared__ bool last;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-    for (int i = 0; i < N; ++i)
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v[i] += __shfl_down_sync(0xffffffffu, v[i], o);
-    if (lane == 0)
-#pragma unroll
-        for (int i = 0; i < N; ++i) sm[wid][i] = v[i];
-    __syncthreads();
-    if (wid == 0) {
-#pragma unroll
-        for (int i = 0; i < N; ++i) {
-            float t = lane < nw ? sm[lane][i] : 0.f;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
-            if (lane == 0) rs.partials[(size_t)blockIdx.x * 8 + i] = (double)t;
-        }
-    }
-    if (threadIdx.x == 0) {
-        __threadfence();
-        last = atomicAdd(rs.ticket, 1u) == gridDim.x - 1;
-    }
-    __syncthreads();
-    if (!last) return false;
-    __threadfence();
-    __shared__ double smd[32 * N];
-    final_sum<N>(rs, out, smd);
-    return threadIdx.x == 0;
-}
-
-__device__ __forceinline__ cx<double> c_of2(double2 a) { return {a.x, a.y}; }
-__device__ __forceinline__ double2 d2_of2(cx<double> a) { return make_double2(a.re, a.im); }
-__device__ __forceinline__ cx<double> cdiv2(cx<double> a, cx<double> b)
-{
-    const double d = b.re * b.re + b.im * b.im;
-    return {(a.re * b.re + a.im * b.im) / d, (a.im * b.re - a.re * b.im) / d};
-}
-
-// Scalar updates of the low-precision BiCGStab, run by one thread of the
-// last block once the grid sums res[] are final (shared by the FP32 and the
-// FP16-storage kernels).
-__device__ void lo_init_update(const double *res, SolverScalars *sc)
-{
-    const double rr = res[0];
-    sc->rr = rr;
-    sc->rho = make_double2(rr, 0.0);
-    sc->rho0 = make_double2(1.0, 0.0);
-    sc->alpha = make_double2(1.0, 0.0);
-    sc->omega = make_double2(1.0, 0.0);
-    sc->beta = make_double2(rr, 0.0);
-    sc->flags = isfinite(rr) ? 0 : FLAG_NAN;
-    if (rr == 0.0) sc->flags |= FLAG_BREAKDOWN;
-}
-
-// alpha = rho / <rhat, v>
-__device__ void lo_alpha_update(const double *res, SolverScalars *sc)
-{
-    const cx<double> rv = mkc(res[0], res[1]);
-    if (!isfinite(rv.re) || !isfinite(rv.im)) sc->flags |= FLAG_NAN;
-    if (rv.re == 0.0 && rv.im == 0.0) {
-        sc->flags |= FLAG_BREAKDOWN;
-        sc->alpha = make_double2(0.0, 0.0);
-    } else {
-        sc->alpha = d2_of2(cdiv2(c_of2(sc->rho), rv));
-    }
-}
+// Grid sums of the low-precision kernels are grid_reduce on float: lanes and
+// warps in FP32, the block partials (one per block) in FP64 by the last
+// block.  The scalar updates are those of the FP64 solver, but for omega.
 
 // omega from <t, s>, <t, t>, <s, s>
-__device__ void lo_omega_update(const double *res, SolverScalars *sc)
+__device__ __forceinline__ void lo_omega_update(double t, SolverScalars *sc)
 {
-    const double tr = res[0], ti = res[1], tt = res[2], ss = res[3];
-    sc->tt = tt;
-    if (!isfinite(tt) || !isfinite(tr) || !isfinite(ti) || !isfinite(ss)) sc->flags |= FLAG_NAN;
-    double2 om = tt > 0.0 ? make_double2(tr / tt, ti / tt) : make_double2(0.0, 0.0);
+    const int lane = threadIdx.x & 31;
+    const double tr = sum_of(t, 0), ti = sum_of(t, 1), tt = sum_of(t, 2), ss = sum_of(t, 3);
+    double om = tt > 0.0 ? t / tt : 0.0;
     // omega stabilisation (Sleijpen & van der Vorst): when t and s are
     // nearly orthogonal, |<t,s>| / (|t||s|) < 0.7, the minimising omega is
     // tiny and BiCGStab loses accuracy in finite precision; enlarge it
-    const double rho_t = (tt > 0.0 && ss > 0.0) ? sqrt(tr * tr + ti * ti) / sqrt(tt * ss) : 1.0;
-    if (rho_t > 0.0 && rho_t < 0.7) {
-        const double f = 0.7 / rho_t;
-        om.x *= f;
-        om.y *= f;
+    // (the squares first: the roots are wanted only then)
+    const double c2 = tr * tr + ti * ti;
+    if (tt > 0.0 && ss > 0.0 && c2 > 0.0 && c2 < 0.5 * (tt * ss)) {
+        const double rho_t = sqrt(c2) / sqrt(tt * ss);
+        if (rho_t < 0.7) om *= 0.7 / rho_t;
     }
-    sc->omega = om;
+    if (lane < 2) (&sc->omega.x)[lane] = om;
+    if (lane == 0) {
+        sc->tt = tt;
+        if (!isfinite(tt) || !isfinite(tr) || !isfinite(ti) || !isfinite(ss)) sc->flags |= FLAG_NAN;
+    }
 }
 
-// rho' = <rhat, r>, rr = |r|^2, beta
-__device__ void lo_xr_update(const double *res, SolverScalars *sc)
+// after r was replaced: rho = <rhat, r> (sums 1, 2), beta from rho0 (rr is
+// sum 0)
+__device__ __forceinline__ void refresh_update(double t, SolverScalars *sc)
 {
-    const cx<double> rho_new = mkc(res[0], res[1]);
-    const cx<double> rho = c_of2(sc->rho), om = c_of2(sc->omega), al = c_of2(sc->alpha);
-    sc->rr = res[2];
-    if (!isfinite(sc->rr) || !isfinite(rho_new.re) || !isfinite(rho_new.im)) sc->flags |= FLAG_NAN;
-    if ((om.re == 0.0 && om.im == 0.0) || (rho.re == 0.0 && rho.im == 0.0))
-        sc->flags |= FLAG_BREAKDOWN;
-    else
-        sc->beta = d2_of2(cdiv2(rho_new, rho) * cdiv2(al, om));
-    if (rho_new.re == 0.0 && rho_new.im == 0.0 && sc->rr > 0.0) sc->flags |= FLAG_BREAKDOWN;
-    sc->rho0 = sc->rho;
-    sc->rho = d2_of2(rho_new);
-}
-
-// after r was replaced: rho = <rhat, r>, beta from rho0 (rr untouched)
-__device__ void lo_rho_update(const double *res, SolverScalars *sc)
-{
-    const cx<double> rho_new = mkc(res[0], res[1]);
-    const cx<double> rho0 = c_of2(sc->rho0), om = c_of2(sc->omega), al = c_of2(sc->alpha);
-    if ((om.re != 0.0 || om.im != 0.0) && (rho0.re != 0.0 || rho0.im != 0.0))
-        sc->beta = d2_of2(cdiv2(rho_new, rho0) * cdiv2(al, om));
-    sc->rho = d2_of2(rho_new);
+    const double rr = sum_of(t, 0);
+    const cx<double> rho_new = mkc(sum_of(t, 1), sum_of(t, 2));
+    const cx<double> rho0 = c_of(sc->rho0), om = c_of(sc->omega), al = c_of(sc->alpha);
+    // rho'/rho0 in lanes 0, 1, alpha/omega in lanes 2, 3
+    const bool second = threadIdx.x & 2;
+    const double q = cdiv_part(second ? al : rho_new, second ? om : rho0);
+    const cx<double> b = mkc(sum_of(q, 0), sum_of(q, 1)) * mkc(sum_of(q, 2), sum_of(q, 3));
+    if ((threadIdx.x & 31) != 0) return;
+    sc->rr = rr;
+    if ((om.re != 0.0 || om.im != 0.0) && (rho0.re != 0.0 || rho0.im != 0.0)) sc->beta = make_double2(b.re, b.im);
+    sc->rho = make_double2(rho_new.re, rho_new.im);
 }
 
 // rhat = r, p = v = 0, xlo = 0; rr = |r|^2, rho = rr, alpha = omega = rho0 = 1
@@ -588,7 +611,7 @@ __global__ void __launch_bounds__(kRedBlock) k_lo_init(long long n, const float4
         xlo[i] = make_float4(0.f, 0.f, 0.f, 0.f);
         acc[0] = fmaf(ri.x, ri.x, fmaf(ri.y, ri.y, fmaf(ri.z, ri.z, fmaf(ri.w, ri.w, acc[0]))));
     }
-    if (grid_reduce_f<1>(acc, rs, rs.result)) lo_init_update(rs.result, sc);
+    grid_reduce<1>(acc, rs, rs.result, [=](double t, const double *) { init_update(t, sc); });
 }
 
 // p = r + beta (p - omega v)
@@ -627,7 +650,7 @@ __device__ __forceinline__ void body_lo_alpha(long long n, const float4 *rhat, c
         acc[0] = fmaf(a.x, b.x, fmaf(a.y, b.y, fmaf(a.z, b.z, fmaf(a.w, b.w, acc[0]))));
         acc[1] = fmaf(a.x, b.y, fmaf(-a.y, b.x, fmaf(a.z, b.w, fmaf(-a.w, b.z, acc[1]))));
     }
-    if (grid_reduce_f<2>(acc, rs, rs.result)) lo_alpha_update(rs.result, sc);
+    grid_reduce<2>(acc, rs, rs.result, [=](double t, const double *) { alpha_update(t, sc); });
 }
 __global__ void __launch_bounds__(kRedBlock) k_lo_alpha(long long n, const float4 *rhat, const float4 *v,
                                                         ReduceScratch rs, SolverScalars *sc)
@@ -669,7 +692,7 @@ __device__ __forceinline__ void body_lo_omega(long long n, const float4 *t, cons
         acc[2] = fmaf(a.x, a.x, fmaf(a.y, a.y, fmaf(a.z, a.z, fmaf(a.w, a.w, acc[2]))));
         acc[3] = fmaf(b.x, b.x, fmaf(b.y, b.y, fmaf(b.z, b.z, fmaf(b.w, b.w, acc[3]))));
     }
-    if (grid_reduce_f<4>(acc, rs, rs.result)) lo_omega_update(rs.result, sc);
+    grid_reduce<4>(acc, rs, rs.result, [=](double t, const double *) { lo_omega_update(t, sc); });
 }
 __global__ void __launch_bounds__(kRedBlock) k_lo_omega(long long n, const float4 *t, const float4 *s,
                                                         ReduceScratch rs, SolverScalars *sc)
@@ -705,7 +728,8 @@ __device__ __forceinline__ void body_lo_xr(long long n, float4 *xlo, const float
         acc[1] += h0.re * r0.im - h0.im * r0.re + h1.re * r1.im - h1.im * r1.re;
         acc[2] += r0.re * r0.re + r0.im * r0.im + r1.re * r1.re + r1.im * r1.im;
     }
-    if (grid_reduce_f<3>(acc, rs, rs.result)) lo_xr_update(rs.result, sc);
+    grid_reduce<3>(acc, rs, rs.result, [=](double t, const double *e) { xr_update(t, e, sc); },
+                   [=] { return xr_ahead(sc); });
 }
 __global__ void __launch_bounds__(kRedBlock) k_lo_xr(long long n, float4 *xlo, const float4 *phat,
                                                      const float4 *shat, const float4 *s, const float4 *t,
@@ -749,7 +773,7 @@ __global__ void __launch_bounds__(kRedBlock) k_lo_init_h(int V, HF r, HF rhat, H
         hst(v, V, x, z);
         P32::store_spinor(xlo, nullptr, V, x, z);
     }
-    if (grid_reduce_f<1>(acc, rs, rs.result)) lo_init_update(rs.result, sc);
+    grid_reduce<1>(acc, rs, rs.result, [=](double t, const double *) { init_update(t, sc); });
 }
 
 __device__ __forceinline__ void body_lo_p_h(int V, HF r, HF v, HF p, const SolverScalars *sc)
@@ -793,7 +817,7 @@ __device__ __forceinline__ void body_lo_alpha_h(int V, HF rhat, HF v, ReduceScra
         hld(v, V, x, b);
         cdot_acc(a, b, acc);
     }
-    if (grid_reduce_f<2>(acc, rs, rs.result)) lo_alpha_update(rs.result, sc);
+    grid_reduce<2>(acc, rs, rs.result, [=](double t, const double *) { alpha_update(t, sc); });
 }
 __global__ void __launch_bounds__(kRedBlock) k_lo_alpha_h(int V, HF rhat, HF v, ReduceScratch rs,
                                                           SolverScalars *sc)
@@ -834,7 +858,7 @@ __device__ __forceinline__ void body_lo_omega_h(int V, HF t, HF s, ReduceScratch
             acc[3] = fmaf(b[k].re, b[k].re, fmaf(b[k].im, b[k].im, acc[3]));
         }
     }
-    if (grid_reduce_f<4>(acc, rs, rs.result)) lo_omega_update(rs.result, sc);
+    grid_reduce<4>(acc, rs, rs.result, [=](double t, const double *) { lo_omega_update(t, sc); });
 }
 __global__ void __launch_bounds__(kRedBlock) k_lo_omega_h(int V, HF t, HF s, ReduceScratch rs, SolverScalars *sc)
 {
@@ -867,7 +891,8 @@ __device__ __forceinline__ void body_lo_xr_h(int V, float4 *xlo, HF phat, HF sha
         hld(rhat, V, x, b);
         cdot_acc(b, a, acc);
     }
-    if (grid_reduce_f<3>(acc, rs, rs.result)) lo_xr_update(rs.result, sc);
+    grid_reduce<3>(acc, rs, rs.result, [=](double t, const double *e) { xr_update(t, e, sc); },
+                   [=] { return xr_ahead(sc); });
 }
 __global__ void __launch_bounds__(kRedBlock) k_lo_xr_h(int V, float4 *xlo, HF phat, HF shat, HF s, HF t, HF r,
                                                        HF rhat, ReduceScratch rs, SolverScalars *sc)
@@ -908,10 +933,7 @@ __global__ void __launch_bounds__(kRedBlock) k_refresh_tail(int V, const void *b
         acc[1] += d[0];
         acc[2] += d[1];
     }
-    if (grid_reduce<3>(acc, rs, rs.result)) {
-        sc->rr = rs.result[0];
-        lo_rho_update(rs.result + 1, sc);
-    }
+    grid_reduce<3>(acc, rs, rs.result, [=](double t, const double *) { refresh_update(t, sc); });
 }
 
 // The step kernels for all members of a lockstep group: member blockIdx.y,
@@ -956,33 +978,24 @@ __global__ void __launch_bounds__(kRedBlock) k_lo_group(int V, const LoMember *m
 // even multi-RHS Schur pass wrote (one member per CTA, the partials summed
 // in a fixed order, so the result does not depend on scheduling).
 template <int STEP>
-__global__ void __launch_bounds__(256) k_lo_group_finalize(int nblk, const double *part, const LoMember *members)
+__global__ void __launch_bounds__(kRedBlock) k_lo_group_finalize(int nblk, const double *part, const LoMember *members)
 {
     const LoMember &a = members[blockIdx.x];
     if (a.sc->skip) return;   // its partials were not written
     const double *p = part + (size_t)blockIdx.x * nblk * 4;
-    double t[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int b = threadIdx.x; b < nblk; b += blockDim.x)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) t[c] += p[(size_t)b * 4 + c];
-    __shared__ double sm[8][4];
+    // warp w adds the partials of sum w % 4
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-    for (int c = 0; c < 4; ++c) t[c] = warp_sum(t[c]);
-    if (lane == 0)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) sm[wid][c] = t[c];
+    double s[1] = {0.0};
+#pragma unroll 4
+    for (int b = (wid / 4) * 32 + lane; b < nblk; b += kRedBlock / 4) s[0] += p[(size_t)b * 4 + wid % 4];
+    const double t = warp_sums(s);
+    __shared__ double fin[kRedWarps];
+    if (lane == 0) fin[wid] = t;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double res[4] = {0.0, 0.0, 0.0, 0.0};
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w)
-#pragma unroll
-            for (int c = 0; c < 4; ++c) res[c] += sm[w][c];
-        if (STEP == LO_STEP_ALPHA)
-            lo_alpha_update(res, a.sc);
-        else
-            lo_omega_update(res, a.sc);
-    }
+    if (wid != 0) return;
+    const double u = lane < 4 ? fin[lane] + fin[lane + 4] : 0.0;
+    if (STEP == LO_STEP_ALPHA) alpha_update(u, a.sc);
+    else lo_omega_update(u, a.sc);
 }
 
 // x (FP64) += xlo (FP32); xlo = 0.  FP32 plane j holds components 2j and
@@ -1013,10 +1026,11 @@ cudaError_t bicg_init(wc_lattice lat, SolverState &S, const double2 *b, double2 
     k_bicg_init<<<WC_GRID(n)>>>(n, b, r, rhat, p, v, S.red, S.scal);
     return cudaGetLastError();
 }
-cudaError_t bicg_p(wc_lattice lat, SolverState &S, const double2 *r, const double2 *v, double2 *p)
+cudaError_t bicg_p(wc_lattice lat, SolverState &S, const double2 *r, const double2 *v, double2 *p, bool norm)
 {
     const long long n = 12LL * lat->g.V;
-    k_bicg_p<<<WC_GRID(n)>>>(n, r, v, p, S.red, S.scal);
+    if (norm) k_bicg_p<true><<<WC_GRID(n)>>>(n, r, v, p, S.red, S.scal);
+    else k_bicg_p<false><<<WC_GRID(n)>>>(n, r, v, p, S.red, S.scal);
     return cudaGetLastError();
 }
 cudaError_t bicg_alpha(wc_lattice lat, SolverState &S, const double2 *rhat, const double2 *v)
@@ -1025,10 +1039,11 @@ cudaError_t bicg_alpha(wc_lattice lat, SolverState &S, const double2 *rhat, cons
     k_bicg_alpha<<<WC_GRID(n)>>>(n, rhat, v, S.red, S.scal);
     return cudaGetLastError();
 }
-cudaError_t bicg_s(wc_lattice lat, SolverState &S, const double2 *r, const double2 *v, double2 *s)
+cudaError_t bicg_s(wc_lattice lat, SolverState &S, const double2 *r, const double2 *v, double2 *s, bool norm)
 {
     const long long n = 12LL * lat->g.V;
-    k_bicg_s<<<WC_GRID(n)>>>(n, r, v, s, S.red, S.scal);
+    if (norm) k_bicg_s<true><<<WC_GRID(n)>>>(n, r, v, s, S.red, S.scal);
+    else k_bicg_s<false><<<WC_GRID(n)>>>(n, r, v, s, S.red, S.scal);
     return cudaGetLastError();
 }
 cudaError_t bicg_omega(wc_lattice lat, SolverState &S, const double2 *t, const double2 *s)
@@ -1150,12 +1165,12 @@ cudaError_t lo_group(LoStep step, wc_lattice lat, int m, const LoMember *members
 {
     if (m < 1 || m > 65535) return cudaErrorInvalidValue;
     const int V = lat->g.V;
-    // about max_blocks blocks in all (each member reduces over its own
-    // gridDim.x partials, at most max_blocks of them)
+    // about eight blocks per SM in all (each member reduces over its own
+    // gridDim.x partials, at most max_blocks = four per SM of them)
     const long long work = half ? (long long)V : 6LL * V;
     long long gx = (work + kRedBlock - 1) / kRedBlock;
-    const long long share = std::max<long long>(1, (max_blocks + m - 1) / m);
-    const long long floor_blocks = std::max(1, max_blocks / 8);   // one per SM
+    const long long share = std::max<long long>(1, (2 * max_blocks + m - 1) / m);
+    const long long floor_blocks = std::max(1, max_blocks / 4);   // one per SM
     gx = std::max<long long>(1, std::min<long long>(std::min<long long>(gx, max_blocks),
                                                     std::max<long long>(share, floor_blocks)));
     const dim3 grid((unsigned)gx, (unsigned)m);

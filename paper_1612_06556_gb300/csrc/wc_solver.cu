@@ -174,11 +174,12 @@ wc_status enqueue_init(wc_lattice lat, SolverState &S, int kind, wc_field x, wc_
 wc_status enqueue_iteration(wc_lattice lat, SolverState &S, const wc_solve_params &p, int kind, wc_field x,
                             const SolverVecs &w)
 {
-    wc_status st = check_cuda(lat, bicg_p(lat, S, d2(w.r), d2(w.v), d2(w.p)), "bicg_p");
+    const bool norm = w.phat != w.p;   // a preconditioner scales its input by |p|, |s|
+    wc_status st = check_cuda(lat, bicg_p(lat, S, d2(w.r), d2(w.v), d2(w.p), norm), "bicg_p");
     if (st == WC_OK) st = apply_precond(lat, S, p, kind, w, w.p, w.phat, &S.scal->pp);
     if (st == WC_OK) st = check_cuda(lat, launch_apply(lat, w.v, w.phat, kind, S), "apply");
     if (st == WC_OK) st = check_cuda(lat, bicg_alpha(lat, S, d2(w.rhat), d2(w.v)), "bicg_alpha");
-    if (st == WC_OK) st = check_cuda(lat, bicg_s(lat, S, d2(w.r), d2(w.v), d2(w.s)), "bicg_s");
+    if (st == WC_OK) st = check_cuda(lat, bicg_s(lat, S, d2(w.r), d2(w.v), d2(w.s), norm), "bicg_s");
     if (st == WC_OK) st = apply_precond(lat, S, p, kind, w, w.s, w.shat, &S.scal->ss);
     if (st == WC_OK) st = check_cuda(lat, launch_apply(lat, w.t, w.shat, kind, S), "apply");
     if (st == WC_OK) st = check_cuda(lat, bicg_omega(lat, S, d2(w.t), d2(w.s)), "bicg_omega");

@@ -12,12 +12,12 @@ int reduce_grid(const ReduceScratch &rs, long long n);
 // r = b - r (r holds M x), rhat = r, p = v = 0; scalars reset
 cudaError_t bicg_init(wc_lattice lat, SolverState &S, const double2 *b, double2 *r, double2 *rhat, double2 *p,
                       double2 *v);
-// p = r + beta (p - omega v); pp = |p|^2
-cudaError_t bicg_p(wc_lattice lat, SolverState &S, const double2 *r, const double2 *v, double2 *p);
+// p = r + beta (p - omega v); with norm pp = |p|^2
+cudaError_t bicg_p(wc_lattice lat, SolverState &S, const double2 *r, const double2 *v, double2 *p, bool norm);
 // alpha = rho / <rhat, v>
 cudaError_t bicg_alpha(wc_lattice lat, SolverState &S, const double2 *rhat, const double2 *v);
-// s = r - alpha v; ss = |s|^2
-cudaError_t bicg_s(wc_lattice lat, SolverState &S, const double2 *r, const double2 *v, double2 *s);
+// s = r - alpha v; with norm ss = |s|^2
+cudaError_t bicg_s(wc_lattice lat, SolverState &S, const double2 *r, const double2 *v, double2 *s, bool norm);
 // omega = <t, s> / <t, t>
 cudaError_t bicg_omega(wc_lattice lat, SolverState &S, const double2 *t, const double2 *s);
 // x += alpha phat + omega shat; r = s - omega t; rho, beta, rr updated

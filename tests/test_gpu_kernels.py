@@ -133,3 +133,24 @@ def test_transfers_turn_rows_round_at_ragged_sizes(dims, prec, offset):
             r, w = torch.view_as_real(got.to(torch.complex128)), torch.view_as_real(want.to(torch.complex128))
             big = w.abs().amax(dim=(1, 2, 3), keepdim=True)
             assert ((r - w).abs() <= 2.0 ** -11 * big * (1 + 1e-5)).all()
+
+
+@pytest.mark.parametrize("dims", [(2, 2, 2, 2), (5, 3, 17, 2), (16, 8, 8, 8), (24, 24, 24, 24)])
+@pytest.mark.parametrize("prec", [0, 1, 2])
+def test_reductions_of_one_two_and_three_sums(dims, prec):
+    """Inner product, norm and axpy with norm from one block (16 sites) to
+    more partials than threads, against numpy on the stored values.  Sums
+    of n = 24 V products in FP64, in trees with at most 12 V / (256 grid) +
+    60 sequential additions: relative error of the sum of magnitudes below
+    1e-13 at these sizes; twice the same bits."""
+    V = int(np.prod(dims))
+    lat = wc().Lattice(dims)
+    a, b = lat.field(prec).load(synth.gaussian_source(dims, 5)), lat.field(prec).load(synth.gaussian_source(dims, 6))
+    na, nb = (f.store(np.zeros((V, 4, 3), complex)) for f in (a, b))
+    mag = np.sum(np.abs(na) * np.abs(nb))
+    assert abs(lat.dot(a, b) - np.vdot(na, nb)) <= 1e-13 * mag
+    assert abs(lat.norm2(a) - np.sum(np.abs(na) ** 2)) <= 1e-13 * np.sum(np.abs(na) ** 2)
+    assert lat.dot(a, b) == lat.dot(a, b) and lat.norm2(b) == lat.norm2(b)
+    got = lat.axpy_norm(0.5 - 0.25j, a, b)
+    tol = {0: 1e-13, 1: 2e-7, 2: 2e-3}[prec]     # the norm is of the values before they are stored
+    assert abs(got - np.sum(np.abs(b.store(np.zeros((V, 4, 3), complex))) ** 2)) <= tol * got
