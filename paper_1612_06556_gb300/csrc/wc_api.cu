@@ -292,6 +292,10 @@ wc_status state_init(wc_lattice lat, SolverState &s)
     if (st == WC_OK)
         st = check_cuda(lat, cudaMallocHost(reinterpret_cast<void **>(&s.scal_host), sizeof(SolverScalars)),
                         "cudaMallocHost");
+    if (st == WC_OK)
+        st = check_cuda(lat, cudaMallocHost(reinterpret_cast<void **>(&s.report), sizeof(StepReport) * kReportSlots),
+                        "cudaMallocHost");
+    for (int i = 0; i < kReportSlots && st == WC_OK; ++i) s.report[i].seq = 0;
     if (st == WC_OK) st = check_cuda(lat, cudaMemset(s.red.ticket, 0, sizeof(unsigned)), "cudaMemset");
     if (st == WC_OK) st = check_cuda(lat, cudaMemset(s.scal, 0, sizeof(SolverScalars)), "cudaMemset");
     if (st != WC_OK) state_free(s);
@@ -315,6 +319,7 @@ void state_free(SolverState &s)
     cudaFreeHost(s.red.host_result);
     cudaFree(s.scal);
     cudaFreeHost(s.scal_host);
+    cudaFreeHost(s.report);
     s = SolverState{};
 }
 

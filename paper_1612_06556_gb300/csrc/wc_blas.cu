@@ -327,6 +327,70 @@ __device__ __forceinline__ void init_update(double t, SolverScalars *sc)
     sc->beta = make_double2(rr, 0.0);  // (rho/rho0)(alpha/omega)
     sc->flags = isfinite(rr) ? 0 : FLAG_NAN;
     if (rr == 0.0) sc->flags |= FLAG_BREAKDOWN;
+    sc->action = ACT_NONE;
+    sc->skip = 0;
+    if (sc->track == TRACK_INNER) {   // the tolerance is relative to this |r|^2
+        sc->tol2 = sc->d2 * rr;
+        if (sc->flags) {
+            sc->action = ACT_STOP;
+            sc->skip = 1;
+        }
+    }
+}
+
+// After a step of a host-driven solve (one thread): does the host have to act
+// before the next one?  The host queues steps ahead of reading these scalars,
+// so this is decided here, and skip keeps the steps already queued from
+// running.
+__device__ __forceinline__ void track_step(SolverScalars *sc)
+{
+    const int f = sc->flags;
+    const double rr = sc->rr;
+    int a = ACT_NONE;
+    if (sc->track == TRACK_NONE) return;
+    if (sc->track == TRACK_FP64 || sc->track == TRACK_INNER) {
+        if (f != 0 || !(rr > sc->tol2)) a = ACT_STOP;
+    } else if ((f & FLAG_NAN) || rr > 1e8 * sc->rr_refresh) {
+        a = ACT_DIVERGED;
+    } else if (f & FLAG_BREAKDOWN) {
+        a = ACT_BREAKDOWN;
+    } else {
+        if (rr > sc->rmax2) sc->rmax2 = rr;
+        const double prev = sc->prev;
+        sc->prev = rr;
+        if (sc->defer2 > 0.0 && rr <= sc->defer2) {
+            a = ACT_DEFER;
+        } else {
+            // deferring, a recurrence below tol but above defer2 refreshes
+            // only once it stops decreasing
+            const bool at_tol = rr <= sc->tol2 && (sc->defer2 <= 0.0 || !(rr < prev));
+            if (rr <= sc->d2 * sc->rmax2 || at_tol) a = ACT_REFRESH;
+        }
+    }
+    sc->action = a;
+    if (a != ACT_NONE) sc->skip = 1;
+}
+
+// one thread: the step's outcome to the host
+__device__ __forceinline__ void report(const SolverScalars *sc, StepReport *rep, unsigned long long seq)
+{
+    if (!rep) return;
+    rep->rr = sc->rr;
+    rep->flags = sc->flags;
+    rep->action = sc->action;
+    __threadfence_system();
+    rep->seq = seq;
+}
+
+__global__ void k_track(SolverScalars *sc, int track, double tol2, double d2, double defer2, double rr)
+{
+    sc->track = track;
+    sc->action = ACT_NONE;
+    sc->skip = 0;
+    sc->tol2 = tol2;
+    sc->d2 = d2;
+    sc->defer2 = defer2;
+    sc->rmax2 = sc->prev = sc->rr_refresh = rr;
 }
 
 // alpha = rho / <rhat, v>
@@ -367,7 +431,8 @@ __device__ __forceinline__ double xr_ahead(const SolverScalars *sc)
 
 // rho' = <rhat, r>, rr = |r|^2, beta = (rho'/rho)(alpha/omega), rho0 = rho,
 // rho = rho'; e: what xr_ahead returned
-__device__ __forceinline__ void xr_update(double t, const double *e, SolverScalars *sc)
+__device__ __forceinline__ void xr_update(double t, const double *e, SolverScalars *sc, StepReport *rep,
+                                          unsigned long long seq)
 {
     const cx<double> rho_new = mkc(sum_of(t, 0), sum_of(t, 1));
     const double rr = sum_of(t, 2);
@@ -384,6 +449,8 @@ __device__ __forceinline__ void xr_update(double t, const double *e, SolverScala
     if (rho_new.re == 0.0 && rho_new.im == 0.0 && rr > 0.0) sc->flags |= FLAG_BREAKDOWN;
     sc->rho0 = sc->rho;
     sc->rho = make_double2(rho_new.re, rho_new.im);
+    track_step(sc);
+    report(sc, rep, seq);
 }
 
 // result[0] = |a|^2 (FP64 field as a flat array)
@@ -423,6 +490,9 @@ template <bool NORM>
 __global__ void __launch_bounds__(kRedBlock) k_bicg_p(long long n, const double2 *r, const double2 *v, double2 *p,
                                                       ReduceScratch rs, SolverScalars *sc)
 {
+    griddep_wait();
+    griddep_launch_dependents();
+    if (sc->skip) return;
     const cx<double> beta = c_of(sc->beta), omega = c_of(sc->omega);
     double acc[1] = {0.0};
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
@@ -443,6 +513,9 @@ __global__ void __launch_bounds__(kRedBlock) k_bicg_p(long long n, const double2
 __global__ void __launch_bounds__(kRedBlock) k_bicg_alpha(long long n, const double2 *rhat, const double2 *v,
                                                           ReduceScratch rs, SolverScalars *sc)
 {
+    griddep_wait();
+    griddep_launch_dependents();
+    if (sc->skip) return;
     double acc[2] = {0.0, 0.0};
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x) {
@@ -458,6 +531,9 @@ template <bool NORM>
 __global__ void __launch_bounds__(kRedBlock) k_bicg_s(long long n, const double2 *r, const double2 *v, double2 *s,
                                                       ReduceScratch rs, SolverScalars *sc)
 {
+    griddep_wait();
+    griddep_launch_dependents();
+    if (sc->skip) return;
     const cx<double> alpha = c_of(sc->alpha);
     double acc[1] = {0.0};
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
@@ -478,6 +554,9 @@ __global__ void __launch_bounds__(kRedBlock) k_bicg_s(long long n, const double2
 __global__ void __launch_bounds__(kRedBlock) k_bicg_omega(long long n, const double2 *t, const double2 *s,
                                                           ReduceScratch rs, SolverScalars *sc)
 {
+    griddep_wait();
+    griddep_launch_dependents();
+    if (sc->skip) return;
     double acc[3] = {0.0, 0.0, 0.0};
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x) {
@@ -494,8 +573,11 @@ __global__ void __launch_bounds__(kRedBlock) k_bicg_omega(long long n, const dou
 __global__ void __launch_bounds__(kRedBlock) k_bicg_xr(long long n, double2 *x, const double2 *phat,
                                                        const double2 *shat, const double2 *s, const double2 *t,
                                                        double2 *r, const double2 *rhat, ReduceScratch rs,
-                                                       SolverScalars *sc)
+                                                       SolverScalars *sc, StepReport *rep, unsigned long long seq)
 {
+    griddep_wait();
+    griddep_launch_dependents();
+    if (sc->skip) return;
     const cx<double> alpha = c_of(sc->alpha), omega = c_of(sc->omega);
     double acc[3] = {0.0, 0.0, 0.0};
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
@@ -511,7 +593,7 @@ __global__ void __launch_bounds__(kRedBlock) k_bicg_xr(long long n, double2 *x, 
         acc[1] += h.re * ri.im - h.im * ri.re;
         acc[2] += ri.re * ri.re + ri.im * ri.im;
     }
-    grid_reduce<3>(acc, rs, rs.result, [=](double t, const double *e) { xr_update(t, e, sc); },
+    grid_reduce<3>(acc, rs, rs.result, [=](double t, const double *e) { xr_update(t, e, sc, rep, seq); },
                    [=] { return xr_ahead(sc); });
 }
 
@@ -582,7 +664,7 @@ __device__ __forceinline__ void lo_omega_update(double t, SolverScalars *sc)
 
 // after r was replaced: rho = <rhat, r> (sums 1, 2), beta from rho0 (rr is
 // sum 0)
-__device__ __forceinline__ void refresh_update(double t, SolverScalars *sc)
+__device__ __forceinline__ void refresh_update(double t, SolverScalars *sc, StepReport *rep, unsigned long long seq)
 {
     const double rr = sum_of(t, 0);
     const cx<double> rho_new = mkc(sum_of(t, 1), sum_of(t, 2));
@@ -595,6 +677,12 @@ __device__ __forceinline__ void refresh_update(double t, SolverScalars *sc)
     sc->rr = rr;
     if ((om.re != 0.0 || om.im != 0.0) && (rho0.re != 0.0 || rho0.im != 0.0)) sc->beta = make_double2(b.re, b.im);
     sc->rho = make_double2(rho_new.re, rho_new.im);
+    if (sc->track == TRACK_RELIABLE) {
+        sc->rmax2 = sc->prev = sc->rr_refresh = rr;
+        sc->action = rr <= sc->tol2 ? ACT_STOP : ACT_NONE;
+        sc->skip = rr <= sc->tol2 ? 1 : 0;
+    }
+    report(sc, rep, seq);
 }
 
 // rhat = r, p = v = 0, xlo = 0; rr = |r|^2, rho = rr, alpha = omega = rho0 = 1
@@ -635,6 +723,8 @@ __device__ __forceinline__ void body_lo_p(long long n, const float4 *r, const fl
 __global__ void __launch_bounds__(kRedBlock) k_lo_p(long long n, const float4 *r, const float4 *v, float4 *p,
                                                     const SolverScalars *sc)
 {
+    griddep_wait();
+    griddep_launch_dependents();
     body_lo_p(n, r, v, p, sc);
 }
 
@@ -655,6 +745,8 @@ __device__ __forceinline__ void body_lo_alpha(long long n, const float4 *rhat, c
 __global__ void __launch_bounds__(kRedBlock) k_lo_alpha(long long n, const float4 *rhat, const float4 *v,
                                                         ReduceScratch rs, SolverScalars *sc)
 {
+    griddep_wait();
+    griddep_launch_dependents();
     body_lo_alpha(n, rhat, v, rs, sc);
 }
 
@@ -675,6 +767,8 @@ __device__ __forceinline__ void body_lo_s(long long n, const float4 *r, const fl
 __global__ void __launch_bounds__(kRedBlock) k_lo_s(long long n, const float4 *r, const float4 *v, float4 *s,
                                                     const SolverScalars *sc)
 {
+    griddep_wait();
+    griddep_launch_dependents();
     body_lo_s(n, r, v, s, sc);
 }
 
@@ -697,6 +791,8 @@ __device__ __forceinline__ void body_lo_omega(long long n, const float4 *t, cons
 __global__ void __launch_bounds__(kRedBlock) k_lo_omega(long long n, const float4 *t, const float4 *s,
                                                         ReduceScratch rs, SolverScalars *sc)
 {
+    griddep_wait();
+    griddep_launch_dependents();
     body_lo_omega(n, t, s, rs, sc);
 }
 
@@ -704,7 +800,8 @@ __global__ void __launch_bounds__(kRedBlock) k_lo_omega(long long n, const float
 __device__ __forceinline__ void body_lo_xr(long long n, float4 *xlo, const float4 *phat,
                                                      const float4 *shat, const float4 *s, const float4 *t,
                                                      float4 *r, const float4 *rhat, ReduceScratch rs,
-                                                     SolverScalars *sc)
+                                                     SolverScalars *sc, StepReport *rep = nullptr,
+                                                     unsigned long long seq = 0)
 {
     if (sc->skip) return;   // a stopped right-hand side of a lockstep batch
     const cx<float> alpha = mkc((float)sc->alpha.x, (float)sc->alpha.y);
@@ -728,15 +825,17 @@ __device__ __forceinline__ void body_lo_xr(long long n, float4 *xlo, const float
         acc[1] += h0.re * r0.im - h0.im * r0.re + h1.re * r1.im - h1.im * r1.re;
         acc[2] += r0.re * r0.re + r0.im * r0.im + r1.re * r1.re + r1.im * r1.im;
     }
-    grid_reduce<3>(acc, rs, rs.result, [=](double t, const double *e) { xr_update(t, e, sc); },
+    grid_reduce<3>(acc, rs, rs.result, [=](double t, const double *e) { xr_update(t, e, sc, rep, seq); },
                    [=] { return xr_ahead(sc); });
 }
 __global__ void __launch_bounds__(kRedBlock) k_lo_xr(long long n, float4 *xlo, const float4 *phat,
                                                      const float4 *shat, const float4 *s, const float4 *t,
                                                      float4 *r, const float4 *rhat, ReduceScratch rs,
-                                                     SolverScalars *sc)
+                                                     SolverScalars *sc, StepReport *rep, unsigned long long seq)
 {
-    body_lo_xr(n, xlo, phat, shat, s, t, r, rhat, rs, sc);
+    griddep_wait();
+    griddep_launch_dependents();
+    body_lo_xr(n, xlo, phat, shat, s, t, r, rhat, rs, sc, rep, seq);
 }
 
 // ------------------------------------------------------------------------
@@ -793,6 +892,8 @@ __device__ __forceinline__ void body_lo_p_h(int V, HF r, HF v, HF p, const Solve
 }
 __global__ void __launch_bounds__(kRedBlock) k_lo_p_h(int V, HF r, HF v, HF p, const SolverScalars *sc)
 {
+    griddep_wait();
+    griddep_launch_dependents();
     body_lo_p_h(V, r, v, p, sc);
 }
 
@@ -822,6 +923,8 @@ __device__ __forceinline__ void body_lo_alpha_h(int V, HF rhat, HF v, ReduceScra
 __global__ void __launch_bounds__(kRedBlock) k_lo_alpha_h(int V, HF rhat, HF v, ReduceScratch rs,
                                                           SolverScalars *sc)
 {
+    griddep_wait();
+    griddep_launch_dependents();
     body_lo_alpha_h(V, rhat, v, rs, sc);
 }
 
@@ -840,6 +943,8 @@ __device__ __forceinline__ void body_lo_s_h(int V, HF r, HF v, HF s, const Solve
 }
 __global__ void __launch_bounds__(kRedBlock) k_lo_s_h(int V, HF r, HF v, HF s, const SolverScalars *sc)
 {
+    griddep_wait();
+    griddep_launch_dependents();
     body_lo_s_h(V, r, v, s, sc);
 }
 
@@ -862,11 +967,14 @@ __device__ __forceinline__ void body_lo_omega_h(int V, HF t, HF s, ReduceScratch
 }
 __global__ void __launch_bounds__(kRedBlock) k_lo_omega_h(int V, HF t, HF s, ReduceScratch rs, SolverScalars *sc)
 {
+    griddep_wait();
+    griddep_launch_dependents();
     body_lo_omega_h(V, t, s, rs, sc);
 }
 
 __device__ __forceinline__ void body_lo_xr_h(int V, float4 *xlo, HF phat, HF shat, HF s, HF t, HF r,
-                                                       HF rhat, ReduceScratch rs, SolverScalars *sc)
+                                                       HF rhat, ReduceScratch rs, SolverScalars *sc,
+                                                       StepReport *rep = nullptr, unsigned long long seq = 0)
 {
     if (sc->skip) return;   // a stopped right-hand side of a lockstep batch
     const cx<float> alpha = mkc((float)sc->alpha.x, (float)sc->alpha.y);
@@ -891,13 +999,16 @@ __device__ __forceinline__ void body_lo_xr_h(int V, float4 *xlo, HF phat, HF sha
         hld(rhat, V, x, b);
         cdot_acc(b, a, acc);
     }
-    grid_reduce<3>(acc, rs, rs.result, [=](double t, const double *e) { xr_update(t, e, sc); },
+    grid_reduce<3>(acc, rs, rs.result, [=](double t, const double *e) { xr_update(t, e, sc, rep, seq); },
                    [=] { return xr_ahead(sc); });
 }
 __global__ void __launch_bounds__(kRedBlock) k_lo_xr_h(int V, float4 *xlo, HF phat, HF shat, HF s, HF t, HF r,
-                                                       HF rhat, ReduceScratch rs, SolverScalars *sc)
+                                                       HF rhat, ReduceScratch rs, SolverScalars *sc,
+                                                       StepReport *rep, unsigned long long seq)
 {
-    body_lo_xr_h(V, xlo, phat, shat, s, t, r, rhat, rs, sc);
+    griddep_wait();
+    griddep_launch_dependents();
+    body_lo_xr_h(V, xlo, phat, shat, s, t, r, rhat, rs, sc, rep, seq);
 }
 
 // End of a reliable update in one pass (the FP64 residual, its
@@ -909,8 +1020,10 @@ __global__ void __launch_bounds__(kRedBlock) k_lo_xr_h(int V, float4 *xlo, HF ph
 template <class PL>
 __global__ void __launch_bounds__(kRedBlock) k_refresh_tail(int V, const void *b, void *r, void *rlo, float *rlo_n,
                                                             const void *rhat, const float *rhat_n, ReduceScratch rs,
-                                                            SolverScalars *sc)
+                                                            SolverScalars *sc, StepReport *rep, unsigned long long seq)
 {
+    griddep_wait();
+    griddep_launch_dependents();
     double acc[3] = {0.0, 0.0, 0.0};
     for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < V; x += gridDim.x * blockDim.x) {
         cx<double> bv[12], rv[12];
@@ -933,7 +1046,7 @@ __global__ void __launch_bounds__(kRedBlock) k_refresh_tail(int V, const void *b
         acc[1] += d[0];
         acc[2] += d[1];
     }
-    grid_reduce<3>(acc, rs, rs.result, [=](double t, const double *) { refresh_update(t, sc); });
+    grid_reduce<3>(acc, rs, rs.result, [=](double t, const double *) { refresh_update(t, sc, rep, seq); });
 }
 
 // The step kernels for all members of a lockstep group: member blockIdx.y,
@@ -1002,6 +1115,8 @@ __global__ void __launch_bounds__(kRedBlock) k_lo_group_finalize(int nblk, const
 // 2j+1 of each site; FP64 plane k holds component k.
 __global__ void k_hp_add_lo(long long n, int V, double2 *x, float4 *xlo)
 {
+    griddep_wait();
+    griddep_launch_dependents();
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x) {
         const long long j = i / V, site = i - j * V;
@@ -1018,6 +1133,7 @@ __global__ void k_hp_add_lo(long long n, int V, double2 *x, float4 *xlo)
 }  // namespace
 
 #define WC_GRID(n) reduce_grid(S.red, (n)), kRedBlock, 0, S.stream
+#define WC_STEP(n) dim3(reduce_grid(S.red, (n))), kRedBlock, S.stream
 
 cudaError_t bicg_init(wc_lattice lat, SolverState &S, const double2 *b, double2 *r, double2 *rhat, double2 *p,
                       double2 *v)
@@ -1029,34 +1145,34 @@ cudaError_t bicg_init(wc_lattice lat, SolverState &S, const double2 *b, double2 
 cudaError_t bicg_p(wc_lattice lat, SolverState &S, const double2 *r, const double2 *v, double2 *p, bool norm)
 {
     const long long n = 12LL * lat->g.V;
-    if (norm) k_bicg_p<true><<<WC_GRID(n)>>>(n, r, v, p, S.red, S.scal);
-    else k_bicg_p<false><<<WC_GRID(n)>>>(n, r, v, p, S.red, S.scal);
+    if (norm) launch_step(S.pdl, k_bicg_p<true>, WC_STEP(n), n, r, v, p, S.red, S.scal);
+    else launch_step(S.pdl, k_bicg_p<false>, WC_STEP(n), n, r, v, p, S.red, S.scal);
     return cudaGetLastError();
 }
 cudaError_t bicg_alpha(wc_lattice lat, SolverState &S, const double2 *rhat, const double2 *v)
 {
     const long long n = 12LL * lat->g.V;
-    k_bicg_alpha<<<WC_GRID(n)>>>(n, rhat, v, S.red, S.scal);
+    launch_step(S.pdl, k_bicg_alpha, WC_STEP(n), n, rhat, v, S.red, S.scal);
     return cudaGetLastError();
 }
 cudaError_t bicg_s(wc_lattice lat, SolverState &S, const double2 *r, const double2 *v, double2 *s, bool norm)
 {
     const long long n = 12LL * lat->g.V;
-    if (norm) k_bicg_s<true><<<WC_GRID(n)>>>(n, r, v, s, S.red, S.scal);
-    else k_bicg_s<false><<<WC_GRID(n)>>>(n, r, v, s, S.red, S.scal);
+    if (norm) launch_step(S.pdl, k_bicg_s<true>, WC_STEP(n), n, r, v, s, S.red, S.scal);
+    else launch_step(S.pdl, k_bicg_s<false>, WC_STEP(n), n, r, v, s, S.red, S.scal);
     return cudaGetLastError();
 }
 cudaError_t bicg_omega(wc_lattice lat, SolverState &S, const double2 *t, const double2 *s)
 {
     const long long n = 12LL * lat->g.V;
-    k_bicg_omega<<<WC_GRID(n)>>>(n, t, s, S.red, S.scal);
+    launch_step(S.pdl, k_bicg_omega, WC_STEP(n), n, t, s, S.red, S.scal);
     return cudaGetLastError();
 }
 cudaError_t bicg_xr(wc_lattice lat, SolverState &S, double2 *x, const double2 *phat, const double2 *shat,
                     const double2 *s, const double2 *t, double2 *r, const double2 *rhat)
 {
     const long long n = 12LL * lat->g.V;
-    k_bicg_xr<<<WC_GRID(n)>>>(n, x, phat, shat, s, t, r, rhat, S.red, S.scal);
+    launch_step(S.pdl, k_bicg_xr, WC_STEP(n), n, x, phat, shat, s, t, r, rhat, S.red, S.scal, S.rep, S.seq);
     return cudaGetLastError();
 }
 cudaError_t residual(wc_lattice lat, SolverState &S, const double2 *b, double2 *r)
@@ -1088,9 +1204,9 @@ cudaError_t lo_p(wc_lattice lat, SolverState &S, wc_field r, wc_field v, wc_fiel
     const int V = lat->g.V;
     const long long n = 6LL * V;
     if (half_vectors(r))
-        k_lo_p_h<<<WC_GRID_SITES(V)>>>(V, hf(r), hf(v), hf(p), S.scal);
+        launch_step(S.pdl, k_lo_p_h, WC_STEP(V), V, hf(r), hf(v), hf(p), S.scal);
     else
-        k_lo_p<<<WC_GRID(n)>>>(n, f4(r), f4(v), f4(p), S.scal);
+        launch_step(S.pdl, k_lo_p, WC_STEP(n), n, f4(r), f4(v), f4(p), S.scal);
     return cudaGetLastError();
 }
 cudaError_t lo_alpha(wc_lattice lat, SolverState &S, wc_field rhat, wc_field v)
@@ -1098,9 +1214,9 @@ cudaError_t lo_alpha(wc_lattice lat, SolverState &S, wc_field rhat, wc_field v)
     const int V = lat->g.V;
     const long long n = 6LL * V;
     if (half_vectors(v))
-        k_lo_alpha_h<<<WC_GRID_SITES(V)>>>(V, hf(rhat), hf(v), S.red, S.scal);
+        launch_step(S.pdl, k_lo_alpha_h, WC_STEP(V), V, hf(rhat), hf(v), S.red, S.scal);
     else
-        k_lo_alpha<<<WC_GRID(n)>>>(n, f4(rhat), f4(v), S.red, S.scal);
+        launch_step(S.pdl, k_lo_alpha, WC_STEP(n), n, f4(rhat), f4(v), S.red, S.scal);
     return cudaGetLastError();
 }
 cudaError_t lo_s(wc_lattice lat, SolverState &S, wc_field r, wc_field v, wc_field s)
@@ -1108,9 +1224,9 @@ cudaError_t lo_s(wc_lattice lat, SolverState &S, wc_field r, wc_field v, wc_fiel
     const int V = lat->g.V;
     const long long n = 6LL * V;
     if (half_vectors(r))
-        k_lo_s_h<<<WC_GRID_SITES(V)>>>(V, hf(r), hf(v), hf(s), S.scal);
+        launch_step(S.pdl, k_lo_s_h, WC_STEP(V), V, hf(r), hf(v), hf(s), S.scal);
     else
-        k_lo_s<<<WC_GRID(n)>>>(n, f4(r), f4(v), f4(s), S.scal);
+        launch_step(S.pdl, k_lo_s, WC_STEP(n), n, f4(r), f4(v), f4(s), S.scal);
     return cudaGetLastError();
 }
 cudaError_t lo_omega(wc_lattice lat, SolverState &S, wc_field t, wc_field s)
@@ -1118,9 +1234,9 @@ cudaError_t lo_omega(wc_lattice lat, SolverState &S, wc_field t, wc_field s)
     const int V = lat->g.V;
     const long long n = 6LL * V;
     if (half_vectors(t))
-        k_lo_omega_h<<<WC_GRID_SITES(V)>>>(V, hf(t), hf(s), S.red, S.scal);
+        launch_step(S.pdl, k_lo_omega_h, WC_STEP(V), V, hf(t), hf(s), S.red, S.scal);
     else
-        k_lo_omega<<<WC_GRID(n)>>>(n, f4(t), f4(s), S.red, S.scal);
+        launch_step(S.pdl, k_lo_omega, WC_STEP(n), n, f4(t), f4(s), S.red, S.scal);
     return cudaGetLastError();
 }
 cudaError_t lo_xr(wc_lattice lat, SolverState &S, wc_field xlo, wc_field phat, wc_field shat, wc_field s,
@@ -1129,21 +1245,21 @@ cudaError_t lo_xr(wc_lattice lat, SolverState &S, wc_field xlo, wc_field phat, w
     const int V = lat->g.V;
     const long long n = 6LL * V;
     if (half_vectors(r))
-        k_lo_xr_h<<<WC_GRID_SITES(V)>>>(V, f4(xlo), hf(phat), hf(shat), hf(s), hf(t), hf(r), hf(rhat), S.red,
-                                         S.scal);
+        launch_step(S.pdl, k_lo_xr_h, WC_STEP(V), V, f4(xlo), hf(phat), hf(shat), hf(s), hf(t), hf(r), hf(rhat), S.red,
+                                         S.scal, S.rep, S.seq);
     else
-        k_lo_xr<<<WC_GRID(n)>>>(n, f4(xlo), f4(phat), f4(shat), f4(s), f4(t), f4(r), f4(rhat), S.red, S.scal);
+        launch_step(S.pdl, k_lo_xr, WC_STEP(n), n, f4(xlo), f4(phat), f4(shat), f4(s), f4(t), f4(r), f4(rhat), S.red, S.scal, S.rep, S.seq);
     return cudaGetLastError();
 }
 cudaError_t refresh_tail(wc_lattice lat, SolverState &S, const wc_field b, wc_field r_hp, wc_field r, wc_field rhat)
 {
     const int V = lat->g.V;
     if (half_vectors(r))
-        k_refresh_tail<P16><<<WC_GRID_SITES(V)>>>(V, b->data, r_hp->data, r->data, r->nrm, rhat->data, rhat->nrm,
-                                                  S.red, S.scal);
+        launch_step(S.pdl, k_refresh_tail<P16>, WC_STEP(V), V, b->data, r_hp->data, r->data, r->nrm, rhat->data, rhat->nrm,
+                                                  S.red, S.scal, S.rep, S.seq);
     else
-        k_refresh_tail<P32><<<WC_GRID_SITES(V)>>>(V, b->data, r_hp->data, r->data, nullptr, rhat->data, nullptr,
-                                                  S.red, S.scal);
+        launch_step(S.pdl, k_refresh_tail<P32>, WC_STEP(V), V, b->data, r_hp->data, r->data, nullptr, rhat->data, nullptr,
+                                                  S.red, S.scal, S.rep, S.seq);
     return cudaGetLastError();
 }
 LoMember lo_member(SolverState &S, wc_field r, wc_field rhat, wc_field p, wc_field v, wc_field s, wc_field t,
@@ -1202,11 +1318,17 @@ cudaError_t lo_group_finalize(LoStep step, int m, int nblk, const double *part, 
     return cudaGetLastError();
 }
 
+cudaError_t track(SolverState &S, int mode, double tol2, double d2, double defer2, double rr)
+{
+    k_track<<<1, 1, 0, S.stream>>>(S.scal, mode, tol2, d2, defer2, rr);
+    return cudaGetLastError();
+}
+
 cudaError_t hp_add_lo(wc_lattice lat, SolverState &S, double2 *x, wc_field xlo_f)
 {
     float4 *xlo = f4(xlo_f);
     const long long n = 6LL * lat->g.V;
-    k_hp_add_lo<<<WC_GRID(n)>>>(n, lat->g.V, x, xlo);
+    launch_step(S.pdl, k_hp_add_lo, WC_STEP(n), n, lat->g.V, x, xlo);
     return cudaGetLastError();
 }
 

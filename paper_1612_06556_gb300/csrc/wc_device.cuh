@@ -185,6 +185,23 @@ struct CloverStore {
     uint4 *c16 = nullptr;     // [9][V]
 };
 
+// Programmatic dependent launch: a kernel launched with the programmatic
+// stream serialization attribute may start while the previous kernel of the
+// stream drains; griddepcontrol.wait then blocks until that kernel has
+// completed and its writes are visible.  launch_dependents lets the next
+// such kernel start once every CTA of this grid is running.  Both are no-ops
+// for kernels launched without the attribute.
+__device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void griddep_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;"); }
+
+// What the host reads after each step of a solve: written by the step's last
+// kernel into page-locked host memory, seq last.
+struct StepReport {
+    double rr;
+    int flags, action;
+    volatile unsigned long long seq;
+};
+
 // Scalars of one BiCGStab solve, resident on the device.
 struct SolverScalars {
     double2 rho, rho0, alpha, omega, beta;
@@ -192,11 +209,20 @@ struct SolverScalars {
     double pp, ss;   // |p|^2, |s|^2 (scales of the defect correction)
     double tt;
     int flags;       // bit 0: breakdown, bit 1: non-finite value
-    int skip;        // lockstep batch: 1 = this right-hand side has stopped, and
-                     // the low-precision step kernels return at once (0 otherwise)
+    int skip;        // 1: the kernels of a solver step return at once -- this
+                     // right-hand side of a lockstep batch has stopped, or a
+                     // host-driven solve has to act before its next step
+    // host-driven solves: what ends or interrupts the run of steps, decided
+    // with the last sum of a step (track_step)
+    int track;       // TRACK_*
+    int action;      // ACT_*
+    double tol2, d2, defer2;        // |r|^2 to reach; delta^2; see reliable_bicgstab
+    double rmax2, prev, rr_refresh; // largest |r|^2 since the last refresh, of the last step, of the refresh
 };
 
 enum { FLAG_BREAKDOWN = 1, FLAG_NAN = 2 };
+enum { TRACK_NONE = 0, TRACK_FP64 = 1, TRACK_RELIABLE = 2, TRACK_INNER = 3 };
+enum { ACT_NONE = 0, ACT_STOP = 1, ACT_DIVERGED = 2, ACT_BREAKDOWN = 3, ACT_DEFER = 4, ACT_REFRESH = 5 };
 
 // Reduction scratch: per-block partial sums and a completion ticket.
 struct ReduceScratch {

@@ -67,15 +67,6 @@ __device__ __forceinline__ void apply_site(const Geom &g, const TileMap &tm, int
     if (valid) apply_site_at<P, KIND>(g, x, U, C, in, in_nrm, out, out_nrm, kappa);
 }
 
-// Programmatic dependent launch: a kernel launched with the programmatic
-// stream serialization attribute may start while the previous kernel of the
-// stream drains; griddepcontrol.wait then blocks until that kernel has
-// completed and its writes are visible.  launch_dependents lets the next
-// such kernel start once every CTA of this grid is running.  Both are no-ops
-// for kernels launched without the attribute.
-__device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void griddep_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;"); }
-
 // Bulk L2 prefetch of n bytes at p (both 16-byte multiples); only a cache
 // hint: L2 is the point of coherence, so data still being written by the
 // previous kernel is read correctly by the loads after griddep_wait().
@@ -114,7 +105,7 @@ constexpr int kFlagPdl = 1;
 template <class P, int KIND, int MINB>
 __global__ void __launch_bounds__(kApplyMaxThreads, MINB)
     k_apply(Geom g, TileMap tm, int nlogical, GaugeStore U, CloverStore C, const void *in, const float *in_nrm,
-            void *out, float *out_nrm, double kappa, int flags)
+            void *out, float *out_nrm, double kappa, int flags, const int *skip)
 {
     if (flags & kFlagPdl) {
         const int x0 = blockIdx.x * blockDim.x;
@@ -123,6 +114,7 @@ __global__ void __launch_bounds__(kApplyMaxThreads, MINB)
         griddep_wait();
     }
     griddep_launch_dependents();
+    if (skip && *skip) return;
     for (int blk = blockIdx.x; blk < nlogical; blk += gridDim.x)
         apply_site<P, KIND>(g, tm, blk, U, C, in, in_nrm, out, out_nrm, kappa);
 }
@@ -132,8 +124,11 @@ __global__ void __launch_bounds__(kApplyMaxThreads, MINB)
 // registers measured the same).
 template <int KIND>
 __global__ void __launch_bounds__(kSplit64 * kSplit64Sites, 3)
-    k_apply_split64(Geom g, GaugeStore U, CloverStore C, const void *in, void *out, double kappa)
+    k_apply_split64(Geom g, GaugeStore U, CloverStore C, const void *in, void *out, double kappa, const int *skip)
 {
+    griddep_wait();
+    griddep_launch_dependents();
+    if (skip && *skip) return;
     __shared__ Split64Mem sm;
     const int s = threadIdx.x & (kSplit64Sites - 1), w = threadIdx.x / kSplit64Sites;
     const int x = blockIdx.x * kSplit64Sites + s;
@@ -217,20 +212,21 @@ int resident_ctas(K kernel, int threads)
     return n;
 }
 
-cudaError_t launch_split64(wc_lattice lat, wc_field out, wc_field in, int kind, cudaStream_t stream)
+cudaError_t launch_split64(wc_lattice lat, wc_field out, wc_field in, int kind, cudaStream_t stream,
+                           const int *skip, bool pdl)
 {
     const Geom &g = lat->g;
-    const dim3 grid((g.V + kSplit64Sites - 1) / kSplit64Sites), block(kSplit64 * kSplit64Sites);
-    if (kind == 0) k_apply_split64<0><<<grid, block, 0, stream>>>(g, lat->gauge, lat->clover, in->data, out->data, lat->kappa);
-    else if (kind == 1) k_apply_split64<1><<<grid, block, 0, stream>>>(g, lat->gauge, lat->clover, in->data, out->data, lat->kappa);
-    else k_apply_split64<2><<<grid, block, 0, stream>>>(g, lat->gauge, lat->clover, in->data, out->data, lat->kappa);
-    return cudaGetLastError();
+    const dim3 grid((g.V + kSplit64Sites - 1) / kSplit64Sites);
+    const auto kern = kind == 0 ? k_apply_split64<0> : kind == 1 ? k_apply_split64<1> : k_apply_split64<2>;
+    return launch_step(pdl && pdl_grid(grid.x), kern, grid, kSplit64 * kSplit64Sites, stream, g, lat->gauge, lat->clover, in->data,
+                       out->data, lat->kappa, skip);
 }
 
 template <class P>
-cudaError_t launch_shape(wc_lattice lat, wc_field out, wc_field in, int kind, int index, cudaStream_t stream)
+cudaError_t launch_shape(wc_lattice lat, wc_field out, wc_field in, int kind, int index, cudaStream_t stream,
+                         const int *skip = nullptr, bool step_pdl = false)
 {
-    if (index == kShapeSplit64) return launch_split64(lat, out, in, kind, stream);
+    if (index == kShapeSplit64) return launch_split64(lat, out, in, kind, stream, skip, step_pdl);
     const ApplyShape &sh = kShapes[index];
     const Geom &g = lat->g;
     TileMap tm{};
@@ -267,10 +263,10 @@ cudaError_t launch_shape(wc_lattice lat, wc_field out, wc_field in, int kind, in
             cfg.attrs = attr;                                                                                 \
             cfg.numAttrs = 1;                                                                                 \
             return cudaLaunchKernelEx(&cfg, kern, g, tm, nlogical, lat->gauge, lat->clover, in->data,         \
-                                      (const float *)in->nrm, out->data, out->nrm, lat->kappa, kFlagPdl);    \
+                                      (const float *)in->nrm, out->data, out->nrm, lat->kappa, kFlagPdl, skip); \
         }                                                                                                     \
         kern<<<grid, sh.threads, 0, stream>>>(g, tm, nlogical, lat->gauge, lat->clover, in->data, in->nrm,    \
-                                              out->data, out->nrm, lat->kappa, 0);                            \
+                                              out->data, out->nrm, lat->kappa, 0, skip);                      \
     } while (0)
     // minimum resident CTAs of 256 threads for caps 1 and 2 (1: not compiled)
     constexpr bool c1 = P::kCaps & 1, c2 = P::kCaps & 2;
@@ -358,7 +354,8 @@ int tune_shape(wc_lattice lat, wc_field out, wc_field in, int kind, cudaStream_t
 }
 
 template <class P>
-cudaError_t launch_apply_p(wc_lattice lat, wc_field out, wc_field in, int kind, cudaStream_t stream)
+cudaError_t launch_apply_p(wc_lattice lat, wc_field out, wc_field in, int kind, cudaStream_t stream,
+                           const int *skip, bool pdl)
 {
     // the double-FP32 operator has its own entry (precision code 3)
     const int pcode = std::is_same<P, PDF>::value ? 3 : (int)in->prec;
@@ -384,7 +381,7 @@ cudaError_t launch_apply_p(wc_lattice lat, wc_field out, wc_field in, int kind, 
             g_shape_choice[key] = choice;
         }
     }
-    return launch_shape<P>(lat, out, in, kind, choice, stream);
+    return launch_shape<P>(lat, out, in, kind, choice, stream, skip, pdl);
 }
 
 // ------------------------------------------------------------------------
@@ -468,15 +465,16 @@ bool apply_shape(wc_lattice lat, wc_prec prec, int kind, int force, int out[6])
 
 int apply_shape_count() { return kNumShapes; }
 
-cudaError_t launch_apply(wc_lattice lat, wc_field out, wc_field in, int kind, cudaStream_t stream)
+cudaError_t launch_apply(wc_lattice lat, wc_field out, wc_field in, int kind, cudaStream_t stream, const int *skip,
+                         bool pdl)
 {
-    if (lat->schur_parent) return launch_schur(lat, out, in, kind == 1, stream);   // half lattice: M^
+    if (lat->schur_parent) return launch_schur(lat, out, in, kind == 1, stream, nullptr, skip, pdl);   // half lattice: M^
     switch (in->prec) {
     case WC_F64:
-        return lat->fp64_arith == WC_ARITH_DF32 ? launch_apply_p<PDF>(lat, out, in, kind, stream)
-                                                : launch_apply_p<P64>(lat, out, in, kind, stream);
-    case WC_F32: return launch_apply_p<P32>(lat, out, in, kind, stream);
-    default: return launch_apply_p<P16>(lat, out, in, kind, stream);
+        return lat->fp64_arith == WC_ARITH_DF32 ? launch_apply_p<PDF>(lat, out, in, kind, stream, skip, pdl)
+                                                : launch_apply_p<P64>(lat, out, in, kind, stream, skip, pdl);
+    case WC_F32: return launch_apply_p<P32>(lat, out, in, kind, stream, skip, pdl);
+    default: return launch_apply_p<P16>(lat, out, in, kind, stream, skip, pdl);
     }
 }
 

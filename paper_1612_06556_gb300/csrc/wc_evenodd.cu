@@ -380,8 +380,11 @@ template <class P, int DAG, int MODE>
 __global__ void __launch_bounds__(128, P::kEoMinBlocks) k_eo(Geom g, int p, GaugeStore U, CloverStore C, CloverStore Ci,
                                             const void *hin, const float *hin_nrm, const void *vin,
                                             const float *vin_nrm, void *out, float *out_nrm, void *out2,
-                                            double beta)
+                                            double beta, const int *skip)
 {
+    griddep_wait();
+    griddep_launch_dependents();
+    if (skip && *skip) return;
     using R = typename P::real;
     const int Vh = g.V >> 1;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -424,8 +427,11 @@ __global__ void __launch_bounds__(128, P::kEoMinBlocks) k_eo(Geom g, int p, Gaug
 template <int DAG, int MODE>
 __global__ void __launch_bounds__(kSplit64 * kSplit64Sites, 3)
     k_eo_split64(Geom g, int p, GaugeStore U, CloverStore C, CloverStore Ci, const void *hin, const double2 *vin,
-                 double2 *out, double2 *out2, double beta)
+                 double2 *out, double2 *out2, double beta, const int *skip)
 {
+    griddep_wait();
+    griddep_launch_dependents();
+    if (skip && *skip) return;
     __shared__ Split64Mem sm;
     const int Vh = g.V >> 1;
     const int s = threadIdx.x & (kSplit64Sites - 1), w = threadIdx.x / kSplit64Sites;
@@ -548,17 +554,17 @@ __global__ void k_merge(Geom g, const void *ev, const float *ev_nrm, const void 
 template <int DAG>
 cudaError_t launch_eo_split64(const wc_lattice_s *full, int parity, int mode, const wc_field_s *hin,
                               const wc_field_s *vin, wc_field_s *out, double beta, cudaStream_t stream,
-                              wc_field_s *out2)
+                              wc_field_s *out2, const int *skip, bool pdl)
 {
     if (mode == 5 && (!out2 || out2->prec != WC_F64)) return cudaErrorInvalidValue;
     const int Vh = full->g.V >> 1;
-    const dim3 grid((Vh + kSplit64Sites - 1) / kSplit64Sites), block(kSplit64 * kSplit64Sites);
+    const dim3 grid((Vh + kSplit64Sites - 1) / kSplit64Sites);
     const void *hd = hin ? hin->data : nullptr;
     const double2 *vd = vin ? static_cast<const double2 *>(vin->data) : nullptr;
     double2 *od = static_cast<double2 *>(out->data), *o2 = out2 ? static_cast<double2 *>(out2->data) : nullptr;
 #define WC_EO(M)                                                                                                 \
-    k_eo_split64<DAG, M><<<grid, block, 0, stream>>>(full->g, parity, full->gauge, full->ceo, full->cinv, hd, vd, \
-                                                     od, o2, beta)
+    return launch_step(pdl && pdl_grid(grid.x), k_eo_split64<DAG, M>, grid, kSplit64 *kSplit64Sites, stream, full->g, parity, full->gauge, \
+                       full->ceo, full->cinv, hd, vd, od, o2, beta, skip)
     switch (mode) {
     case 0: WC_EO(0); break;
     case 1: WC_EO(1); break;
@@ -568,26 +574,26 @@ cudaError_t launch_eo_split64(const wc_lattice_s *full, int parity, int mode, co
     default: WC_EO(5);
     }
 #undef WC_EO
-    return cudaGetLastError();
 }
 
 template <class P, int DAG>
 cudaError_t launch_eo_p(const wc_lattice_s *full, int parity, int mode, const wc_field_s *hin, const wc_field_s *vin,
-                        wc_field_s *out, double beta, cudaStream_t stream, wc_field_s *out2)
+                        wc_field_s *out, double beta, cudaStream_t stream, wc_field_s *out2, const int *skip,
+                        bool pdl)
 {
     const int Vh = full->g.V >> 1;
     // CTAs of 128 sites; on small lattices (fewer than two such CTAs per SM)
     // CTAs of 32, so that the sites spread over more SMs
     const int threads = Vh < 2 * 128 * sm_count() ? 32 : 128;
-    dim3 grid((Vh + threads - 1) / threads), block(threads);
+    const dim3 grid((Vh + threads - 1) / threads);
     const void *hd = hin ? hin->data : nullptr;
     const float *hn = hin ? hin->nrm : nullptr;
     const void *vd = vin ? vin->data : nullptr;
     const float *vn = vin ? vin->nrm : nullptr;
     void *o2 = out2 ? out2->data : nullptr;
 #define WC_EO(M)                                                                                                \
-    k_eo<P, DAG, M><<<grid, block, 0, stream>>>(full->g, parity, full->gauge, full->ceo, full->cinv, hd, hn,    \
-                                                vd, vn, out->data, out->nrm, o2, beta)
+    return launch_step(pdl && pdl_grid(grid.x), k_eo<P, DAG, M>, grid, threads, stream, full->g, parity, full->gauge, full->ceo,    \
+                       full->cinv, hd, hn, vd, vn, out->data, out->nrm, o2, beta, skip)
     switch (mode) {
     case 0: WC_EO(0); break;
     case 1: WC_EO(1); break;
@@ -603,27 +609,27 @@ cudaError_t launch_eo_p(const wc_lattice_s *full, int parity, int mode, const wc
         }
     }
 #undef WC_EO
-    return cudaGetLastError();
 }
 
 }  // namespace
 
 // one parity-stencil step on half fields of the full lattice `full`
 cudaError_t launch_eo(const wc_lattice_s *full, int parity, int mode, int dagger, const wc_field_s *hin,
-                      const wc_field_s *vin, wc_field_s *out, double beta, cudaStream_t stream, wc_field_s *out2)
+                      const wc_field_s *vin, wc_field_s *out, double beta, cudaStream_t stream, wc_field_s *out2,
+                      const int *skip, bool pdl)
 {
     const wc_prec pr = out->prec;
     if (pr == WC_F64 && full->fp64_arith == WC_ARITH_DF32)
-        return dagger ? launch_eo_p<PDF, 1>(full, parity, mode, hin, vin, out, beta, stream, out2)
-                      : launch_eo_p<PDF, 0>(full, parity, mode, hin, vin, out, beta, stream, out2);
+        return dagger ? launch_eo_p<PDF, 1>(full, parity, mode, hin, vin, out, beta, stream, out2, skip, pdl)
+                      : launch_eo_p<PDF, 0>(full, parity, mode, hin, vin, out, beta, stream, out2, skip, pdl);
     if (pr == WC_F64)
-        return dagger ? launch_eo_split64<1>(full, parity, mode, hin, vin, out, beta, stream, out2)
-                      : launch_eo_split64<0>(full, parity, mode, hin, vin, out, beta, stream, out2);
+        return dagger ? launch_eo_split64<1>(full, parity, mode, hin, vin, out, beta, stream, out2, skip, pdl)
+                      : launch_eo_split64<0>(full, parity, mode, hin, vin, out, beta, stream, out2, skip, pdl);
     if (pr == WC_F32)
-        return dagger ? launch_eo_p<P32, 1>(full, parity, mode, hin, vin, out, beta, stream, out2)
-                      : launch_eo_p<P32, 0>(full, parity, mode, hin, vin, out, beta, stream, out2);
-    return dagger ? launch_eo_p<P16, 1>(full, parity, mode, hin, vin, out, beta, stream, out2)
-                  : launch_eo_p<P16, 0>(full, parity, mode, hin, vin, out, beta, stream, out2);
+        return dagger ? launch_eo_p<P32, 1>(full, parity, mode, hin, vin, out, beta, stream, out2, skip, pdl)
+                      : launch_eo_p<P32, 0>(full, parity, mode, hin, vin, out, beta, stream, out2, skip, pdl);
+    return dagger ? launch_eo_p<P16, 1>(full, parity, mode, hin, vin, out, beta, stream, out2, skip, pdl)
+                  : launch_eo_p<P16, 0>(full, parity, mode, hin, vin, out, beta, stream, out2, skip, pdl);
 }
 
 // od may be NULL: only the even half is written
@@ -662,19 +668,22 @@ cudaError_t launch_merge(const wc_lattice_s *full, const wc_field_s *ev, const w
 
 // out = M^ in (or M^+ in) on half fields of the half lattice `half`: t = A_oo^-1 H_oe in,
 // out = A_ee in - k^2 H_eo t.  t: the half lattice's scratch of out's precision.
-cudaError_t launch_schur(wc_lattice half, wc_field out, wc_field in, int dagger, cudaStream_t stream, wc_field tmp)
+cudaError_t launch_schur(wc_lattice half, wc_field out, wc_field in, int dagger, cudaStream_t stream, wc_field tmp,
+                         const int *skip, bool pdl)
 {
     const wc_lattice_s *full = half->schur_parent;
     wc_field_s *t = tmp ? tmp : half->schur_tmp[out->prec];
-    cudaError_t e = launch_eo(full, 1, 0, dagger, in, nullptr, t, 0.0, stream);
-    if (e == cudaSuccess) e = launch_eo(full, 0, 1, dagger, t, in, out, -full->kappa * full->kappa, stream);
+    cudaError_t e = launch_eo(full, 1, 0, dagger, in, nullptr, t, 0.0, stream, nullptr, skip, pdl);
+    if (e == cudaSuccess)
+        e = launch_eo(full, 0, 1, dagger, t, in, out, -full->kappa * full->kappa, stream, nullptr, skip, pdl);
     return e;
 }
 
-cudaError_t launch_apply(wc_lattice lat, wc_field out, wc_field in, int kind, SolverState &S)
+cudaError_t launch_apply(wc_lattice lat, wc_field out, wc_field in, int kind, SolverState &S, bool step)
 {
-    if (!lat->schur_parent) return launch_apply(lat, out, in, kind, S.stream);
-    return launch_schur(lat, out, in, kind == 1, S.stream, S.work[kSchurSlot + out->prec]);
+    const int *skip = step ? &S.scal->skip : nullptr;
+    if (!lat->schur_parent) return launch_apply(lat, out, in, kind, S.stream, skip, S.pdl);
+    return launch_schur(lat, out, in, kind == 1, S.stream, S.work[kSchurSlot + out->prec], skip, S.pdl);
 }
 
 wc_status build_clover_inverse(wc_lattice lat)

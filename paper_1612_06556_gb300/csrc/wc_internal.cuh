@@ -45,6 +45,7 @@ namespace wc {
 // even and odd halves of the final full residual of an even-odd solve) and
 // the stream the solve is queued on.  A lattice owns one for its single-RHS
 // calls; a batched solve creates one per RHS.
+constexpr int kReportSlots = 2;
 constexpr int kSchurSlot = 24;
 constexpr int kEoSlot = 27;
 constexpr int kRasEoSlot = 32;
@@ -53,6 +54,12 @@ constexpr int kEoResSlot = 44;
 struct SolverState {
     SolverScalars *scal = nullptr;
     SolverScalars *scal_host = nullptr;
+    StepReport *report = nullptr;   // pinned, kReportSlots of them
+    // set while a step of a host-driven solve is queued: its report, and
+    // programmatic dependent launches (launch_step)
+    StepReport *rep = nullptr;
+    unsigned long long seq = 0;
+    bool pdl = false;
     ReduceScratch red;
     wc_field_s *work[46] = {};
     cudaStream_t stream = nullptr;
@@ -138,12 +145,15 @@ inline size_t spinor_bytes(wc_prec p, int V)
 }
 
 // launchers implemented in the .cu files (all asynchronous on `stream`)
+// skip (nullable): a device flag whose nonzero value makes the kernels return
+// at once
 cudaError_t launch_apply(wc_lattice lat, wc_field out, wc_field in, int kind /*0 M, 1 Mdag, 2 H*/,
-                         cudaStream_t stream);
+                         cudaStream_t stream, const int *skip = nullptr, bool pdl = false);
 // The operator of a solve on S.stream; on a half lattice (M^) the odd-site
 // intermediate is the state's own (slot kSchurSlot + precision, when it
-// exists), so that solves on one lattice may run concurrently.
-cudaError_t launch_apply(wc_lattice lat, wc_field out, wc_field in, int kind, SolverState &S);
+// exists), so that solves on one lattice may run concurrently.  step: the
+// operator of a solver step, which returns at once when S.scal->skip is set.
+cudaError_t launch_apply(wc_lattice lat, wc_field out, wc_field in, int kind, SolverState &S, bool step = false);
 cudaError_t launch_copy(wc_lattice lat, wc_field dst, wc_field src, double scale, const double *dev_scale,
                         int invert_scale, cudaStream_t stream);
 // RAS on block Schur complements, on half-lattice (even-site) fields of the
@@ -158,6 +168,33 @@ cudaError_t launch_ras(wc_lattice lat, wc_field out, wc_field in, const wc_ras_p
 cudaError_t launch_build_clover(wc_lattice lat, double csw, double kappa, cudaStream_t stream);
 
 bool apply_shape(wc_lattice lat, wc_prec prec, int kind, int force, int out[6]);
+
+// Whether an operator kernel of so many CTAs is launched as a programmatic
+// dependent: its CTAs are then placed while those of the kernel before it
+// still hold their SMs, so that a grid of about one CTA per SM gets two on
+// some SMs and none on others (FP64 M at 8^4 12 -> 20 us, 76 instead of 63 us
+// per solver step); from two per SM on it gains (FP32 even-odd reliable step
+// at 16^4 103 -> 97 us, 16^3x32 131 -> 122, 24^3x32 287 -> 276).
+inline bool pdl_grid(unsigned ctas) { return (int)ctas >= 2 * sm_count(); }
+
+// Launch of a solver-step kernel; pdl: as a programmatic dependent of the
+// kernel before it on the stream (the kernel begins with griddep_wait), which
+// takes its launch latency out of the chain of small kernels.  Not while the
+// stream is being captured.
+template <class... K, class... A>
+cudaError_t launch_step(bool pdl, void (*kernel)(K...), dim3 grid, int block, cudaStream_t stream, A... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(block);
+    cfg.stream = stream;
+    cfg.attrs = attr;
+    cfg.numAttrs = pdl ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, K(args)...);
+}
 
 // WC_OK when the whole-lattice operator of lat can be applied: gauge field
 // (and, with need_clover, the clover term) loaded, and lat not a sub-domain,
@@ -192,11 +229,11 @@ int schur_multi_blocks(wc_lattice half);
 // tmp: a half-lattice field of out's precision for the odd-site
 // intermediate (nullptr: the half lattice's own, shared by its callers)
 cudaError_t launch_schur(wc_lattice half, wc_field out, wc_field in, int dagger, cudaStream_t stream,
-                         wc_field tmp = nullptr);
+                         wc_field tmp = nullptr, const int *skip = nullptr, bool pdl = false);
 // out2: the second output of mode 5 (nullptr for the other modes)
 cudaError_t launch_eo(const wc_lattice_s *full, int parity, int mode, int dagger, const wc_field_s *hin,
                       const wc_field_s *vin, wc_field_s *out, double beta, cudaStream_t stream,
-                      wc_field_s *out2 = nullptr);
+                      wc_field_s *out2 = nullptr, const int *skip = nullptr, bool pdl = false);
 cudaError_t launch_split(const wc_lattice_s *full, const wc_field_s *f, wc_field_s *ev, wc_field_s *od,
                          cudaStream_t stream);
 cudaError_t launch_merge(const wc_lattice_s *full, const wc_field_s *ev, const wc_field_s *od, wc_field_s *f,

@@ -17,8 +17,12 @@
 // correction in which the low-precision preconditioner only ever sees a
 // unit-norm vector, while residuals, inner products and the solution update
 // stay FP64 on the GPU.  Every scalar (rho, alpha, omega, beta, norms) is
-// computed on the device by the last block of the fused reduction kernels;
-// the host reads one small struct per iteration to test convergence.
+// computed on the device by the last block of the fused reduction kernels,
+// and so is whether the host has to act (convergence, a refresh, breakdown).
+// The host reads one small struct per step; without a preconditioner it has
+// queued the next step before it waits for this one's (StepQueue): a step
+// that must not run finds the skip word set and its kernels return at once.
+// Waiting first had left the GPU idle for 25 to 30 us per step.
 //
 // The other drivers here: the reliable-update solver (the same recurrence
 // in FP32 with FP64 refreshes of x and r), the nested three-level solver
@@ -27,6 +31,7 @@
 #include <math.h>
 #include <stdlib.h>
 
+#include <atomic>
 #include <chrono>
 #include <new>
 
@@ -83,6 +88,65 @@ wc_status read_scalars(wc_lattice lat, SolverState &S)
     if (st == WC_OK) st = check_cuda(lat, cudaStreamSynchronize(S.stream), "sync(scalars)");
     return st;
 }
+
+namespace {
+
+// Steps of a host-driven solve in the order they are queued, each reporting
+// into its slot of page-locked memory (no copy, event or synchronisation on
+// the stream, which would also break the chain of dependent launches).
+// ahead: the step after the one that is waited for is queued first.
+struct StepQueue {
+    wc_lattice lat;
+    SolverState &S;
+    bool ahead;
+    unsigned long long due[kReportSlots] = {};
+    int head = 0;       // slot of the oldest step not waited for
+    int queued = 0;
+
+    template <class Enqueue>
+    wc_status push(Enqueue enqueue)
+    {
+        const int slot = (head + queued) % kReportSlots;
+        due[slot] = ++S.seq;
+        S.rep = &S.report[slot];
+        S.pdl = true;
+        const wc_status st = enqueue();
+        S.rep = nullptr;
+        S.pdl = false;
+        if (st == WC_OK) ++queued;
+        return st;
+    }
+    wc_status pop(StepReport *h)
+    {
+        StepReport &r = S.report[head];
+        for (unsigned spin = 1; r.seq != due[head]; ++spin) {
+            if (spin % 4096 != 0) continue;
+            // an error on the stream would leave the report unwritten
+            const cudaError_t e = cudaStreamQuery(S.stream);
+            if (e == cudaErrorNotReady || (e == cudaSuccess && r.seq == due[head])) continue;
+            return check_cuda(lat, e == cudaSuccess ? cudaErrorUnknown : e, "solver step");
+        }
+        std::atomic_thread_fence(std::memory_order_acquire);
+        h->rr = r.rr;
+        h->flags = r.flags;
+        h->action = r.action;
+        head = (head + 1) % kReportSlots;
+        --queued;
+        return WC_OK;
+    }
+    // the scalars after the next step; more: another step may follow it
+    template <class Enqueue>
+    wc_status step(Enqueue enqueue, bool more, StepReport *h)
+    {
+        wc_status st = queued ? WC_OK : push(enqueue);
+        if (st == WC_OK && ahead && more) st = push(enqueue);
+        return st == WC_OK ? pop(h) : st;
+    }
+    // a step queued ahead of the host's action does not run
+    void drop() { queued = 0; }
+};
+
+}  // namespace
 
 static wc_status eo_ras_temps(wc_lattice lat, SolverState &S, wc_prec prec);
 
@@ -177,11 +241,11 @@ wc_status enqueue_iteration(wc_lattice lat, SolverState &S, const wc_solve_param
     const bool norm = w.phat != w.p;   // a preconditioner scales its input by |p|, |s|
     wc_status st = check_cuda(lat, bicg_p(lat, S, d2(w.r), d2(w.v), d2(w.p), norm), "bicg_p");
     if (st == WC_OK) st = apply_precond(lat, S, p, kind, w, w.p, w.phat, &S.scal->pp);
-    if (st == WC_OK) st = check_cuda(lat, launch_apply(lat, w.v, w.phat, kind, S), "apply");
+    if (st == WC_OK) st = check_cuda(lat, launch_apply(lat, w.v, w.phat, kind, S, true), "apply");
     if (st == WC_OK) st = check_cuda(lat, bicg_alpha(lat, S, d2(w.rhat), d2(w.v)), "bicg_alpha");
     if (st == WC_OK) st = check_cuda(lat, bicg_s(lat, S, d2(w.r), d2(w.v), d2(w.s), norm), "bicg_s");
     if (st == WC_OK) st = apply_precond(lat, S, p, kind, w, w.s, w.shat, &S.scal->ss);
-    if (st == WC_OK) st = check_cuda(lat, launch_apply(lat, w.t, w.shat, kind, S), "apply");
+    if (st == WC_OK) st = check_cuda(lat, launch_apply(lat, w.t, w.shat, kind, S, true), "apply");
     if (st == WC_OK) st = check_cuda(lat, bicg_omega(lat, S, d2(w.t), d2(w.s)), "bicg_omega");
     if (st == WC_OK)
         st = check_cuda(lat, bicg_xr(lat, S, d2(x), d2(w.phat), d2(w.shat), d2(w.s), d2(w.t), d2(w.r), d2(w.rhat)),
@@ -390,6 +454,11 @@ static wc_status bicgstab_impl(wc_lattice lat, SolverState &S, int kind, wc_fiel
     if (iters_done == 0) st = x_is_zero(lat, S, x, &x_zero);
     if (st != WC_OK) return st;
 
+    // a preconditioned step takes milliseconds: nothing to gain ahead of it
+    StepQueue q{lat, S, p.precond == WC_PRECOND_NONE && p.solver != WC_SOLVER_NESTED};
+    st = check_cuda(lat, track(S, TRACK_FP64, tol2), "track");
+    if (st != WC_OK) return st;
+    const auto step = [&] { return enqueue_iteration(lat, S, p, kind, x, w); };
     for (int restart = 0; restart <= p.max_restarts; ++restart) {
         inf.restarts = restart;
         st = enqueue_init(lat, S, kind, x, b, w, restart == 0 && x_zero);
@@ -406,11 +475,11 @@ static wc_status bicgstab_impl(wc_lattice lat, SolverState &S, int kind, wc_fiel
         }
         bool breakdown = false;
         while (inf.iters < p.max_iter) {
-            st = enqueue_iteration(lat, S, p, kind, x, w);
-            if (st == WC_OK) st = read_scalars(lat, S);
+            StepReport h;
+            st = q.step(step, inf.iters + 1 < p.max_iter, &h);
             if (st != WC_OK) return st;
             ++inf.iters;
-            const SolverScalars &h = *S.scal_host;
+            if (h.action != ACT_NONE) q.drop();
             if (h.flags & FLAG_NAN) {
                 result = set_error(lat, WC_ERR_NAN, "non-finite value in BiCGStab");
                 break;
@@ -505,11 +574,11 @@ wc_status enqueue_lo_iteration(wc_lattice lat, SolverState &S, const wc_solve_pa
 {
     wc_status st = check_cuda(lat, lo_p(lat, S, w.r, w.v, w.p), "lo_p");
     if (st == WC_OK) st = lo_precond(lat, S, p, kind, w, w.p, w.phat);
-    if (st == WC_OK) st = check_cuda(lat, launch_apply(lat, w.v, w.phat, kind, S), "apply");
+    if (st == WC_OK) st = check_cuda(lat, launch_apply(lat, w.v, w.phat, kind, S, true), "apply");
     if (st == WC_OK) st = check_cuda(lat, lo_alpha(lat, S, w.rhat, w.v), "lo_alpha");
     if (st == WC_OK) st = check_cuda(lat, lo_s(lat, S, w.r, w.v, w.s), "lo_s");
     if (st == WC_OK) st = lo_precond(lat, S, p, kind, w, w.s, w.shat);
-    if (st == WC_OK) st = check_cuda(lat, launch_apply(lat, w.t, w.shat, kind, S), "apply");
+    if (st == WC_OK) st = check_cuda(lat, launch_apply(lat, w.t, w.shat, kind, S, true), "apply");
     if (st == WC_OK) st = check_cuda(lat, lo_omega(lat, S, w.t, w.s), "lo_omega");
     if (st == WC_OK)
         st = check_cuda(lat, lo_xr(lat, S, w.xlo, w.phat, w.shat, w.s, w.t, w.r, w.rhat),
@@ -583,20 +652,20 @@ static wc_status nested_inner(wc_lattice lat, SolverState &S, const wc_solve_par
     const double itol = (p.inner_tol > 0.0 && p.inner_tol < 1.0) ? p.inner_tol : 0.01;
     const int iters = p.inner_iters > 0 ? p.inner_iters : 100;
     st = check_cuda(lat, launch_copy(lat, w.r, u, 1.0, norm2_dev, 1, I.stream), "cast to unit norm");
+    if (st == WC_OK) st = check_cuda(lat, track(I, TRACK_INNER, 0.0, itol * itol), "track");
     if (st == WC_OK)
         st = check_cuda(lat, lo_init(lat, I, w.r, w.rhat, w.p, w.v, w.xlo), "lo_init");
-    if (st == WC_OK) st = read_scalars(lat, I);
     if (st != WC_OK) return st;
-    const double rr0 = I.scal_host->rr;
-    for (int it = 0; it < iters && rr0 > 0.0; ++it) {
-        st = enqueue_lo_iteration(lat, I, p, kind, w);
-        if (st == WC_OK) st = read_scalars(lat, I);
+    // (a residual that is zero or not finite stops before the first step)
+    StepQueue q{lat, I, p.precond == WC_PRECOND_NONE};
+    StepReport h{};
+    for (int it = 0; it < iters; ++it) {
+        st = q.step([&] { return enqueue_lo_iteration(lat, I, p, kind, w); }, it + 1 < iters, &h);
         if (st != WC_OK) return st;
-        const SolverScalars &h = *I.scal_host;
-        if (h.flags != 0 || !(h.rr > itol * itol * rr0)) break;
+        if (h.action != ACT_NONE) break;
     }
     // a blown-up inner solve (NaN) falls back to the identity preconditioner
-    if (I.scal_host->flags & FLAG_NAN)
+    if (h.flags & FLAG_NAN)
         return check_cuda(lat, launch_copy(lat, uhat, u, 1.0, nullptr, 0, I.stream), "copy");
     return check_cuda(lat, launch_copy(lat, uhat, w.xlo, 1.0, norm2_dev, 0, I.stream), "cast back");
 }
@@ -666,31 +735,32 @@ wc_status reliable_bicgstab(wc_lattice lat, SolverState &S, int kind, wc_field x
             break;
         }
         st = check_cuda(lat, launch_copy(lat, w.r, r_hp, 1.0, nullptr, 0, S.stream), "cast residual");
+        if (st == WC_OK) st = check_cuda(lat, track(S, TRACK_RELIABLE, tol2, d2, defer_rr, rr_true), "track");
         if (st == WC_OK)
             st = check_cuda(lat, lo_init(lat, S, w.r, w.rhat, w.p, w.v, w.xlo), "lo_init");
         if (st != WC_OK) return st;
-        double rmax2 = rr_true, rr_refresh = rr_true, rr_prev = rr_true;
         bool breakdown = false, converged = false, diverged = false;
+        // a preconditioned step takes milliseconds: nothing to gain ahead of it
+        StepQueue q{lat, S, p.precond == WC_PRECOND_NONE};
+        const auto step = [&] { return enqueue_lo_iteration(lat, S, p, kind, w); };
         while (inf.iters < p.max_iter) {
-            st = enqueue_lo_iteration(lat, S, p, kind, w);
-            if (st == WC_OK) st = read_scalars(lat, S);
+            StepReport h;
+            st = q.step(step, inf.iters + 1 < p.max_iter, &h);
             if (st != WC_OK) return st;
             ++inf.iters;
-            const SolverScalars h = *S.scal_host;
-            if ((h.flags & FLAG_NAN) || h.rr > 1e8 * rr_refresh) {
+            if (h.action == ACT_NONE) continue;
+            q.drop();
+            if (h.action == ACT_DIVERGED) {
                 // the FP32 recurrence blew up: drop its pending correction and
                 // restart from the last FP64-verified iterate
                 diverged = true;
                 break;
             }
-            if (h.flags & FLAG_BREAKDOWN) {
+            if (h.action == ACT_BREAKDOWN) {
                 breakdown = true;
                 break;
             }
-            if (h.rr > rmax2) rmax2 = h.rr;
-            const double prev = rr_prev;
-            rr_prev = h.rr;
-            if (defer_rr > 0.0 && h.rr <= defer_rr) {
+            if (h.action == ACT_DEFER) {
                 // the caller confirms with its own true residual: fold the
                 // correction only
                 st = check_cuda(lat, hp_add_lo(lat, S, static_cast<double2 *>(x->data), w.xlo), "hp_add_lo");
@@ -700,25 +770,20 @@ wc_status reliable_bicgstab(wc_lattice lat, SolverState &S, int kind, wc_field x
                 converged = true;
                 break;
             }
-            // deferring, a recurrence below tol but above defer_rr refreshes
-            // only once it stops decreasing
-            const bool at_tol = h.rr <= tol2 && (defer_rr <= 0.0 || !(h.rr < prev));
-            if (h.rr <= d2 * rmax2 || at_tol) {
-                // reliable update: fold the FP32 correction into the FP64
-                // solution and restart the recurrence from the true residual
-                // (its low-precision copy and rho in the same pass)
-                st = enqueue_refresh_full(lat, S, kind, x, b, r_hp, w);
-                if (st == WC_OK) st = read_scalars(lat, S);
-                if (st != WC_OK) return st;
-                rr_true = S.scal_host->rr;
-                inf.true_rel_resid = sqrt(rr_true / bb);
-                if (rr_true <= tol2) {
-                    converged = true;
-                    break;
-                }
-                rmax2 = rr_true;
-                rr_refresh = rr_true;
-                rr_prev = rr_true;
+            // reliable update: fold the FP32 correction into the FP64
+            // solution and restart the recurrence from the true residual
+            // (its low-precision copy and rho in the same pass); the step
+            // after it runs unless the true residual has reached tol
+            st = q.push([&] { return enqueue_refresh_full(lat, S, kind, x, b, r_hp, w); });
+            if (st == WC_OK && q.ahead && inf.iters < p.max_iter) st = q.push(step);
+            if (st == WC_OK) st = q.pop(&h);
+            if (st != WC_OK) return st;
+            rr_true = h.rr;
+            inf.true_rel_resid = sqrt(rr_true / bb);
+            if (rr_true <= tol2) {
+                q.drop();
+                converged = true;
+                break;
             }
         }
         if (converged) {

@@ -44,6 +44,9 @@ cudaError_t lo_xr(wc_lattice lat, SolverState &S, wc_field xlo, wc_field phat, w
 // r_hp = b - r_hp (r_hp holds op x), rr = |r_hp|^2, r = r_hp in the Krylov
 // storage, rho = <rhat, r> and beta recomputed: one pass (FP64 b and r_hp)
 cudaError_t refresh_tail(wc_lattice lat, SolverState &S, const wc_field b, wc_field r_hp, wc_field r, wc_field rhat);
+// what ends a run of steps of a host-driven solve (see SolverScalars), with
+// |r|^2 = rr at its start; clears skip
+cudaError_t track(SolverState &S, int mode, double tol2 = 0.0, double d2 = 0.0, double defer2 = 0.0, double rr = 0.0);
 // x (FP64) += xlo (FP32); xlo = 0
 cudaError_t hp_add_lo(wc_lattice lat, SolverState &S, double2 *x, wc_field xlo);
 

@@ -154,3 +154,70 @@ def test_reductions_of_one_two_and_three_sums(dims, prec):
     got = lat.axpy_norm(0.5 - 0.25j, a, b)
     tol = {0: 1e-13, 1: 2e-7, 2: 2e-3}[prec]     # the norm is of the values before they are stored
     assert abs(got - np.sum(np.abs(b.store(np.zeros((V, 4, 3), complex))) ** 2)) <= tol * got
+
+
+SOLVERS = [dict(), dict(even_odd=True), dict(solver=1), dict(solver=1, even_odd=True), dict(solver=1, even_odd=True, krylov_prec=2),
+           dict(solver=2, even_odd=True), dict(solver=2)]
+
+
+@pytest.mark.parametrize("kw", SOLVERS)
+def test_steps_queued_ahead_do_not_run(kw):
+    """A host-driven solve queues a step before it has seen the last one's
+    outcome: it stops after exactly max_iter steps, goes on from there, and
+    two solves of one source take the same steps to the same bits."""
+    dims, kappa, csw, tbc = (6, 4, 4, 8), 0.12, 1.0, -1
+    U = synth.exp_links(dims, 0.3, 91)
+    lat = make_lattice(dims, U, csw, kappa, tbc)
+    src = synth.gaussian_source(dims, 92)
+    b = lat.field(0).load(src)
+    xs, infos = [], []
+    for _ in range(2):
+        x = lat.field(0)
+        infos.append(lat.solve(x, b, tol=1e-10, **kw))
+        xs.append(x.store(np.zeros_like(src)))
+    assert infos[0].iters == infos[1].iters and np.array_equal(xs[0], xs[1])
+    r = src - oracle.apply_M(dims, tbc, kappa, csw, U, xs[0])
+    assert np.linalg.norm(r) <= 1.5e-10 * np.linalg.norm(src)
+    for n in (1, 2, 3):
+        if n >= infos[0].iters:
+            continue
+        x = lat.field(0)
+        info = lat.solve(x, b, tol=1e-10, max_iter=n, check=False, **kw)
+        assert info.iters == n and info.status != 0
+        assert lat.solve(x, b, tol=1e-10, **kw).status == 0
+
+
+def test_solves_of_two_threads_on_their_own_streams():
+    """Each thread solves on its own lattice and stream; the solutions have
+    the bits of the same solves one after the other."""
+    import threading
+
+    import torch
+    dims, kappa, csw, tbc = (4, 6, 4, 8), 0.12, 1.0, -1
+    kinds = [dict(), dict(solver=1, even_odd=True), dict(solver=2, even_odd=True)]
+    lats, srcs, streams = [], [], []
+    for k in range(3):
+        streams.append(torch.cuda.Stream())
+        U = synth.exp_links(dims, 0.3, 95 + k)
+        lats.append(wc().Lattice(dims, tbc, stream=streams[k]).load_gauge(U).load_clover(csw, kappa))
+        srcs.append(synth.gaussian_source(dims, 97 + k))
+
+    def solve(k, out):
+        for _ in range(4):
+            x, b = lats[k].field(0), lats[k].field(0).load(srcs[k])
+            lats[k].solve(x, b, tol=1e-10, **kinds[k])
+            out.append(x.store(np.zeros_like(srcs[k])))
+
+    alone = [[] for _ in kinds]
+    for k in range(3):
+        solve(k, alone[k])
+    together = [[] for _ in kinds]
+    threads = [threading.Thread(target=solve, args=(k, together[k])) for k in range(3)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    for k in range(3):
+        assert len(together[k]) == 4
+        for a in together[k]:
+            assert np.array_equal(a, alone[k][0])
