@@ -231,6 +231,9 @@ void free_clover(CloverStore &c)
     cudaFree(c.cdf);
     cudaFree(c.c32);
     cudaFree(c.c16);
+    cudaFree(c.a32);
+    cudaFree(c.a16);
+    cudaFree(c.a16b);
     c = CloverStore{};
 }
 
@@ -253,6 +256,16 @@ wc_status check_field(wc_lattice lat, wc_field f, const char *name)
 }
 
 }  // namespace
+
+// the FP32 and FP16 parts of a store of A
+wc_status alloc_clover_a(wc_lattice lat, CloverStore &c)
+{
+    const size_t V = lat->g.V;
+    wc_status st = check_cuda(lat, dalloc(&c.a32, sizeof(float4) * 13 * V), "cudaMalloc(clover)");
+    if (st == WC_OK) st = check_cuda(lat, dalloc(&c.a16, sizeof(uint4) * 6 * V), "cudaMalloc(clover)");
+    if (st == WC_OK) st = check_cuda(lat, dalloc(&c.a16b, sizeof(uint2) * V), "cudaMalloc(clover)");
+    return st;
+}
 
 // readers of the per-translation-unit violation counters (checked build)
 std::vector<cudaError_t (*)(unsigned *)> &check_readers()
@@ -661,8 +674,7 @@ wc_status wc_load_clover(wc_lattice lat, double csw, double kappa)
     if (!c.c64) {
         st = check_cuda(lat, dalloc(&c.c64, sizeof(double2) * 36 * (size_t)V), "cudaMalloc(clover)");
         if (st == WC_OK) st = check_cuda(lat, dalloc(&c.cdf, sizeof(float4) * 36 * (size_t)V), "cudaMalloc(clover)");
-        if (st == WC_OK) st = check_cuda(lat, dalloc(&c.c32, sizeof(float4) * 18 * (size_t)V), "cudaMalloc(clover)");
-        if (st == WC_OK) st = check_cuda(lat, dalloc(&c.c16, sizeof(uint4) * 9 * (size_t)V), "cudaMalloc(clover)");
+        if (st == WC_OK) st = alloc_clover_a(lat, c);
         if (st != WC_OK) {
             free_clover(c);
             return st;

@@ -308,7 +308,7 @@ __global__ void __launch_bounds__(128) k_store_clover(int V, CloverStore C)
     if (x >= V) return;
     double r[36];
     P64::load_clover(C, V, x, b, r);
-    store_clover_block<false>(C, V, x, b, r);
+    store_clover_a<false>(C, V, x, b, r);
 }
 
 }  // namespace

@@ -20,7 +20,18 @@
 //           index 3*s_local + colour): per block 6 real diagonal entries then
 //           the 15 complex entries below the diagonal in row order
 //           (1,0) (2,0) (2,1) (3,0) ... (5,4); 72 reals per site
-//           F64: double2 [36][V]       F32: float4 [18][V]    F16: uint4 [9][V]
+//           F64: double2 [36][V]; the inverse A^-1 of the even-odd kernels
+//           F32: float4 [18][V]    F16: uint4 [9][V]
+//           A itself in FP32 and FP16: a block is 1 + [[P, Q^+], [Q, -P]]
+//           with P traceless Hermitian and Q any 3x3 matrix (field strengths
+//           times csw kappa), 26 reals: the words (P00, P11), P10, P20, P21,
+//           Q00, Q01, ... Q22 of two reals each, 13 per block
+//           F32: float4 [13][V], block b in planes 6 b .. 6 b + 5 and half b
+//           of plane 12;   F16: uint4 [6][V], block b in planes 3 b .. 3 b +
+//           2, and uint2 [V], word b: the block's last
+//           208 / 104 bytes a site instead of 288 / 144, and the stored
+//           values are the small ones: rounding 1 + P to the storage had
+//           cost up to 2^-24 / 2^-11 of 1
 //   FP64 links and clover are also kept split into double-FP32 pairs (same
 //   planes, float4 = hi, lo of the real part, hi, lo of the imaginary part)
 //   for the double-FP32 operator (wc_df.cuh).
@@ -181,8 +192,11 @@ struct GaugeStore {
 struct CloverStore {
     double2 *c64 = nullptr;   // [36][V]
     float4 *cdf = nullptr;    // [36][V] c64 as double-FP32 pairs
-    float4 *c32 = nullptr;    // [18][V]
-    uint4 *c16 = nullptr;     // [9][V]
+    float4 *c32 = nullptr;    // [18][V]  the inverse only
+    uint4 *c16 = nullptr;     // [9][V]   the inverse only
+    float4 *a32 = nullptr;    // [13][V]  A only
+    uint4 *a16 = nullptr;     // [6][V]   A only
+    uint2 *a16b = nullptr;    // [V]      A only
 };
 
 // Programmatic dependent launch: a kernel launched with the programmatic
@@ -560,16 +574,45 @@ struct P16 {
     }
 };
 
-// one packed block (36 reals) at position pos of a clover store in the other
-// precisions, and in FP64 too when F64; 16-byte stores, but for the 8 bytes
-// of each block in the binary16 word the two blocks share
+// one packed block of A (36 reals) at position pos of its store in the other
+// precisions, and in FP64 too when F64
 template <bool F64>
-__device__ __forceinline__ void store_clover_block(const CloverStore &S, int V, int pos, int b, const double r[36])
+__device__ __forceinline__ void store_clover_a(const CloverStore &S, int V, int pos, int b, const double r[36])
 {
 #pragma unroll
     for (int q = 0; q < 18; ++q) {
         const double2 v = make_double2(r[2 * q], r[2 * q + 1]);
         if (F64) S.c64[((size_t)b * 18 + q) * V + pos] = v;
+        S.cdf[((size_t)b * 18 + q) * V + pos] = df_pack(v);
+    }
+    // words of two reals: (P00, P11), the lower entries of P, the rows of Q
+    constexpr int at[13] = {0, 3, 4, 5, 6, 7, 8, 9, 10, 11, 13, 14, 15};
+    float2 w[13];
+    w[0] = make_float2((float)(r[0] - 1.0), (float)(r[1] - 1.0));
+#pragma unroll
+    for (int q = 1; q < 13; ++q) w[q] = make_float2((float)r[2 * at[q]], (float)r[2 * at[q] + 1]);
+#pragma unroll
+    for (int q = 0; q < 6; ++q)
+        S.a32[((size_t)b * 6 + q) * V + pos] = make_float4(w[2 * q].x, w[2 * q].y, w[2 * q + 1].x, w[2 * q + 1].y);
+    reinterpret_cast<float2 *>(S.a32 + (size_t)12 * V + pos)[b] = w[12];
+    unsigned h[13];
+#pragma unroll
+    for (int q = 0; q < 13; ++q) h[q] = c2h(w[q].x, w[q].y);
+#pragma unroll
+    for (int q = 0; q < 3; ++q)
+        S.a16[((size_t)b * 3 + q) * V + pos] = make_uint4(h[4 * q], h[4 * q + 1], h[4 * q + 2], h[4 * q + 3]);
+    reinterpret_cast<unsigned *>(S.a16b + pos)[b] = h[12];
+}
+
+// one packed block (36 reals) of the inverse at position pos of its store, in
+// all precisions; 16-byte stores, but for the 8 bytes of each block in the
+// binary16 word the two blocks share
+__device__ __forceinline__ void store_clover_block(const CloverStore &S, int V, int pos, int b, const double r[36])
+{
+#pragma unroll
+    for (int q = 0; q < 18; ++q) {
+        const double2 v = make_double2(r[2 * q], r[2 * q + 1]);
+        S.c64[((size_t)b * 18 + q) * V + pos] = v;
         S.cdf[((size_t)b * 18 + q) * V + pos] = df_pack(v);
     }
 #pragma unroll
@@ -604,6 +647,78 @@ __device__ __forceinline__ void clover_block_mul(const R r[36], const cx<R> v[6]
             y[i] = cfma(l, v[j], y[i]);        // lower entry (i, j)
             y[j] = cfma_conj(l, v[i], y[j]);   // its mirror (j, i) = conj(l)
         }
+    }
+}
+
+// y = s y + A v for block b of A in FP32 or FP16 storage: word(k) returns the
+// reals of word k as float2.  HAVE: y holds a value (s ignored otherwise).
+// The words are used as they arrive, so that few of them are live together.
+template <bool HAVE, class Word>
+__device__ __forceinline__ void clover_a_mul(Word word, const cx<float> v[6], cx<float> y[6], float s)
+{
+    const float2 d01 = word(0);
+    const float d[3] = {d01.x, d01.y, -(d01.x + d01.y)};
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+        const float di = i < 3 ? d[i] : -d[i - 3];
+        const cx<float> u = HAVE ? mkc(fmaf(s, y[i].re, v[i].re), fmaf(s, y[i].im, v[i].im)) : v[i];
+        y[i] = mkc(fmaf(di, v[i].re, u.re), fmaf(di, v[i].im, u.im));
+    }
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {   // P10, P20, P21
+        const int i = q == 0 ? 1 : 2, j = q == 2 ? 1 : 0;
+        const float2 e = word(1 + q);
+        const cx<float> l = mkc(e.x, e.y);
+        y[i] = cfma(l, v[j], y[i]);
+        y[j] = cfma_conj(l, v[i], y[j]);
+        y[3 + i] = cfma(l, -v[3 + j], y[3 + i]);
+        y[3 + j] = cfma_conj(l, -v[3 + i], y[3 + j]);
+    }
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            const float2 e = word(4 + 3 * i + j);
+            const cx<float> l = mkc(e.x, e.y);
+            y[3 + i] = cfma(l, v[j], y[3 + i]);
+            y[j] = cfma_conj(l, v[3 + i], y[j]);
+        }
+}
+
+// word k of block b at position pos
+__device__ __forceinline__ float2 clover_a_word(P32, const CloverStore &C, int V, int pos, int b, int k)
+{
+    const float4 w = __ldg(C.a32 + (size_t)(k < 12 ? 6 * b + (k >> 1) : 12) * V + pos);
+    return (k < 12 ? k & 1 : b) ? make_float2(w.z, w.w) : make_float2(w.x, w.y);
+}
+
+// binary16 word k (two halves) of block b at position pos
+__device__ __forceinline__ unsigned clover_a_half(const CloverStore &C, int V, int pos, int b, int k)
+{
+    if (k == 12) {
+        const uint2 w = __ldg(C.a16b + pos);
+        return b ? w.y : w.x;
+    }
+    const uint4 w = __ldg(C.a16 + (size_t)(3 * b + (k >> 2)) * V + pos);
+    return (k & 3) == 0 ? w.x : (k & 3) == 1 ? w.y : (k & 3) == 2 ? w.z : w.w;
+}
+__device__ __forceinline__ float2 clover_a_word(P16, const CloverStore &C, int V, int pos, int b, int k)
+{
+    const cx<float> f = h2c(clover_a_half(C, V, pos, b, k));
+    return make_float2(f.re, f.im);
+}
+
+// y = A v for block b at position pos of the store of A
+template <class P>
+__device__ __forceinline__ void clover_a(const CloverStore &C, int V, int pos, int b, const cx<typename P::real> v[6],
+                                         cx<typename P::real> y[6])
+{
+    if constexpr (sizeof(typename P::real) == sizeof(float)) {
+        clover_a_mul<false>([&](int k) { return clover_a_word(P(), C, V, pos, b, k); }, v, y, 0.f);
+    } else {
+        typename P::real r[36];
+        P::load_clover(C, V, pos, b, r);
+        clover_block_mul(r, v, y);
     }
 }
 

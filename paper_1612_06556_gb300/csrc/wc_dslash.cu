@@ -85,11 +85,12 @@ __device__ __forceinline__ void prefetch_block(const Geom &g, const GaugeStore &
     const size_t V = g.V;
     if (std::is_same<P, P32>::value) {
         if (i < 12) prefetch_l2(U.u32 + i * V + x0, 16u * n);                   // [4][3][V] float4
-        else if (i < 30) prefetch_l2(C.c32 + (i - 12) * V + x0, 16u * n);      // [18][V] float4
+        else if (i < 25) prefetch_l2(C.a32 + (i - 12) * V + x0, 16u * n);      // [13][V] float4
     } else if (std::is_same<P, P16>::value) {
         if (i < 4) prefetch_l2(U.u16a + i * V + x0, 16u * n);                   // [4][V] uint4
         else if (i < 8) prefetch_l2(U.u16b + (i - 4) * V + x0, 8u * n);        // [4][V] uint2
-        else if (i < 17) prefetch_l2(C.c16 + (i - 8) * V + x0, 16u * n);       // [9][V] uint4
+        else if (i < 14) prefetch_l2(C.a16 + (i - 8) * V + x0, 16u * n);       // [6][V] uint4
+        else if (i < 15) prefetch_l2(C.a16b + x0, 8u * n);                     // [V] uint2
     }
 }
 

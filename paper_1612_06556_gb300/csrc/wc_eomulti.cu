@@ -48,22 +48,21 @@ struct EoMultiArgs {
     double *part;
 };
 
-// the staged words of one site: 4 forward and 4 backward links, the block
+// the staged words of one site: 4 forward and 4 backward links, then the
+// block of the pass: A^-1 (MODE 0) or A (MODE 1, see CloverStore)
 template <class P>
 struct EoMStage;
 
 template <>
 struct EoMStage<P32> {
     using W = float4;
-    static constexpr int kWords = 24 + 18;   // links [fwd/bwd][mu][3], block [18]
+    template <int MODE>
+    static constexpr int words = 24 + (MODE == 0 ? 18 : 13);   // links [fwd/bwd][mu][3], block
     static __device__ __forceinline__ W link_word(const GaugeStore &U, int V, int mu, int x, int j)
     {
         return __ldg(U.u32 + ((size_t)mu * 3 + j) * V + x);
     }
-    static __device__ __forceinline__ W block_word(const CloverStore &C, int V, int pos, int q)
-    {
-        return __ldg(C.c32 + (size_t)q * V + pos);
-    }
+    template <int MODE>
     static __device__ __forceinline__ void stage(const GaugeStore &U, const CloverStore &C, int V, int item, int x,
                                                  int xb_mu[4], int pos, W &out)
     {
@@ -72,7 +71,7 @@ struct EoMStage<P32> {
         else if (item < 24)
             out = link_word(U, V, (item - 12) / 3, xb_mu[(item - 12) / 3], (item - 12) % 3);
         else
-            out = block_word(C, V, pos, item - 24);
+            out = __ldg((MODE == 0 ? C.c32 : C.a32) + (size_t)(item - 24) * V + pos);
     }
     // the two stored rows of link lam = 4 bwd + mu
     static __device__ __forceinline__ void rows(const W (*st)[kEoMSites], int s, int lam, cx<float> a[6])
@@ -85,15 +84,28 @@ struct EoMStage<P32> {
             a[2 * j + 1] = mkc(v.z, v.w);
         }
     }
-    static __device__ __forceinline__ void block(const W (*st)[kEoMSites], int s, int b, float r[36])
+    // y = A^-1 v or A v, block b
+    template <int MODE>
+    static __device__ __forceinline__ void block_mul(const W (*st)[kEoMSites], int s, int b, const cx<float> v[6],
+                                                     cx<float> y[6])
     {
+        if (MODE == 0) {
+            float r[36];
 #pragma unroll
-        for (int q = 0; q < 9; ++q) {
-            const float4 v = st[24 + 9 * b + q][s];
-            r[4 * q] = v.x;
-            r[4 * q + 1] = v.y;
-            r[4 * q + 2] = v.z;
-            r[4 * q + 3] = v.w;
+            for (int q = 0; q < 9; ++q) {
+                const float4 w = st[24 + 9 * b + q][s];
+                r[4 * q] = w.x;
+                r[4 * q + 1] = w.y;
+                r[4 * q + 2] = w.z;
+                r[4 * q + 3] = w.w;
+            }
+            clover_block_mul(r, v, y);
+        } else {
+            const auto word = [&](int k) {
+                const float4 w = st[24 + (k < 12 ? 6 * b + (k >> 1) : 12)][s];
+                return (k < 12 ? k & 1 : b) ? make_float2(w.z, w.w) : make_float2(w.x, w.y);
+            };
+            clover_a_mul<false>(word, v, y, 0.f);
         }
     }
 };
@@ -102,8 +114,10 @@ template <>
 struct EoMStage<P16> {
     using W = uint4;
     // links: [fwd/bwd][mu] as (uint4 row 0 + entry (1,0)) then the uint2
-    // (entries (1,1), (1,2)) of two directions per word; block [9]
-    static constexpr int kWords = 8 + 4 + 9;
+    // (entries (1,1), (1,2)) of two directions per word; block [9] or [6 + 1]
+    template <int MODE>
+    static constexpr int words = 8 + 4 + (MODE == 0 ? 9 : 7);
+    template <int MODE>
     static __device__ __forceinline__ void stage(const GaugeStore &U, const CloverStore &C, int V, int item, int x,
                                                  int xb_mu[4], int pos, W &out)
     {
@@ -117,8 +131,13 @@ struct EoMStage<P16> {
             const uint2 a = __ldg(U.u16b + (size_t)mu0 * V + (bwd ? xb_mu[mu0] : x));
             const uint2 b = __ldg(U.u16b + (size_t)(mu0 + 1) * V + (bwd ? xb_mu[mu0 + 1] : x));
             out = make_uint4(a.x, a.y, b.x, b.y);
-        } else {
+        } else if (MODE == 0) {
             out = __ldg(C.c16 + (size_t)(item - 12) * V + pos);
+        } else if (item < 18) {
+            out = __ldg(C.a16 + (size_t)(item - 12) * V + pos);
+        } else {
+            const uint2 a = __ldg(C.a16b + pos);
+            out = make_uint4(a.x, a.y, 0u, 0u);
         }
     }
     static __device__ __forceinline__ void rows(const W (*st)[kEoMSites], int s, int lam, cx<float> a[6])
@@ -134,16 +153,30 @@ struct EoMStage<P16> {
         a[4] = h2c((mu & 1) ? w.z : w.x);
         a[5] = h2c((mu & 1) ? w.w : w.y);
     }
-    static __device__ __forceinline__ void block(const W (*st)[kEoMSites], int s, int b, float r[36])
+    static __device__ __forceinline__ unsigned part(const uint4 &v, int k)
     {
+        return k == 0 ? v.x : k == 1 ? v.y : k == 2 ? v.z : v.w;
+    }
+    template <int MODE>
+    static __device__ __forceinline__ void block_mul(const W (*st)[kEoMSites], int s, int b, const cx<float> v[6],
+                                                     cx<float> y[6])
+    {
+        if (MODE == 0) {
+            float r[36];
 #pragma unroll
-        for (int k = 0; k < 18; ++k) {
-            const int q = 18 * b + k;   // half2 index among the 36 of a site
-            const uint4 v = st[12 + (q >> 2)][s];
-            const unsigned w = (q & 3) == 0 ? v.x : (q & 3) == 1 ? v.y : (q & 3) == 2 ? v.z : v.w;
-            const cx<float> f = h2c(w);
-            r[2 * k] = f.re;
-            r[2 * k + 1] = f.im;
+            for (int k = 0; k < 18; ++k) {
+                const int q = 18 * b + k;   // half2 index among the 36 of a site
+                const cx<float> f = h2c(part(st[12 + (q >> 2)][s], q & 3));
+                r[2 * k] = f.re;
+                r[2 * k + 1] = f.im;
+            }
+            clover_block_mul(r, v, y);
+        } else {
+            const auto word = [&](int k) {
+                const cx<float> f = h2c(k < 12 ? part(st[12 + 3 * b + (k >> 2)][s], k & 3) : part(st[18][s], b));
+                return make_float2(f.re, f.im);
+            };
+            clover_a_mul<false>(word, v, y, 0.f);
         }
     }
 };
@@ -221,7 +254,7 @@ __global__ void __maxnreg__(80) k_eo_multi(Geom g, int p, GaugeStore U, CloverSt
                                                                    double beta)
 {
     using W = typename EoMStage<P>::W;
-    constexpr int NW = EoMStage<P>::kWords;
+    constexpr int NW = EoMStage<P>::template words<MODE>;
     __shared__ W st[NW][kEoMSites];
     __shared__ float2 r3[8][3][kEoMSites];   // third rows of the 8 links
     const int Vh = g.V >> 1;
@@ -238,7 +271,7 @@ __global__ void __maxnreg__(80) k_eo_multi(Geom g, int p, GaugeStore U, CloverSt
             xb[mu] = wc_idx(c[mu] == 0 ? x + (g.L[mu] - 1) * g.stride[mu] : x - g.stride[mu], g.V);
         const int pos = wc_idx(p * Vh + i, g.V);
         for (int item = r; item < NW; item += blockDim.x / kEoMSites)
-            EoMStage<P>::stage(U, Blk, g.V, item, x, xb, pos, st[item][s]);
+            EoMStage<P>::template stage<MODE>(U, Blk, g.V, item, x, xb, pos, st[item][s]);
     }
     __syncthreads();
     // the third row of every staged link, once per site
@@ -274,11 +307,7 @@ __global__ void __maxnreg__(80) k_eo_multi(Geom g, int p, GaugeStore U, CloverSt
         P::load_spinor(a.vin[r], a.vin_nrm[r], FULL ? g.V : Vh, FULL ? x : i, v);
     }
 #pragma unroll
-    for (int b = 0; b < 2; ++b) {
-        float blk[36];
-        EoMStage<P>::block(st, s, b, blk);
-        clover_block_mul(blk, v + 6 * b, o + 6 * b);
-    }
+    for (int b = 0; b < 2; ++b) EoMStage<P>::template block_mul<MODE>(st, s, b, v + 6 * b, o + 6 * b);
     if (MODE == 1)
 #pragma unroll
         for (int k = 0; k < 12; ++k) o[k] = o[k] + bt * h[k];

@@ -246,9 +246,9 @@ __global__ void __launch_bounds__(64) k_clover_invert(Geom g, CloverStore C, Clo
     const int pos = ((c[0] + c[1] + c[2] + c[3]) & 1) * (V >> 1) + (x >> 1);
     double r[36], inv[36];
     P64::load_clover(C, V, x, b, r);
-    store_clover_block<true>(Ce, V, pos, b, r);
+    store_clover_a<true>(Ce, V, pos, b, r);
     if (!invert_block(r, inv) && !invert_block_pivoted(r, inv)) atomicExch(bad, 1);
-    store_clover_block<true>(Ci, V, pos, b, inv);
+    store_clover_block(Ci, V, pos, b, inv);
 }
 
 // ------------------------------------------------------------------------
@@ -303,14 +303,17 @@ __device__ __forceinline__ void eo_hop_dir(const Geom &g, const GaugeStore &U, c
     }
 }
 
-// y = A v at position pos of a parity-ordered clover store (A or A^-1)
-template <class P>
+// y = A v (INV: A^-1 v) at position pos of the parity-ordered store
+template <class P, bool INV>
 __device__ __forceinline__ void clover_eo(const CloverStore &S, int V, int pos, const cx<typename P::real> v[12],
                                           cx<typename P::real> y[12])
 {
     if constexpr (std::is_same<P, PDF>::value) {   // compact form (instruction cache)
         clover_block_rt<P>(S, V, pos, 0, v, y);
         clover_block_rt<P>(S, V, pos, 1, v + 6, y + 6);
+    } else if constexpr (!INV) {
+        clover_a<P>(S, V, pos, 0, v, y);
+        clover_a<P>(S, V, pos, 1, v + 6, y + 6);
     } else {
         using R = typename P::real;
         R r0[36], r1[36];
@@ -349,7 +352,7 @@ __device__ __forceinline__ void eo_tail(const Geom &g, int p, const CloverStore 
     } else {
         P::load_spinor(vin, vin_nrm, Vh, i, v);
         if (MODE == 1) {
-            clover_eo<P>(C, g.V, wc_idx(p * Vh + i, g.V), v, o);
+            clover_eo<P, false>(C, g.V, wc_idx(p * Vh + i, g.V), v, o);
 #pragma unroll
             for (int k = 0; k < 12; ++k) o[k] = o[k] + bt * h[k];
             P::store_spinor(out, out_nrm, Vh, i, o);
@@ -363,13 +366,13 @@ __device__ __forceinline__ void eo_tail(const Geom &g, int p, const CloverStore 
             return;
         }
     }
-    clover_eo<P>(Ci, g.V, wc_idx(p * Vh + i, g.V), v, o);
+    clover_eo<P, true>(Ci, g.V, wc_idx(p * Vh + i, g.V), v, o);
     P::store_spinor(out, out_nrm, Vh, i, o);
     if constexpr (MODE == 5) {
         // the residual of x_o as the caller receives it (the stored value)
         cx<R> y[12];
         P::as_stored(o);
-        clover_eo<P>(C, g.V, wc_idx(p * Vh + i, g.V), o, y);
+        clover_eo<P, false>(C, g.V, wc_idx(p * Vh + i, g.V), o, y);
 #pragma unroll
         for (int k = 0; k < 12; ++k) y[k] = v[k] - y[k];
         P::store_spinor(out2, nullptr, Vh, i, y);
@@ -696,10 +699,14 @@ wc_status build_clover_inverse(wc_lattice lat)
         st = check_cuda(lat, cudaMalloc(&c->c64, sizeof(double2) * 36 * (size_t)V), "cudaMalloc(clover inverse)");
         if (st == WC_OK)
             st = check_cuda(lat, cudaMalloc(&c->cdf, sizeof(float4) * 36 * (size_t)V), "cudaMalloc(clover inverse)");
-        if (st == WC_OK)
-            st = check_cuda(lat, cudaMalloc(&c->c32, sizeof(float4) * 18 * (size_t)V), "cudaMalloc(clover inverse)");
-        if (st == WC_OK)
-            st = check_cuda(lat, cudaMalloc(&c->c16, sizeof(uint4) * 9 * (size_t)V), "cudaMalloc(clover inverse)");
+        if (c == &lat->cinv) {
+            if (st == WC_OK)
+                st = check_cuda(lat, cudaMalloc(&c->c32, sizeof(float4) * 18 * (size_t)V), "cudaMalloc(clover inverse)");
+            if (st == WC_OK)
+                st = check_cuda(lat, cudaMalloc(&c->c16, sizeof(uint4) * 9 * (size_t)V), "cudaMalloc(clover inverse)");
+        } else if (st == WC_OK) {
+            st = alloc_clover_a(lat, *c);
+        }
         if (st != WC_OK) return st;
     }
     int *bad = nullptr;

@@ -234,11 +234,7 @@ __global__ void __launch_bounds__(kHaloThreads) k_apply_surface(Geom g, HaloGeom
         cx<float> p[12];
         P32::load_spinor(in, nullptr, g.V, x, p);
 #pragma unroll
-        for (int b = 0; b < 2; ++b) {
-            float r[36];
-            P32::load_clover(C, g.V, x, b, r);
-            clover_block_mul(r, p + 6 * b, acc + 6 * b);
-        }
+        for (int b = 0; b < 2; ++b) clover_a<P32>(C, g.V, x, b, p + 6 * b, acc + 6 * b);
     }
     const float k = (float)(-kappa);
     constexpr int SF = KIND == 1 ? +1 : -1;
@@ -324,8 +320,9 @@ cudaError_t extract_clover(wc_lattice sub, cudaStream_t stream)
     CloverStore &d = sub->clover;
     cudaError_t e = extract(sub, s.c64, d.c64, 36, stream);
     if (e == cudaSuccess) e = extract(sub, s.cdf, d.cdf, 36, stream);
-    if (e == cudaSuccess) e = extract(sub, s.c32, d.c32, 18, stream);
-    if (e == cudaSuccess) e = extract(sub, s.c16, d.c16, 9, stream);
+    if (e == cudaSuccess) e = extract(sub, s.a32, d.a32, 13, stream);
+    if (e == cudaSuccess) e = extract(sub, s.a16, d.a16, 6, stream);
+    if (e == cudaSuccess) e = extract(sub, s.a16b, d.a16b, 1, stream);
     return e;
 }
 

@@ -2,16 +2,16 @@
 // for up to kMrhsMax fields of one lattice in one launch.
 //
 // The right-hand sides of a propagator share the gauge field and the clover
-// term, which are 480 of the 672 bytes per site of a single FP32 apply.  A
+// term, which are 400 of the 592 bytes per site of a single FP32 apply.  A
 // CTA covers kMrhsSites consecutive sites for all n right-hand sides: it
 // first stages, once, the 4 forward links of its sites, the 4 backward links
 // U_mu(x - mu) of their neighbours and their clover blocks in shared memory
-// (42 float4 per site, coalesced along the sites), then thread (s, r)
+// (37 float4 per site, coalesced along the sites), then thread (s, r)
 // computes site s of right-hand side r, reading links and clover from
 // shared memory and the 9 spinors of field r from global memory (neighbours
 // through L1/L2); the third row of each link is rebuilt once per site
 // after staging.  Compulsory bytes per site and right-hand side:
-// 2 x 96 (spinor in, out) + 480 / n, i.e. 232 B at n = 12 against 672 B for
+// 2 x 96 (spinor in, out) + 400 / n, i.e. 225 B at n = 12 against 592 B for
 // separate applies.  The arithmetic per (site, right-hand side) is that of
 // the single-field operator (spin projection, two-row links with the third
 // row rebuilt, clover first, then -kappa times the hops).
@@ -23,7 +23,7 @@ namespace wc {
 namespace {
 
 constexpr int kMrhsSites = 32;
-constexpr int kStageF4 = 42;   // float4 per site: 12 forward link, 12 backward link, 18 clover
+constexpr int kStageF4 = 37;   // float4 per site: 12 forward link, 12 backward link, 13 clover
 
 struct MrhsArgs {
     int n;
@@ -110,8 +110,8 @@ __global__ void __maxnreg__(80)
                 const int mu = (item - 12) / 3, j = (item - 12) % 3;
                 const int xb = wc_idx(c[mu] == 0 ? x + (g.L[mu] - 1) * g.stride[mu] : x - g.stride[mu], g.V);
                 v = __ldg(U.u32 + ((size_t)mu * 3 + j) * g.V + xb);
-            } else {                                       // clover plane item - 24 of [18][V]
-                v = __ldg(C.c32 + (size_t)(item - 24) * g.V + x);
+            } else {                                       // clover plane item - 24 of [13][V]
+                v = __ldg(C.a32 + (size_t)(item - 24) * g.V + x);
             }
             st[item][s] = v;
         }
@@ -136,16 +136,11 @@ __global__ void __maxnreg__(80)
         P32::load_spinor(in, nullptr, g.V, x, p);
 #pragma unroll
         for (int b = 0; b < 2; ++b) {
-            float cl[36];
-#pragma unroll
-            for (int q = 0; q < 9; ++q) {
-                const float4 v = st[24 + 9 * b + q][s];
-                cl[4 * q] = v.x;
-                cl[4 * q + 1] = v.y;
-                cl[4 * q + 2] = v.z;
-                cl[4 * q + 3] = v.w;
-            }
-            clover_block_mul(cl, p + 6 * b, acc + 6 * b);
+            const auto word = [&](int k) {
+                const float4 w = st[24 + (k < 12 ? 6 * b + (k >> 1) : 12)][s];
+                return (k < 12 ? k & 1 : b) ? make_float2(w.z, w.w) : make_float2(w.x, w.y);
+            };
+            clover_a_mul<false>(word, p + 6 * b, acc + 6 * b, 0.f);
         }
     }
     const float k = (float)(-kappa);

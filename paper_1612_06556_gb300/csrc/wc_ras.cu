@@ -27,7 +27,7 @@
 // other CTA's shared memory (distributed shared memory).  alpha is summed
 // from per-warp FP32 partials of both CTAs in one fixed order, so both CTAs
 // get the same alpha; two cluster barriers per MR step (after the partial
-// sums, after the r update).  The clover term (72 reals per site) does not
+// sums, after the r update).  The clover term (52 reals per site) does not
 // fit beside r and the links and is read from global memory.
 //
 // k_ras (FP16 storage, and block shapes the cluster kernel does not take:
@@ -260,9 +260,7 @@ __global__ void __launch_bounds__(kRasMaxThreads, 1)
             for (int b = 0; b < 2; ++b) {
                 cx<float> rl[6];
                 sm_load_block(r, rg.ne, l, b, rl);
-                float cl[36];
-                P::load_clover(C, V, gs[j], b, cl);
-                clover_block_mul(cl, rl, q + 6 * b);
+                clover_a<P>(C, V, gs[j], b, rl, q + 6 * b);
             }
             // one direction at a time (not unrolled): bounds the registers
             // the scheduler spends on loads in flight
@@ -357,47 +355,6 @@ struct RasLinks<P32> {
         reconstruct_row2(a, c);
     }
 };
-
-// y = s y + B v for one packed Hermitian 6x6 clover block whose 18 complex
-// pairs are produced one at a time by fetch(p) (p = 0..2: the diagonal
-// reals 2p, 2p+1; p = 3..17: lower entry p - 3 in row order), consumed as
-// they arrive so that the 36 reals are never live together
-// (accumulating form: y = s y + B v)
-template <class Fetch>
-__device__ __forceinline__ void clover_block_stream(Fetch fetch, const cx<float> v[6], cx<float> y[6], float s)
-{
-#pragma unroll
-    for (int p = 0; p < 3; ++p) {
-        const float2 d = fetch(p);
-        y[2 * p] = mkc(fmaf(d.x, v[2 * p].re, s * y[2 * p].re), fmaf(d.x, v[2 * p].im, s * y[2 * p].im));
-        y[2 * p + 1] =
-            mkc(fmaf(d.y, v[2 * p + 1].re, s * y[2 * p + 1].re), fmaf(d.y, v[2 * p + 1].im, s * y[2 * p + 1].im));
-    }
-    int k = 3;
-#pragma unroll
-    for (int a = 1; a < 6; ++a) {
-#pragma unroll
-        for (int b = 0; b < a; ++b) {
-            const float2 e = fetch(k++);
-            const cx<float> l = mkc(e.x, e.y);
-            y[a] = cfma(l, v[b], y[a]);        // lower entry (a, b)
-            y[b] = cfma_conj(l, v[a], y[b]);   // its mirror (b, a) = conj(l)
-        }
-    }
-}
-
-// FP32 clover block b of global site x
-__device__ __forceinline__ void clover32_mul(const CloverStore &C, int V, int x, int b, const cx<float> v[6],
-                                             cx<float> y[6], float s)
-{
-    const float4 *p0 = C.c32 + (size_t)b * 9 * V + x;
-    clover_block_stream(
-        [&](int p) {
-            const float4 c = __ldg(p0 + (size_t)(p >> 1) * V);
-            return (p & 1) ? make_float2(c.z, c.w) : make_float2(c.x, c.y);
-        },
-        v, y, s);
-}
 
 // q[c], q[3+c], q[6+c], q[9+c] += the spin reconstruction of the two-spinor
 // components (w0, w1) of colour c (the per-colour form of reconstruct_add)
@@ -615,7 +572,7 @@ __global__ void __cluster_dims__(kRasNC, 1, 1) __launch_bounds__(kRasCThreads, 1
             for (int b = 0; b < 2; ++b) {
                 cx<float> rl[6];
                 sm_load_block(r, np, i, b, rl);
-                clover32_mul(C, V, site, b, rl, q + 6 * b, mk);
+                clover_a_mul<true>([&](int k) { return clover_a_word(P(), C, V, site, b, k); }, rl, q + 6 * b, mk);
             }
             // <q, r> and <q, q>, one plane of r at a time
 #pragma unroll
@@ -873,9 +830,7 @@ __global__ void __launch_bounds__(kRasEoMaxThreads, 1)
             for (int b = 0; b < 2; ++b) {
                 cx<float> rl[6];
                 sm_load_block(r, nh, j, b, rl);
-                float cl[36];
-                P::load_clover(A, V, wc_idx(ge >> 1, V), b, cl);
-                clover_block_mul(cl, rl, q + 6 * b);
+                clover_a<P>(A, V, wc_idx(ge >> 1, V), b, rl, q + 6 * b);
             }
             cx<float> rl[12];
             sm_load(r, nh, j, rl);

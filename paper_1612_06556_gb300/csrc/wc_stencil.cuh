@@ -327,7 +327,7 @@ __device__ __forceinline__ float fma_h(unsigned short a, unsigned short b, float
 __device__ __forceinline__ unsigned short lo16(unsigned w) { return (unsigned short)(w & 0xffffu); }
 __device__ __forceinline__ unsigned short hi16(unsigned w) { return (unsigned short)(w >> 16); }
 
-// y = B v for clover block b (FP16 store, site x) and the unscaled FP16
+// y = A v for clover block b (FP16 store, site x) and the unscaled FP16
 // centre spinor components v (half2 words (re, im), spins 2b, 2b + 1)
 __device__ __forceinline__ void clover_block_h(const CloverStore &C, int V, int x, int b, const unsigned v[6],
                                                cx<float> y[6])
@@ -340,32 +340,34 @@ __device__ __forceinline__ void clover_block_h(const CloverStore &C, int V, int 
         nvr[i] = vr[i] ^ 0x8000u;
         nvi[i] = vi[i] ^ 0x8000u;
     }
-    const uint4 *p = C.c16 + x;
-    auto entry = [&](int q) {   // half2 word q (0..17) of block b
-        const int gq = 18 * b + q;
-        const uint4 w = __ldg(p + (size_t)(gq >> 2) * V);
-        return (gq & 3) == 0 ? w.x : ((gq & 3) == 1 ? w.y : ((gq & 3) == 2 ? w.z : w.w));
+    // y = v + diag(d, -d) v, d = (P00, P11, -(P00 + P11))
+    const cx<float> d01 = h2c(clover_a_half(C, V, x, b, 0));
+    const float d[3] = {d01.re, d01.im, -(d01.re + d01.im)};
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+        const cx<float> f = h2c(v[i]);
+        const float di = i < 3 ? d[i] : -d[i - 3];
+        y[i] = mkc(fmaf(di, f.re, f.re), fmaf(di, f.im, f.im));
+    }
+    // y[a] += l v[c]; y[c] += conj(l) v[a]
+    const auto off = [&](unsigned l, int a, int c) {
+        const unsigned short lr = lo16(l), li = hi16(l);
+        y[a].re = fma_h(lr, vr[c], fma_h(li, nvi[c], y[a].re));
+        y[a].im = fma_h(lr, vi[c], fma_h(li, vr[c], y[a].im));
+        y[c].re = fma_h(lr, vr[a], fma_h(li, vi[a], y[c].re));
+        y[c].im = fma_h(lr, vi[a], fma_h(li, nvr[a], y[c].im));
     };
 #pragma unroll
-    for (int q = 0; q < 3; ++q) {   // diagonal reals 2q, 2q + 1
-        const unsigned d = entry(q);
-        y[2 * q] = mkc(fma_h(lo16(d), vr[2 * q], 0.f), fma_h(lo16(d), vi[2 * q], 0.f));
-        y[2 * q + 1] = mkc(fma_h(hi16(d), vr[2 * q + 1], 0.f), fma_h(hi16(d), vi[2 * q + 1], 0.f));
+    for (int q = 0; q < 3; ++q) {   // P10, P20, P21, and -P below
+        const int i = q == 0 ? 1 : 2, j = q == 2 ? 1 : 0;
+        const unsigned l = clover_a_half(C, V, x, b, 1 + q);
+        off(l, i, j);
+        off(l ^ 0x80008000u, 3 + i, 3 + j);
     }
-    int k = 3;
 #pragma unroll
-    for (int a = 1; a < 6; ++a) {
+    for (int i = 0; i < 3; ++i)
 #pragma unroll
-        for (int c = 0; c < a; ++c) {
-            const unsigned l = entry(k++);
-            const unsigned short lr = lo16(l), li = hi16(l);
-            // y[a] += l v[c]; y[c] += conj(l) v[a]
-            y[a].re = fma_h(lr, vr[c], fma_h(li, nvi[c], y[a].re));
-            y[a].im = fma_h(lr, vi[c], fma_h(li, vr[c], y[a].im));
-            y[c].re = fma_h(lr, vr[a], fma_h(li, vi[a], y[c].re));
-            y[c].im = fma_h(lr, vi[a], fma_h(li, nvr[a], y[c].im));
-        }
-    }
+        for (int j = 0; j < 3; ++j) off(clover_a_half(C, V, x, b, 4 + 3 * i + j), 3 + i, j);
 }
 
 // a + S b for binary16 a, b, exactly rounded to FP32 (the FP32 sum of the
@@ -703,9 +705,7 @@ __device__ __forceinline__ void apply_site_at(const Geom &g, int x, const GaugeS
         P::load_spinor(in, in_nrm, g.V, x, p);
 #pragma unroll
         for (int b = 0; b < 2; ++b) {
-            R r[36];
-            P::load_clover(C, g.V, x, b, r);
-            clover_block_mul(r, p + 6 * b, acc + 6 * b);
+            clover_a<P>(C, g.V, x, b, p + 6 * b, acc + 6 * b);
         }
     }
     const R k = KIND == 2 ? R(1) : R(-kappa);
