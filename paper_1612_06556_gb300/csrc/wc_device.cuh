@@ -287,7 +287,6 @@ struct P64 {
     // cap 2) and the minimum resident 256-thread CTAs that cap 1 stands for
     static constexpr int kCaps = 0;   // ALU-bound on the FP64 pipe: no cap
     static constexpr int kCap1MinBlocks = 1;
-    static constexpr int kEoMinBlocks = 1;   // even-odd kernel: minimum resident CTAs of 128
     static __device__ __forceinline__ void load_spinor(const void *d, const float *, int V, int x,
                                                        cx<double> s[12])
     {
@@ -312,10 +311,6 @@ struct P64 {
 #pragma unroll
         for (int k = 0; k < 12; ++k) p[(size_t)k * V + x] = make_double2(s[k].re, s[k].im);
     }
-    // s as a store_spinor followed by a load_spinor returns it (computed in
-    // registers: load_spinor reads through the non-coherent path, which need
-    // not see a write of the same kernel)
-    static __device__ __forceinline__ void as_stored(cx<double> s[12]) {}
     // U_mu(x): a[0..2] = row 0, a[3..5] = row 1, c[0..2] = row 2
     static __device__ __forceinline__ void load_link(const GaugeStore &g, int V, int mu, int x,
                                                      cx<double> a[6], cx<double> c[3])
@@ -350,7 +345,6 @@ struct P32 {
     using real = float;
     static constexpr int kCaps = 3;   // cap 1: 64 registers, cap 2: 85
     static constexpr int kCap1MinBlocks = 4;
-    static constexpr int kEoMinBlocks = 1;
     static __device__ __forceinline__ void load_spinor(const void *d, const float *, int V, int x,
                                                        cx<float> s[12])
     {
@@ -376,7 +370,9 @@ struct P32 {
         for (int j = 0; j < 6; ++j)
             p[(size_t)j * V + x] = make_float4(s[2 * j].re, s[2 * j].im, s[2 * j + 1].re, s[2 * j + 1].im);
     }
-    // s as a store_spinor followed by a load_spinor returns it
+    // s as a store_spinor followed by a load_spinor returns it (computed in
+    // registers: load_spinor reads through the non-coherent path, which need
+    // not see a write of the same kernel)
     static __device__ __forceinline__ void as_stored(cx<float> s[12]) {}
     static __device__ __forceinline__ void load_link(const GaugeStore &g, int V, int mu, int x,
                                                      cx<float> a[6], cx<float> c[3])
@@ -412,7 +408,6 @@ struct PDF {
     using real = df;
     static constexpr int kCaps = 1;   // cap 1: 128 registers (2 CTAs of 256)
     static constexpr int kCap1MinBlocks = 2;
-    static constexpr int kEoMinBlocks = 4;   // 128 registers: latency-bound, occupancy pays
     static __device__ __forceinline__ void load_spinor(const void *d, const float *, int V, int x, cx<df> s[12])
     {
         const double2 *p = static_cast<const double2 *>(d);
@@ -433,13 +428,6 @@ struct PDF {
 #pragma unroll
         for (int k = 0; k < 12; ++k) p[(size_t)k * V + x] = make_double2(df_to_double(s[k].re), df_to_double(s[k].im));
     }
-    // s as a store_spinor followed by a load_spinor returns it
-    static __device__ __forceinline__ void as_stored(cx<df> s[12])
-    {
-#pragma unroll
-        for (int k = 0; k < 12; ++k)
-            s[k] = {df_from_double(df_to_double(s[k].re)), df_from_double(df_to_double(s[k].im))};
-    }
     static __device__ __forceinline__ void load_link(const GaugeStore &g, int V, int mu, int x, cx<df> a[6],
                                                      cx<df> c[3])
     {
@@ -454,18 +442,6 @@ struct PDF {
             const float4 v = __ldg(p + (size_t)(6 + k) * V);
             c[k] = {df(v.x, v.y), df(v.z, v.w)};
         }
-    }
-    // real entry t (0..5: the diagonal) and complex lower entry m (0..14) of
-    // block b at position x
-    static __device__ __forceinline__ df clover_real(const CloverStore &c, int V, int x, int b, int t)
-    {
-        const float4 v = __ldg(c.cdf + (size_t)(b * 18 + (t >> 1)) * V + x);
-        return (t & 1) ? df(v.z, v.w) : df(v.x, v.y);
-    }
-    static __device__ __forceinline__ cx<df> clover_lower(const CloverStore &c, int V, int x, int b, int m)
-    {
-        const float4 v = __ldg(c.cdf + (size_t)(b * 18 + 3 + m) * V + x);
-        return {df(v.x, v.y), df(v.z, v.w)};
     }
     static __device__ __forceinline__ void load_clover(const CloverStore &c, int V, int x, int b, df r[36])
     {
@@ -483,7 +459,6 @@ struct P16 {
     using real = float;
     static constexpr int kCaps = 3;   // cap 1: 64 registers, cap 2: 85
     static constexpr int kCap1MinBlocks = 4;
-    static constexpr int kEoMinBlocks = 1;
     // stored (unit-scaled) values; returns the site's scale, to be folded
     // into a later coefficient instead of multiplying all 24 components
     static __device__ __forceinline__ float load_spinor_raw(const void *d, const float *nrm, int V, int x,

@@ -21,6 +21,7 @@
 
 #include "wc_internal.cuh"
 #include "wc_stencil.cuh"
+#include "wc_dfsplit.cuh"
 
 namespace wc {
 
@@ -161,6 +162,44 @@ __global__ void __launch_bounds__(kSplit64 * kSplit64Sites, 3)
     }
 }
 
+// The same in double-FP32 arithmetic (wc_dfsplit.cuh).  HDF: in holds split
+// values.
+template <int KIND, bool HDF>
+__global__ void __launch_bounds__(kSplit64 * kSplit64Sites, dfs::kCtas)
+    k_apply_splitdf(Geom g, GaugeStore U, CloverStore C, const void *in, void *out, double kappa, const int *skip)
+{
+    griddep_wait();
+    griddep_launch_dependents();
+    if (skip && *skip) return;
+    __shared__ dfs::Mem sm;
+    const int s = threadIdx.x & (kSplit64Sites - 1), w = threadIdx.x / kSplit64Sites;
+    const int x = blockIdx.x * kSplit64Sites + s;
+    const bool valid = x < g.V;
+    if (valid) {
+        int c[4];
+        site_coords_fast(g, x, c);
+        dfs::hops<KIND == 1 ? +1 : -1, HDF>(g, U, in, g.V, x, c, sm, w, s, [](int y) { return y; });
+    }
+    __syncthreads();
+    if (!valid) return;
+    double2 *o = static_cast<double2 *>(out) + (size_t)3 * w * g.V + x;
+    if (KIND == 2) {
+#pragma unroll
+        for (int r = 0; r < 3; ++r) o[(size_t)r * g.V] = dfs::to_double(dfs::sum(sm, 3 * w + r, s));
+        return;
+    }
+    const df mk(-kappa);
+    f2::z2 v[6];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) v[k] = dfs::load<HDF>(in, g.V, 6 * (w >> 1) + k, x);
+    dfs::Sum y[3];
+#pragma unroll
+    for (int r = 0; r < 3; ++r) y[r] = dfs::first_term(mk, dfs::sum(sm, 3 * w + r, s));
+    dfs::clover_rows(C, g.V, x, w, v, y);
+#pragma unroll
+    for (int r = 0; r < 3; ++r) o[(size_t)r * g.V] = dfs::to_double(dfs::finish(y[r]));
+}
+
 // ---- launch shapes and their autotuner ---------------------------------
 
 struct ApplyShape {
@@ -189,6 +228,10 @@ constexpr int kNumShapes = sizeof(kShapes) / sizeof(kShapes[0]);
 // against 39 us, 8^4 14 / 39, 12^4 49 / 60, 16^3x32 247 / 266, 24^3x32
 // 828 / 863, 17x19x21x23 299 / 331, 32^3x64 3960-4016 / 4014-4022), so
 // nothing is timed for it.
+// In double-FP32 arithmetic it is one more candidate to time: each hop there
+// splits its spinor anew, which costs more than it gains on large lattices
+// (8^4 17 against 47 us, 16^3x32 181 / 218, 24^3x32 605 / 608, 32^3x64 2924 /
+// 2550); a solve splits its vector once (launch_apply_df).
 constexpr int kShapeSplit64 = kNumShapes;
 
 // caps: bit c-1 set if register cap c is compiled for the operator (P::kCaps)
@@ -213,12 +256,16 @@ int resident_ctas(K kernel, int threads)
     return n;
 }
 
+template <class P>
 cudaError_t launch_split64(wc_lattice lat, wc_field out, wc_field in, int kind, cudaStream_t stream,
                            const int *skip, bool pdl)
 {
     const Geom &g = lat->g;
     const dim3 grid((g.V + kSplit64Sites - 1) / kSplit64Sites);
-    const auto kern = kind == 0 ? k_apply_split64<0> : kind == 1 ? k_apply_split64<1> : k_apply_split64<2>;
+    const auto k64 = kind == 0 ? k_apply_split64<0> : kind == 1 ? k_apply_split64<1> : k_apply_split64<2>;
+    const auto kdf = kind == 0 ? k_apply_splitdf<0, false>
+                               : kind == 1 ? k_apply_splitdf<1, false> : k_apply_splitdf<2, false>;
+    const auto kern = std::is_same<P, PDF>::value ? kdf : k64;
     return launch_step(pdl && pdl_grid(grid.x), kern, grid, kSplit64 * kSplit64Sites, stream, g, lat->gauge, lat->clover, in->data,
                        out->data, lat->kappa, skip);
 }
@@ -227,7 +274,7 @@ template <class P>
 cudaError_t launch_shape(wc_lattice lat, wc_field out, wc_field in, int kind, int index, cudaStream_t stream,
                          const int *skip = nullptr, bool step_pdl = false)
 {
-    if (index == kShapeSplit64) return launch_split64(lat, out, in, kind, stream, skip, step_pdl);
+    if (index == kShapeSplit64) return launch_split64<P>(lat, out, in, kind, stream, skip, step_pdl);
     const ApplyShape &sh = kShapes[index];
     const Geom &g = lat->g;
     TileMap tm{};
@@ -325,11 +372,12 @@ int tune_shape(wc_lattice lat, wc_field out, wc_field in, int kind, cudaStream_t
         npair = k + 1;
     }
     cudaGetLastError();
-    float best_ms[kNumShapes];
-    for (int i = 0; i < kNumShapes; ++i) best_ms[i] = 1e30f;
+    constexpr int n = kNumShapes + std::is_same<P, PDF>::value;   // with kShapeSplit64
+    float best_ms[n];
+    for (int i = 0; i < n; ++i) best_ms[i] = 1e30f;
     for (int round = 0; round < 3; ++round) {
-        for (int i = 0; i < kNumShapes; ++i) {
-            if (!shape_fits(lat->g, kShapes[i], P::kCaps)) continue;
+        for (int i = 0; i < n; ++i) {
+            if (i < kNumShapes && !shape_fits(lat->g, kShapes[i], P::kCaps)) continue;
             if (launch_shape<P>(lat, out, in, kind, i, stream) != cudaSuccess) continue;
             cudaEventRecord(e0, stream);
             for (int r = 0; r < 16; ++r)
@@ -342,7 +390,7 @@ int tune_shape(wc_lattice lat, wc_field out, wc_field in, int kind, cudaStream_t
         }
     }
     int best = 0;
-    for (int i = 1; i < kNumShapes; ++i)
+    for (int i = 1; i < n; ++i)
         if (best_ms[i] < best_ms[best]) best = i;
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
@@ -477,6 +525,18 @@ cudaError_t launch_apply(wc_lattice lat, wc_field out, wc_field in, int kind, cu
     case WC_F32: return launch_apply_p<P32>(lat, out, in, kind, stream, skip, pdl);
     default: return launch_apply_p<P16>(lat, out, in, kind, stream, skip, pdl);
     }
+}
+
+cudaError_t launch_apply_df(wc_lattice lat, wc_field out, wc_field in, wc_field split, int kind, cudaStream_t stream,
+                            const int *skip, bool pdl)
+{
+    cudaError_t e = launch_to_df(12LL * lat->g.V, in, split, stream, skip, pdl);
+    if (e != cudaSuccess) return e;
+    const Geom &g = lat->g;
+    const dim3 grid((g.V + kSplit64Sites - 1) / kSplit64Sites);
+    const auto kern = kind == 0 ? k_apply_splitdf<0, true> : kind == 1 ? k_apply_splitdf<1, true> : k_apply_splitdf<2, true>;
+    return launch_step(pdl && pdl_grid(grid.x), kern, grid, kSplit64 * kSplit64Sites, stream, g, lat->gauge, lat->clover,
+                       split->data, out->data, lat->kappa, skip);
 }
 
 cudaError_t launch_copy(wc_lattice lat, wc_field dst, wc_field src, double scale, const double *dev_scale,

@@ -17,10 +17,12 @@
 // holds Lx/2 sites of each parity and i is unique within a parity.
 #include <math.h>
 
+#include <algorithm>
 #include <new>
 
 #include "wc_internal.cuh"
 #include "wc_stencil.cuh"
+#include "wc_dfsplit.cuh"
 
 namespace wc {
 
@@ -308,10 +310,7 @@ template <class P, bool INV>
 __device__ __forceinline__ void clover_eo(const CloverStore &S, int V, int pos, const cx<typename P::real> v[12],
                                           cx<typename P::real> y[12])
 {
-    if constexpr (std::is_same<P, PDF>::value) {   // compact form (instruction cache)
-        clover_block_rt<P>(S, V, pos, 0, v, y);
-        clover_block_rt<P>(S, V, pos, 1, v + 6, y + 6);
-    } else if constexpr (!INV) {
+    if constexpr (!INV) {
         clover_a<P>(S, V, pos, 0, v, y);
         clover_a<P>(S, V, pos, 1, v + 6, y + 6);
     } else {
@@ -341,7 +340,7 @@ __device__ __forceinline__ void clover_eo(const CloverStore &S, int V, int pos, 
 template <class P, int MODE>
 __device__ __forceinline__ void eo_tail(const Geom &g, int p, const CloverStore &C, const CloverStore &Ci,
                                         const void *vin, const float *vin_nrm, void *out, float *out_nrm,
-                                        void *out2, double beta, int Vh, int i, const cx<typename P::real> h[12])
+                                        double beta, int Vh, int i, const cx<typename P::real> h[12])
 {
     using R = typename P::real;
     cx<R> v[12], o[12];
@@ -358,7 +357,7 @@ __device__ __forceinline__ void eo_tail(const Geom &g, int p, const CloverStore 
             P::store_spinor(out, out_nrm, Vh, i, o);
             return;
         }
-        if (MODE == 2 || MODE == 3 || MODE == 5)
+        if (MODE == 2 || MODE == 3)
 #pragma unroll
             for (int k = 0; k < 12; ++k) v[k] = v[k] + bt * h[k];
         if (MODE == 2) {
@@ -368,22 +367,16 @@ __device__ __forceinline__ void eo_tail(const Geom &g, int p, const CloverStore 
     }
     clover_eo<P, true>(Ci, g.V, wc_idx(p * Vh + i, g.V), v, o);
     P::store_spinor(out, out_nrm, Vh, i, o);
-    if constexpr (MODE == 5) {
-        // the residual of x_o as the caller receives it (the stored value)
-        cx<R> y[12];
-        P::as_stored(o);
-        clover_eo<P, false>(C, g.V, wc_idx(p * Vh + i, g.V), o, y);
-#pragma unroll
-        for (int k = 0; k < 12; ++k) y[k] = v[k] - y[k];
-        P::store_spinor(out2, nullptr, Vh, i, y);
-    }
 }
 
+// (FP32 and FP16 fields.  One CTA per SM is all that is asked of the register
+// allocation: without that it keeps fewer loads in flight, a solver step at
+// 16^3x32 in binary16 136 instead of 122 us.)
 template <class P, int DAG, int MODE>
-__global__ void __launch_bounds__(128, P::kEoMinBlocks) k_eo(Geom g, int p, GaugeStore U, CloverStore C, CloverStore Ci,
+__global__ void __launch_bounds__(128, 1) k_eo(Geom g, int p, GaugeStore U, CloverStore C, CloverStore Ci,
                                             const void *hin, const float *hin_nrm, const void *vin,
-                                            const float *vin_nrm, void *out, float *out_nrm, void *out2,
-                                            double beta, const int *skip)
+                                            const float *vin_nrm, void *out, float *out_nrm, double beta,
+                                            const int *skip)
 {
     griddep_wait();
     griddep_launch_dependents();
@@ -394,34 +387,19 @@ __global__ void __launch_bounds__(128, P::kEoMinBlocks) k_eo(Geom g, int p, Gaug
     if (i >= Vh) return;
     int c[4];
     const int x = full_site(g, i, p, c);
-    if constexpr (std::is_same<P, PDF>::value) {
-        // compact form (instruction cache): hops and clover rows in runtime
-        // loops.  Measured at 24^3x32 (even-odd FP64-class solve, 40 such
-        // passes): the site-local A / A^-1 products in FP64 on the FP64 pipe
-        // 2 % slower, with the two x hops in FP64 too 8 % slower, and a
-        // 168- or 255-register cap (12 or 8 warps per SM, no spills) 2 % and
-        // 23 % slower than this form at 128 registers and 16 warps.
-        cx<R> h[12];
+    cx<R> h[12];
 #pragma unroll
-        for (int k = 0; k < 12; ++k) h[k] = mkc(R(0.0f, 0.0f), R(0.0f, 0.0f));
-        if (MODE != 4)
-            hops_rt<P, DAG ? +1 : -1>(g, U, hin, hin_nrm, Vh, x, c, R(1.0f, 0.0f), h, [](int y) { return y >> 1; });
-        eo_tail<P, MODE>(g, p, C, Ci, vin, vin_nrm, out, out_nrm, out2, beta, Vh, i, h);
-    } else {
-        cx<R> h[12];
-#pragma unroll
-        for (int k = 0; k < 12; ++k) h[k] = mkc(R(0), R(0));
-        if (MODE != 4) {
-            constexpr int SF = DAG ? +1 : -1;
-            constexpr int SB = -SF;
-            const R one = R(1);
-            eo_hop_dir<P, 0, SF, SB>(g, U, hin, hin_nrm, Vh, x, c, one, h);
-            eo_hop_dir<P, 1, SF, SB>(g, U, hin, hin_nrm, Vh, x, c, one, h);
-            eo_hop_dir<P, 2, SF, SB>(g, U, hin, hin_nrm, Vh, x, c, one, h);
-            eo_hop_dir<P, 3, SF, SB>(g, U, hin, hin_nrm, Vh, x, c, one, h);
-        }
-        eo_tail<P, MODE>(g, p, C, Ci, vin, vin_nrm, out, out_nrm, out2, beta, Vh, i, h);
+    for (int k = 0; k < 12; ++k) h[k] = mkc(R(0), R(0));
+    if (MODE != 4) {
+        constexpr int SF = DAG ? +1 : -1;
+        constexpr int SB = -SF;
+        const R one = R(1);
+        eo_hop_dir<P, 0, SF, SB>(g, U, hin, hin_nrm, Vh, x, c, one, h);
+        eo_hop_dir<P, 1, SF, SB>(g, U, hin, hin_nrm, Vh, x, c, one, h);
+        eo_hop_dir<P, 2, SF, SB>(g, U, hin, hin_nrm, Vh, x, c, one, h);
+        eo_hop_dir<P, 3, SF, SB>(g, U, hin, hin_nrm, Vh, x, c, one, h);
     }
+    eo_tail<P, MODE>(g, p, C, Ci, vin, vin_nrm, out, out_nrm, beta, Vh, i, h);
 }
 
 // k_eo in FP64 on four warps per 32 sites (hop_split64): warp w finishes
@@ -517,6 +495,120 @@ __global__ void __launch_bounds__(kSplit64 * kSplit64Sites, 3)
     }
 }
 
+// An FP64 half field as z2 values (wc_dfsplit.cuh), for the hops of the next
+// pass: each of its spinors is read eight times.
+__global__ void __launch_bounds__(256) k_to_df(long long n, const double2 *__restrict__ in, float4 *__restrict__ out,
+                                               const int *skip)
+{
+    griddep_wait();
+    griddep_launch_dependents();
+    if (skip && *skip) return;
+#pragma unroll 4
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+        out[i] = dfs::to4(dfs::of_double(in[i]));
+}
+
+// k_eo of FP64 fields in double-FP32 arithmetic, on four warps per 32 sites as
+// k_eo_split64.  HDF, ODF: hin / out is kept as z2 values.
+template <int DAG, int MODE, bool HDF, bool ODF>
+__global__ void __launch_bounds__(kSplit64 * kSplit64Sites, dfs::kCtas)
+    k_eo_splitdf(Geom g, int p, GaugeStore U, CloverStore C, CloverStore Ci, const void *hin, const double2 *vin,
+                 void *out, double2 *out2, double beta, const int *skip)
+{
+    using dfs::z2;
+    griddep_wait();
+    griddep_launch_dependents();
+    if (skip && *skip) return;
+    __shared__ dfs::Mem sm;
+    const int Vh = g.V >> 1;
+    const int s = threadIdx.x & (kSplit64Sites - 1), w = threadIdx.x / kSplit64Sites;
+    const int i = blockIdx.x * kSplit64Sites + s;
+    const bool valid = i < Vh;
+    if (MODE != 4 && valid) {
+        int c[4];
+        const int x = full_site(g, i, p, c);
+        dfs::hops<DAG ? +1 : -1, HDF>(g, U, hin, Vh, x, c, sm, w, s, [](int y) { return y >> 1; });
+    }
+    __syncthreads();
+    const df bt(beta);
+    z2 v[3], vb[6];
+    if (valid) {
+#pragma unroll
+        for (int r = 0; r < 3; ++r) {
+            const int k = 3 * w + r;
+            const z2 h = MODE == 4 ? dfs::zero() : dfs::sum(sm, k, s);
+            if (MODE == 0) {
+                v[r] = h;
+            } else if (MODE == 1) {
+                dfs::Sum t = dfs::first_term(bt, h);
+                v[r] = dfs::finish(t);
+            } else {
+                const z2 a = dfs::of_double(__ldg(vin + (size_t)k * Vh + i));
+                dfs::Sum t = dfs::start(a);
+                if (MODE != 4) dfs::add_term(t, bt, h);
+                v[r] = dfs::finish(t);
+            }
+        }
+    }
+    // component k is read and written only by its own warp until the barrier
+    const auto share = [&](const z2 a[3]) {
+        if (valid)
+#pragma unroll
+            for (int r = 0; r < 3; ++r) sm[0][3 * w + r][s] = dfs::to4(a[r]);
+        __syncthreads();
+        if (valid)
+#pragma unroll
+            for (int k = 0; k < 6; ++k) vb[k] = dfs::of4(sm[0][(w >> 1) * 6 + k][s]);
+    };
+    const auto store = [&](const z2 a[3]) {
+#pragma unroll
+        for (int r = 0; r < 3; ++r) {
+            const size_t at = (size_t)(3 * w + r) * Vh + i;
+            if (ODF) static_cast<float4 *>(out)[at] = dfs::to4(a[r]);
+            else static_cast<double2 *>(out)[at] = dfs::to_double(a[r]);
+        }
+    };
+    if (MODE == 2) {
+        if (valid) store(v);
+        return;
+    }
+    const int pos = wc_idx(p * Vh + (valid ? i : 0), g.V);
+    if (MODE == 1) {
+        if (!valid) return;
+        const double2 *q = vin + (size_t)(w >> 1) * 6 * Vh + i;
+#pragma unroll
+        for (int k = 0; k < 6; ++k) vb[k] = dfs::of_double(__ldg(q + (size_t)k * Vh));
+        dfs::Sum y[3] = {dfs::start(v[0]), dfs::start(v[1]), dfs::start(v[2])};
+        dfs::clover_rows(C, g.V, pos, w, vb, y);
+        const z2 o[3] = {dfs::finish(y[0]), dfs::finish(y[1]), dfs::finish(y[2])};
+        store(o);
+        return;
+    }
+    share(v);
+    z2 o[3];
+    if (valid) {
+        dfs::Sum y[3] = {dfs::start(dfs::zero()), dfs::start(dfs::zero()), dfs::start(dfs::zero())};
+        dfs::clover_rows(Ci, g.V, pos, w, vb, y);
+#pragma unroll
+        for (int r = 0; r < 3; ++r) o[r] = dfs::finish(y[r]);
+        store(o);
+    }
+    if (MODE == 5) {
+        // the residual of x_o as the caller receives it (the stored value)
+        if (valid)
+#pragma unroll
+            for (int r = 0; r < 3; ++r) o[r] = dfs::of_double(dfs::to_double(o[r]));
+        __syncthreads();   // vb is read
+        share(o);
+        if (valid) {
+            dfs::Sum y[3] = {dfs::start(dfs::neg(v[0])), dfs::start(dfs::neg(v[1])), dfs::start(dfs::neg(v[2]))};
+            dfs::clover_rows(C, g.V, pos, w, vb, y);
+#pragma unroll
+            for (int r = 0; r < 3; ++r) out2[(size_t)(3 * w + r) * Vh + i] = dfs::to_double(dfs::neg(dfs::finish(y[r])));
+        }
+    }
+}
+
 // full field <-> the two half fields (parity 0 = even, 1 = odd)
 template <class P>
 __global__ void k_split(Geom g, const void *full, const float *full_nrm, void *ev, float *ev_nrm, void *od,
@@ -579,10 +671,45 @@ cudaError_t launch_eo_split64(const wc_lattice_s *full, int parity, int mode, co
 #undef WC_EO
 }
 
+template <int DAG>
+cudaError_t launch_eo_splitdf(const wc_lattice_s *full, int parity, int mode, const wc_field_s *hin,
+                              const wc_field_s *vin, wc_field_s *out, double beta, cudaStream_t stream,
+                              wc_field_s *out2, const int *skip, bool pdl, int split)
+{
+    if (mode == 5 && (!out2 || out2->prec != WC_F64)) return cudaErrorInvalidValue;
+    const bool hdf = split & kEoInSplit, odf = split & kEoOutSplit;
+    if (odf && mode != 0 && mode != 4) return cudaErrorInvalidValue;
+    const int Vh = full->g.V >> 1;
+    const dim3 grid((Vh + kSplit64Sites - 1) / kSplit64Sites);
+    const void *hd = hin ? hin->data : nullptr;
+    const double2 *vd = vin ? static_cast<const double2 *>(vin->data) : nullptr;
+    double2 *o2 = out2 ? static_cast<double2 *>(out2->data) : nullptr;
+#define WC_EO(M, H, O)                                                                                                \
+    return launch_step(pdl && pdl_grid(grid.x), k_eo_splitdf<DAG, M, H, O>, grid, kSplit64 *kSplit64Sites, stream,    \
+                       full->g, parity, full->gauge, full->ceo, full->cinv, hd, vd, out->data, o2, beta, skip)
+#define WC_EO_H(M) \
+    if (hdf) WC_EO(M, true, false); \
+    WC_EO(M, false, false)
+    switch (mode) {
+    case 0:
+        if (hdf && odf) WC_EO(0, true, true);
+        if (odf) WC_EO(0, false, true);
+        WC_EO_H(0);
+    case 1: WC_EO_H(1);
+    case 2: WC_EO_H(2);
+    case 3: WC_EO_H(3);
+    case 4:
+        if (odf) WC_EO(4, false, true);
+        WC_EO(4, false, false);
+    default: WC_EO_H(5);
+    }
+#undef WC_EO_H
+#undef WC_EO
+}
+
 template <class P, int DAG>
 cudaError_t launch_eo_p(const wc_lattice_s *full, int parity, int mode, const wc_field_s *hin, const wc_field_s *vin,
-                        wc_field_s *out, double beta, cudaStream_t stream, wc_field_s *out2, const int *skip,
-                        bool pdl)
+                        wc_field_s *out, double beta, cudaStream_t stream, const int *skip, bool pdl)
 {
     const int Vh = full->g.V >> 1;
     // CTAs of 128 sites; on small lattices (fewer than two such CTAs per SM)
@@ -593,23 +720,16 @@ cudaError_t launch_eo_p(const wc_lattice_s *full, int parity, int mode, const wc
     const float *hn = hin ? hin->nrm : nullptr;
     const void *vd = vin ? vin->data : nullptr;
     const float *vn = vin ? vin->nrm : nullptr;
-    void *o2 = out2 ? out2->data : nullptr;
 #define WC_EO(M)                                                                                                \
     return launch_step(pdl && pdl_grid(grid.x), k_eo<P, DAG, M>, grid, threads, stream, full->g, parity, full->gauge, full->ceo,    \
-                       full->cinv, hd, hn, vd, vn, out->data, out->nrm, o2, beta, skip)
+                       full->cinv, hd, hn, vd, vn, out->data, out->nrm, beta, skip)
     switch (mode) {
     case 0: WC_EO(0); break;
     case 1: WC_EO(1); break;
     case 2: WC_EO(2); break;
     case 3: WC_EO(3); break;
     case 4: WC_EO(4); break;
-    default:
-        if constexpr (std::is_same<P, PDF>::value) {
-            if (!out2 || out2->prec != WC_F64) return cudaErrorInvalidValue;
-            WC_EO(5);
-        } else {
-            return cudaErrorInvalidValue;
-        }
+    default: return cudaErrorInvalidValue;   // mode 5: FP64 fields only
     }
 #undef WC_EO
 }
@@ -619,20 +739,34 @@ cudaError_t launch_eo_p(const wc_lattice_s *full, int parity, int mode, const wc
 // one parity-stencil step on half fields of the full lattice `full`
 cudaError_t launch_eo(const wc_lattice_s *full, int parity, int mode, int dagger, const wc_field_s *hin,
                       const wc_field_s *vin, wc_field_s *out, double beta, cudaStream_t stream, wc_field_s *out2,
-                      const int *skip, bool pdl)
+                      const int *skip, bool pdl, int split)
 {
     const wc_prec pr = out->prec;
     if (pr == WC_F64 && full->fp64_arith == WC_ARITH_DF32)
-        return dagger ? launch_eo_p<PDF, 1>(full, parity, mode, hin, vin, out, beta, stream, out2, skip, pdl)
-                      : launch_eo_p<PDF, 0>(full, parity, mode, hin, vin, out, beta, stream, out2, skip, pdl);
+        return dagger ? launch_eo_splitdf<1>(full, parity, mode, hin, vin, out, beta, stream, out2, skip, pdl, split)
+                      : launch_eo_splitdf<0>(full, parity, mode, hin, vin, out, beta, stream, out2, skip, pdl, split);
+    if (split) return cudaErrorInvalidValue;
     if (pr == WC_F64)
         return dagger ? launch_eo_split64<1>(full, parity, mode, hin, vin, out, beta, stream, out2, skip, pdl)
                       : launch_eo_split64<0>(full, parity, mode, hin, vin, out, beta, stream, out2, skip, pdl);
     if (pr == WC_F32)
-        return dagger ? launch_eo_p<P32, 1>(full, parity, mode, hin, vin, out, beta, stream, out2, skip, pdl)
-                      : launch_eo_p<P32, 0>(full, parity, mode, hin, vin, out, beta, stream, out2, skip, pdl);
-    return dagger ? launch_eo_p<P16, 1>(full, parity, mode, hin, vin, out, beta, stream, out2, skip, pdl)
-                  : launch_eo_p<P16, 0>(full, parity, mode, hin, vin, out, beta, stream, out2, skip, pdl);
+        return dagger ? launch_eo_p<P32, 1>(full, parity, mode, hin, vin, out, beta, stream, skip, pdl)
+                      : launch_eo_p<P32, 0>(full, parity, mode, hin, vin, out, beta, stream, skip, pdl);
+    return dagger ? launch_eo_p<P16, 1>(full, parity, mode, hin, vin, out, beta, stream, skip, pdl)
+                  : launch_eo_p<P16, 0>(full, parity, mode, hin, vin, out, beta, stream, skip, pdl);
+}
+
+cudaError_t launch_to_df(long long n, const wc_field_s *in, wc_field_s *out, cudaStream_t stream, const int *skip,
+                         bool pdl)
+{
+    const int blocks = (int)std::min<long long>((n + 255) / 256, 8 * sm_count());
+    return launch_step(pdl && pdl_grid(blocks), k_to_df, dim3(blocks), 256, stream, n,
+                       static_cast<const double2 *>(in->data), static_cast<float4 *>(out->data), skip);
+}
+
+bool eo_split(const wc_lattice_s *full, const wc_field_s *f)
+{
+    return f->prec == WC_F64 && full->fp64_arith == WC_ARITH_DF32;
 }
 
 // od may be NULL: only the even half is written
@@ -676,16 +810,27 @@ cudaError_t launch_schur(wc_lattice half, wc_field out, wc_field in, int dagger,
 {
     const wc_lattice_s *full = half->schur_parent;
     wc_field_s *t = tmp ? tmp : half->schur_tmp[out->prec];
-    cudaError_t e = launch_eo(full, 1, 0, dagger, in, nullptr, t, 0.0, stream, nullptr, skip, pdl);
+    // in double-FP32 the passes exchange split values: out holds those of in
+    // until the second pass writes it
+    const bool df = eo_split(full, out);
+    cudaError_t e = df ? launch_to_df(6LL * full->g.V, in, out, stream, skip, pdl) : cudaSuccess;
     if (e == cudaSuccess)
-        e = launch_eo(full, 0, 1, dagger, t, in, out, -full->kappa * full->kappa, stream, nullptr, skip, pdl);
+        e = launch_eo(full, 1, 0, dagger, df ? out : in, nullptr, t, 0.0, stream, nullptr, skip, pdl,
+                      df ? kEoInSplit | kEoOutSplit : 0);
+    if (e == cudaSuccess)
+        e = launch_eo(full, 0, 1, dagger, t, in, out, -full->kappa * full->kappa, stream, nullptr, skip, pdl,
+                      df ? kEoInSplit : 0);
     return e;
 }
 
 cudaError_t launch_apply(wc_lattice lat, wc_field out, wc_field in, int kind, SolverState &S, bool step)
 {
     const int *skip = step ? &S.scal->skip : nullptr;
-    if (!lat->schur_parent) return launch_apply(lat, out, in, kind, S.stream, skip, S.pdl);
+    if (!lat->schur_parent) {
+        wc_field split = S.work[kDfSlot];
+        if (split && eo_split(lat, in)) return launch_apply_df(lat, out, in, split, kind, S.stream, skip, S.pdl);
+        return launch_apply(lat, out, in, kind, S.stream, skip, S.pdl);
+    }
     return launch_schur(lat, out, in, kind == 1, S.stream, S.work[kSchurSlot + out->prec], skip, S.pdl);
 }
 

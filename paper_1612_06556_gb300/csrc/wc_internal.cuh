@@ -42,7 +42,8 @@ namespace wc {
 // b_e, b_o, x_e, x_o, b^_e of an even-odd solve, 32-35: full-lattice FP32
 // and FP16 in/out fields of the RAS preconditioner of an even-odd solve,
 // 36-43: the low-precision BiCGStab vectors when they are FP16, 44-45: the
-// even and odd halves of the final full residual of an even-odd solve) and
+// even and odd halves of the final full residual of an even-odd solve, 46:
+// the split copy of a full-lattice vector in double-FP32 arithmetic) and
 // the stream the solve is queued on.  A lattice owns one for its single-RHS
 // calls; a batched solve creates one per RHS.
 constexpr int kReportSlots = 2;
@@ -51,6 +52,7 @@ constexpr int kEoSlot = 27;
 constexpr int kRasEoSlot = 32;
 constexpr int kHalfKrylovSlot = 36;
 constexpr int kEoResSlot = 44;
+constexpr int kDfSlot = 46;
 struct SolverState {
     SolverScalars *scal = nullptr;
     SolverScalars *scal_host = nullptr;
@@ -61,7 +63,7 @@ struct SolverState {
     unsigned long long seq = 0;
     bool pdl = false;
     ReduceScratch red;
-    wc_field_s *work[46] = {};
+    wc_field_s *work[47] = {};
     cudaStream_t stream = nullptr;
     SolverState *inner = nullptr;   // state of a nested inner solve, created on first use
 };
@@ -234,7 +236,17 @@ cudaError_t launch_schur(wc_lattice half, wc_field out, wc_field in, int dagger,
 // out2: the second output of mode 5 (nullptr for the other modes)
 cudaError_t launch_eo(const wc_lattice_s *full, int parity, int mode, int dagger, const wc_field_s *hin,
                       const wc_field_s *vin, wc_field_s *out, double beta, cudaStream_t stream,
-                      wc_field_s *out2 = nullptr, const int *skip = nullptr, bool pdl = false);
+                      wc_field_s *out2 = nullptr, const int *skip = nullptr, bool pdl = false, int split = 0);
+// In double-FP32 arithmetic hin (kEoInSplit) or the output of modes 0 and 4
+// (kEoOutSplit) may be held as split values (wc_dfsplit.cuh) in an FP64 half
+// field: launch_to_df makes them, eo_split says whether f is of that kind.
+constexpr int kEoInSplit = 1, kEoOutSplit = 2;
+cudaError_t launch_to_df(long long n /*complex values*/, const wc_field_s *in, wc_field_s *out, cudaStream_t stream,
+                         const int *skip = nullptr, bool pdl = false);
+// the whole-lattice operator in double-FP32, in split into `split` first
+cudaError_t launch_apply_df(wc_lattice lat, wc_field out, wc_field in, wc_field split, int kind, cudaStream_t stream,
+                            const int *skip, bool pdl);
+bool eo_split(const wc_lattice_s *full, const wc_field_s *f);
 cudaError_t launch_split(const wc_lattice_s *full, const wc_field_s *f, wc_field_s *ev, wc_field_s *od,
                          cudaStream_t stream);
 cudaError_t launch_merge(const wc_lattice_s *full, const wc_field_s *ev, const wc_field_s *od, wc_field_s *f,

@@ -163,6 +163,7 @@ wc_status solver_vectors(wc_lattice lat, SolverState &S, const wc_solve_params &
     w->shat = w->s;
     w->lo_in = w->lo_out = nullptr;
     if (st == WC_OK && lat->schur_parent) state_work(lat, S, kSchurSlot + WC_F64, WC_F64, &st);
+    if (st == WC_OK && !lat->schur_parent && lat->fp64_arith == WC_ARITH_DF32) state_work(lat, S, kDfSlot, WC_F64, &st);
     if (st == WC_OK && (p.precond == WC_PRECOND_RAS || p.solver == WC_SOLVER_NESTED)) {
         w->phat = state_work(lat, S, 6, WC_F64, &st);
         if (st == WC_OK) w->shat = state_work(lat, S, 7, WC_F64, &st);
@@ -284,14 +285,23 @@ wc_status eo_reconstruct_residual(wc_lattice lat, int kind, wc_field be, wc_fiel
     wc_field ro = st == WC_OK ? state_work(h, R, kEoResSlot + 1, WC_F64, &st) : nullptr;
     if (st != WC_OK) return st;
     const double k = lat->kappa;
-    st = check_cuda(lat, launch_eo(lat, 1, 5, kind, xe, bo, xo, k, s, ro), "x_o and r_o");
-    if (st == WC_OK) st = check_cuda(lat, launch_eo(lat, 0, 1, kind, xo, xe, re, -k, s), "(M x)_e");
-    if (st == WC_OK) st = check_cuda(lat, launch_merge(lat, xe, xo, x, s), "merge");
-    if (st == WC_OK) st = check_cuda(lat, residual(h, R, d2(be), d2(re)), "residual");
+    // in double-FP32, re and then ro hold the split values of the vector that
+    // the hops read, until a pass writes re and after |r_o|^2 is taken
+    const bool df = eo_split(lat, xe);
+    if (df) st = check_cuda(lat, launch_to_df(6LL * lat->g.V, xe, re, s), "split x_e");
+    if (st == WC_OK)
+        st = check_cuda(lat, launch_eo(lat, 1, 5, kind, df ? re : xe, bo, xo, k, s, ro, nullptr, false,
+                                       df ? kEoInSplit : 0), "x_o and r_o");
     if (st == WC_OK) st = check_cuda(lat, norm2_to_result(h, R, d2(ro)), "norm2");
     if (st == WC_OK)
         st = check_cuda(lat, cudaMemcpyAsync(R.red.host_result, R.red.result, sizeof(double), cudaMemcpyDeviceToHost, s),
                         "copy");
+    if (st == WC_OK && df) st = check_cuda(lat, launch_to_df(6LL * lat->g.V, xo, ro, s), "split x_o");
+    if (st == WC_OK)
+        st = check_cuda(lat, launch_eo(lat, 0, 1, kind, df ? ro : xo, xe, re, -k, s, nullptr, nullptr, false,
+                                       df ? kEoInSplit : 0), "(M x)_e");
+    if (st == WC_OK) st = check_cuda(lat, launch_merge(lat, xe, xo, x, s), "merge");
+    if (st == WC_OK) st = check_cuda(lat, residual(h, R, d2(be), d2(re)), "residual");
     if (st == WC_OK) st = read_scalars(h, R);
     if (st == WC_OK) *rr = R.scal_host->rr + R.red.host_result[0];
     return st;
@@ -372,8 +382,10 @@ static wc_status eo_bicgstab(wc_lattice lat, int kind, wc_field x, wc_field b, c
     const double k = lat->kappa;
     if (st == WC_OK) st = check_cuda(lat, launch_split(lat, b, be, bo, s), "split");
     if (st == WC_OK) st = check_cuda(lat, launch_split(lat, x, xe, xo, s), "split");
-    if (st == WC_OK) st = check_cuda(lat, launch_eo(lat, 1, 4, kind, nullptr, bo, t, 0.0, s), "A_oo^-1 b_o");
-    if (st == WC_OK) st = check_cuda(lat, launch_eo(lat, 0, 2, kind, t, be, bh, k, s), "b^_e");
+    if (st == WC_OK) st = check_cuda(lat, launch_eo(lat, 1, 4, kind, nullptr, bo, t, 0.0, s, nullptr, nullptr, false,
+                                        eo_split(lat, t) ? kEoOutSplit : 0), "A_oo^-1 b_o");
+    if (st == WC_OK) st = check_cuda(lat, launch_eo(lat, 0, 2, kind, t, be, bh, k, s, nullptr, nullptr, false,
+                                        eo_split(lat, t) ? kEoInSplit : 0), "b^_e");
     double bb = 0.0, bbh = 0.0;
     if (st == WC_OK) st = reduce_norm2(lat, b, &bb);
     if (st == WC_OK) st = reduce_norm2(h, bh, &bbh);
@@ -542,6 +554,7 @@ wc_status lo_vectors(wc_lattice lat, SolverState &S, const wc_solve_params &p, L
     const wc_prec kp = half ? WC_F16 : WC_F32;
     if (st == WC_OK && lat->schur_parent) state_work(lat, S, kSchurSlot + kp, kp, &st);
     if (st == WC_OK && lat->schur_parent) state_work(lat, S, kSchurSlot + WC_F64, WC_F64, &st);
+    if (st == WC_OK && !lat->schur_parent && lat->fp64_arith == WC_ARITH_DF32) state_work(lat, S, kDfSlot, WC_F64, &st);
     // RAS on FP16 storage when either the vectors or inner_prec are FP16
     const bool ras16 = half || p.inner_prec == WC_F16;
     if (st == WC_OK && p.precond == WC_PRECOND_RAS) st = eo_ras_temps(lat, S, ras16 ? WC_F16 : WC_F32);

@@ -142,9 +142,8 @@ namespace wc {
 // A double-FP32 site costs ~20 k instructions; written out per direction
 // (as the FP32/FP16/FP64 kernels are) the code no longer fits the
 // instruction cache (ncu: half of the fetches miss, 65 % of the stalls are
-// "no instruction").  These forms run the eight hops and the clover rows as
-// loops with a runtime index, so that one copy of the SU(3) product and of
-// the clover row is in the code.
+// "no instruction").  These forms run the eight hops as a loop with a runtime
+// index, so that one copy of the SU(3) product is in the code.
 
 template <class R>
 __device__ __forceinline__ void project_rt(int mu, int s, const cx<R> p[12], cx<R> h[6])
@@ -242,35 +241,6 @@ __device__ __forceinline__ void hops_rt(const Geom &g, const GaugeStore &U, cons
         P::load_link(U, g.V, mu, fwd ? x : y, u, r2);
         su3_mul_rt(!fwd, u, r2, h, coef, w);
         reconstruct_add_rt(mu, s, acc, w);
-    }
-}
-
-// y = A v for clover block b of the packed store (rows in a runtime loop;
-// each row reads its six entries: diagonal, lower (i, j) and the conjugate
-// of lower (j, i))
-template <class P>
-__device__ __forceinline__ void clover_block_rt(const CloverStore &C, int V, int x, int b,
-                                                const cx<typename P::real> v[6], cx<typename P::real> y[6])
-{
-    using R = typename P::real;
-#pragma unroll 1
-    for (int i = 0; i < 6; ++i) {
-        cx<R> acc = mkc(R(0.0f, 0.0f), R(0.0f, 0.0f));
-#pragma unroll
-        for (int j = 0; j < 6; ++j) {
-            cx<R> e;
-            if (j == i) {
-                e = cx<R>{P::clover_real(C, V, x, b, i), R(0.0f, 0.0f)};
-            } else {
-                const int hi = i > j ? i : j, lo = i > j ? j : i;
-                const cx<R> l = P::clover_lower(C, V, x, b, hi * (hi - 1) / 2 + lo);
-                e = j < i ? l : conj(l);
-            }
-            acc = cfma(e, v[j], acc);
-        }
-#pragma unroll
-        for (int r = 0; r < 6; ++r)
-            if (r == i) y[r] = acc;
     }
 }
 

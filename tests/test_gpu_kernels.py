@@ -221,3 +221,52 @@ def test_solves_of_two_threads_on_their_own_streams():
         assert len(together[k]) == 4
         for a in together[k]:
             assert np.array_equal(a, alone[k][0])
+
+
+@pytest.mark.parametrize("dims,tbc", [((2, 2, 2, 2), -1), ((3, 5, 2, 7), 1), ((5, 3, 7, 4), -1), ((8, 4, 4, 4), -1)])
+def test_double_fp32_operator_with_directions_on_four_warps(dims, tbc):
+    """M, M^+ and H in double-FP32 arithmetic on ragged volumes, by the kernel
+    that splits its input per hop (whatever shape is chosen), and by the
+    solves, which split a vector once: one step from x = 0 gives the same
+    x as the FP64 arithmetic's to 1e-11 (the step's scalars amplify the
+    2^-45 of the operator)."""
+    csw, kappa = 1.2, 0.12
+    U = synth.haar_links(dims, 160 + sum(dims))
+    lat = make_lattice(dims, U, csw, kappa, tbc)
+    op = oracle.Operator(dims, U, csw, kappa, tbc)
+    psi = synth.gaussian_source(dims, 161)
+    F64 = wc().F64
+    fi, fo, fx = lat.field(F64).load(psi), lat.field(F64), lat.field(F64)
+    lat.solve(fx, fi, tol=1e-13, max_iter=2, max_restarts=0, check=False)
+    x64 = fx.store(np.zeros_like(psi))
+    lat.set_fp64_arith(wc().ARITH_DF32)
+    ref = {"M": op.M(psi), "Mdag": op.Mdag(psi), "hop": oracle.apply_hop(dims, tbc, U, psi)}
+    for name in ref:
+        getattr(lat, "apply_" + name)(fo, fi)
+        assert_elementwise(fo.store(np.zeros_like(psi)), ref[name], 1e-12)
+    fx = lat.field(F64)
+    lat.solve(fx, fi, tol=1e-13, max_iter=2, max_restarts=0, check=False)
+    assert_elementwise(fx.store(np.zeros_like(psi)), x64, 1e-11)
+
+
+@pytest.mark.parametrize("dims,tbc", [((2, 2, 2, 2), -1), ((6, 2, 10, 4), 1), ((4, 4, 4, 4), -1)])
+@pytest.mark.parametrize("arith", [0, 1])
+def test_even_odd_passes_of_a_solve(dims, tbc, arith):
+    """The source preparation, reconstruction and both residual halves of an
+    even-odd solve (modes 4, 2, 5, 1) in FP64 and double-FP32: stopped after
+    one step, the reported residual is the oracle's of the returned x; M and
+    M^+ (the force's two solves) to 1e-12."""
+    csw, kappa = 1.1, 0.11
+    U = synth.exp_links(dims, 0.4, 171)
+    lat = make_lattice(dims, U, csw, kappa, tbc).set_fp64_arith(arith)
+    src = synth.gaussian_source(dims, 172)
+    b, x = lat.field(0).load(src), lat.field(0)
+    info = lat.solve(x, b, tol=1e-30, max_iter=1, max_restarts=0, even_odd=True, check=False)
+    r = src - oracle.apply_M(dims, tbc, kappa, csw, U, x.store(np.zeros_like(src)))
+    rel = np.linalg.norm(r) / np.linalg.norm(src)
+    assert abs(info.true_rel_resid - rel) <= 1e-11 * max(1.0, rel) + 1e-13
+    F = np.zeros((int(np.prod(dims)), 4, 3, 3), complex)
+    S = lat.action_force(b, F, tol=1e-13, even_odd=True)
+    S0, F0, _, _ = oracle.action_and_force(oracle.Operator(dims, U, csw, kappa, tbc), src, tol=1e-14)
+    assert abs(S - S0) <= 1e-11 * S0
+    assert_elementwise(F, F0, 1e-9)
