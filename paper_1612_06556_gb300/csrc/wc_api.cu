@@ -816,7 +816,7 @@ wc_status wc_apply_multi(wc_lattice lat, int n, wc_field *outs, wc_field *ins, i
     }
     wc_status st = require_operator(lat);
     if (st != WC_OK) return st;
-    return check_cuda(lat, launch_apply_multi(lat, n, outs, ins, dagger ? 1 : 0, nullptr, lat->stream),
+    return check_cuda(lat, launch_apply_multi(lat, n, outs, ins, dagger ? 1 : 0, lat->stream),
                       "apply_multi");
 }
 

@@ -317,7 +317,7 @@ wc_status enqueue_group_step(wc_lattice half, const std::vector<int> &idx, Resou
     }
     const bool hv = R.LW[idx[0]].v->prec == WC_F16;
     const bool fused = !hv && part;
-    const int mb = R.S[idx[0]].red.max_blocks, nblk = schur_multi_blocks(half);
+    const int mb = R.S[idx[0]].red.max_blocks, nblk = schur_multi_blocks(half, m);
     std::vector<wc_field> rh(m);
     for (int k = 0; k < m; ++k) rh[k] = R.LW[idx[k]].rhat;
     wc_status st = check_cuda(half, lo_group(LO_STEP_P, half, m, dm, hv, mb, s), "lo_p");
@@ -651,7 +651,7 @@ static wc_status batch_core(int n, const wc_lattice *lats, wc_field *xs, wc_fiel
             if (R.LW[i0].v->prec == WC_F32)
                 st = check_cuda(nullptr, cudaMalloc(reinterpret_cast<void **>(&R.d_part[g]),
                                                     sizeof(double) * 4 * members[g].size() *
-                                                        (size_t)schur_multi_blocks(lats[i0])),
+                                                        (size_t)schur_multi_blocks(lats[i0], (int)members[g].size())),
                                 "cudaMalloc");
             if (st != WC_OK) break;
             std::vector<LoMember> tab;

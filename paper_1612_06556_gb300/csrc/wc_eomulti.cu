@@ -7,11 +7,16 @@
 // In one pass a site reads its 8 links (4 forward U_mu(x), 4 backward
 // U_mu(x - mu)) and one clover-type block (A^-1 on the odd pass, A on the
 // even pass): 672 B per site in FP32, 336 B in FP16 storage, against 96 /
-// 52 B per spinor read or written.  A CTA covers kEoMSites consecutive
+// 52 B per spinor read or written.  A CTA covers S consecutive
 // sites of one parity for all n right-hand sides: it stages those shared
 // words once in shared memory (coalesced along the sites), then thread
 // (s, r) computes site s of right-hand side r from the staged links and
-// block and the 8 neighbour spinors of field r (through L1/L2).  The third
+// block and the 8 neighbour spinors of field r (through L1/L2).  A CTA takes
+// 32 sites for up to 6 fields and 16 above: more and smaller CTAs on an SM,
+// one of them staging while the others compute (M^ at 24^3x32 in FP32, 16 /
+// 32 sites: 5 fields 314 / 317 us, 6 321 / 333, 8 393 / 410, 12 559 / 585, 16
+// 748 / 978; binary16: 5 258 / 237, 6 252 / 251, 8 311 / 320, 12 440 / 472, 16
+// 583 / 771; at 64 registers 16 sites spill, 696 for 12 FP32 fields).  The third
 // row of each link is rebuilt once per site after staging (into shared
 // memory), not once per right-hand side.  The arithmetic per (site,
 // right-hand side) is otherwise that of the single-field pass (spin
@@ -27,8 +32,6 @@
 namespace wc {
 
 namespace {
-
-constexpr int kEoMSites = 32;
 
 struct EoMultiArgs {
     int n;
@@ -74,7 +77,8 @@ struct EoMStage<P32> {
             out = __ldg((MODE == 0 ? C.c32 : C.a32) + (size_t)(item - 24) * V + pos);
     }
     // the two stored rows of link lam = 4 bwd + mu
-    static __device__ __forceinline__ void rows(const W (*st)[kEoMSites], int s, int lam, cx<float> a[6])
+    template <int S>
+    static __device__ __forceinline__ void rows(const W (*st)[S], int s, int lam, cx<float> a[6])
     {
         const int base = (lam >= 4 ? 12 : 0) + 3 * (lam & 3);
 #pragma unroll
@@ -85,8 +89,8 @@ struct EoMStage<P32> {
         }
     }
     // y = A^-1 v or A v, block b
-    template <int MODE>
-    static __device__ __forceinline__ void block_mul(const W (*st)[kEoMSites], int s, int b, const cx<float> v[6],
+    template <int MODE, int S>
+    static __device__ __forceinline__ void block_mul(const W (*st)[S], int s, int b, const cx<float> v[6],
                                                      cx<float> y[6])
     {
         if (MODE == 0) {
@@ -140,7 +144,8 @@ struct EoMStage<P16> {
             out = make_uint4(a.x, a.y, 0u, 0u);
         }
     }
-    static __device__ __forceinline__ void rows(const W (*st)[kEoMSites], int s, int lam, cx<float> a[6])
+    template <int S>
+    static __device__ __forceinline__ void rows(const W (*st)[S], int s, int lam, cx<float> a[6])
     {
         const int mu = lam & 3;
         const bool bwd = lam >= 4;
@@ -157,8 +162,8 @@ struct EoMStage<P16> {
     {
         return k == 0 ? v.x : k == 1 ? v.y : k == 2 ? v.z : v.w;
     }
-    template <int MODE>
-    static __device__ __forceinline__ void block_mul(const W (*st)[kEoMSites], int s, int b, const cx<float> v[6],
+    template <int MODE, int S>
+    static __device__ __forceinline__ void block_mul(const W (*st)[S], int s, int b, const cx<float> v[6],
                                                      cx<float> y[6])
     {
         if (MODE == 0) {
@@ -182,51 +187,50 @@ struct EoMStage<P16> {
 };
 
 // the two hops of direction MU of site x (full index, coordinates c) of the
-// half field `in` (opposite parity), links from the stage
-// link lam (mu, or 4 + mu for U_mu(x - mu)) of site s from the stage: the
-// two stored rows and the third row rebuilt once per site at staging
-template <class P>
-__device__ __forceinline__ void eom_link(const typename EoMStage<P>::W (*st)[kEoMSites],
-                                         const float2 (*r3)[3][kEoMSites], int s, int lam, cx<float> a[6],
-                                         cx<float> c[3])
-{
-    EoMStage<P>::rows(st, s, lam, a);
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-        const float2 v = r3[lam][j][s];
-        c[j] = mkc(v.x, v.y);
-    }
-}
-
-// (FIN: `in` is a full-lattice field, read at the full index)
-template <class P, int MU, int SF, int SB, bool FIN>
-__device__ __forceinline__ void eom_hops(const Geom &g, const typename EoMStage<P>::W (*st)[kEoMSites],
-                                        const float2 (*r3)[3][kEoMSites], int s, const void *in,
-                                        const float *in_nrm, int Vh, int x, const int c[4], cx<float> acc[12])
+// half field `in` (opposite parity), or (FIN) of a full-lattice field read at
+// the full index; links from the stage, their third rows rebuilt there
+template <class P, int MU, int SF, bool FIN, int S>
+__device__ __forceinline__ void eom_hops(const Geom &g, const typename EoMStage<P>::W (*st)[S],
+                                        const float2 (*r3)[3][S], int s, const void *in, const float *in_nrm, int Vh,
+                                        int x, const int c[4], cx<float> acc[12])
 {
     const int Vin = FIN ? g.V : Vh;
     const int L = g.L[MU], stride = g.stride[MU];
+    const bool wf = c[MU] == L - 1, wb = c[MU] == 0;
+    const int xf = wc_idx(wf ? x - (L - 1) * stride : x + stride, g.V);
+    const int xb = wc_idx(wb ? x + (L - 1) * stride : x - stride, g.V);
+    const auto load = [&](int y, bool wrap, cx<float> p[12]) {   // the factor of the hop
+        const float scale = P::load_spinor_raw(in, in_nrm, Vin, FIN ? y : y >> 1, p);
+        return (MU == 3 && wrap) ? (float)g.tbc * scale : scale;
+    };
+    const auto link = [&](int lam, cx<float> u[6], cx<float> r2[3]) {
+        EoMStage<P>::rows(st, s, lam, u);
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            const float2 v = r3[lam][j][s];
+            r2[j] = mkc(v.x, v.y);
+        }
+    };
+    const auto scaled = [&](float f, cx<float> h[6]) {
+        if (std::is_same<P, P32>::value && (MU != 3 || f == 1.f)) return;
+#pragma unroll
+        for (int k = 0; k < 6; ++k) h[k] = f * h[k];
+    };
     {
-        const bool wrap = c[MU] == L - 1;
-        const int xf = wc_idx(wrap ? x - (L - 1) * stride : x + stride, g.V);
-        cx<float> p[12], h[6], u[6], r2[3], w[6];
-        const float scale = P::load_spinor_raw(in, in_nrm, Vin, FIN ? xf : xf >> 1, p);
-        const float coef = ((MU == 3 && wrap) ? (float)g.tbc : 1.f) * scale;
+        cx<float> p[12], h[6], u[6], r2[3];
+        const float f = load(xf, wf, p);
         project<MU, SF>(p, h);
-        eom_link<P>(st, r3, s, MU, u, r2);
-        su3_mul(u, r2, h, coef, w);
-        reconstruct_add<MU, SF>(acc, w);
+        scaled(f, h);
+        link(MU, u, r2);
+        mul_reconstruct_add<MU, SF, true>(u, r2, h, acc);
     }
     {
-        const bool wrap = c[MU] == 0;
-        const int xb = wc_idx(wrap ? x + (L - 1) * stride : x - stride, g.V);
-        cx<float> p[12], h[6], u[6], r2[3], w[6];
-        const float scale = P::load_spinor_raw(in, in_nrm, Vin, FIN ? xb : xb >> 1, p);
-        const float coef = ((MU == 3 && wrap) ? (float)g.tbc : 1.f) * scale;
-        project<MU, SB>(p, h);
-        eom_link<P>(st, r3, s, 4 + MU, u, r2);
-        su3_adj_mul(u, r2, h, coef, w);
-        reconstruct_add<MU, SB>(acc, w);
+        cx<float> p[12], h[6], u[6], r2[3];
+        const float f = load(xb, wb, p);
+        project<MU, -SF>(p, h);
+        scaled(f, h);
+        link(4 + MU, u, r2);
+        mul_reconstruct_add<MU, -SF, false>(u, r2, h, acc);
     }
 }
 
@@ -248,20 +252,20 @@ __device__ __forceinline__ int eom_full_site(const Geom &g, int i, int p, int c[
 // it, so wc_apply_schur_multi needs no split and merge passes (at
 // 16^3x32 with 12 FP32 fields two launches instead of 26: 48 of them, 264
 // us, in an M^+ M^ pair before).
-template <class P, int DAG, int MODE, bool FULL>
+template <class P, int DAG, int MODE, bool FULL, int S>
 __global__ void __maxnreg__(80) k_eo_multi(Geom g, int p, GaugeStore U, CloverStore Blk,
                                                                    const __grid_constant__ EoMultiArgs a,
                                                                    double beta)
 {
     using W = typename EoMStage<P>::W;
     constexpr int NW = EoMStage<P>::template words<MODE>;
-    __shared__ W st[NW][kEoMSites];
-    __shared__ float2 r3[8][3][kEoMSites];   // third rows of the 8 links
+    __shared__ W st[NW][S];
+    __shared__ float2 r3[8][3][S];   // third rows of the 8 links
     const int Vh = g.V >> 1;
-    const int i0 = blockIdx.x * kEoMSites;
-    // blockDim is a multiple of kEoMSites: a thread stages and computes the
+    const int i0 = blockIdx.x * S;
+    // blockDim is a multiple of S: a thread stages and computes the
     // same site s
-    const int s = threadIdx.x % kEoMSites, r = threadIdx.x / kEoMSites, i = i0 + s;
+    const int s = threadIdx.x % S, r = threadIdx.x / S, i = i0 + s;
     int c[4] = {0, 0, 0, 0}, x = 0;
     if (i < Vh) {
         x = eom_full_site(g, i, p, c);
@@ -270,13 +274,13 @@ __global__ void __maxnreg__(80) k_eo_multi(Geom g, int p, GaugeStore U, CloverSt
         for (int mu = 0; mu < 4; ++mu)
             xb[mu] = wc_idx(c[mu] == 0 ? x + (g.L[mu] - 1) * g.stride[mu] : x - g.stride[mu], g.V);
         const int pos = wc_idx(p * Vh + i, g.V);
-        for (int item = r; item < NW; item += blockDim.x / kEoMSites)
+        for (int item = r; item < NW; item += blockDim.x / S)
             EoMStage<P>::template stage<MODE>(U, Blk, g.V, item, x, xb, pos, st[item][s]);
     }
     __syncthreads();
     // the third row of every staged link, once per site
-    for (int q = threadIdx.x; q < 8 * kEoMSites; q += blockDim.x) {
-        const int ss = q % kEoMSites, lam = q / kEoMSites;
+    for (int q = threadIdx.x; q < 8 * S; q += blockDim.x) {
+        const int ss = q % S, lam = q / S;
         if (i0 + ss >= Vh) continue;
         cx<float> u[6], c3[3];
         EoMStage<P>::rows(st, ss, lam, u);
@@ -286,18 +290,18 @@ __global__ void __maxnreg__(80) k_eo_multi(Geom g, int p, GaugeStore U, CloverSt
     }
     __syncthreads();
     if (r >= a.n) return;
-    if (a.skip[r] && *a.skip[r]) return;   // the whole warp: one field per warp
+    if (a.skip[r] && *a.skip[r]) return;   // all S threads of the field
     float red[4] = {0.f, 0.f, 0.f, 0.f};
     if (i < Vh) {
     constexpr int SF = DAG ? +1 : -1;
-    constexpr int SB = -SF;
+    constexpr bool FIN = FULL && MODE == 0;
     cx<float> h[12];
 #pragma unroll
     for (int k = 0; k < 12; ++k) h[k] = mkc(0.f, 0.f);
-    eom_hops<P, 0, SF, SB, FULL && MODE == 0>(g, st, r3, s, a.hin[r], a.hin_nrm[r], Vh, x, c, h);
-    eom_hops<P, 1, SF, SB, FULL && MODE == 0>(g, st, r3, s, a.hin[r], a.hin_nrm[r], Vh, x, c, h);
-    eom_hops<P, 2, SF, SB, FULL && MODE == 0>(g, st, r3, s, a.hin[r], a.hin_nrm[r], Vh, x, c, h);
-    eom_hops<P, 3, SF, SB, FULL && MODE == 0>(g, st, r3, s, a.hin[r], a.hin_nrm[r], Vh, x, c, h);
+    eom_hops<P, 0, SF, FIN>(g, st, r3, s, a.hin[r], a.hin_nrm[r], Vh, x, c, h);
+    eom_hops<P, 1, SF, FIN>(g, st, r3, s, a.hin[r], a.hin_nrm[r], Vh, x, c, h);
+    eom_hops<P, 2, SF, FIN>(g, st, r3, s, a.hin[r], a.hin_nrm[r], Vh, x, c, h);
+    eom_hops<P, 3, SF, FIN>(g, st, r3, s, a.hin[r], a.hin_nrm[r], Vh, x, c, h);
     cx<float> v[12], o[12];
     const float bt = (float)beta;
     if (MODE == 0) {
@@ -339,24 +343,26 @@ __global__ void __maxnreg__(80) k_eo_multi(Geom g, int p, GaugeStore U, CloverSt
     }
     }   // i < Vh
     if (MODE == 1 && a.red != 0) {
-        // the warp holds the 32 sites of this CTA for field r
+        // S adjacent lanes hold the sites of this CTA for field r; the other
+        // field of the warp may have left it
+        const unsigned lanes = S == 32 ? 0xffffffffu : 0xffffu << (threadIdx.x & 16);
 #pragma unroll
         for (int c = 0; c < 4; ++c)
 #pragma unroll
-            for (int o2 = 16; o2 > 0; o2 >>= 1) red[c] += __shfl_xor_sync(0xffffffffu, red[c], o2);
+            for (int o2 = S / 2; o2 > 0; o2 >>= 1) red[c] += __shfl_xor_sync(lanes, red[c], o2);
         if (s == 0)
 #pragma unroll
             for (int c = 0; c < 4; ++c) a.part[((size_t)r * gridDim.x + blockIdx.x) * 4 + c] = (double)red[c];
     }
 }
 
-template <class P, int DAG, bool FULL>
-cudaError_t launch_eom(const wc_lattice_s *full, int n, wc_field_s *const *outs, wc_field_s *const *ins,
+template <class P, int DAG, bool FULL, int S>
+cudaError_t launch_eom_s(const wc_lattice_s *full, int n, wc_field_s *const *outs, wc_field_s *const *ins,
                        wc_field_s *const *tmps, const int *const *skip, int red, wc_field const *dots, double *part,
                        cudaStream_t stream)
 {
     const int Vh = full->g.V >> 1;
-    const dim3 grid((Vh + kEoMSites - 1) / kEoMSites), block(kEoMSites * n);
+    const dim3 grid((Vh + S - 1) / S), block(S * n);
     EoMultiArgs a{};
     a.n = n;
     for (int r = 0; r < n; ++r) {
@@ -367,7 +373,7 @@ cudaError_t launch_eom(const wc_lattice_s *full, int n, wc_field_s *const *outs,
         a.out_nrm[r] = tmps[r]->nrm;
     }
     // odd sites: tmp = A_oo^-1 H_oe in
-    k_eo_multi<P, DAG, 0, FULL><<<grid, block, 0, stream>>>(full->g, 1, full->gauge, full->cinv, a, 0.0);
+    k_eo_multi<P, DAG, 0, FULL, S><<<grid, block, 0, stream>>>(full->g, 1, full->gauge, full->cinv, a, 0.0);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     // even sites: out = A_ee in - kappa^2 H_eo tmp
@@ -382,9 +388,20 @@ cudaError_t launch_eom(const wc_lattice_s *full, int n, wc_field_s *const *outs,
     a.red = red;
     a.part = part;
     for (int r = 0; r < n && red == 1; ++r) a.dot[r] = dots[r]->data;
-    k_eo_multi<P, DAG, 1, FULL><<<grid, block, 0, stream>>>(full->g, 0, full->gauge, full->ceo, a,
+    k_eo_multi<P, DAG, 1, FULL, S><<<grid, block, 0, stream>>>(full->g, 0, full->gauge, full->ceo, a,
                                                       -full->kappa * full->kappa);
     return cudaGetLastError();
+}
+
+constexpr int kEomSmall = 6;   // fields up to which a CTA takes 32 sites
+
+template <class P, int DAG, bool FULL>
+cudaError_t launch_eom(const wc_lattice_s *full, int n, wc_field_s *const *outs, wc_field_s *const *ins,
+                       wc_field_s *const *tmps, const int *const *skip, int red, wc_field const *dots, double *part,
+                       cudaStream_t stream)
+{
+    return n > kEomSmall ? launch_eom_s<P, DAG, FULL, 16>(full, n, outs, ins, tmps, skip, red, dots, part, stream)
+                         : launch_eom_s<P, DAG, FULL, 32>(full, n, outs, ins, tmps, skip, red, dots, part, stream);
 }
 
 }  // namespace
@@ -406,7 +423,11 @@ cudaError_t launch_schur_multi(wc_lattice half, int n, wc_field const *outs, wc_
     return cudaErrorInvalidValue;
 }
 
-int schur_multi_blocks(wc_lattice half) { return (half->g.V + kEoMSites - 1) / kEoMSites; }
+int schur_multi_blocks(wc_lattice half, int n)
+{
+    const int S = n > kEomSmall ? 16 : 32;
+    return (half->g.V + S - 1) / S;
+}
 
 }  // namespace wc
 

@@ -212,10 +212,10 @@ cudaError_t extract_clover(wc_lattice sub, cudaStream_t stream);
 
 // multi-right-hand-side FP32 operator (wc_mrhs.cu): outs[r] = M ins[r]
 // (kind 0) or M^+ ins[r] (kind 1) for r < n <= kMrhsMax, links and clover
-// read once per site; active (nullable, device): 0 skips right-hand side r
+// read once per site
 constexpr int kMrhsMax = 16;
 cudaError_t launch_apply_multi(wc_lattice lat, int n, const wc_field *outs, const wc_field *ins, int kind,
-                               const int *active, cudaStream_t stream);
+                               cudaStream_t stream);
 
 // multi-right-hand-side Schur operator (wc_eomulti.cu): outs[r] = M^ ins[r]
 // (M^+ with dagger) for FP32 or FP16 half-lattice fields of the half lattice
@@ -224,9 +224,9 @@ cudaError_t launch_apply_multi(wc_lattice lat, int n, const wc_field *outs, cons
 cudaError_t launch_schur_multi(wc_lattice half, int n, wc_field const *outs, wc_field const *ins,
                                wc_field const *tmps, int dagger, const int *const *skip, cudaStream_t stream,
                                int red = 0, wc_field const *dots = nullptr, double *part = nullptr);
-// CTAs of one multi-RHS Schur pass on the half lattice `half` (the second
-// dimension of its partial sums)
-int schur_multi_blocks(wc_lattice half);
+// CTAs of one multi-RHS Schur pass of n fields on the half lattice `half` (the
+// second dimension of its partial sums)
+int schur_multi_blocks(wc_lattice half, int n);
 
 // even-odd preconditioning (wc_evenodd.cu)
 // tmp: a half-lattice field of out's precision for the odd-site

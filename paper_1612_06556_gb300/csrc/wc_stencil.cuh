@@ -89,6 +89,40 @@ __device__ __forceinline__ void reconstruct_add(cx<R> acc[12], const cx<R> w[6])
     }
 }
 
+// acc += the spin reconstruction of W h, W = U (FWD) or U^+, one colour of W
+// h at a time: the two-spinor product is never live as a whole, which keeps a
+// kernel of many warps per SM in 64 registers
+template <int MU, int S, bool FWD, class R>
+__device__ __forceinline__ void mul_reconstruct_add(const cx<R> u[6], const cx<R> r2[3], const cx<R> h[6], cx<R> acc[12])
+{
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        const cx<R> m0 = FWD ? (c < 2 ? u[3 * c] : r2[0]) : conj(u[c]),
+                    m1 = FWD ? (c < 2 ? u[3 * c + 1] : r2[1]) : conj(u[3 + c]),
+                    m2 = FWD ? (c < 2 ? u[3 * c + 2] : r2[2]) : conj(r2[c]);
+        cx<R> w0 = m0 * h[0], w1 = m0 * h[3];
+        w0 = cfma(m1, h[1], w0);
+        w1 = cfma(m1, h[4], w1);
+        w0 = cfma(m2, h[2], w0);
+        w1 = cfma(m2, h[5], w1);
+        acc[c] = acc[c] + w0;
+        acc[3 + c] = acc[3 + c] + w1;
+        if (MU == 0) {
+            acc[6 + c] = acc[6 + c] - sgn<S>(times_i(w1));
+            acc[9 + c] = acc[9 + c] - sgn<S>(times_i(w0));
+        } else if (MU == 1) {
+            acc[6 + c] = acc[6 + c] - sgn<S>(w1);
+            acc[9 + c] = acc[9 + c] + sgn<S>(w0);
+        } else if (MU == 2) {
+            acc[6 + c] = acc[6 + c] - sgn<S>(times_i(w0));
+            acc[9 + c] = acc[9 + c] + sgn<S>(times_i(w1));
+        } else {
+            acc[6 + c] = acc[6 + c] + sgn<S>(w0);
+            acc[9 + c] = acc[9 + c] + sgn<S>(w1);
+        }
+    }
+}
+
 // w = coef * U h  (per spin of the two-spinor)
 template <class R>
 __device__ __forceinline__ void su3_mul(const cx<R> u[6], const cx<R> r2[3], const cx<R> h[6], R coef,

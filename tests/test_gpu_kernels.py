@@ -270,3 +270,47 @@ def test_even_odd_passes_of_a_solve(dims, tbc, arith):
     S0, F0, _, _ = oracle.action_and_force(oracle.Operator(dims, U, csw, kappa, tbc), src, tol=1e-14)
     assert abs(S - S0) <= 1e-11 * S0
     assert_elementwise(F, F0, 1e-9)
+
+
+@pytest.mark.parametrize("n", [4, 5, 6, 7, 16])
+@pytest.mark.parametrize("dims,tbc", [((3, 5, 2, 3), -1), ((4, 4, 4, 4), 1), ((6, 2, 2, 6), -1)])
+def test_multi_field_operators_on_16_and_32_sites(n, dims, tbc):
+    """M and M^+ of n fields on both sides of the rule for a CTA's sites (4
+    and 6 fields), on ragged volumes and odd n (a warp of one and a half
+    fields); the Schur form where all extents are even."""
+    csw, kappa = 1.2, 0.12
+    U = synth.haar_links(dims, 190 + n)
+    lat = make_lattice(dims, U, csw, kappa, tbc)
+    op = oracle.Operator(dims, U, csw, kappa, tbc)
+    srcs = [synth.gaussian_source(dims, 200 + r) for r in range(n)]
+    ins, outs = [lat.field(1).load(s) for s in srcs], [lat.field(1) for _ in srcs]
+    for dagger in (False, True):
+        lat.apply_multi(outs, ins, dagger)
+        for s, f in zip(srcs, outs):
+            assert_elementwise(f.store(np.zeros_like(s)), op.Mdag(s) if dagger else op.M(s), 1e-5)
+    if any(d % 2 for d in dims):
+        return
+    eo = EvenOdd(dims, tbc, kappa, U, op.T)
+    for prec in (1, 2):
+        ins, outs = [lat.field(prec).load(s) for s in srcs], [lat.field(prec) for _ in srcs]
+        lat.apply_schur_multi(outs, ins, True)
+        for s, f in zip(srcs, outs):
+            assert_elementwise(f.store(np.zeros_like(s)), eo.schur(s, True), TOL[prec])
+
+
+@pytest.mark.parametrize("n", [5, 7, 12])
+def test_lockstep_group_whose_members_stop_apart(n):
+    """The fused inner products of a lockstep group with n members, one of
+    which has a zero source: its lanes leave while the other field of the
+    warp goes on."""
+    dims, kappa, csw, tbc = (4, 4, 4, 6), 0.12, 1.0, -1
+    U = synth.exp_links(dims, 0.3, 210)
+    lat = make_lattice(dims, U, csw, kappa, tbc)
+    srcs = [synth.gaussian_source(dims, 211 + r) if r != 2 else np.zeros((int(np.prod(dims)), 4, 3), complex) for r in range(n)]
+    xs = [lat.field(0) for _ in srcs]
+    infos = wc().solve_batch([lat] * n, xs, [lat.field(0).load(s) for s in srcs], tol=1e-10, solver=wc().SOLVER_RELIABLE,
+                             even_odd=True)
+    for s, x, info in zip(srcs, xs, infos):
+        sol = x.store(np.zeros_like(s))
+        r = s - oracle.apply_M(dims, tbc, kappa, csw, U, sol)
+        assert info.status == 0 and np.linalg.norm(r) <= 1.5e-10 * np.linalg.norm(s)
