@@ -33,14 +33,38 @@
 // second term gives the same F as c W_k(Xi^+), so only the Hermitian
 // Xh = Xi + Xi^+ enters (k_xi stores it, 9 reals per plane and site), and
 //   sum_k W_k(Xh_k) = U [ Xh(c1) T + L1 (S2 Xh(x) + (Xh(c2) L2 + L2 Xh(c3)) L3) ]
-// with S2 = L2 L3 and T = L1 S2: eight 3x3 products per leaf pair (nu, d)
-// instead of twenty-one for the four insertions taken one by one.
+// with S2 = L2 L3 and T = L1 S2.
+//
+// The four links of a plaquette see the same insertions, so k_force_plaq
+// forms their sum once per plaquette and carries it from link to link.  Let
+// L0 = U_a(x), L1 = U_b(x+a), V = U_a(x+b), W = U_b(x) be the links of the
+// plaquette of (a, b), a < b, at x, P = L0 L1 V^+ W^+, Z0, Z1, Z2, Z3 = Xh_ab at
+// x, x+a, x+a+b, x+b, G = sum_k W_k the sum for the link L0, and Hm(M) = (M +
+// M^+)/2.  As c is imaginary, F = TA(c M) = c Hm(M) - trace, and of G only H =
+// Hm(G) is needed:
+//   G = (L0 (Z1 L1 + L1 Z2) V^+ + L0 L1 V^+ Z3) W^+ + P Z0.
+// Beginning the loop at another corner moves one insertion from the end of the
+// product to its front, which adds a commutator [Z, P] there, and Hm([Z, P]) =
+// Hm(Z X) with X = P - P^+.  In units of c with sigma = +1 the links get
+//   U_a(x)     H
+//   U_b(x)     -(H + Hm(Z0 X))
+//   U_b(x+a)   H1 - Hm(Z1 X1),      H1 + X1 = L0^+ (H + X) L0
+//   U_a(x+b)   -(H3 + Hm(Z3 X3)),   H3 + X3 = W^+ (H + Hm(Z0 X) + X) W
+// (Hermitian and anti-Hermitian parts of the carried matrix): about 1680 FP64
+// operations per plaquette, 10 000 a site, where the four insertions of each
+// leaf pair taken link by link are 19 000.  k_force_link adds the six
+// contributions of a link and its hopping part; two planes at a time, the
+// pairs (xy, zt), (xz, yt), (yz, xt) that contain every direction once.
+//
+// Everything here is bound by the FP64 pipe.  At 16^3x32 (k_xi + the force):
+// 244 + 4650 us link by link; now the plaquettes 3 x 794, the last link pass 313.
 
 #include <math.h>
 
 #include "wc_internal.cuh"
 #include "wc_solver.cuh"
 #include "wc_solver_kernels.cuh"
+#include "wc_stencil.cuh"
 
 namespace wc {
 
@@ -76,25 +100,7 @@ __device__ __forceinline__ M3 dag(const M3 &a)
     return r;
 }
 
-__device__ __forceinline__ M3 ident()
-{
-    M3 r;
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) r.m[i][j] = mkc(i == j ? 1.0 : 0.0, 0.0);
-    return r;
-}
-
-__device__ __forceinline__ void add_scaled(M3 &acc, cx<double> s, const M3 &a)
-{
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) acc.m[i][j] = cfma(s, a.m[i][j], acc.m[i][j]);
-}
-
-__device__ M3 link(const GaugeStore &g, int V, int mu, int x)
+__device__ __forceinline__ M3 link(const GaugeStore &g, int V, int mu, int x)
 {
     cx<double> u[6], r2[3];
     P64::load_link(g, V, mu, x, u, r2);
@@ -108,48 +114,10 @@ __device__ M3 link(const GaugeStore &g, int V, int mu, int x)
     return r;
 }
 
-__device__ __forceinline__ int shift(const Geom &g, const int c[4], int mu, int dmu, int nu, int dnu)
-{
-    int d[4] = {c[0], c[1], c[2], c[3]};
-    d[mu] = (d[mu] + dmu + g.L[mu]) % g.L[mu];
-    d[nu] = (d[nu] + dnu + g.L[nu]) % g.L[nu];
-    return d[0] + g.stride[1] * d[1] + g.stride[2] * d[2] + g.stride[3] * d[3];
-}
-
 // plane index of (a, b), a < b: xy xz xt yz yt zt
 __device__ __forceinline__ int plane_of(int a, int b)
 {
     return a == 0 ? b - 1 : a == 1 ? b + 1 : 5;
-}
-
-// 2x2 block of sigma_ab on spin pair blk (chiral basis), as complex entries
-// sigma_xy = -s3, sigma_xz = s2, sigma_yz = -s1 on both pairs;
-// sigma_xt = eta s1, sigma_yt = eta s2, sigma_zt = eta s3, eta = -1, +1
-__device__ __forceinline__ void sigma_block(int plane, int blk, cx<double> s[2][2])
-{
-    const double eta = blk == 0 ? -1.0 : 1.0;
-    int pauli;
-    double sg;
-    switch (plane) {
-    case 0: pauli = 3; sg = -1.0; break;   // xy
-    case 1: pauli = 2; sg = 1.0; break;    // xz
-    case 2: pauli = 1; sg = eta; break;    // xt
-    case 3: pauli = 1; sg = -1.0; break;   // yz
-    case 4: pauli = 2; sg = eta; break;    // yt
-    default: pauli = 3; sg = eta; break;   // zt
-    }
-    const cx<double> z = mkc(0.0, 0.0);
-    s[0][0] = s[0][1] = s[1][0] = s[1][1] = z;
-    if (pauli == 1) {
-        s[0][1] = mkc(sg, 0.0);
-        s[1][0] = mkc(sg, 0.0);
-    } else if (pauli == 2) {
-        s[0][1] = mkc(0.0, -sg);
-        s[1][0] = mkc(0.0, sg);
-    } else {
-        s[0][0] = mkc(sg, 0.0);
-        s[1][1] = mkc(-sg, 0.0);
-    }
 }
 
 // Hermitian 3x3 matrix: real diagonal d, upper entries o = (h01, h02, h12)
@@ -209,225 +177,394 @@ __device__ __forceinline__ M3 zero3()
     return r;
 }
 
+__device__ __forceinline__ M3 mul_dag(const M3 &a, const M3 &b) { return mul(a, dag(b)); }
+
+// off-diagonal entry q of an H3 / X3: rows and columns
+__device__ __forceinline__ int off_row(int q) { return q == 2 ? 1 : 0; }
+__device__ __forceinline__ int off_col(int q) { return q == 0 ? 1 : 2; }
+
+// anti-Hermitian 3x3 matrix: i d on the diagonal, upper entries o
+struct X3 {
+    double d[3];
+    cx<double> o[3];
+};
+
+__device__ __forceinline__ H3 operator+(const H3 &a, const H3 &b)
+{
+    H3 r;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        r.d[k] = a.d[k] + b.d[k];
+        r.o[k] = a.o[k] + b.o[k];
+    }
+    return r;
+}
+
+// entry (i, j) of X, i != j
+__device__ __forceinline__ cx<double> xoff(const X3 &x, int i, int j)
+{
+    const cx<double> v = x.o[i + j - 1];
+    return i < j ? v : -conj(v);
+}
+
+// 2 Hm(E W^+ + P Z)
+__device__ __forceinline__ H3 herm2(const M3 &e, const M3 &w, const M3 &p, const H3 &z)
+{
+    // entry (i, j) of E W^+ + P Z
+    const auto at = [&](int i, int j) {
+        cx<double> s = mkc(0.0, 0.0);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) s = cfma_conj(w.m[j][k], e.m[i][k], s);
+        s.re = fma(p.m[i][j].re, z.d[j], s.re);
+        s.im = fma(p.m[i][j].im, z.d[j], s.im);
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+            if (k != j) s = cfma(p.m[i][k], hoff(z, k, j), s);
+        return s;
+    };
+    H3 r;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        double s = 0.0;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) s = fma(e.m[i][k].re, w.m[i][k].re, fma(e.m[i][k].im, w.m[i][k].im, s));
+        s = fma(p.m[i][i].re, z.d[i], s);
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+            if (k != i) {
+                const cx<double> h = hoff(z, k, i);
+                s = fma(p.m[i][k].re, h.re, fma(-p.m[i][k].im, h.im, s));
+            }
+        r.d[i] = 2.0 * s;
+    }
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        const int i = off_row(q), j = off_col(q);
+        r.o[q] = at(i, j) + conj(at(j, i));
+    }
+    return r;
+}
+
+// 2 Hm(Z X)
+__device__ __forceinline__ H3 herm2_zx(const H3 &z, const X3 &x)
+{
+    H3 r;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        double s = 0.0;   // Re (Z X)_ii: Z_ii times the imaginary X_ii drops out
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+            if (k != i) {
+                const cx<double> h = hoff(z, i, k), a = xoff(x, k, i);
+                s = fma(h.re, a.re, fma(-h.im, a.im, s));
+            }
+        r.d[i] = 2.0 * s;
+    }
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        const int i = off_row(q), j = off_col(q), k = 3 - i - j;
+        const auto at = [&](int a, int b) {
+            const cx<double> xab = xoff(x, a, b), zab = hoff(z, a, b);
+            cx<double> s = mkc(z.d[a] * xab.re, z.d[a] * xab.im);
+            s.re = fma(-zab.im, x.d[b], s.re);   // Z_ab i X_bb
+            s.im = fma(zab.re, x.d[b], s.im);
+            return cfma(hoff(z, a, k), xoff(x, k, b), s);
+        };
+        r.o[q] = at(i, j) + conj(at(j, i));
+    }
+    return r;
+}
+
+// U^+ (h + x) U as its Hermitian and anti-Hermitian parts, twice each
+__device__ __forceinline__ void carry2(const H3 &h, const X3 &x, const M3 &u, H3 &hc, X3 &xc)
+{
+    M3 m;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) m.m[i][i] = mkc(h.d[i], x.d[i]);
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        const int i = off_row(q), j = off_col(q);
+        m.m[i][j] = h.o[q] + x.o[q];
+        m.m[j][i] = conj(h.o[q] - x.o[q]);
+    }
+    const M3 t = mul(m, u);
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            cx<double> s = cmul_conj(u.m[0][i], t.m[0][j]);
+            s = cfma_conj(u.m[1][i], t.m[1][j], s);
+            m.m[i][j] = cfma_conj(u.m[2][i], t.m[2][j], s);
+        }
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        hc.d[i] = 2.0 * m.m[i][i].re;
+        xc.d[i] = 2.0 * m.m[i][i].im;
+    }
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        const cx<double> a = m.m[off_row(q)][off_col(q)], b = conj(m.m[off_col(q)][off_row(q)]);
+        hc.o[q] = a + b;
+        xc.o[q] = a - b;
+    }
+}
+
+__device__ __forceinline__ void store_h3(double *p, int V, int x, const H3 &h)
+{
+#pragma unroll
+    for (int k = 0; k < 3; ++k) p[(size_t)k * V + x] = h.d[k];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        p[(size_t)(3 + 2 * k) * V + x] = h.o[k].re;
+        p[(size_t)(4 + 2 * k) * V + x] = h.o[k].im;
+    }
+}
+
+__device__ __forceinline__ H3 load_h3(const double *p, int V, int x)
+{
+    H3 h;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) h.d[k] = __ldg(p + (size_t)k * V + x);
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+        h.o[k] = mkc(__ldg(p + (size_t)(3 + 2 * k) * V + x), __ldg(p + (size_t)(4 + 2 * k) * V + x));
+    return h;
+}
+
 // Xh_ab(y) = Xi + Xi^+ for the six planes, Xi the traceless part of
 // sum_{s,t} sigma_ab[s][t] X_t(y) Y_s(y)^+.  Layout [6][9][V] doubles:
-// h00 h11 h22, re/im of h01, h02, h12.
-__global__ void k_xi(Geom g, const double2 *X, const double2 *Y, double *xh)
+// h00 h11 h22, re/im of h01, h02, h12.  On spin pair 0 / 1 sigma is (s1, s2, s3
+// the Pauli matrices) xy -s3, xz s2, xt -/+s1, yz -s1, yt -/+s2, zt -/+s3: the
+// Hermitian parts of the three Pauli sums of each pair, added and subtracted.
+__global__ void __launch_bounds__(64) k_xi(Geom g, const double2 *X, const double2 *Y, double *xh)
 {
     const int y = blockIdx.x * blockDim.x + threadIdx.x;
     if (y >= g.V) return;
     const int V = g.V;
-    cx<double> xs[12], ys[12];
+    H3 s[2][3];   // [pair][Pauli]: S + S^+
 #pragma unroll
-    for (int k = 0; k < 12; ++k) {
-        const double2 a = X[(size_t)k * V + y], b = Y[(size_t)k * V + y];
-        xs[k] = mkc(a.x, a.y);
-        ys[k] = mkc(b.x, b.y);
+    for (int b = 0; b < 2; ++b) {
+        cx<double> x[6], w[6];
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+            const double2 u = __ldg(X + (size_t)(6 * b + k) * V + y), v = __ldg(Y + (size_t)(6 * b + k) * V + y);
+            x[k] = mkc(u.x, u.y);
+            w[k] = mkc(v.x, v.y);
+        }
+        // O_st = X_t Y_s^+
+        const auto o = [&](int sp, int t, int i, int j) { return cmul_conj(w[3 * sp + j], x[3 * t + i]); };
+        const auto osub = [&](int sp, int t, int i, int j, cx<double> a) { return cfma_conj(w[3 * sp + j], -x[3 * t + i], a); };
+#pragma unroll
+        for (int q = 0; q < 6; ++q) {   // the diagonal, then the three pairs (i, j)
+            const int i = q < 3 ? q : off_row(q - 3), j = q < 3 ? q : off_col(q - 3);
+            const cx<double> a01 = o(0, 1, i, j), a10 = o(1, 0, i, j), a3 = osub(1, 1, i, j, o(0, 0, i, j));
+            const cx<double> p1 = a01 + a10, p2 = times_i(a10 - a01);
+            if (q < 3) {
+                s[b][0].d[q] = 2.0 * p1.re;
+                s[b][1].d[q] = 2.0 * p2.re;
+                s[b][2].d[q] = 2.0 * a3.re;
+            } else {
+                const cx<double> c01 = o(0, 1, j, i), c10 = o(1, 0, j, i), c3 = osub(1, 1, j, i, o(0, 0, j, i));
+                s[b][0].o[q - 3] = p1 + conj(c01 + c10);
+                s[b][1].o[q - 3] = p2 + conj(times_i(c10 - c01));
+                s[b][2].o[q - 3] = a3 + conj(c3);
+            }
+        }
     }
+    // planes xy xz xt yz yt zt: Pauli matrix and the signs of the two pairs
+    constexpr int pauli[6] = {2, 1, 0, 0, 1, 2};
+    constexpr double s0[6] = {-1.0, 1.0, -1.0, -1.0, -1.0, -1.0}, s1[6] = {-1.0, 1.0, 1.0, -1.0, 1.0, 1.0};
 #pragma unroll
     for (int pl = 0; pl < 6; ++pl) {
-        M3 Z = zero3();
-#pragma unroll
-        for (int blk = 0; blk < 2; ++blk) {
-            cx<double> sg[2][2];
-            sigma_block(pl, blk, sg);
-#pragma unroll
-            for (int s = 0; s < 2; ++s)
-#pragma unroll
-                for (int t = 0; t < 2; ++t) {
-                    const cx<double> w = sg[s][t];
-                    if (w.re == 0.0 && w.im == 0.0) continue;
-                    const int ss = 2 * blk + s, tt = 2 * blk + t;
-#pragma unroll
-                    for (int i = 0; i < 3; ++i)
-#pragma unroll
-                        for (int j = 0; j < 3; ++j)
-                            Z.m[i][j] = cfma(w, xs[3 * tt + i] * conj(ys[3 * ss + j]), Z.m[i][j]);
-                }
-        }
-        const double tr = (2.0 / 3.0) * (Z.m[0][0].re + Z.m[1][1].re + Z.m[2][2].re);
-        double *o = xh + (size_t)pl * 9 * V + y;
-        o[0] = 2.0 * Z.m[0][0].re - tr;
-        o[(size_t)V] = 2.0 * Z.m[1][1].re - tr;
-        o[2 * (size_t)V] = 2.0 * Z.m[2][2].re - tr;
-        const int ij[3][2] = {{0, 1}, {0, 2}, {1, 2}};
+        const H3 &a = s[0][pauli[pl]], &c = s[1][pauli[pl]];
+        H3 h;
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            const cx<double> v = Z.m[ij[k][0]][ij[k][1]] + conj(Z.m[ij[k][1]][ij[k][0]]);
-            o[(size_t)(3 + 2 * k) * V] = v.re;
-            o[(size_t)(4 + 2 * k) * V] = v.im;
+            h.d[k] = s0[pl] * a.d[k] + s1[pl] * c.d[k];
+            h.o[k] = mkc(s0[pl] * a.o[k].re + s1[pl] * c.o[k].re, s0[pl] * a.o[k].im + s1[pl] * c.o[k].im);
         }
+        const double t = (1.0 / 3.0) * (h.d[0] + h.d[1] + h.d[2]);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) h.d[k] -= t;
+        store_h3(xh + (size_t)pl * 9 * V, V, y, h);
     }
 }
 
-__device__ __forceinline__ H3 load_xh(const double *xh, int V, int plane, int y)
+// The contributions of one plaquette to its four links (see above), twice
+// each, in units of c: slot 0 U_a(x), 1 U_b(x), 2 U_b(x+a), 3 U_a(x+b), at the
+// index of x.  Plane (planes.x, planes.y) for blockIdx.y = 0, (planes.z,
+// planes.w) for 1; ws: [2 planes][4 slots][9][V].
+__global__ void __launch_bounds__(64) k_force_plaq(Geom g, GaugeStore G, const double *xh, int4 planes, double *ws)
 {
-    const double *p = xh + (size_t)plane * 9 * V + y;
-    H3 h;
-#pragma unroll
-    for (int k = 0; k < 3; ++k) h.d[k] = __ldg(p + (size_t)k * V);
-#pragma unroll
-    for (int k = 0; k < 3; ++k) h.o[k] = mkc(__ldg(p + (size_t)(3 + 2 * k) * V), __ldg(p + (size_t)(4 + 2 * k) * V));
-    return h;
-}
-
-// (1 + s gamma_mu) psi as a full spinor (chiral basis)
-__device__ __forceinline__ void project_full(int mu, int s, const cx<double> p[12], cx<double> o[12])
-{
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        const cx<double> u0 = p[c], u1 = p[3 + c], d0 = p[6 + c], d1 = p[9 + c];
-        const double sd = (double)s;
-        cx<double> h0, h1, l0, l1;
-        if (mu == 0) {
-            h0 = u0 + sd * times_i(d1);
-            h1 = u1 + sd * times_i(d0);
-            l0 = (-sd) * times_i(h1);
-            l1 = (-sd) * times_i(h0);
-        } else if (mu == 1) {
-            h0 = u0 + sd * d1;
-            h1 = u1 - sd * d0;
-            l0 = (-sd) * h1;
-            l1 = sd * h0;
-        } else if (mu == 2) {
-            h0 = u0 + sd * times_i(d0);
-            h1 = u1 - sd * times_i(d1);
-            l0 = (-sd) * times_i(h0);
-            l1 = sd * times_i(h1);
-        } else {
-            h0 = u0 + sd * d0;
-            h1 = u1 + sd * d1;
-            l0 = sd * h0;
-            l1 = sd * h1;
-        }
-        o[c] = h0;
-        o[3 + c] = h1;
-        o[6 + c] = l0;
-        o[9 + c] = l1;
-    }
-}
-
-__device__ __forceinline__ void load_sp(const double2 *f, int V, int x, cx<double> s[12])
-{
-#pragma unroll
-    for (int k = 0; k < 12; ++k) {
-        const double2 v = __ldg(f + (size_t)k * V + x);
-        s[k] = mkc(v.x, v.y);
-    }
-}
-
-// acc + sum_s a_s b_s^+ (a, b spinors; 3x3 colour outer products summed over spin)
-__device__ __forceinline__ void fma_outer(const cx<double> a[12], const cx<double> b[12], M3 &acc)
-{
-#pragma unroll
-    for (int s = 0; s < 4; ++s)
-#pragma unroll
-        for (int p = 0; p < 3; ++p)
-#pragma unroll
-            for (int q = 0; q < 3; ++q) acc.m[p][q] = cfma(a[3 * s + p], conj(b[3 * s + q]), acc.m[p][q]);
-}
-
-// The four insertions of the leaf pair (nu, D) with U = L0 factored out:
-// Xh(c1) T + L1 (S2 Xh(x) + (Xh(c2) L2 + L2 Xh(c3)) L3), S2 = L2 L3, T = L1 S2.
-template <int D>
-__device__ __forceinline__ M3 leaf_pair(const Geom &g, const GaugeStore &G, const double *xh, int x, const int c[4],
-                                        int mu, int nu, int pl, int c1)
-{
+    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    if (x >= g.V) return;
     const int V = g.V;
-    const int c2 = shift(g, c, mu, 1, nu, D), c3 = shift(g, c, mu, 0, nu, D);
-    const M3 L2 = dag(link(G, V, mu, c3));                          // c2 -> c3
-    const M3 L3 = D == 1 ? dag(link(G, V, nu, x)) : link(G, V, nu, c3);   // c3 -> x
-    const M3 S2 = mul(L2, L3);
-    M3 K = zero3();
-    fma_hm(load_xh(xh, V, pl, c2), L2, K);
-    fma_mh(L2, load_xh(xh, V, pl, c3), K);
-    K = mul(K, L3);
-    fma_mh(S2, load_xh(xh, V, pl, x), K);
-    const M3 L1 = D == 1 ? link(G, V, nu, c1) : dag(link(G, V, nu, c2));  // c1 -> c2
-    M3 E = mul(L1, K);
-    const M3 T = mul(L1, S2);
-    fma_hm(load_xh(xh, V, pl, c1), T, E);
-    return E;
-}
-
-// one thread per link (x, mu): F = TA(U H), canonical layout [V][4][3][3]
-__global__ void __launch_bounds__(128) k_force(Geom g, GaugeStore G, const double2 *X, const double2 *Y,
-                                               const double *xh, double kappa, double csw, double2 *F)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= 4 * g.V) return;
-    const int V = g.V;
-    const int x = i % V, mu = i / V;
+    const int a = blockIdx.y ? planes.z : planes.x, b = blockIdx.y ? planes.w : planes.y;
+    const double *xp = xh + (size_t)plane_of(a, b) * 9 * V;
+    double *w0 = ws + (size_t)blockIdx.y * 36 * V;
     int c[4];
     site_coords(g, x, c);
-    M3 H = zero3();
-
-    // clover part: H = -(i csw kappa / 4) sum_{nu, d} sigma E(nu, d)
-    if (csw != 0.0) {
-        M3 A = zero3();
-        const int c1 = shift(g, c, mu, 1, mu, 0);
-#pragma unroll 1
-        for (int nu = 0; nu < 4; ++nu) {
-            if (nu == mu) continue;
-            const int pl = plane_of(mu < nu ? mu : nu, mu < nu ? nu : mu);
-            // d = +1 runs counter-clockwise in the (a, b) plane when mu < nu
-            const double sp = mu < nu ? 1.0 : -1.0;
-            const M3 Ep = leaf_pair<1>(g, G, xh, x, c, mu, nu, pl, c1);
-#pragma unroll
-            for (int a = 0; a < 3; ++a)
-#pragma unroll
-                for (int b = 0; b < 3; ++b) A.m[a][b] = A.m[a][b] + sp * Ep.m[a][b];
-            const M3 Em = leaf_pair<-1>(g, G, xh, x, c, mu, nu, pl, c1);
-#pragma unroll
-            for (int a = 0; a < 3; ++a)
-#pragma unroll
-                for (int b = 0; b < 3; ++b) A.m[a][b] = A.m[a][b] - sp * Em.m[a][b];
-        }
-        const double beta = -csw * kappa / 4.0;
-#pragma unroll
-        for (int a = 0; a < 3; ++a)
-#pragma unroll
-            for (int b = 0; b < 3; ++b) H.m[a][b] = beta * times_i(A.m[a][b]);
-    }
-
-    // hopping part: H += 2 kappa p sum_s [((1-g) X(x+mu))_s Y_s(x)^+ + Y_s(x+mu) ((1+g) X(x))_s^+]
+    const int xa = wc_idx(c[a] == g.L[a] - 1 ? x - (g.L[a] - 1) * g.stride[a] : x + g.stride[a], V);
+    const int xb = wc_idx(c[b] == g.L[b] - 1 ? x - (g.L[b] - 1) * g.stride[b] : x + g.stride[b], V);
+    const int xab = wc_idx(c[b] == g.L[b] - 1 ? xa - (g.L[b] - 1) * g.stride[b] : xa + g.stride[b], V);
+    const M3 L0 = link(G, V, a, x), W = link(G, V, b, x);
+    const H3 Z0 = load_h3(xp, V, x);
+    H3 H;
+    X3 X;
     {
-        const bool wrap = c[mu] == g.L[mu] - 1;
-        const int xf = wrap ? x - (g.L[mu] - 1) * g.stride[mu] : x + g.stride[mu];
-        const double k2 = 2.0 * kappa * ((mu == 3 && wrap) ? (double)g.tbc : 1.0);
-        M3 Z = zero3();
-        cx<double> a[12], b[12];
-        load_sp(X, V, xf, b);
-        project_full(mu, -1, b, a);
-        load_sp(Y, V, x, b);
-        fma_outer(a, b, Z);
-        load_sp(X, V, x, b);
-        project_full(mu, +1, b, a);
-        load_sp(Y, V, xf, b);
-        fma_outer(b, a, Z);
+        const M3 L1 = link(G, V, b, xa), Vd = dag(link(G, V, a, xb));
+        M3 t = zero3();
+        fma_hm(load_h3(xp, V, xa), L1, t);
+        fma_mh(L1, load_h3(xp, V, xab), t);
+        M3 E = mul(mul(L0, t), Vd);
+        const M3 C = mul(mul(L0, L1), Vd);
+        fma_mh(C, load_h3(xp, V, xb), E);
+        const M3 P = mul_dag(C, W);
+        H = herm2(E, W, P, Z0);
+#pragma unroll
+        for (int i = 0; i < 3; ++i) X.d[i] = 2.0 * P.m[i][i].im;
+#pragma unroll
+        for (int q = 0; q < 3; ++q) X.o[q] = P.m[off_row(q)][off_col(q)] - conj(P.m[off_col(q)][off_row(q)]);
+    }
+    // H is 2 Hm(G); below hc, xc are twice the carried H and X
+    store_h3(w0, V, x, H);
+    H3 hc;
+    X3 xc;
+    carry2(H, X, L0, hc, xc);
+    {
+        const H3 k = herm2_zx(load_h3(xp, V, xa), xc);   // 4 Hm(Z1 X1)
+        H3 r;
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            r.d[q] = 0.5 * (hc.d[q] - k.d[q]);
+            r.o[q] = 0.5 * (hc.o[q] - k.o[q]);
+        }
+        store_h3(w0 + (size_t)18 * V, V, x, r);
+    }
+    H = H + herm2_zx(Z0, X);
+    H3 n;
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        n.d[q] = -H.d[q];
+        n.o[q] = -H.o[q];
+    }
+    store_h3(w0 + (size_t)9 * V, V, x, n);
+    carry2(H, X, W, hc, xc);
+    {
+        const H3 k = herm2_zx(load_h3(xp, V, xb), xc);
+        H3 r;
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            r.d[q] = -0.5 * (hc.d[q] + k.d[q]);
+            r.o[q] = -0.5 * (hc.o[q] + k.o[q]);
+        }
+        store_h3(w0 + (size_t)27 * V, V, x, r);
+    }
+}
+
+// two-spinor of (1 + S g_mu) psi at site x of an FP64 field
+template <int MU, int S>
+__device__ __forceinline__ void half_spinor(const double2 *f, int V, int x, cx<double> h[6])
+{
+    cx<double> p[12];
+    P64::load_spinor(f, nullptr, V, x, p);
+    project<MU, S>(p, h);
+}
+
+// Z += sum over two spins of a_s b_s^+
+__device__ __forceinline__ void fma_outer2(const cx<double> a[6], const cx<double> b[6], M3 &z)
+{
+#pragma unroll
+    for (int s = 0; s < 2; ++s)
 #pragma unroll
         for (int p = 0; p < 3; ++p)
 #pragma unroll
-            for (int q = 0; q < 3; ++q) H.m[p][q] = H.m[p][q] + k2 * Z.m[p][q];
-    }
+            for (int q = 0; q < 3; ++q) z.m[p][q] = cfma_conj(b[3 * s + q], a[3 * s + p], z.m[p][q]);
+}
 
-    // F = TA(U H) = (G - G^+)/2 - tr(G - G^+)/6
-    const M3 Gm = mul(link(G, V, mu, x), H);
-    M3 D;
-#pragma unroll
-    for (int p = 0; p < 3; ++p)
-#pragma unroll
-        for (int q = 0; q < 3; ++q) D.m[p][q] = Gm.m[p][q] - conj(Gm.m[q][p]);
-    const cx<double> tr = (1.0 / 6.0) * (D.m[0][0] + D.m[1][1] + D.m[2][2]);
+// sum_s [((1-g) X(x+mu))_s Y_s(x)^+ + Y_s(x+mu) ((1+g) X(x))_s^+]: 1 -+ g is
+// Hermitian and twice a projector, so the sums over four spins are those over
+// the two spins of both projected spinors
+template <int MU>
+__device__ __forceinline__ M3 hop_outer(const double2 *X, const double2 *Y, int V, int x, int xf)
+{
+    M3 z = zero3();
+    cx<double> a[6], b[6];
+    half_spinor<MU, -1>(X, V, xf, a);
+    half_spinor<MU, -1>(Y, V, x, b);
+    fma_outer2(a, b, z);
+    half_spinor<MU, +1>(Y, V, xf, a);
+    half_spinor<MU, +1>(X, V, x, b);
+    fma_outer2(a, b, z);
+    return z;
+}
+
+// Link (x, mu), mu = blockIdx.y: the contributions of the planes of this step
+// added to those parked in F (9 doubles of a link's 18); with LAST, the hopping
+// part too and F = TA(G) in the canonical layout [V][4][3][3].
+template <bool FIRST, bool LAST>
+__global__ void __launch_bounds__(64) k_force_link(Geom g, GaugeStore G, const double2 *X, const double2 *Y, int4 planes,
+                                                   const double *ws, double kappa, double csw, double2 *F)
+{
+    const int x = blockIdx.x * blockDim.x + threadIdx.x, mu = blockIdx.y;
+    if (x >= g.V) return;
+    const int V = g.V;
+    int c[4];
+    site_coords(g, x, c);
+    H3 h = {};
     double2 *out = F + ((size_t)x * 4 + mu) * 9;
+    if (csw != 0.0) {
+        // the plane of this step that contains mu: (a, b) with a = mu or b = mu
+        const int second = mu == planes.z || mu == planes.w;
+        const int a = second ? planes.z : planes.x, b = second ? planes.w : planes.y;
+        const double *w0 = ws + (size_t)second * 36 * V;
+        const int nu = mu == a ? b : a;
+        const int xd = wc_idx(c[nu] == 0 ? x + (g.L[nu] - 1) * g.stride[nu] : x - g.stride[nu], V);
+        h = load_h3(w0 + (size_t)(mu == a ? 0 : 9) * V, V, x) + load_h3(w0 + (size_t)(mu == a ? 27 : 18) * V, V, xd);
+        if (!FIRST) {
+            H3 p;
+            const double2 d0 = out[0], d1 = out[1];
+            p.d[0] = d0.x, p.d[1] = d0.y, p.d[2] = d1.x;
 #pragma unroll
-    for (int p = 0; p < 3; ++p)
-#pragma unroll
-        for (int q = 0; q < 3; ++q) {
-            cx<double> f = 0.5 * D.m[p][q];
-            if (p == q) f = f - tr;
-            out[3 * p + q] = make_double2(f.re, f.im);
+            for (int k = 0; k < 3; ++k) {
+                const double2 v = out[2 + k];
+                p.o[k] = mkc(v.x, v.y);
+            }
+            h = h + p;
         }
+    }
+    if (!LAST) {
+        out[0] = make_double2(h.d[0], h.d[1]);
+        out[1] = make_double2(h.d[2], 0.0);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) out[2 + k] = make_double2(h.o[k].re, h.o[k].im);
+        return;
+    }
+    const bool wrap = c[mu] == g.L[mu] - 1;
+    const int xf = wc_idx(wrap ? x - (g.L[mu] - 1) * g.stride[mu] : x + g.stride[mu], V);
+    const double k2 = kappa * ((mu == 3 && wrap) ? (double)g.tbc : 1.0);
+    M3 z;
+    if (mu == 0) z = hop_outer<0>(X, Y, V, x, xf);
+    else if (mu == 1) z = hop_outer<1>(X, Y, V, x, xf);
+    else if (mu == 2) z = hop_outer<2>(X, Y, V, x, xf);
+    else z = hop_outer<3>(X, Y, V, x, xf);
+    const M3 u = mul(link(G, V, mu, x), z);
+    // G - G^+ = 2 kappa p (U z - (U z)^+) + 2 c H, H = h / 2, c = -i csw kappa / 4
+    const double cb = -csw * kappa / 8.0;
+    const double f0 = fma(cb, h.d[0], 2.0 * k2 * u.m[0][0].im), f1 = fma(cb, h.d[1], 2.0 * k2 * u.m[1][1].im),
+                 f2 = fma(cb, h.d[2], 2.0 * k2 * u.m[2][2].im);
+    const double t = (1.0 / 3.0) * (f0 + f1 + f2);
+    out[0] = make_double2(0.0, f0 - t);
+    out[4] = make_double2(0.0, f1 - t);
+    out[8] = make_double2(0.0, f2 - t);
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        const int i = off_row(q), j = off_col(q);
+        const cx<double> d = u.m[i][j] - conj(u.m[j][i]);
+        const cx<double> v = mkc(fma(k2, d.re, -cb * h.o[q].im), fma(k2, d.im, cb * h.o[q].re));
+        out[3 * i + j] = make_double2(v.re, v.im);
+        out[3 * j + i] = make_double2(-v.re, v.im);
+    }
 }
 
 bool is_device_ptr(const void *p)
@@ -446,19 +583,25 @@ bool is_device_ptr(const void *p)
 wc_status force_from_solutions(wc_lattice lat, wc_field X, wc_field Y, double2 *dst)
 {
     const int V = lat->g.V;
+    cudaStream_t s = lat->stream;
+    const double2 *x = static_cast<const double2 *>(X->data), *y = static_cast<const double2 *>(Y->data);
+    // Xh of the six planes, then the link contributions of two planes
     double *xh = nullptr;
-    wc_status st = check_cuda(lat, cudaMalloc(&xh, sizeof(double) * 54 * (size_t)V), "cudaMalloc(xh)");
+    wc_status st = check_cuda(lat, cudaMalloc(&xh, sizeof(double) * (54 + 72) * (size_t)V), "cudaMalloc(force)");
     if (st != WC_OK) return st;
-    k_xi<<<(V + 127) / 128, 128, 0, lat->stream>>>(lat->g, static_cast<const double2 *>(X->data),
-                                                   static_cast<const double2 *>(Y->data), xh);
-    st = check_launch(lat, "xi");
-    if (st == WC_OK) {
-        k_force<<<(4 * V + 127) / 128, 128, 0, lat->stream>>>(lat->g, lat->gauge, static_cast<const double2 *>(X->data),
-                                                           static_cast<const double2 *>(Y->data), xh, lat->kappa,
-                                                           lat->csw, dst);
-        st = check_launch(lat, "force");
+    double *ws = xh + (size_t)54 * V;
+    const int4 pair[3] = {make_int4(0, 1, 2, 3), make_int4(0, 2, 1, 3), make_int4(1, 2, 0, 3)};
+    const unsigned blocks = (V + 63) / 64;
+    const bool clover = lat->csw != 0.0;
+    if (clover) k_xi<<<blocks, 64, 0, s>>>(lat->g, x, y, xh);
+    for (int p = clover ? 0 : 2; p < 3; ++p) {
+        if (clover) k_force_plaq<<<dim3(blocks, 2), 64, 0, s>>>(lat->g, lat->gauge, xh, pair[p], ws);
+        const auto kern = p == 2 ? (clover ? k_force_link<false, true> : k_force_link<true, true>)
+                                 : p == 0 ? k_force_link<true, false> : k_force_link<false, false>;
+        kern<<<dim3(blocks, 4), 64, 0, s>>>(lat->g, lat->gauge, x, y, pair[p], ws, lat->kappa, lat->csw, dst);
     }
-    cudaStreamSynchronize(lat->stream);
+    st = check_launch(lat, "force");
+    cudaStreamSynchronize(s);
     cudaFree(xh);
     return st;
 }

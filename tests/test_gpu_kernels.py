@@ -314,3 +314,24 @@ def test_lockstep_group_whose_members_stop_apart(n):
         sol = x.store(np.zeros_like(s))
         r = s - oracle.apply_M(dims, tbc, kappa, csw, U, sol)
         assert info.status == 0 and np.linalg.norm(r) <= 1.5e-10 * np.linalg.norm(s)
+
+
+@pytest.mark.parametrize("dims,tbc", [((2, 2, 2, 2), -1), ((2, 4, 6, 2), 1), ((3, 2, 5, 3), -1), ((4, 4, 4, 6), -1)])
+@pytest.mark.parametrize("csw", [0.0, 1.3])
+def test_force_from_shared_plaquettes(dims, tbc, csw):
+    """The force where a plaquette's corners wrap onto each other (extent 2),
+    on odd and ragged volumes, with and without the clover part: every link
+    against the oracle (its F of the same solutions; solves to 1e-13), and
+    traceless and anti-Hermitian to rounding."""
+    kappa = 0.11
+    U = synth.haar_links(dims, 230 + sum(dims))
+    lat = make_lattice(dims, U, csw, kappa, tbc)
+    phi = synth.gaussian_source(dims, 231)
+    F = np.full((int(np.prod(dims)), 4, 3, 3), 9.0, complex)      # old contents must not matter
+    S = lat.action_force(lat.field(0).load(phi), F, tol=1e-13)
+    S0, F0, _, _ = oracle.action_and_force(oracle.Operator(dims, U, csw, kappa, tbc), phi, tol=1e-14)
+    assert abs(S - S0) <= 1e-11 * S0
+    assert_elementwise(F, F0, 1e-9)
+    scale = np.abs(F).max()
+    assert np.abs(F + F.conj().swapaxes(-1, -2)).max() == 0.0
+    assert np.abs(np.trace(F, axis1=-2, axis2=-1)).max() <= 1e-14 * scale
