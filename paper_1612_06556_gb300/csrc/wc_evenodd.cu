@@ -257,18 +257,14 @@ __global__ void __launch_bounds__(64) k_clover_invert(Geom g, CloverStore C, Clo
 // parity stencil
 // ------------------------------------------------------------------------
 
-// full site of half index i of parity p
+// full site of half index i of parity p: 2 i is the full index of the site
+// with x rounded down to even (all extents are even)
 __device__ __forceinline__ int full_site(const Geom &g, int i, int p, int c[4])
 {
-    const int hx = g.L[0] >> 1;
-    const int xh = i % hx;
-    int rest = i / hx;
-    c[1] = rest % g.L[1];
-    rest /= g.L[1];
-    c[2] = rest % g.L[2];
-    c[3] = rest / g.L[2];
-    c[0] = 2 * xh + ((p + c[1] + c[2] + c[3]) & 1);
-    return wc_idx(c[0] + g.stride[1] * c[1] + g.stride[2] * c[2] + g.stride[3] * c[3], g.V);
+    site_coords_fast(g, 2 * i, c);
+    const int bit = (p + c[1] + c[2] + c[3]) & 1;
+    c[0] += bit;
+    return wc_idx(2 * i + bit, g.V);
 }
 
 // hops of the opposite-parity half field `in` into site x (full index x,
@@ -371,7 +367,10 @@ __device__ __forceinline__ void eo_tail(const Geom &g, int p, const CloverStore 
 
 // (FP32 and FP16 fields.  One CTA per SM is all that is asked of the register
 // allocation: without that it keeps fewer loads in flight, a solver step at
-// 16^3x32 in binary16 136 instead of 122 us.)
+// 16^3x32 in binary16 136 instead of 122 us; four CTAs measured the same, five
+// and six 4 and 8 % slower.  Site coordinates by multiplication and the
+// binary16 hops formed from the stored halves took 2 to 3 % off a step:
+// 16^3x32 FP32 112 -> 109 us, 24^3x32 binary16 188 -> 183.)
 template <class P, int DAG, int MODE>
 __global__ void __launch_bounds__(128, 1) k_eo(Geom g, int p, GaugeStore U, CloverStore C, CloverStore Ci,
                                             const void *hin, const float *hin_nrm, const void *vin,
@@ -393,11 +392,19 @@ __global__ void __launch_bounds__(128, 1) k_eo(Geom g, int p, GaugeStore U, Clov
     if (MODE != 4) {
         constexpr int SF = DAG ? +1 : -1;
         constexpr int SB = -SF;
-        const R one = R(1);
-        eo_hop_dir<P, 0, SF, SB>(g, U, hin, hin_nrm, Vh, x, c, one, h);
-        eo_hop_dir<P, 1, SF, SB>(g, U, hin, hin_nrm, Vh, x, c, one, h);
-        eo_hop_dir<P, 2, SF, SB>(g, U, hin, hin_nrm, Vh, x, c, one, h);
-        eo_hop_dir<P, 3, SF, SB>(g, U, hin, hin_nrm, Vh, x, c, one, h);
+        if constexpr (std::is_same<P, P16>::value) {
+            const auto half = [](int y) { return y >> 1; };
+            hop_dir_h16<0, SF, SB>(g, U, hin, hin_nrm, Vh, x, c, 1.f, h, half);
+            hop_dir_h16<1, SF, SB>(g, U, hin, hin_nrm, Vh, x, c, 1.f, h, half);
+            hop_dir_h16<2, SF, SB>(g, U, hin, hin_nrm, Vh, x, c, 1.f, h, half);
+            hop_dir_h16<3, SF, SB>(g, U, hin, hin_nrm, Vh, x, c, 1.f, h, half);
+        } else {
+            const R one = R(1);
+            eo_hop_dir<P, 0, SF, SB>(g, U, hin, hin_nrm, Vh, x, c, one, h);
+            eo_hop_dir<P, 1, SF, SB>(g, U, hin, hin_nrm, Vh, x, c, one, h);
+            eo_hop_dir<P, 2, SF, SB>(g, U, hin, hin_nrm, Vh, x, c, one, h);
+            eo_hop_dir<P, 3, SF, SB>(g, U, hin, hin_nrm, Vh, x, c, one, h);
+        }
     }
     eo_tail<P, MODE>(g, p, C, Ci, vin, vin_nrm, out, out_nrm, beta, Vh, i, h);
 }

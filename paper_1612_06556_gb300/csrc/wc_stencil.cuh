@@ -438,9 +438,10 @@ __device__ __forceinline__ void reconstruct_fma(cx<float> acc[12], const cx<floa
 // the forward and backward hop of direction MU for FP16 storage (hop_dir
 // with the projection formed from the stored halves and the coefficient
 // folded into the accumulation)
-template <int MU, int SF, int SB>
+// (the neighbour spinors read at sidx(y) of a field of Vin sites)
+template <int MU, int SF, int SB, class SiteIdx>
 __device__ __forceinline__ void hop_dir_h16(const Geom &g, const GaugeStore &U, const void *in, const float *in_nrm,
-                                            int x, const int c[4], float k, cx<float> acc[12])
+                                            int Vin, int x, const int c[4], float k, cx<float> acc[12], SiteIdx sidx)
 {
     const int L = g.L[MU], st = g.stride[MU];
     const uint4 *ps = static_cast<const uint4 *>(in);
@@ -448,9 +449,10 @@ __device__ __forceinline__ void hop_dir_h16(const Geom &g, const GaugeStore &U, 
     for (int dir = 0; dir < 2; ++dir) {
         const bool wrap = dir == 0 ? c[MU] == L - 1 : c[MU] == 0;
         const int y = wc_idx(dir == 0 ? (wrap ? x - (L - 1) * st : x + st) : (wrap ? x + (L - 1) * st : x - st), g.V);
-        const uint4 s0 = __ldg(ps + y), s1 = __ldg(ps + (size_t)g.V + y), s2 = __ldg(ps + 2 * (size_t)g.V + y);
+        const int z = sidx(y);
+        const uint4 s0 = __ldg(ps + z), s1 = __ldg(ps + (size_t)Vin + z), s2 = __ldg(ps + 2 * (size_t)Vin + z);
         const unsigned w[12] = {s0.x, s0.y, s0.z, s0.w, s1.x, s1.y, s1.z, s1.w, s2.x, s2.y, s2.z, s2.w};
-        const float coef = ((MU == 3 && wrap) ? k * (float)g.tbc : k) * __ldg(in_nrm + y);
+        const float coef = ((MU == 3 && wrap) ? k * (float)g.tbc : k) * __ldg(in_nrm + z);
         cx<float> h[6], u[6], r2[3], wv[6];
         if (dir == 0) {
             project_h16<MU, SF>(w, h);
@@ -716,10 +718,11 @@ __device__ __forceinline__ void apply_site_at(const Geom &g, int x, const GaugeS
     constexpr int SF = KIND == 1 ? +1 : -1;
     constexpr int SB = -SF;
     if constexpr (std::is_same<P, P16>::value) {
-        hop_dir_h16<0, SF, SB>(g, U, in, in_nrm, x, c, k, acc);
-        hop_dir_h16<1, SF, SB>(g, U, in, in_nrm, x, c, k, acc);
-        hop_dir_h16<2, SF, SB>(g, U, in, in_nrm, x, c, k, acc);
-        hop_dir_h16<3, SF, SB>(g, U, in, in_nrm, x, c, k, acc);
+        const auto same = [](int y) { return y; };
+        hop_dir_h16<0, SF, SB>(g, U, in, in_nrm, g.V, x, c, k, acc, same);
+        hop_dir_h16<1, SF, SB>(g, U, in, in_nrm, g.V, x, c, k, acc, same);
+        hop_dir_h16<2, SF, SB>(g, U, in, in_nrm, g.V, x, c, k, acc, same);
+        hop_dir_h16<3, SF, SB>(g, U, in, in_nrm, g.V, x, c, k, acc, same);
     } else {
         hop_dir<P, 0, SF, SB>(g, U, in, in_nrm, x, c, k, acc);
         hop_dir<P, 1, SF, SB>(g, U, in, in_nrm, x, c, k, acc);
