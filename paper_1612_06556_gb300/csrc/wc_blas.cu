@@ -22,113 +22,10 @@
 #include <algorithm>
 
 #include "wc_internal.cuh"
+#include "wc_reduce.cuh"
 #include "wc_solver_kernels.cuh"
 
 namespace wc {
-
-namespace {
-
-constexpr int kRedBlock = 256;
-
-// Sums of v[0..N) over the lanes, N = 1, 2 or 4: lane l returns the sum of
-// v[l / (32 / N)].
-template <int N, class T>
-__device__ __forceinline__ T warp_sums(T (&v)[N])
-{
-    static_assert(N == 1 || N == 2 || N == 4, "one, two or four sums");
-    const int lane = threadIdx.x & 31;
-#pragma unroll
-    for (int half = N / 2, o = 16; half > 0; half /= 2, o /= 2) {
-        const bool up = (lane & o) != 0;
-#pragma unroll
-        for (int i = 0; i < half; ++i) {
-            const T give = up ? v[i] : v[half + i], keep = up ? v[half + i] : v[i];
-            v[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
-        }
-    }
-#pragma unroll
-    for (int o = 16 / N; o > 0; o /= 2) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
-    return v[0];
-}
-
-constexpr int kRedWarps = kRedBlock / 32;
-
-// Sum i over w[.][k] where warp k of the block has put its sums (lane i * 8 +
-// k of the calling warp reads it): every lane of i * 8 .. i * 8 + 7.
-template <int N, class T>
-__device__ __forceinline__ T block_sums(const T (&w)[N][kRedWarps])
-{
-    static_assert(kRedWarps == 8, "eight warps");
-    const int lane = threadIdx.x & 31;
-    T u = lane < N * 8 ? w[lane >> 3][lane & 7] : T(0);
-#pragma unroll
-    for (int o = 4; o > 0; o /= 2) u += __shfl_xor_sync(0xffffffffu, u, o);
-    return u;
-}
-
-struct NoUpdate {
-    __device__ void operator()(double, const double *) const {}
-};
-struct NoAhead {
-    __device__ double operator()() const { return 0.0; }
-};
-
-}  // namespace
-
-// Reduce v[0..M) over the grid (blocks of kRedBlock threads, one dimension x).
-// The last block to arrive leaves the grid sums in out[0..M), summed in a
-// fixed order, and its warp 0 calls post(t, extra) with sum i in lane i
-// (zero above).  ahead() runs meanwhile in the last warp of that block;
-// extra[l] is what lane l of it returned.
-template <int M, class T, class Post = NoUpdate, class Ahead = NoAhead>
-__device__ __forceinline__ void grid_reduce(T (&acc)[M], const ReduceScratch &rs, double *out, Post post = Post(),
-                                            Ahead ahead = Ahead())
-{
-    constexpr int N = M == 3 ? 4 : M;
-    __shared__ T sm[N][kRedWarps];
-    __shared__ double fin[kRedWarps], extra[32];
-    __shared__ bool last;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    T v[N];
-#pragma unroll
-    for (int i = 0; i < N; ++i) v[i] = i < M ? acc[i] : T(0);
-    const T t = warp_sums(v);
-    if (lane % (32 / N) == 0) sm[lane / (32 / N)][wid] = t;
-    __syncthreads();
-    if (wid == 0) {
-        const T u = block_sums(sm);
-        if (lane < N * 8 && (lane & 7) == 0) {
-            rs.partials[(size_t)blockIdx.x * 8 + (lane >> 3)] = (double)u;
-            __threadfence();
-        }
-        __syncwarp();
-        if (lane == 0) last = atomicAdd(rs.ticket, 1u) == gridDim.x - 1;
-    }
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
-    // warp w adds the partials of sum w % N
-    double s = 0.0;
-    const int i = wid % N;
-    if (i < M) {
-#pragma unroll 4
-        for (int b = (wid / N) * 32 + lane; b < (int)gridDim.x; b += kRedBlock / N)
-            s += __ldcg(rs.partials + (size_t)b * 8 + i);
-        double one[1] = {s};
-        s = warp_sums(one);
-    }
-    if (lane == 0) fin[wid] = s;
-    if (wid == kRedWarps - 1) extra[lane] = ahead();
-    __syncthreads();
-    if (wid != 0) return;
-    double u = lane < kRedWarps ? fin[lane] : 0.0;
-#pragma unroll
-    for (int o = N; o < kRedWarps; o *= 2) u += __shfl_xor_sync(0xffffffffu, u, o);
-    if (lane >= M) u = 0.0;
-    if (lane < M) out[lane] = u;
-    if (lane == 0) *rs.ticket = 0u;
-    post(u, extra);
-}
 
 int reduce_grid(const ReduceScratch &rs, long long n)
 {
@@ -299,21 +196,6 @@ __device__ __forceinline__ cx<double> ld(const double2 *p, long long i)
     return {v.x, v.y};
 }
 __device__ __forceinline__ void st(double2 *p, long long i, cx<double> a) { p[i] = make_double2(a.re, a.im); }
-__device__ __forceinline__ cx<double> c_of(double2 a) { return {a.x, a.y}; }
-
-// ---- scalar updates, run by one warp -------------------------------------
-// t: sum i of the reduction in lane i.
-
-__device__ __forceinline__ double sum_of(double t, int i) { return __shfl_sync(0xffffffffu, t, i); }
-
-// a / b, the real part in even lanes, the imaginary part in odd ones
-__device__ __forceinline__ double cdiv_part(cx<double> a, cx<double> b)
-{
-    const bool im = threadIdx.x & 1;
-    const double d = b.re * b.re + b.im * b.im;
-    const double p = im ? a.im : a.re, q = im ? -a.re : a.im;
-    return (p * b.re + q * b.im) / d;
-}
 
 __device__ __forceinline__ void init_update(double t, SolverScalars *sc)
 {
@@ -391,34 +273,6 @@ __global__ void k_track(SolverScalars *sc, int track, double tol2, double d2, do
     sc->d2 = d2;
     sc->defer2 = defer2;
     sc->rmax2 = sc->prev = sc->rr_refresh = rr;
-}
-
-// alpha = rho / <rhat, v>
-__device__ __forceinline__ void alpha_update(double t, SolverScalars *sc)
-{
-    const int lane = threadIdx.x & 31;
-    const cx<double> rv = mkc(sum_of(t, 0), sum_of(t, 1));
-    const double a = cdiv_part(c_of(sc->rho), rv);
-    const bool zero = rv.re == 0.0 && rv.im == 0.0;
-    if (lane < 2) (&sc->alpha.x)[lane] = zero ? 0.0 : a;
-    if (lane == 0) {
-        if (!isfinite(rv.re) || !isfinite(rv.im)) sc->flags |= FLAG_NAN;
-        if (zero) sc->flags |= FLAG_BREAKDOWN;
-    }
-}
-
-// omega = <t, s> / <t, t>
-__device__ __forceinline__ void omega_update(double t, SolverScalars *sc)
-{
-    const int lane = threadIdx.x & 31;
-    const double tt = sum_of(t, 2);
-    const bool bad = !isfinite(tt) || !isfinite(sum_of(t, 0)) || !isfinite(sum_of(t, 1));
-    const double om = t / tt;
-    if (lane < 2) (&sc->omega.x)[lane] = tt > 0.0 ? om : 0.0;
-    if (lane == 0) {
-        sc->tt = tt;
-        if (bad) sc->flags |= FLAG_NAN;
-    }
 }
 
 // alpha / omega in lanes 0, 1 and 1 / rho in lanes 2, 3, while the sums of
@@ -639,28 +493,6 @@ __device__ __forceinline__ void st4(float4 *p, long long i, cx<float> a, cx<floa
 // Grid sums of the low-precision kernels are grid_reduce on float: lanes and
 // warps in FP32, the block partials (one per block) in FP64 by the last
 // block.  The scalar updates are those of the FP64 solver, but for omega.
-
-// omega from <t, s>, <t, t>, <s, s>
-__device__ __forceinline__ void lo_omega_update(double t, SolverScalars *sc)
-{
-    const int lane = threadIdx.x & 31;
-    const double tr = sum_of(t, 0), ti = sum_of(t, 1), tt = sum_of(t, 2), ss = sum_of(t, 3);
-    double om = tt > 0.0 ? t / tt : 0.0;
-    // omega stabilisation (Sleijpen & van der Vorst): when t and s are
-    // nearly orthogonal, |<t,s>| / (|t||s|) < 0.7, the minimising omega is
-    // tiny and BiCGStab loses accuracy in finite precision; enlarge it
-    // (the squares first: the roots are wanted only then)
-    const double c2 = tr * tr + ti * ti;
-    if (tt > 0.0 && ss > 0.0 && c2 > 0.0 && c2 < 0.5 * (tt * ss)) {
-        const double rho_t = sqrt(c2) / sqrt(tt * ss);
-        if (rho_t < 0.7) om *= 0.7 / rho_t;
-    }
-    if (lane < 2) (&sc->omega.x)[lane] = om;
-    if (lane == 0) {
-        sc->tt = tt;
-        if (!isfinite(tt) || !isfinite(tr) || !isfinite(ti) || !isfinite(ss)) sc->flags |= FLAG_NAN;
-    }
-}
 
 // after r was replaced: rho = <rhat, r> (sums 1, 2), beta from rho0 (rr is
 // sum 0)

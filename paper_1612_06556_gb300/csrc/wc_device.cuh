@@ -240,7 +240,7 @@ enum { ACT_NONE = 0, ACT_STOP = 1, ACT_DIVERGED = 2, ACT_BREAKDOWN = 3, ACT_DEFE
 
 // Reduction scratch: per-block partial sums and a completion ticket.
 struct ReduceScratch {
-    double *partials = nullptr;   // [max_blocks][8]
+    double *partials = nullptr;   // [2 max_blocks][4]
     unsigned *ticket = nullptr;
     double *result = nullptr;     // [8] final sums (device)
     double *host_result = nullptr;  // [8] pinned host mirror

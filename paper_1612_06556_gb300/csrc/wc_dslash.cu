@@ -20,6 +20,7 @@
 #include <type_traits>
 
 #include "wc_internal.cuh"
+#include "wc_reduce.cuh"
 #include "wc_stencil.cuh"
 #include "wc_dfsplit.cuh"
 
@@ -160,6 +161,49 @@ __global__ void __launch_bounds__(kSplit64 * kSplit64Sites, 3)
         o[(size_t)r * g.V] = KIND == 2 ? make_double2(h.re, h.im)
                                        : make_double2(fma(-kappa, h.re, y[r].re), fma(-kappa, h.im, y[r].im));
     }
+}
+
+// k_apply_split64 as the operator of a solver step: the pass also forms the
+// sums of alpha (or OMEGA: of omega) with `ss.with`.
+template <int KIND, bool OMEGA>
+__global__ void __launch_bounds__(kSplit64 * kSplit64Sites, 3)
+    k_apply_split64_sum(Geom g, GaugeStore U, CloverStore C, const void *in, void *out, double kappa, StepSum ss)
+{
+    griddep_wait();
+    griddep_launch_dependents();
+    if (ss.sc->skip) return;
+    __shared__ Split64Mem sm;
+    const int s = threadIdx.x & (kSplit64Sites - 1), w = threadIdx.x / kSplit64Sites;
+    const int x = blockIdx.x * kSplit64Sites + s;
+    const bool valid = x < g.V;
+    if (valid) {
+        int c[4];
+        site_coords_fast(g, x, c);
+        hop_split64<KIND == 1 ? +1 : -1>(g, U, in, g.V, x, c, sm, w, s, [](int y) { return y; });
+    }
+    __syncthreads();
+    double acc[step_sums<OMEGA, double>] = {};
+    if (valid) {
+        cx<double> v[6], y[3], a[3];
+        const double2 *p = static_cast<const double2 *>(in) + (size_t)(w >> 1) * 6 * g.V + x;
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+            const double2 b = __ldg(p + (size_t)k * g.V);
+            v[k] = mkc(b.x, b.y);
+        }
+        clover_rows64(C, g.V, x, w, v, y);
+#pragma unroll
+        for (int r = 0; r < 3; ++r) {
+            const size_t k = (size_t)(3 * w + r) * g.V + x;
+            const cx<double> h = sum_split64(sm, 3 * w + r, s);
+            y[r] = mkc(fma(-kappa, h.re, y[r].re), fma(-kappa, h.im, y[r].im));
+            static_cast<double2 *>(out)[k] = make_double2(y[r].re, y[r].im);
+            const double2 b = __ldg(static_cast<const double2 *>(ss.with) + k);
+            a[r] = mkc(b.x, b.y);
+        }
+        add_step_sums<OMEGA, 3>(y, a, acc);
+    }
+    reduce_step_sums<OMEGA, kSplit64, double>(acc, ss);
 }
 
 // The same in double-FP32 arithmetic (wc_dfsplit.cuh).  HDF: in holds split
@@ -525,6 +569,24 @@ cudaError_t launch_apply(wc_lattice lat, wc_field out, wc_field in, int kind, cu
     case WC_F32: return launch_apply_p<P32>(lat, out, in, kind, stream, skip, pdl);
     default: return launch_apply_p<P16>(lat, out, in, kind, stream, skip, pdl);
     }
+}
+
+cudaError_t launch_apply64_sum(wc_lattice lat, wc_field out, wc_field in, int kind, cudaStream_t stream,
+                               const StepSum &ss, bool omega, bool pdl)
+{
+    const Geom &g = lat->g;
+    {
+        // a launch shape that a caller has pinned stays in use
+        std::lock_guard<std::mutex> lk(g_shape_mutex);
+        if (g_shape_choice.emplace(std::array<int, 6>{g.L[0], g.L[1], g.L[2], g.L[3], (int)WC_F64, kind}, kShapeSplit64)
+                .first->second != kShapeSplit64)
+            return cudaErrorNotSupported;
+    }
+    const dim3 grid((g.V + kSplit64Sites - 1) / kSplit64Sites);
+    const auto kern = kind == 0 ? (omega ? k_apply_split64_sum<0, true> : k_apply_split64_sum<0, false>)
+                                : (omega ? k_apply_split64_sum<1, true> : k_apply_split64_sum<1, false>);
+    return launch_step(pdl && pdl_grid(grid.x), kern, grid, kSplit64 * kSplit64Sites, stream, g, lat->gauge, lat->clover,
+                       in->data, out->data, lat->kappa, ss);
 }
 
 cudaError_t launch_apply_df(wc_lattice lat, wc_field out, wc_field in, wc_field split, int kind, cudaStream_t stream,

@@ -21,6 +21,8 @@
 #include <new>
 
 #include "wc_internal.cuh"
+#include "wc_reduce.cuh"
+#include "wc_solver_kernels.cuh"
 #include "wc_stencil.cuh"
 #include "wc_dfsplit.cuh"
 
@@ -331,6 +333,19 @@ __device__ __forceinline__ void clover_eo(const CloverStore &S, int V, int pos, 
 //           vin = b_o, h = H_oe x_e, beta = k: the reconstructed x_o and
 //           the odd-site residual b_o - (A_oo x_o - k H_oe x_e) of the
 //           x_o as stored, in one pass; FP64 fields only)
+// o = C v + beta h
+template <class P>
+__device__ __forceinline__ void add_clover_eo(const Geom &g, int p, const CloverStore &C, double beta, int Vh, int i,
+                                              const cx<typename P::real> v[12], const cx<typename P::real> h[12],
+                                              cx<typename P::real> o[12])
+{
+    using R = typename P::real;
+    const R bt = R(beta);
+    clover_eo<P, false>(C, g.V, wc_idx(p * Vh + i, g.V), v, o);
+#pragma unroll
+    for (int k = 0; k < 12; ++k) o[k] = o[k] + bt * h[k];
+}
+
 // The site-local part of k_eo after the hops h: everything but the hops,
 // in the arithmetic of P.
 template <class P, int MODE>
@@ -347,9 +362,7 @@ __device__ __forceinline__ void eo_tail(const Geom &g, int p, const CloverStore 
     } else {
         P::load_spinor(vin, vin_nrm, Vh, i, v);
         if (MODE == 1) {
-            clover_eo<P, false>(C, g.V, wc_idx(p * Vh + i, g.V), v, o);
-#pragma unroll
-            for (int k = 0; k < 12; ++k) o[k] = o[k] + bt * h[k];
+            add_clover_eo<P>(g, p, C, beta, Vh, i, v, h, o);
             P::store_spinor(out, out_nrm, Vh, i, o);
             return;
         }
@@ -363,6 +376,33 @@ __device__ __forceinline__ void eo_tail(const Geom &g, int p, const CloverStore 
     }
     clover_eo<P, true>(Ci, g.V, wc_idx(p * Vh + i, g.V), v, o);
     P::store_spinor(out, out_nrm, Vh, i, o);
+}
+
+// h = the hops of hin (opposite parity) to full-lattice site x; 0 without HOP
+template <class P, int DAG, bool HOP>
+__device__ __forceinline__ void eo_hops(const Geom &g, const GaugeStore &U, const void *hin, const float *hin_nrm, int Vh,
+                                        int x, const int c[4], cx<typename P::real> h[12])
+{
+    using R = typename P::real;
+#pragma unroll
+    for (int k = 0; k < 12; ++k) h[k] = mkc(R(0), R(0));
+    if (HOP) {
+        constexpr int SF = DAG ? +1 : -1;
+        constexpr int SB = -SF;
+        if constexpr (std::is_same<P, P16>::value) {
+            const auto half = [](int y) { return y >> 1; };
+            hop_dir_h16<0, SF, SB>(g, U, hin, hin_nrm, Vh, x, c, 1.f, h, half);
+            hop_dir_h16<1, SF, SB>(g, U, hin, hin_nrm, Vh, x, c, 1.f, h, half);
+            hop_dir_h16<2, SF, SB>(g, U, hin, hin_nrm, Vh, x, c, 1.f, h, half);
+            hop_dir_h16<3, SF, SB>(g, U, hin, hin_nrm, Vh, x, c, 1.f, h, half);
+        } else {
+            const R one = R(1);
+            eo_hop_dir<P, 0, SF, SB>(g, U, hin, hin_nrm, Vh, x, c, one, h);
+            eo_hop_dir<P, 1, SF, SB>(g, U, hin, hin_nrm, Vh, x, c, one, h);
+            eo_hop_dir<P, 2, SF, SB>(g, U, hin, hin_nrm, Vh, x, c, one, h);
+            eo_hop_dir<P, 3, SF, SB>(g, U, hin, hin_nrm, Vh, x, c, one, h);
+        }
+    }
 }
 
 // (FP32 and FP16 fields.  One CTA per SM is all that is asked of the register
@@ -387,25 +427,7 @@ __global__ void __launch_bounds__(128, 1) k_eo(Geom g, int p, GaugeStore U, Clov
     int c[4];
     const int x = full_site(g, i, p, c);
     cx<R> h[12];
-#pragma unroll
-    for (int k = 0; k < 12; ++k) h[k] = mkc(R(0), R(0));
-    if (MODE != 4) {
-        constexpr int SF = DAG ? +1 : -1;
-        constexpr int SB = -SF;
-        if constexpr (std::is_same<P, P16>::value) {
-            const auto half = [](int y) { return y >> 1; };
-            hop_dir_h16<0, SF, SB>(g, U, hin, hin_nrm, Vh, x, c, 1.f, h, half);
-            hop_dir_h16<1, SF, SB>(g, U, hin, hin_nrm, Vh, x, c, 1.f, h, half);
-            hop_dir_h16<2, SF, SB>(g, U, hin, hin_nrm, Vh, x, c, 1.f, h, half);
-            hop_dir_h16<3, SF, SB>(g, U, hin, hin_nrm, Vh, x, c, 1.f, h, half);
-        } else {
-            const R one = R(1);
-            eo_hop_dir<P, 0, SF, SB>(g, U, hin, hin_nrm, Vh, x, c, one, h);
-            eo_hop_dir<P, 1, SF, SB>(g, U, hin, hin_nrm, Vh, x, c, one, h);
-            eo_hop_dir<P, 2, SF, SB>(g, U, hin, hin_nrm, Vh, x, c, one, h);
-            eo_hop_dir<P, 3, SF, SB>(g, U, hin, hin_nrm, Vh, x, c, one, h);
-        }
-    }
+    eo_hops<P, DAG, MODE != 4>(g, U, hin, hin_nrm, Vh, x, c, h);
     eo_tail<P, MODE>(g, p, C, Ci, vin, vin_nrm, out, out_nrm, beta, Vh, i, h);
 }
 
@@ -500,6 +522,79 @@ __global__ void __launch_bounds__(kSplit64 * kSplit64Sites, 3)
             store(out2, y);
         }
     }
+}
+
+// k_eo in mode 1 as the second half of a solver step's operator: the pass
+// also forms the sums of alpha (or OMEGA: of omega) with `ss.with`, in CTAs
+// of W warps.  The sums are those of out as stored.
+template <class P, int DAG, int W, bool OMEGA>
+__global__ void __launch_bounds__(32 * W, 1) k_eo_sum(Geom g, int p, GaugeStore U, CloverStore C, const void *hin,
+                                                      const float *hin_nrm, const void *vin, const float *vin_nrm,
+                                                      void *out, float *out_nrm, double beta, StepSum ss)
+{
+    griddep_wait();
+    griddep_launch_dependents();
+    if (ss.sc->skip) return;
+    using R = typename P::real;
+    const int Vh = g.V >> 1;
+    const int i = blockIdx.x * 32 * W + threadIdx.x;
+    R acc[step_sums<OMEGA, R>] = {};
+    if (i < Vh) {
+        int c[4];
+        const int x = full_site(g, i, p, c);
+        cx<R> h[12], v[12], o[12];
+        eo_hops<P, DAG, true>(g, U, hin, hin_nrm, Vh, x, c, h);
+        P::load_spinor(vin, vin_nrm, Vh, i, v);
+        add_clover_eo<P>(g, p, C, beta, Vh, i, v, h, o);
+        P::store_spinor(out, out_nrm, Vh, i, o);
+        P::as_stored(o);
+        P::load_spinor(ss.with, ss.with_nrm, Vh, i, v);
+        add_step_sums<OMEGA, 12>(o, v, acc);
+    }
+    reduce_step_sums<OMEGA, W, R>(acc, ss);
+}
+
+// The same in FP64 on four warps per 32 sites (k_eo_split64).
+template <int DAG, bool OMEGA>
+__global__ void __launch_bounds__(kSplit64 * kSplit64Sites, 3)
+    k_eo_split64_sum(Geom g, int p, GaugeStore U, CloverStore C, const void *hin, const double2 *vin, double2 *out,
+                     double beta, StepSum ss)
+{
+    griddep_wait();
+    griddep_launch_dependents();
+    if (ss.sc->skip) return;
+    __shared__ Split64Mem sm;
+    const int Vh = g.V >> 1;
+    const int s = threadIdx.x & (kSplit64Sites - 1), w = threadIdx.x / kSplit64Sites;
+    const int i = blockIdx.x * kSplit64Sites + s;
+    const bool valid = i < Vh;
+    if (valid) {
+        int c[4];
+        const int x = full_site(g, i, p, c);
+        hop_split64<DAG ? +1 : -1>(g, U, hin, Vh, x, c, sm, w, s, [](int y) { return y >> 1; });
+    }
+    __syncthreads();
+    double acc[step_sums<OMEGA, double>] = {};
+    if (valid) {
+        cx<double> vb[6], o[3], a[3];
+        const double2 *q = vin + (size_t)(w >> 1) * 6 * Vh + i;
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+            const double2 b = __ldg(q + (size_t)k * Vh);
+            vb[k] = mkc(b.x, b.y);
+        }
+        clover_rows64(C, g.V, wc_idx(p * Vh + i, g.V), w, vb, o);
+#pragma unroll
+        for (int r = 0; r < 3; ++r) {
+            const size_t k = (size_t)(3 * w + r) * Vh + i;
+            o[r] = o[r] + beta * sum_split64(sm, 3 * w + r, s);
+            out[k] = make_double2(o[r].re, o[r].im);
+            const double2 b = __ldg(static_cast<const double2 *>(ss.with) + k);
+            a[r] = mkc(b.x, b.y);
+        }
+        add_step_sums<OMEGA, 3>(o, a, acc);
+    }
+    reduce_step_sums<OMEGA, kSplit64, double>(acc, ss);
 }
 
 // An FP64 half field as z2 values (wc_dfsplit.cuh), for the hops of the next
@@ -714,14 +809,16 @@ cudaError_t launch_eo_splitdf(const wc_lattice_s *full, int parity, int mode, co
 #undef WC_EO
 }
 
+// CTAs of 128 sites; on small lattices (fewer than two such CTAs per SM)
+// CTAs of 32, so that the sites spread over more SMs
+int eo_threads(int Vh) { return Vh < 2 * 128 * sm_count() ? 32 : 128; }
+
 template <class P, int DAG>
 cudaError_t launch_eo_p(const wc_lattice_s *full, int parity, int mode, const wc_field_s *hin, const wc_field_s *vin,
                         wc_field_s *out, double beta, cudaStream_t stream, const int *skip, bool pdl)
 {
     const int Vh = full->g.V >> 1;
-    // CTAs of 128 sites; on small lattices (fewer than two such CTAs per SM)
-    // CTAs of 32, so that the sites spread over more SMs
-    const int threads = Vh < 2 * 128 * sm_count() ? 32 : 128;
+    const int threads = eo_threads(Vh);
     const dim3 grid((Vh + threads - 1) / threads);
     const void *hd = hin ? hin->data : nullptr;
     const float *hn = hin ? hin->nrm : nullptr;
@@ -739,6 +836,29 @@ cudaError_t launch_eo_p(const wc_lattice_s *full, int parity, int mode, const wc
     default: return cudaErrorInvalidValue;   // mode 5: FP64 fields only
     }
 #undef WC_EO
+}
+
+template <class P, int DAG>
+cudaError_t launch_eo_sum(const wc_lattice_s *full, const wc_field_s *hin, const wc_field_s *vin, wc_field_s *out,
+                          double beta, cudaStream_t stream, const StepSum &ss, bool omega, bool pdl)
+{
+    const int Vh = full->g.V >> 1, threads = eo_threads(Vh);
+    const dim3 grid((Vh + threads - 1) / threads);
+    const auto kern = threads == 32 ? (omega ? k_eo_sum<P, DAG, 1, true> : k_eo_sum<P, DAG, 1, false>)
+                                    : (omega ? k_eo_sum<P, DAG, 4, true> : k_eo_sum<P, DAG, 4, false>);
+    return launch_step(pdl && pdl_grid(grid.x), kern, grid, threads, stream, full->g, 0, full->gauge, full->ceo,
+                       hin->data, hin->nrm, vin->data, vin->nrm, out->data, out->nrm, beta, ss);
+}
+
+template <int DAG>
+cudaError_t launch_eo_sum64(const wc_lattice_s *full, const wc_field_s *hin, const wc_field_s *vin, wc_field_s *out,
+                            double beta, cudaStream_t stream, const StepSum &ss, bool omega, bool pdl)
+{
+    const dim3 grid(((full->g.V >> 1) + kSplit64Sites - 1) / kSplit64Sites);
+    const auto kern = omega ? k_eo_split64_sum<DAG, true> : k_eo_split64_sum<DAG, false>;
+    return launch_step(pdl && pdl_grid(grid.x), kern, grid, kSplit64 * kSplit64Sites, stream, full->g, 0, full->gauge,
+                       full->ceo, hin->data, static_cast<const double2 *>(vin->data), static_cast<double2 *>(out->data),
+                       beta, ss);
 }
 
 }  // namespace
@@ -839,6 +959,41 @@ cudaError_t launch_apply(wc_lattice lat, wc_field out, wc_field in, int kind, So
         return launch_apply(lat, out, in, kind, S.stream, skip, S.pdl);
     }
     return launch_schur(lat, out, in, kind == 1, S.stream, S.work[kSchurSlot + out->prec], skip, S.pdl);
+}
+
+cudaError_t launch_apply_sum(wc_lattice lat, wc_field out, wc_field in, int kind, SolverState &S, bool omega,
+                             wc_field with)
+{
+    const StepSum ss{with->data, with->nrm, S.red, S.scal};
+    const wc_prec pr = out->prec;
+    const wc_lattice_s *full = lat->schur_parent;
+    // sites and warps of a CTA of the pass that would form the sums
+    const int sites = pr == WC_F64 ? kSplit64Sites : eo_threads(lat->g.V), warps = pr == WC_F64 ? kSplit64 : sites / 32;
+    const bool fused = (full ? !eo_split(full, out) : pr == WC_F64 && !eo_split(lat, out)) && kind != 2 &&
+                       sum_in_pass(S.red, (lat->g.V + sites - 1) / sites, warps);
+    if (fused && !full) {
+        const cudaError_t e = launch_apply64_sum(lat, out, in, kind, S.stream, ss, omega, S.pdl);
+        if (e != cudaErrorNotSupported) return e;
+    } else if (fused) {
+        const bool dag = kind == 1;
+        const int *skip = &S.scal->skip;
+        wc_field_s *t = S.work[kSchurSlot + pr] ? S.work[kSchurSlot + pr] : lat->schur_tmp[pr];
+        const double beta = -full->kappa * full->kappa;
+        cudaError_t e = launch_eo(full, 1, 0, dag, in, nullptr, t, 0.0, S.stream, nullptr, skip, S.pdl);
+        if (e != cudaSuccess) return e;
+#define WC_SUM(F, ...) F<__VA_ARGS__>(full, t, in, out, beta, S.stream, ss, omega, S.pdl)
+        if (pr == WC_F64) return dag ? WC_SUM(launch_eo_sum64, 1) : WC_SUM(launch_eo_sum64, 0);
+        if (pr == WC_F32) return dag ? WC_SUM(launch_eo_sum, P32, 1) : WC_SUM(launch_eo_sum, P32, 0);
+        return dag ? WC_SUM(launch_eo_sum, P16, 1) : WC_SUM(launch_eo_sum, P16, 0);
+#undef WC_SUM
+    }
+    const cudaError_t e = launch_apply(lat, out, in, kind, S, true);
+    if (e != cudaSuccess) return e;
+    if (pr == WC_F64) {
+        const double2 *o = static_cast<const double2 *>(out->data), *a = static_cast<const double2 *>(with->data);
+        return omega ? bicg_omega(lat, S, o, a) : bicg_alpha(lat, S, a, o);
+    }
+    return omega ? lo_omega(lat, S, out, with) : lo_alpha(lat, S, with, out);
 }
 
 wc_status build_clover_inverse(wc_lattice lat)

@@ -156,6 +156,16 @@ cudaError_t launch_apply(wc_lattice lat, wc_field out, wc_field in, int kind /*0
 // exists), so that solves on one lattice may run concurrently.  step: the
 // operator of a solver step, which returns at once when S.scal->skip is set.
 cudaError_t launch_apply(wc_lattice lat, wc_field out, wc_field in, int kind, SolverState &S, bool step = false);
+// out = op in of a solver step, then alpha = rho / <with, out> or (omega) the
+// omega of <out, with> / <out, out> into S.scal, from sums that the operator
+// pass forms itself on small grids (sum_in_pass, wc_reduce.cuh)
+cudaError_t launch_apply_sum(wc_lattice lat, wc_field out, wc_field in, int kind, SolverState &S, bool omega,
+                             wc_field with);
+// the FP64 operator of the whole lattice in that form; cudaErrorNotSupported
+// under another launch shape
+struct StepSum;
+cudaError_t launch_apply64_sum(wc_lattice lat, wc_field out, wc_field in, int kind, cudaStream_t stream,
+                               const StepSum &ss, bool omega, bool pdl);
 cudaError_t launch_copy(wc_lattice lat, wc_field dst, wc_field src, double scale, const double *dev_scale,
                         int invert_scale, cudaStream_t stream);
 // RAS on block Schur complements, on half-lattice (even-site) fields of the

@@ -242,12 +242,10 @@ wc_status enqueue_iteration(wc_lattice lat, SolverState &S, const wc_solve_param
     const bool norm = w.phat != w.p;   // a preconditioner scales its input by |p|, |s|
     wc_status st = check_cuda(lat, bicg_p(lat, S, d2(w.r), d2(w.v), d2(w.p), norm), "bicg_p");
     if (st == WC_OK) st = apply_precond(lat, S, p, kind, w, w.p, w.phat, &S.scal->pp);
-    if (st == WC_OK) st = check_cuda(lat, launch_apply(lat, w.v, w.phat, kind, S, true), "apply");
-    if (st == WC_OK) st = check_cuda(lat, bicg_alpha(lat, S, d2(w.rhat), d2(w.v)), "bicg_alpha");
+    if (st == WC_OK) st = check_cuda(lat, launch_apply_sum(lat, w.v, w.phat, kind, S, false, w.rhat), "apply, alpha");
     if (st == WC_OK) st = check_cuda(lat, bicg_s(lat, S, d2(w.r), d2(w.v), d2(w.s), norm), "bicg_s");
     if (st == WC_OK) st = apply_precond(lat, S, p, kind, w, w.s, w.shat, &S.scal->ss);
-    if (st == WC_OK) st = check_cuda(lat, launch_apply(lat, w.t, w.shat, kind, S, true), "apply");
-    if (st == WC_OK) st = check_cuda(lat, bicg_omega(lat, S, d2(w.t), d2(w.s)), "bicg_omega");
+    if (st == WC_OK) st = check_cuda(lat, launch_apply_sum(lat, w.t, w.shat, kind, S, true, w.s), "apply, omega");
     if (st == WC_OK)
         st = check_cuda(lat, bicg_xr(lat, S, d2(x), d2(w.phat), d2(w.shat), d2(w.s), d2(w.t), d2(w.r), d2(w.rhat)),
                         "bicg_xr");
@@ -587,12 +585,10 @@ wc_status enqueue_lo_iteration(wc_lattice lat, SolverState &S, const wc_solve_pa
 {
     wc_status st = check_cuda(lat, lo_p(lat, S, w.r, w.v, w.p), "lo_p");
     if (st == WC_OK) st = lo_precond(lat, S, p, kind, w, w.p, w.phat);
-    if (st == WC_OK) st = check_cuda(lat, launch_apply(lat, w.v, w.phat, kind, S, true), "apply");
-    if (st == WC_OK) st = check_cuda(lat, lo_alpha(lat, S, w.rhat, w.v), "lo_alpha");
+    if (st == WC_OK) st = check_cuda(lat, launch_apply_sum(lat, w.v, w.phat, kind, S, false, w.rhat), "apply, alpha");
     if (st == WC_OK) st = check_cuda(lat, lo_s(lat, S, w.r, w.v, w.s), "lo_s");
     if (st == WC_OK) st = lo_precond(lat, S, p, kind, w, w.s, w.shat);
-    if (st == WC_OK) st = check_cuda(lat, launch_apply(lat, w.t, w.shat, kind, S, true), "apply");
-    if (st == WC_OK) st = check_cuda(lat, lo_omega(lat, S, w.t, w.s), "lo_omega");
+    if (st == WC_OK) st = check_cuda(lat, launch_apply_sum(lat, w.t, w.shat, kind, S, true, w.s), "apply, omega");
     if (st == WC_OK)
         st = check_cuda(lat, lo_xr(lat, S, w.xlo, w.phat, w.shat, w.s, w.t, w.r, w.rhat),
                         "lo_xr");

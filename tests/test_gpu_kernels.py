@@ -335,3 +335,50 @@ def test_force_from_shared_plaquettes(dims, tbc, csw):
     scale = np.abs(F).max()
     assert np.abs(F + F.conj().swapaxes(-1, -2)).max() == 0.0
     assert np.abs(np.trace(F, axis1=-2, axis2=-1)).max() <= 1e-14 * scale
+
+
+@pytest.mark.parametrize("kw,dims", [
+    # FP64, whole lattice: CTAs of 32 sites, the last grid that forms its sums
+    # in the operator pass (152 SMs) and the first that does not
+    (dict(), (2, 2, 2, 2)), (dict(), (5, 3, 7, 9)), (dict(), (8, 8, 8, 76)), (dict(), (8, 8, 8, 78)),
+    (dict(even_odd=True), (2, 2, 2, 2)), (dict(even_odd=True), (6, 2, 10, 4)),
+    # low precisions: CTAs of one warp up to 9728 even sites, of four from 38912 on
+    (dict(even_odd=True, solver=1, krylov_prec=1), (2, 2, 2, 2)),
+    (dict(even_odd=True, solver=1, krylov_prec=1), (6, 2, 10, 4)),
+    (dict(even_odd=True, solver=1, krylov_prec=1), (8, 8, 8, 38)),
+    (dict(even_odd=True, solver=1, krylov_prec=1), (8, 8, 8, 40)),
+    (dict(even_odd=True, solver=1, krylov_prec=1), (10, 14, 18, 34)),
+    (dict(even_odd=True, solver=1, krylov_prec=2), (6, 2, 10, 4)),
+    (dict(even_odd=True, solver=1, krylov_prec=2), (10, 14, 18, 34))])
+def test_sums_formed_by_the_operator_pass(kw, dims):
+    """x after one step from x = 0 is alpha b + omega s: the scalars of a step
+    whether its operator passes form the sums or separate passes do.  The
+    source lives on even sites, so that M^ is all that an even-odd step
+    applies to it.  x is first order in both scalars and in the vectors as
+    stored: the tolerance of the Krylov vectors."""
+    U = synth.exp_links(dims, 0.3, 121)
+    lat = make_lattice(dims, U, 1.0, 0.12, -1)
+    eo = bool(kw)
+    c = np.indices(dims[::-1]).sum(axis=0).reshape(-1) % 2 == 0
+    src = synth.gaussian_source(dims, 122)
+    if eo:
+        src = src * c.reshape(-1, *[1] * (src.ndim - 1))
+    f, g = lat.field(0), lat.field(0)
+
+    def op(a):
+        (lat.apply_schur if eo else lat.apply_M)(g, f.load(a))
+        return g.store(np.zeros_like(a))
+
+    v = op(src)
+    alpha = np.vdot(src, src) / np.vdot(src, v)
+    s = src - alpha * v
+    t = op(s)
+    assert abs(np.vdot(t, s)) > 0.75 * np.linalg.norm(t) * np.linalg.norm(s)     # omega as it is
+    ref = alpha * src + np.vdot(t, s) / np.vdot(t, t) * s
+    x = lat.field(0)
+    info = lat.solve(x, lat.field(0).load(src), tol=1e-14, max_iter=1, check=False, **kw)
+    assert info.iters == 1
+    out = x.store(np.zeros_like(src))
+    if eo:
+        out = out * c.reshape(-1, *[1] * (src.ndim - 1))
+    assert np.linalg.norm(out - ref) <= TOL[kw.get("krylov_prec", 0)] * np.linalg.norm(ref)
