@@ -843,38 +843,116 @@ __global__ void __launch_bounds__(kRedBlock) k_lo_xr_h(int V, float4 *xlo, HF ph
     body_lo_xr_h(V, xlo, phat, shat, s, t, r, rhat, rs, sc, rep, seq);
 }
 
+// Six components (two spins) of a site: half h of a field of V sites, as the
+// lanes of a half-warp hold them.  store: s in Krylov storage, s left as a
+// load would return it; the lanes of the two halves of a site are 16 apart.
+template <class PL>
+struct HalfSite;
+
+template <>
+struct HalfSite<P32> {
+    static __device__ __forceinline__ void store(void *d, float *, int V, int x, int h, cx<float> s[6], bool valid)
+    {
+        float4 *p = static_cast<float4 *>(d) + (size_t)3 * h * V + x;
+        if (valid)
+#pragma unroll
+            for (int q = 0; q < 3; ++q)
+                p[(size_t)q * V] = make_float4(s[2 * q].re, s[2 * q].im, s[2 * q + 1].re, s[2 * q + 1].im);
+    }
+    static __device__ __forceinline__ void load(const void *d, const float *, int V, int x, int h, cx<float> s[6])
+    {
+        const float4 *p = static_cast<const float4 *>(d) + (size_t)3 * h * V + x;
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            const float4 w = __ldg(p + (size_t)q * V);
+            s[2 * q] = mkc(w.x, w.y);
+            s[2 * q + 1] = mkc(w.z, w.w);
+        }
+    }
+};
+
+// (the second of the three words of a site belongs to both halves)
+template <>
+struct HalfSite<P16> {
+    static __device__ __forceinline__ void store(void *d, float *nrm, int V, int x, int h, cx<float> s[6], bool valid)
+    {
+        float m = 0.f;
+#pragma unroll
+        for (int k = 0; k < 6; ++k) m = fmax3(m, fabsf(s[k].re), fabsf(s[k].im));
+        m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 16));
+        const float inv = m > 0.f ? 1.f / m : 0.f;
+        unsigned w[6];
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+            w[k] = c2h(s[k].re * inv, s[k].im * inv);
+            s[k] = m * h2c(w[k]);
+        }
+        if (!valid) return;
+        uint4 *p = static_cast<uint4 *>(d) + x;
+        p[h ? (size_t)2 * V : 0] = h ? make_uint4(w[2], w[3], w[4], w[5]) : make_uint4(w[0], w[1], w[2], w[3]);
+        reinterpret_cast<uint2 *>(p + V)[h] = h ? make_uint2(w[0], w[1]) : make_uint2(w[4], w[5]);
+        if (h == 0) nrm[x] = m;
+    }
+    static __device__ __forceinline__ void load(const void *d, const float *nrm, int V, int x, int h, cx<float> s[6])
+    {
+        const uint4 *p = static_cast<const uint4 *>(d) + x;
+        const float sc = __ldg(nrm + x);
+        const uint4 a = __ldg(p + (h ? (size_t)2 * V : 0));
+        const uint2 b = __ldg(reinterpret_cast<const uint2 *>(p + V) + h);
+        const unsigned w[6] = {h ? b.x : a.x, h ? b.y : a.y, h ? a.x : a.z, h ? a.y : a.w, h ? a.z : b.x, h ? a.w : b.y};
+#pragma unroll
+        for (int k = 0; k < 6; ++k) s[k] = sc * h2c(w[k]);
+    }
+};
+
 // End of a reliable update in one pass (the FP64 residual, its
 // low-precision copy and the new rho of the recurrence): r = b - r (r holds
 // op x), rr = |r|^2; rlo = r rounded to the Krylov storage PL (FP32, or
 // FP16 with its per-site scale); rho = <rhat, rlo> of the stored rlo and
-// beta from rho0, alpha, omega of the last step (lo_rho_update).  One site
-// per thread.
+// beta from rho0, alpha, omega of the last step (refresh_update).  Half a
+// site per thread, 16 sites per warp: with a site per thread the half lattice
+// of 16^3x32 filled 256 of the 608 blocks, and that of 24^3x32 took some of
+// them two turns and some one: FP32 at 16^3x32 50 -> 43 us beside a solve's other
+// kernels and 37 -> 31 in a batch, binary16 at 24^3x32 75 -> 59.
 template <class PL>
-__global__ void __launch_bounds__(kRedBlock) k_refresh_tail(int V, const void *b, void *r, void *rlo, float *rlo_n,
+__global__ void __launch_bounds__(kRedBlock) k_refresh_tail(int V, const double2 *b, double2 *r, void *rlo, float *rlo_n,
                                                             const void *rhat, const float *rhat_n, ReduceScratch rs,
                                                             SolverScalars *sc, StepReport *rep, unsigned long long seq)
 {
     griddep_wait();
     griddep_launch_dependents();
     double acc[3] = {0.0, 0.0, 0.0};
-    for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < V; x += gridDim.x * blockDim.x) {
-        cx<double> bv[12], rv[12];
-        P64::load_spinor(b, nullptr, V, x, bv);
-        P64::load_spinor(r, nullptr, V, x, rv);
-        cx<float> lo[12];
+    const int lane = threadIdx.x & 31, h = lane >> 4;
+    for (int t = blockIdx.x * kRedWarps + (threadIdx.x >> 5); t * 16 < V; t += gridDim.x * kRedWarps) {
+        const int x = t * 16 + (lane & 15);
+        const bool valid = x < V;
+        cx<float> lo[6], hat[6];
 #pragma unroll
-        for (int k = 0; k < 12; ++k) {
-            rv[k] = bv[k] - rv[k];
-            acc[0] += rv[k].re * rv[k].re + rv[k].im * rv[k].im;
-            lo[k] = mkc((float)rv[k].re, (float)rv[k].im);
+        for (int k = 0; k < 6; ++k) lo[k] = hat[k] = mkc(0.f, 0.f);
+        if (valid) {
+            const size_t at = (size_t)6 * h * V + x;
+            double2 bv[6], rv[6];
+#pragma unroll
+            for (int k = 0; k < 6; ++k) {
+                bv[k] = __ldg(b + at + (size_t)k * V);
+                rv[k] = r[at + (size_t)k * V];
+            }
+            HalfSite<PL>::load(rhat, rhat_n, V, x, h, hat);
+#pragma unroll
+            for (int k = 0; k < 6; ++k) {
+                const double2 d = make_double2(bv[k].x - rv[k].x, bv[k].y - rv[k].y);
+                r[at + (size_t)k * V] = d;
+                acc[0] = fma(d.x, d.x, fma(d.y, d.y, acc[0]));
+                lo[k] = mkc((float)d.x, (float)d.y);
+            }
         }
-        P64::store_spinor(r, nullptr, V, x, rv);
-        PL::store_spinor(rlo, rlo_n, V, x, lo);
-        PL::as_stored(lo);
-        cx<float> h[12];
-        PL::load_spinor(rhat, rhat_n, V, x, h);
+        HalfSite<PL>::store(rlo, rlo_n, V, x, h, lo, valid);
         float d[2] = {0.f, 0.f};
-        cdot_acc(h, lo, d);
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+            d[0] = fmaf(hat[k].re, lo[k].re, fmaf(hat[k].im, lo[k].im, d[0]));
+            d[1] = fmaf(hat[k].re, lo[k].im, fmaf(-hat[k].im, lo[k].re, d[1]));
+        }
         acc[1] += d[0];
         acc[2] += d[1];
     }
@@ -921,9 +999,13 @@ __global__ void __launch_bounds__(kRedBlock) k_lo_group(int V, const LoMember *m
 
 // The alpha or omega scalars of every member from the partial sums the
 // even multi-RHS Schur pass wrote (one member per CTA, the partials summed
-// in a fixed order, so the result does not depend on scheduling).
+// in a fixed order, so the result does not depend on scheduling).  A CTA
+// waits for its reads, one partial for 16 sites: 32 warps instead of 8, with
+// eight reads of each in flight, took 4096 partials from 16.1 to 11.2 us
+// (omega) and 13.7 to 9.4 (alpha).
+constexpr int kFinalBlock = 1024;
 template <int STEP>
-__global__ void __launch_bounds__(kRedBlock) k_lo_group_finalize(int nblk, const double *part, const LoMember *members)
+__global__ void __launch_bounds__(kFinalBlock) k_lo_group_finalize(int nblk, const double *part, const LoMember *members)
 {
     const LoMember &a = members[blockIdx.x];
     if (a.sc->skip) return;   // its partials were not written
@@ -931,14 +1013,18 @@ __global__ void __launch_bounds__(kRedBlock) k_lo_group_finalize(int nblk, const
     // warp w adds the partials of sum w % 4
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     double s[1] = {0.0};
-#pragma unroll 4
-    for (int b = (wid / 4) * 32 + lane; b < nblk; b += kRedBlock / 4) s[0] += p[(size_t)b * 4 + wid % 4];
+#pragma unroll 8
+    for (int b = (wid / 4) * 32 + lane; b < nblk; b += kFinalBlock / 4) s[0] += p[(size_t)b * 4 + wid % 4];
     const double t = warp_sums(s);
-    __shared__ double fin[kRedWarps];
+    __shared__ double fin[kFinalBlock / 32];
     if (lane == 0) fin[wid] = t;
     __syncthreads();
     if (wid != 0) return;
-    const double u = lane < 4 ? fin[lane] + fin[lane + 4] : 0.0;
+    // lane l: the sum l % 4 of warp l
+    double u = fin[lane];
+#pragma unroll
+    for (int o = 4; o < 32; o *= 2) u += __shfl_xor_sync(0xffffffffu, u, o);
+    if (lane >= 4) u = 0.0;
     if (STEP == LO_STEP_ALPHA) alpha_update(u, a.sc);
     else lo_omega_update(u, a.sc);
 }
@@ -1086,12 +1172,9 @@ cudaError_t lo_xr(wc_lattice lat, SolverState &S, wc_field xlo, wc_field phat, w
 cudaError_t refresh_tail(wc_lattice lat, SolverState &S, const wc_field b, wc_field r_hp, wc_field r, wc_field rhat)
 {
     const int V = lat->g.V;
-    if (half_vectors(r))
-        launch_step(S.pdl, k_refresh_tail<P16>, WC_STEP(V), V, b->data, r_hp->data, r->data, r->nrm, rhat->data, rhat->nrm,
-                                                  S.red, S.scal, S.rep, S.seq);
-    else
-        launch_step(S.pdl, k_refresh_tail<P32>, WC_STEP(V), V, b->data, r_hp->data, r->data, nullptr, rhat->data, nullptr,
-                                                  S.red, S.scal, S.rep, S.seq);
+    const auto kern = half_vectors(r) ? k_refresh_tail<P16> : k_refresh_tail<P32>;
+    launch_step(S.pdl, kern, WC_STEP(2LL * ((V + 15) / 16 * 16)), V, static_cast<const double2 *>(b->data),
+                static_cast<double2 *>(r_hp->data), r->data, r->nrm, rhat->data, rhat->nrm, S.red, S.scal, S.rep, S.seq);
     return cudaGetLastError();
 }
 LoMember lo_member(SolverState &S, wc_field r, wc_field rhat, wc_field p, wc_field v, wc_field s, wc_field t,
@@ -1142,9 +1225,9 @@ cudaError_t lo_group_finalize(LoStep step, int m, int nblk, const double *part, 
 {
     if (m < 1 || nblk < 1) return cudaErrorInvalidValue;
     if (step == LO_STEP_ALPHA)
-        k_lo_group_finalize<LO_STEP_ALPHA><<<m, 256, 0, stream>>>(nblk, part, members);
+        k_lo_group_finalize<LO_STEP_ALPHA><<<m, kFinalBlock, 0, stream>>>(nblk, part, members);
     else if (step == LO_STEP_OMEGA)
-        k_lo_group_finalize<LO_STEP_OMEGA><<<m, 256, 0, stream>>>(nblk, part, members);
+        k_lo_group_finalize<LO_STEP_OMEGA><<<m, kFinalBlock, 0, stream>>>(nblk, part, members);
     else
         return cudaErrorInvalidValue;
     return cudaGetLastError();

@@ -382,3 +382,23 @@ def test_sums_formed_by_the_operator_pass(kw, dims):
     if eo:
         out = out * c.reshape(-1, *[1] * (src.ndim - 1))
     assert np.linalg.norm(out - ref) <= TOL[kw.get("krylov_prec", 0)] * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("dims", [(2, 2, 2, 2), (3, 5, 3, 7), (4, 4, 4, 6)])
+@pytest.mark.parametrize("krylov", [1, 2])
+def test_refresh_on_half_warps_of_ragged_lattices(dims, krylov):
+    """A refresh replaces the recurrence's residual 16 sites to a warp.  Lost
+    sites or a wrong rho would leave the recurrence with another residual than
+    the true one: the solve would need further refreshes and steps, and it
+    would not take the steps of the FP64 solve within a factor of two."""
+    kappa, csw, tbc = 0.12, 1.0, -1
+    U = synth.exp_links(dims, 0.3, 131)
+    lat = make_lattice(dims, U, csw, kappa, tbc)
+    src = synth.gaussian_source(dims, 132)
+    b = lat.field(0).load(src)
+    plain = lat.solve(lat.field(0), b, tol=1e-11)
+    x = lat.field(0)
+    info = lat.solve(x, b, tol=1e-11, solver=1, krylov_prec=krylov)
+    r = src - oracle.apply_M(dims, tbc, kappa, csw, U, x.store(np.zeros_like(src)))
+    assert np.linalg.norm(r) <= 1.5e-11 * np.linalg.norm(src)
+    assert info.iters <= 2 * plain.iters + 4
