@@ -6,11 +6,15 @@
 // im.lo), operated on by paired instructions (wc_df2.cuh).  Sums of products
 // are formed as compensated dot products (Ogita, Rump and Oishi 2005, "Dot2"):
 // every product's rounding error, its cross terms and the error of adding it
-// to the running sum go into one FP32 error sum, and hi + lo is normalised
-// once per sum: 12 paired instructions a term and a chain of six through the
-// running sum, where a multiply-add of double-word numbers that normalises
-// each time takes 16 and a chain of twelve.  What the stencil sums are
-// accurate to stays the same, about 2^-45 of the largest terms.
+// to the running sum go into one FP32 error sum.  That sum is rounded at its
+// own size, so it is kept small: hi + lo is normalised every second term (13.5
+// paired instructions a term and a chain of seven through the running sum,
+// where a multiply-add of double-word numbers that normalises each time takes
+// 16 and a chain of twelve), and the diagonal of a clover block, its largest
+// term, comes last.  Relative errors against FP64, M / M^: 5.1e-15 / 1.5e-14 at
+// kappa 0.12, 5.6e-15 / 1.7e-14 at 0.137, csw 1.9 (a site per thread with
+// double-word multiply-adds: 6.6e-15 / 1.5e-14, 8.5e-15 / 1.7e-14; one
+// normalisation per sum: 2.2e-14 / 2.3e-14, 5 % faster).
 //
 // One site per thread at 128 registers spilled 1 KB and ran 22 500 warp
 // instructions per 32 sites of an even-odd pass in 38 % of the issue slots;
@@ -29,9 +33,10 @@ using f2::u64;
 using f2::z2;
 
 constexpr int kSites = kSplit64Sites;
-// CTAs per SM: 128 registers, no spills; even-odd passes at 24^3x32 172 + 137
-// us, 198 + 146 with three (168 registers), 179 + 141 with five (96, 100 B of
-// spills); 324 + 295 us with a site per thread
+// CTAs per SM: 128 registers, no spills; even-odd passes at 24^3x32 178 + 144
+// us (before the normalisation of every second term: 172 + 137
+// with four CTAs, 198 + 146 with three (168 registers), 179 + 141 with five (96, 100 B of
+// spills)); 324 + 295 us with a site per thread
 constexpr int kCtas = 4;
 using Mem = float4[kSplit64][12][kSites];   // z2 as float4 (H, L)
 
@@ -85,14 +90,26 @@ __device__ __forceinline__ void add_term(Sum &t, df b, z2 x)
 {
     const u64 nb = f2::pk(-b.hi, -b.hi), bh = f2::pk(b.hi, b.hi), bl = f2::pk(b.lo, b.lo);
     const u64 np = f2::mul(nb, x.h);              // -fl(b x)
-    t.e = f2::add(t.e, f2::fma(bh, x.h, np));     // its rounding error
-    t.e = f2::fma(bh, x.l, t.e);
-    t.e = f2::fma(bl, x.h, t.e);
+    const u64 q = f2::fma(bl, x.h, f2::fma(bh, x.l, f2::fma(bh, x.h, np)));   // its rounding error, the cross terms
     const u64 s = f2::sub(t.s, np);               // TwoSum(t.s, -np)
     const u64 bb = f2::sub(s, t.s);
     const u64 e1 = f2::sub(t.s, f2::sub(s, bb)), e2 = f2::add(np, bb);
-    t.e = f2::add(t.e, f2::sub(e1, e2));
+    t.e = f2::add(t.e, f2::add(q, f2::sub(e1, e2)));
     t.s = s;
+}
+// the error sum back below half a unit of s
+__device__ __forceinline__ void normalise(Sum &t)
+{
+    const u64 hi = f2::add(t.s, t.e);
+    t.e = f2::sub(t.e, f2::sub(hi, t.s));
+    t.s = hi;
+}
+// + (re + i im) x, with ix = i x
+__device__ __forceinline__ void add_pair(Sum &t, df re, z2 x, df im, z2 ix)
+{
+    add_term(t, re, x);
+    add_term(t, im, ix);
+    normalise(t);
 }
 // the first term
 __device__ __forceinline__ Sum first_term(df b, z2 x)
@@ -161,7 +178,7 @@ __device__ __forceinline__ void link_mul(const GaugeStore &U, int V, int mu, int
                 const float4 m = ADJ ? u[3 * j + i] : u[3 * i + j];
                 const df re(m.x, m.y), im = ADJ ? df(-m.z, -m.w) : df(m.z, m.w);
                 if (j == 0) t = first_term(re, h[3 * s]);
-                else add_term(t, re, h[3 * s + j]);
+                else normalise(t), add_term(t, re, h[3 * s + j]);
                 add_term(t, im, ih[j]);
             }
             w[3 * s + i] = finish(t);
@@ -229,8 +246,6 @@ __device__ __forceinline__ void clover_rows_at(const CloverStore &C, int V, int 
         const float4 a = __ldg(p + (size_t)V), e = __ldg(p + (size_t)2 * V);
         d[0] = df(a.z, a.w), d[1] = df(e.x, e.y), d[2] = df(e.z, e.w);
     }
-#pragma unroll
-    for (int r = 0; r < 3; ++r) add_term(y[r], d[r], v[I0 + r]);
     z2 iv[6];
 #pragma unroll
     for (int k = 0; k < 6; ++k) iv[k] = times_i(v[k]);
@@ -243,14 +258,16 @@ __device__ __forceinline__ void clover_rows_at(const CloverStore &C, int V, int 
             const float4 e = __ldg(p + (size_t)(3 + i * (i - 1) / 2 + j) * V);
             const df re(e.x, e.y), im(e.z, e.w);
             if (row) {
-                add_term(y[i - I0], re, v[j]);
-                add_term(y[i - I0], im, iv[j]);
+                add_pair(y[i - I0], re, v[j], im, iv[j]);
             }
             if (col) {   // the mirror entry: conjugate
-                add_term(y[j - I0], re, v[i]);
-                add_term(y[j - I0], -im, iv[i]);
+                add_pair(y[j - I0], re, v[i], -im, iv[i]);
             }
         }
+    // the diagonal, the largest term, at the end: the error sums of the others
+    // stay small
+#pragma unroll
+    for (int r = 0; r < 3; ++r) add_term(y[r], d[r], v[I0 + r]);
 }
 
 __device__ __forceinline__ void clover_rows(const CloverStore &C, int V, int x, int w, const z2 v[6], Sum y[3])

@@ -206,11 +206,14 @@ __global__ void __launch_bounds__(kSplit64 * kSplit64Sites, 3)
     reduce_step_sums<OMEGA, kSplit64, double>(acc, ss);
 }
 
-// The same in double-FP32 arithmetic (wc_dfsplit.cuh).  HDF: in holds split
-// values.
+// The same with the hops in double-FP32 arithmetic (wc_dfsplit.cuh); HDF: hin
+// holds split values of in.  The clover term stays in FP64: its 66
+// instructions per warp run on the FP64 units while the other warps' hops
+// fill the FP32 pipes, and the largest term of out keeps all its bits.
 template <int KIND, bool HDF>
 __global__ void __launch_bounds__(kSplit64 * kSplit64Sites, dfs::kCtas)
-    k_apply_splitdf(Geom g, GaugeStore U, CloverStore C, const void *in, void *out, double kappa, const int *skip)
+    k_apply_splitdf(Geom g, GaugeStore U, CloverStore C, const void *hin, const void *in, void *out, double kappa,
+                    const int *skip)
 {
     griddep_wait();
     griddep_launch_dependents();
@@ -222,26 +225,27 @@ __global__ void __launch_bounds__(kSplit64 * kSplit64Sites, dfs::kCtas)
     if (valid) {
         int c[4];
         site_coords_fast(g, x, c);
-        dfs::hops<KIND == 1 ? +1 : -1, HDF>(g, U, in, g.V, x, c, sm, w, s, [](int y) { return y; });
+        dfs::hops<KIND == 1 ? +1 : -1, HDF>(g, U, hin, g.V, x, c, sm, w, s, [](int y) { return y; });
     }
     __syncthreads();
     if (!valid) return;
-    double2 *o = static_cast<double2 *>(out) + (size_t)3 * w * g.V + x;
-    if (KIND == 2) {
+    cx<double> y[3];
+    if (KIND != 2) {
+        cx<double> v[6];
+        const double2 *p = static_cast<const double2 *>(in) + (size_t)(w >> 1) * 6 * g.V + x;
 #pragma unroll
-        for (int r = 0; r < 3; ++r) o[(size_t)r * g.V] = dfs::to_double(dfs::sum(sm, 3 * w + r, s));
-        return;
+        for (int k = 0; k < 6; ++k) {
+            const double2 a = __ldg(p + (size_t)k * g.V);
+            v[k] = mkc(a.x, a.y);
+        }
+        clover_rows64(C, g.V, x, w, v, y);
     }
-    const df mk(-kappa);
-    f2::z2 v[6];
+    double2 *o = static_cast<double2 *>(out) + (size_t)3 * w * g.V + x;
 #pragma unroll
-    for (int k = 0; k < 6; ++k) v[k] = dfs::load<HDF>(in, g.V, 6 * (w >> 1) + k, x);
-    dfs::Sum y[3];
-#pragma unroll
-    for (int r = 0; r < 3; ++r) y[r] = dfs::first_term(mk, dfs::sum(sm, 3 * w + r, s));
-    dfs::clover_rows(C, g.V, x, w, v, y);
-#pragma unroll
-    for (int r = 0; r < 3; ++r) o[(size_t)r * g.V] = dfs::to_double(dfs::finish(y[r]));
+    for (int r = 0; r < 3; ++r) {
+        const double2 h = dfs::to_double(dfs::sum(sm, 3 * w + r, s));
+        o[(size_t)r * g.V] = KIND == 2 ? h : make_double2(fma(-kappa, h.x, y[r].re), fma(-kappa, h.y, y[r].im));
+    }
 }
 
 // ---- launch shapes and their autotuner ---------------------------------
@@ -306,12 +310,16 @@ cudaError_t launch_split64(wc_lattice lat, wc_field out, wc_field in, int kind, 
 {
     const Geom &g = lat->g;
     const dim3 grid((g.V + kSplit64Sites - 1) / kSplit64Sites);
-    const auto k64 = kind == 0 ? k_apply_split64<0> : kind == 1 ? k_apply_split64<1> : k_apply_split64<2>;
-    const auto kdf = kind == 0 ? k_apply_splitdf<0, false>
-                               : kind == 1 ? k_apply_splitdf<1, false> : k_apply_splitdf<2, false>;
-    const auto kern = std::is_same<P, PDF>::value ? kdf : k64;
-    return launch_step(pdl && pdl_grid(grid.x), kern, grid, kSplit64 * kSplit64Sites, stream, g, lat->gauge, lat->clover, in->data,
-                       out->data, lat->kappa, skip);
+    if constexpr (std::is_same<P, PDF>::value) {
+        const auto kern = kind == 0 ? k_apply_splitdf<0, false>
+                                    : kind == 1 ? k_apply_splitdf<1, false> : k_apply_splitdf<2, false>;
+        return launch_step(pdl && pdl_grid(grid.x), kern, grid, kSplit64 * kSplit64Sites, stream, g, lat->gauge,
+                           lat->clover, in->data, in->data, out->data, lat->kappa, skip);
+    } else {
+        const auto kern = kind == 0 ? k_apply_split64<0> : kind == 1 ? k_apply_split64<1> : k_apply_split64<2>;
+        return launch_step(pdl && pdl_grid(grid.x), kern, grid, kSplit64 * kSplit64Sites, stream, g, lat->gauge,
+                           lat->clover, in->data, out->data, lat->kappa, skip);
+    }
 }
 
 template <class P>
@@ -598,7 +606,7 @@ cudaError_t launch_apply_df(wc_lattice lat, wc_field out, wc_field in, wc_field 
     const dim3 grid((g.V + kSplit64Sites - 1) / kSplit64Sites);
     const auto kern = kind == 0 ? k_apply_splitdf<0, true> : kind == 1 ? k_apply_splitdf<1, true> : k_apply_splitdf<2, true>;
     return launch_step(pdl && pdl_grid(grid.x), kern, grid, kSplit64 * kSplit64Sites, stream, g, lat->gauge, lat->clover,
-                       split->data, out->data, lat->kappa, skip);
+                       split->data, in->data, out->data, lat->kappa, skip);
 }
 
 cudaError_t launch_copy(wc_lattice lat, wc_field dst, wc_field src, double scale, const double *dev_scale,

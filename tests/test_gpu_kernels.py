@@ -402,3 +402,27 @@ def test_refresh_on_half_warps_of_ragged_lattices(dims, krylov):
     r = src - oracle.apply_M(dims, tbc, kappa, csw, U, x.store(np.zeros_like(src)))
     assert np.linalg.norm(r) <= 1.5e-11 * np.linalg.norm(src)
     assert info.iters <= 2 * plain.iters + 4
+
+
+@pytest.mark.parametrize("dims", [(4, 4, 4, 6), (8, 8, 8, 8)])
+@pytest.mark.parametrize("kappa,csw", [(0.12, 1.0), (0.137, 1.9)])
+def test_double_fp32_operators_keep_their_accuracy(dims, kappa, csw):
+    """Relative L2 distance of the double-FP32 operators from the FP64 ones.
+    A pair of floats rounds at 2^-49 = 1.8e-15.  With a chain of double-word
+    multiply-adds per row, M stood at 6.6e-15 (kappa 0.12) and 8.5e-15 and M^,
+    two dot products longer, at 1.53e-14 and 1.74e-14: the dot products may not
+    be worse."""
+    U = synth.exp_links(dims, 0.3, 141)
+    lat = make_lattice(dims, U, csw, kappa, -1)
+    src = synth.gaussian_source(dims, 142)
+    f, g = lat.field(0).load(src), lat.field(0)
+    out = {}
+    for arith in (0, 1):
+        lat.set_fp64_arith(arith)
+        for name, op in (("M", lat.apply_M), ("S", lat.apply_schur)):
+            op(g, f)
+            out[name, arith] = g.store(np.zeros_like(src))
+    bound = {"M": 6.6e-15 if kappa == 0.12 else 8.5e-15, "S": 1.53e-14 if kappa == 0.12 else 1.74e-14}
+    for name in ("M", "S"):
+        a, b = out[name, 0], out[name, 1]
+        assert np.linalg.norm(a - b) <= bound[name] * np.linalg.norm(a), name
