@@ -8,7 +8,7 @@ One step = one application of M = (1 + T) - kappa H to an FP32 colour-spinor
 field on the 24^3x32 lattice (Haar-like SU(3) links, csw = 1.0,
 kappa = 0.125, antiperiodic time, Z2 source), inputs resident in HBM.
 GFlop/s counts 1320 (hopping) + 504 (clover) = 1824 flops per site.  Every
-step reads links + clover + input spinor = 297 MB (> 129 MB L2) and steps
+step reads links + clover + input spinor = 262 MB (> 129 MB L2) and steps
 rotate over 4 input/output field pairs.
 
 Under torchrun (N > 1) every rank runs an independent replica of the
@@ -38,9 +38,9 @@ sys.path.insert(0, ROOT)
 
 FLOPS_PER_SITE = 1320 + 504
 # compulsory bytes per site of one M apply: in + out spinor, 4 forward links,
-# clover (FP32 and FP16: 12-real links; FP16: per-site FP32 scale with each
-# spinor; FP64: 18-real links)
-BYTES_PER_SITE = {"f32": 96 + 96 + 192 + 288, "f16": 52 + 52 + 96 + 144, "f64": 192 + 192 + 576 + 576}
+# clover (FP32 and FP16: 12-real links, the 2 x 26 independent reals of A;
+# FP16: per-site FP32 scale with each spinor; FP64: 18-real links, 72 reals)
+BYTES_PER_SITE = {"f32": 96 + 96 + 192 + 208, "f16": 52 + 52 + 96 + 104, "f64": 192 + 192 + 576 + 576}
 CFG = 2  # the 24^3x32 FP32 workload
 METRIC = "Wilson-Clover apply GFlop/s & % HBM roofline; mixed vs FP64 solve time to 1e-10"
 
@@ -52,8 +52,8 @@ NCU_TRAFFIC = {
     # the other lexicographic shapes run the same kernel body), from the
     # capture summarised in profiles/apply_fp32_24x24x24x32.md; valid while
     # the operator's device sources hash to sources_sha
-    "sources_sha": "b010e33ca36fe672",
-    "bytes_per_launch": 292184064,
+    "sources_sha": "a1c1240f8c1d4bb2",
+    "bytes_per_launch": 255279104,
 }
 
 
@@ -551,7 +551,7 @@ def batch_comparison(wc, args):
 def multi_rhs_apply(wc, lat, dims, single_ms, stream, n=12, reps=100):
     """The 12 spin-colour sources of a propagator through one multi-RHS
     launch (wc_apply_multi) on the same lattice: links and clover read once
-    per site for all 12 fields, 192 + 480/12 = 232 B per site and field."""
+    per site for all 12 fields, 192 + 400/12 = 225 B per site and field."""
     import torch
     import synth
     V = int(np.prod(dims))
@@ -569,7 +569,7 @@ def multi_rhs_apply(wc, lat, dims, single_ms, stream, n=12, reps=100):
     ms = e0.elapsed_time(e1) / reps
     for f in ins + outs:
         f.close()
-    bps = 192 + 480 / n
+    bps = 192 + 400 / n
     peak, _ = measured_peaks()
     gbs = bps * n * V / (ms * 1e-3) / 1e9
     return {"rhs": n, "ms_per_launch": ms, "gflops": FLOPS_PER_SITE * V * n / (ms * 1e-3) / 1e9,

@@ -261,8 +261,8 @@ wc_status wc_apply_hop(wc_lattice lat, wc_field out, wc_field in);
  * the solver is applied per source; the sources share U and A):
  * outs[r] = M ins[r] (dagger = 0) or M^+ ins[r] (dagger != 0), r < n,
  * 1 <= n <= 16, all FP32 fields of lat.  One launch reads the links and the
- * clover term once per site for all n fields: 192 + 480/n bytes per site and
- * field instead of 672.  Every out distinct from every other out and every
+ * clover term once per site for all n fields: 192 + 400/n bytes per site and
+ * field instead of 592.  Every out distinct from every other out and every
  * in.  Asynchronous on the lattice stream; WC_ERR_ARG for other precisions
  * or sizes, before any launch. */
 wc_status wc_apply_multi(wc_lattice lat, int n, wc_field *outs, wc_field *ins, int dagger);

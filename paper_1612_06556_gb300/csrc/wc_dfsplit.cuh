@@ -34,9 +34,9 @@ using f2::z2;
 
 constexpr int kSites = kSplit64Sites;
 // CTAs per SM: 128 registers, no spills; even-odd passes at 24^3x32 178 + 144
-// us (before the normalisation of every second term: 172 + 137
-// with four CTAs, 198 + 146 with three (168 registers), 179 + 141 with five (96, 100 B of
-// spills)); 324 + 295 us with a site per thread
+// us, 324 + 295 with a site per thread.  (Before the normalisation of every
+// second term: 172 + 137 us, 198 + 146 with three CTAs (168 registers), 179 +
+// 141 with five (96 registers, 100 B of spills).)
 constexpr int kCtas = 4;
 using Mem = float4[kSplit64][12][kSites];   // z2 as float4 (H, L)
 

@@ -6,8 +6,8 @@
 // The right-hand sides of a propagator share the gauge field, A and A^-1.
 // In one pass a site reads its 8 links (4 forward U_mu(x), 4 backward
 // U_mu(x - mu)) and one clover-type block (A^-1 on the odd pass, A on the
-// even pass): 672 B per site in FP32, 336 B in FP16 storage, against 96 /
-// 52 B per spinor read or written.  A CTA covers S consecutive
+// even pass): 672 / 592 B per site in FP32, 336 / 296 B in FP16 storage,
+// against 96 / 52 B per spinor read or written.  A CTA covers S consecutive
 // sites of one parity for all n right-hand sides: it stages those shared
 // words once in shared memory (coalesced along the sites), then thread
 // (s, r) computes site s of right-hand side r from the staged links and
