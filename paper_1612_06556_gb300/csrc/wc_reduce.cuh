@@ -202,7 +202,7 @@ __device__ __forceinline__ void lo_omega_update(double t, SolverScalars *sc)
 // 222; at 16^3x32 (512 CTAs of four) 121.7 and 116.3.
 inline bool sum_in_pass(const ReduceScratch &rs, int ctas, int warps)
 {
-    return ctas <= rs.max_blocks / 2 * warps;
+    return ctas <= rs.max_blocks / 2 * warps && ctas <= 2 * rs.max_blocks;   // the partials hold four sums of each
 }
 
 struct StepSum {
