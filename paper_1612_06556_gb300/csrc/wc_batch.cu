@@ -883,7 +883,8 @@ static wc_status batch_even_odd(int n, const wc_lattice *lats, wc_field *xs, wc_
             qi.tol = p->tol * scale[i];
             wc_solve_info sub{};
             H[i]->st.stream = lat->stream;
-            const wc_status sr = bicgstab(H[i], H[i]->st, 0, F(i, 2), F(i, 4), qi, &sub, infos[i].iters, bbh[i]);
+            const wc_status sr = idle_after(H[i], lat->stream, bicgstab(H[i], H[i]->st, 0, F(i, 2), F(i, 4), qi, &sub,
+                                                                        infos[i].iters, bbh[i]), &sub);
             if (sr != WC_OK && sr != WC_ERR_NOT_CONVERGED && sr != WC_ERR_BREAKDOWN) st = sr;
             infos[i].iters = sub.iters;
             infos[i].restarts += 1 + sub.restarts;

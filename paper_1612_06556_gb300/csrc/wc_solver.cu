@@ -142,7 +142,10 @@ struct StepQueue {
         if (st == WC_OK && ahead && more) st = push(enqueue);
         return st == WC_OK ? pop(h) : st;
     }
-    // a step queued ahead of the host's action does not run
+    // a step queued ahead of the host's action does not run: its kernels find
+    // the skip word set.  They stay on the stream, so whatever clears the word
+    // (track) must come after them there, and a solve must leave no such step
+    // behind when it returns (idle_after)
     void drop() { queued = 0; }
 };
 
@@ -341,11 +344,24 @@ wc_status bicgstab(wc_lattice lat, SolverState &S, int kind, wc_field x, wc_fiel
 static wc_status eo_bicgstab(wc_lattice lat, int kind, wc_field x, wc_field b, const wc_solve_params &p,
                              wc_solve_info *info);
 
+// The end of a solve on `stream`, whatever its outcome: a step queued ahead
+// and dropped is done with the solver state before the caller can start the
+// next solve, on this stream or another.
+wc_status idle_after(wc_lattice lat, cudaStream_t stream, wc_status st, wc_solve_info *info)
+{
+    const cudaError_t e = cudaStreamSynchronize(stream);
+    if (st != WC_OK || e == cudaSuccess) return st;
+    st = check_cuda(lat, e, "sync(solve)");
+    if (info) info->status = st;
+    return st;
+}
+
 wc_status bicgstab(wc_lattice lat, int kind, wc_field x, wc_field b, const wc_solve_params &p, wc_solve_info *info)
 {
     lat->st.stream = lat->stream;
-    if (p.even_odd) return eo_bicgstab(lat, kind, x, b, p, info);
-    return bicgstab(lat, lat->st, kind, x, b, p, info, 0, -1.0);
+    return idle_after(lat, lat->stream,
+                      p.even_odd ? eo_bicgstab(lat, kind, x, b, p, info)
+                                 : bicgstab(lat, lat->st, kind, x, b, p, info, 0, -1.0), info);
 }
 
 // Even-odd solve of op x = b (op = M, or M^+ for kind 1):

@@ -47,7 +47,10 @@ wc_status eo_reconstruct_residual(wc_lattice lat, int kind, wc_field be, wc_fiel
 wc_status bicgstab(wc_lattice lat, SolverState &S, int kind, wc_field x, wc_field b, const wc_solve_params &p,
                    wc_solve_info *info, int iters_done, double bb, double defer_rr = 0.0,
                    bool *unconfirmed = nullptr);
-// Same with the lattice's own state and stream.
+// Waits for `stream` at the end of a solve that returned st: a step queued
+// ahead may still be on it.  st, or the status of the wait.
+wc_status idle_after(wc_lattice lat, cudaStream_t stream, wc_status st, wc_solve_info *info);
+// Same with the lattice's own state and stream, idle on return.
 wc_status bicgstab(wc_lattice lat, int kind, wc_field x, wc_field b, const wc_solve_params &p, wc_solve_info *info);
 
 // FP32 vectors of the reliable-update solver (r, rhat, p, v, s, t, phat,
