@@ -197,7 +197,20 @@ __device__ __forceinline__ cx<double> ld(const double2 *p, long long i)
 }
 __device__ __forceinline__ void st(double2 *p, long long i, cx<double> a) { p[i] = make_double2(a.re, a.im); }
 
-__device__ __forceinline__ void init_update(double t, SolverScalars *sc)
+// one thread: the outcome of a step (or of the start of a run of steps) to the
+// host
+__device__ __forceinline__ void report(const SolverScalars *sc, StepReport *rep, unsigned long long seq)
+{
+    if (!rep) return;
+    rep->rr = sc->rr;
+    rep->flags = sc->flags;
+    rep->action = sc->action;
+    __threadfence_system();
+    rep->seq = seq;
+}
+
+__device__ __forceinline__ void init_update(double t, SolverScalars *sc, StepReport *rep = nullptr,
+                                            unsigned long long seq = 0)
 {
     if ((threadIdx.x & 31) != 0) return;
     const double rr = t;
@@ -218,6 +231,7 @@ __device__ __forceinline__ void init_update(double t, SolverScalars *sc)
             sc->skip = 1;
         }
     }
+    report(sc, rep, seq);
 }
 
 // After a step of a host-driven solve (one thread): does the host have to act
@@ -251,17 +265,6 @@ __device__ __forceinline__ void track_step(SolverScalars *sc)
     }
     sc->action = a;
     if (a != ACT_NONE) sc->skip = 1;
-}
-
-// one thread: the step's outcome to the host
-__device__ __forceinline__ void report(const SolverScalars *sc, StepReport *rep, unsigned long long seq)
-{
-    if (!rep) return;
-    rep->rr = sc->rr;
-    rep->flags = sc->flags;
-    rep->action = sc->action;
-    __threadfence_system();
-    rep->seq = seq;
 }
 
 __global__ void k_track(SolverScalars *sc, int track, double tol2, double d2, double defer2, double rr)
@@ -519,7 +522,8 @@ __device__ __forceinline__ void refresh_update(double t, SolverScalars *sc, Step
 
 // rhat = r, p = v = 0, xlo = 0; rr = |r|^2, rho = rr, alpha = omega = rho0 = 1
 __global__ void __launch_bounds__(kRedBlock) k_lo_init(long long n, const float4 *r, float4 *rhat, float4 *p,
-                                                       float4 *v, float4 *xlo, ReduceScratch rs, SolverScalars *sc)
+                                                       float4 *v, float4 *xlo, ReduceScratch rs, SolverScalars *sc,
+                                                       StepReport *rep, unsigned long long seq)
 {
     float acc[1] = {0.f};
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
@@ -531,7 +535,7 @@ __global__ void __launch_bounds__(kRedBlock) k_lo_init(long long n, const float4
         xlo[i] = make_float4(0.f, 0.f, 0.f, 0.f);
         acc[0] = fmaf(ri.x, ri.x, fmaf(ri.y, ri.y, fmaf(ri.z, ri.z, fmaf(ri.w, ri.w, acc[0]))));
     }
-    grid_reduce<1>(acc, rs, rs.result, [=](double t, const double *) { init_update(t, sc); });
+    grid_reduce<1>(acc, rs, rs.result, [=](double t, const double *) { init_update(t, sc, rep, seq); });
 }
 
 // p = r + beta (p - omega v)
@@ -688,7 +692,8 @@ __device__ __forceinline__ void hst(const HF &f, int V, int x, const cx<float> s
 }
 
 __global__ void __launch_bounds__(kRedBlock) k_lo_init_h(int V, HF r, HF rhat, HF p, HF v, float4 *xlo,
-                                                         ReduceScratch rs, SolverScalars *sc)
+                                                         ReduceScratch rs, SolverScalars *sc, StepReport *rep,
+                                                         unsigned long long seq)
 {
     float acc[1] = {0.f};
     for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < V; x += gridDim.x * blockDim.x) {
@@ -704,7 +709,7 @@ __global__ void __launch_bounds__(kRedBlock) k_lo_init_h(int V, HF r, HF rhat, H
         hst(v, V, x, z);
         P32::store_spinor(xlo, nullptr, V, x, z);
     }
-    grid_reduce<1>(acc, rs, rs.result, [=](double t, const double *) { init_update(t, sc); });
+    grid_reduce<1>(acc, rs, rs.result, [=](double t, const double *) { init_update(t, sc, rep, seq); });
 }
 
 __device__ __forceinline__ void body_lo_p_h(int V, HF r, HF v, HF p, const SolverScalars *sc)
@@ -1112,9 +1117,9 @@ cudaError_t lo_init(wc_lattice lat, SolverState &S, wc_field r, wc_field rhat, w
     const int V = lat->g.V;
     const long long n = 6LL * V;
     if (half_vectors(r))
-        k_lo_init_h<<<WC_GRID_SITES(V)>>>(V, hf(r), hf(rhat), hf(p), hf(v), f4(xlo), S.red, S.scal);
+        k_lo_init_h<<<WC_GRID_SITES(V)>>>(V, hf(r), hf(rhat), hf(p), hf(v), f4(xlo), S.red, S.scal, S.rep, S.seq);
     else
-        k_lo_init<<<WC_GRID(n)>>>(n, f4(r), f4(rhat), f4(p), f4(v), f4(xlo), S.red, S.scal);
+        k_lo_init<<<WC_GRID(n)>>>(n, f4(r), f4(rhat), f4(p), f4(v), f4(xlo), S.red, S.scal, S.rep, S.seq);
     return cudaGetLastError();
 }
 cudaError_t lo_p(wc_lattice lat, SolverState &S, wc_field r, wc_field v, wc_field p)

@@ -91,8 +91,8 @@ wc_status read_scalars(wc_lattice lat, SolverState &S)
 
 namespace {
 
-// Steps of a host-driven solve in the order they are queued, each reporting
-// into its slot of page-locked memory (no copy, event or synchronisation on
+// Steps of a host-driven solve (or its start) in the order they are queued,
+// each reporting into its slot of page-locked memory (no copy, event or synchronisation on
 // the stream, which would also break the chain of dependent launches).
 // ahead: the step after the one that is waited for is queued first.
 struct StepQueue {
@@ -678,17 +678,17 @@ static wc_status nested_inner(wc_lattice lat, SolverState &S, const wc_solve_par
     const int iters = p.inner_iters > 0 ? p.inner_iters : 100;
     st = check_cuda(lat, launch_copy(lat, w.r, u, 1.0, norm2_dev, 1, I.stream), "cast to unit norm");
     if (st == WC_OK) st = check_cuda(lat, track(I, TRACK_INNER, 0.0, itol * itol), "track");
-    if (st == WC_OK)
-        st = check_cuda(lat, lo_init(lat, I, w.r, w.rhat, w.p, w.v, w.xlo), "lo_init");
     if (st != WC_OK) return st;
-    // (a residual that is zero or not finite stops before the first step)
+    // the start reports as a step does: a residual that is zero or not finite
+    // ends the inner solve there (the step queued behind it does not run)
     StepQueue q{lat, I, p.precond == WC_PRECOND_NONE};
     StepReport h{};
-    for (int it = 0; it < iters; ++it) {
-        st = q.step([&] { return enqueue_lo_iteration(lat, I, p, kind, w); }, it + 1 < iters, &h);
-        if (st != WC_OK) return st;
-        if (h.action != ACT_NONE) break;
-    }
+    const auto step = [&] { return enqueue_lo_iteration(lat, I, p, kind, w); };
+    st = q.push([&] { return check_cuda(lat, lo_init(lat, I, w.r, w.rhat, w.p, w.v, w.xlo), "lo_init"); });
+    if (st == WC_OK && q.ahead) st = q.push(step);
+    if (st == WC_OK) st = q.pop(&h);
+    for (int it = 0; it < iters && st == WC_OK && h.action == ACT_NONE; ++it) st = q.step(step, it + 1 < iters, &h);
+    if (st != WC_OK) return st;
     // a blown-up inner solve (NaN) falls back to the identity preconditioner
     if (h.flags & FLAG_NAN)
         return check_cuda(lat, launch_copy(lat, uhat, u, 1.0, nullptr, 0, I.stream), "copy");

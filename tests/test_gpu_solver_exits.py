@@ -48,3 +48,37 @@ def test_a_returned_solve_has_left_its_stream(kw):
     if not kw.get("even_odd"):
         info = lat.solve(lat.field(0), b, tol=1e-10, max_restarts=1, check=False, **kw)
         assert info.status != 0 and s.query()
+
+
+NESTED = [dict(precond=p, krylov_prec=k, even_odd=e) for p in (0, 1) for k in (1, 2) for e in (False, True)]
+
+
+@pytest.mark.parametrize("kw", NESTED)
+def test_nested_solve_whose_half_step_is_exact(kw):
+    """M = 1 (kappa = 0, csw = 0) and a point source: the first half step is
+    exact, so the second inner solve starts from a zero vector and has to
+    return a zero correction."""
+    dims = (4, 4, 4, 6)
+    U = synth.exp_links(dims, 0.3, 311)
+    lat = make_lattice(dims, U, 0.0, 0.0, TBC)
+    src = np.zeros((int(np.prod(dims)), 4, 3), complex)
+    src[0, 1, 2] = 1.0
+    x = lat.field(0)
+    info = lat.solve(x, lat.field(0).load(src), tol=1e-10, solver=2, block=(2, 2, 2, 2), overlap=0, mr_iters=2,
+                     **kw)
+    assert info.status == 0
+    assert np.abs(x.store(np.zeros_like(src)) - src).max() <= 1e-10
+
+
+@pytest.mark.parametrize("kw", NESTED[::2])
+def test_nested_solve_on_links_with_a_nan(kw):
+    """The inner solves meet a NaN, their second one in its source: the solve
+    ends as WC_ERR_NAN (6)."""
+    dims = (4, 4, 4, 6)
+    U = synth.exp_links(dims, 0.3, 312)
+    U[0, 0, 1, 1] = np.nan      # (the third row is rebuilt from the other two)
+    lat = make_lattice(dims, U, 0.0, KAPPA, TBC)
+    src = synth.gaussian_source(dims, 313)
+    info = lat.solve(lat.field(0), lat.field(0).load(src), tol=1e-10, solver=2, check=False,
+                     block=(2, 2, 2, 2), overlap=0, mr_iters=2, **kw)
+    assert info.status == 6
