@@ -38,6 +38,7 @@ wc_status set_error(wc_lattice lat, wc_status st, const std::string &msg)
 wc_status check_cuda(wc_lattice lat, cudaError_t e, const char *what)
 {
     if (e == cudaSuccess) return WC_OK;
+    cudaGetLastError();   // reported here: not again by the next launch check
     return set_error(lat, WC_ERR_CUDA, std::string(what) + ": " + cudaGetErrorString(e));
 }
 
@@ -225,18 +226,6 @@ void free_gauge(GaugeStore &g)
     g = GaugeStore{};
 }
 
-void free_clover(CloverStore &c)
-{
-    cudaFree(c.c64);
-    cudaFree(c.cdf);
-    cudaFree(c.c32);
-    cudaFree(c.c16);
-    cudaFree(c.a32);
-    cudaFree(c.a16);
-    cudaFree(c.a16b);
-    c = CloverStore{};
-}
-
 wc_status need_staging(wc_lattice lat, size_t bytes)
 {
     if (lat->staging_bytes >= bytes) return WC_OK;
@@ -256,6 +245,18 @@ wc_status check_field(wc_lattice lat, wc_field f, const char *name)
 }
 
 }  // namespace
+
+void free_clover(CloverStore &c)
+{
+    cudaFree(c.c64);
+    cudaFree(c.cdf);
+    cudaFree(c.c32);
+    cudaFree(c.c16);
+    cudaFree(c.a32);
+    cudaFree(c.a16);
+    cudaFree(c.a16b);
+    c = CloverStore{};
+}
 
 // the FP32 and FP16 parts of a store of A
 wc_status alloc_clover_a(wc_lattice lat, CloverStore &c)

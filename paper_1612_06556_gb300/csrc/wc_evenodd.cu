@@ -1014,7 +1014,10 @@ wc_status build_clover_inverse(wc_lattice lat)
         } else if (st == WC_OK) {
             st = alloc_clover_a(lat, *c);
         }
-        if (st != WC_OK) return st;
+        if (st != WC_OK) {
+            free_clover(*c);   // c64 says that a store is complete
+            return st;
+        }
     }
     int *bad = nullptr;
     st = check_cuda(lat, cudaMalloc(&bad, sizeof(int)), "cudaMalloc");

@@ -177,6 +177,7 @@ cudaError_t launch_ras(wc_lattice lat, wc_field out, wc_field in, const wc_ras_p
                        cudaStream_t stream);
 
 wc_status alloc_clover_a(wc_lattice lat, CloverStore &c);
+void free_clover(CloverStore &c);
 // the clover term of lat's links into lat->clover (wc_clover.cu)
 cudaError_t launch_build_clover(wc_lattice lat, double csw, double kappa, cudaStream_t stream);
 

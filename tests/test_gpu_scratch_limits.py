@@ -1,0 +1,49 @@
+"""Calls that run out of device memory: the error, and the call after it."""
+import gc
+
+import numpy as np
+import pytest
+
+import synth
+from gpu_common import make_lattice, wc
+
+pytestmark = pytest.mark.gpu
+
+MB = 1 << 20
+
+
+def _leave(mbytes):
+    """A tensor that leaves about so much device memory free."""
+    import torch
+    gc.collect()
+    torch.cuda.empty_cache()
+    free = torch.cuda.mem_get_info()[0]
+    return torch.empty(free - mbytes * MB, dtype=torch.uint8, device="cuda")
+
+
+@pytest.mark.parametrize("left", [100, 300])
+def test_even_odd_call_after_one_that_ran_out_of_memory(left):
+    """At 16^3x32 the inverse clover term takes 208 MB and the parity-ordered
+    one 192 MB, 75 MB of each in its first array: with 100 MB left the second
+    array of the first store does not fit, with 300 MB that of the second.
+    The call reports it, and with memory free again the next one is right."""
+    import torch
+    dims, kappa, csw, tbc = (16, 16, 16, 32), 0.12, 1.0, -1
+    U = synth.pool_links(dims, 321)
+    src = synth.gaussian_source(dims, 322)
+    ref_lat = make_lattice(dims, U, csw, kappa, tbc)
+    f, g = ref_lat.field(0).load(src), ref_lat.field(0)
+    ref_lat.apply_schur(g, f)
+    ref = g.store(np.zeros_like(src))
+    ref_lat.close()
+    lat = make_lattice(dims, U, csw, kappa, tbc)
+    f, g = lat.field(0).load(src), lat.field(0)
+    lat.sync()
+    hog = _leave(left)
+    with pytest.raises(wc().WCError) as e:
+        lat.apply_schur(g, f)
+    assert e.value.status == 2
+    del hog
+    torch.cuda.empty_cache()
+    lat.apply_schur(g, f)
+    assert np.array_equal(g.store(np.zeros_like(src)), ref)
