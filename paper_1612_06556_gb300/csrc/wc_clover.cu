@@ -2,29 +2,28 @@
 //
 // Fhat_munu(x) = (1/8)[(Q - Q^+) - tr(Q - Q^+)/3], Q the sum of the four
 // plaquette leaves at x.  The four leaves that pass through one plaquette
-// are the same loop begun at its four corners, so each plaquette P of x is
-// formed once and its anti-Hermitian part X = P - P^+ (9 reals) carried to
-// the other corners:
-//   at x + mu        U_mu(x)^+ X U_mu(x)
-//   at x + nu        U_nu(x)^+ X U_nu(x)
-//   at x + mu + nu   U_nu(x+mu)^+ [U_mu(x)^+ X U_mu(x)] U_nu(x+mu)
-// A carry costs 144 FP64 operations (X U with an imaginary diagonal 90, the
-// upper triangle of U^+ (X U) 54), the plaquette 306: 738 per site and plane
-// against 12 products of 108 for the four leaves taken site by site.  The
+// are the same loop begun at its four corners.  With its two-link paths
+//   A = U_mu(x) U_nu(x+mu)         B = U_nu(x) U_mu(x+nu)
+//   C = U_nu(x+mu) U_mu(x+nu)^+    D = U_mu(x)^+ U_nu(x)
+// they are
+//   at x  A B^+     at x + mu + nu  B^+ A     at x + mu  C D^+     at x + nu  D^+ C
+// of which only the anti-Hermitian part X = P - P^+ (9 reals) is wanted: four
+// products of 108 FP64 operations and four X of 96 per plaquette, 816 a site and
+// plane, against 12 products of 108 for the four leaves taken site by site.
+// (Forming X once and carrying it to the other corners, U^+ X U, takes 738, but
+// U^+ U = 1 only as far as the links are unitary: for links rounded to FP32 the
+// term was off by 4e-9, and its rounding errors were a fifth larger.)  The
 // build is bound by the FP64 pipe (one warp instruction per 64 cycles on
-// each of its four units per SM).  A new configuration at 16^3x32 (links,
-// clover term, inverse, one FP64 Schur application, export): 4047 -> 1913 us
-// together with the inversion by 3x3 blocks; the leaves site by site were
-// 1929 us of it, the elimination of every block 1637 us.
+// each of its four units per SM); at 16^3x32 it took 1929 us site by site.
 //
-// k_leaves writes the four carried X per plaquette at the index of x, plane
+// k_leaves writes the four X per plaquette at the index of x, plane
 // by plane; k_gather adds the leaves that arrive at a site (fixed order)
 // and forms the clover entries; two planes per pass, since the entries need
 // the pairs (xy, zt), (yz, xt), (xz, yt).  The leaves of two planes are 576 B
 // a site, the size of the double-FP32 copy of the clover term, which is
 // written last and holds them until then.  One thread per
-// (site, plane) in k_leaves: six times as many warps as sites / 32, which
-// is what small lattices need to reach all FP64 units.
+// (site, plane, pair of leaves) in k_leaves: twelve times as many warps as
+// sites / 32, which is what small lattices need to reach all FP64 units.
 #include "wc_internal.cuh"
 
 namespace wc {
@@ -71,6 +70,16 @@ __device__ __forceinline__ M3 m3_mul(const M3 &a, const M3 &b)
     return r;
 }
 
+__device__ __forceinline__ M3 m3_dag(const M3 &a)
+{
+    M3 r;
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) r.m[i][j] = conj(a.m[j][i]);
+    return r;
+}
+
 // a * conj(b), accumulated
 __device__ __forceinline__ cx<double> mul_conj(cx<double> a, cx<double> b, cx<double> acc)
 {
@@ -104,42 +113,6 @@ __device__ __forceinline__ X3 anti_of_abdag(const M3 &a, const M3 &b)
         x.o[q] = u - conj(l);
     }
     return x;
-}
-
-// U^+ X U
-__device__ __forceinline__ X3 carry(const X3 &x, const M3 &u)
-{
-    M3 t;   // X U
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-        const cx<double> u0 = u.m[0][j], u1 = u.m[1][j], u2 = u.m[2][j];
-        cx<double> s = mkc(-x.d[0] * u0.im, x.d[0] * u0.re);
-        s = cfma(x.o[0], u1, s);
-        t.m[0][j] = cfma(x.o[1], u2, s);
-        s = mkc(-x.d[1] * u1.im, x.d[1] * u1.re);
-        s = cfma_conj(x.o[0], -u0, s);
-        t.m[1][j] = cfma(x.o[2], u2, s);
-        s = mkc(-x.d[2] * u2.im, x.d[2] * u2.re);
-        s = cfma_conj(x.o[1], -u0, s);
-        t.m[2][j] = cfma_conj(x.o[2], -u1, s);
-    }
-    X3 r;
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-        double s = 0.0;
-#pragma unroll
-        for (int k = 0; k < 3; ++k) s = fma(u.m[k][i].re, t.m[k][i].im, fma(-u.m[k][i].im, t.m[k][i].re, s));
-        r.d[i] = s;
-    }
-#pragma unroll
-    for (int q = 0; q < 3; ++q) {
-        const int i = q == 2 ? 1 : 0, j = q == 0 ? 1 : 2;
-        cx<double> s = mkc(0.0, 0.0);
-#pragma unroll
-        for (int k = 0; k < 3; ++k) s = cfma_conj(u.m[k][i], t.m[k][j], s);
-        r.o[q] = s;
-    }
-    return r;
 }
 
 // scratch of one plane: double [4 corners][9][V]
@@ -176,8 +149,9 @@ __device__ __forceinline__ int down(const Geom &g, int x, const int c[4], int mu
 }
 
 // Leaves of the plaquettes of plane (planes.x, planes.y) (blockIdx.y = 0) or
-// (planes.z, planes.w) (blockIdx.y = 1).  200 registers: ten warps per SM, two
-// or three per FP64 unit, whose 64-cycle issue they keep busy.
+// (planes.z, planes.w) (blockIdx.y = 1): A B^+ and B^+ A (blockIdx.z = 0), or C D^+
+// and D^+ C (blockIdx.z = 1).  The two pairs in one thread take 254 registers,
+// or 1.8 KB of spills at 168.
 __global__ void __launch_bounds__(64) k_leaves(Geom g, GaugeStore G, int4 planes, double *ws)
 {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
@@ -188,17 +162,16 @@ __global__ void __launch_bounds__(64) k_leaves(Geom g, GaugeStore G, int4 planes
     int c[4];
     site_coords(g, x, c);
     const int xm = up(g, x, c, mu), xn = up(g, x, c, nu);
-    const M3 um = load_u(G, V, mu, x), un = load_u(G, V, nu, x), un_m = load_u(G, V, nu, xm);
-    X3 a;
-    {
-        const M3 pa = m3_mul(um, un_m), pb = m3_mul(un, load_u(G, V, mu, xn));
-        a = anti_of_abdag(pa, pb);
+    M3 a, b;
+    if (blockIdx.z == 0) {
+        a = m3_mul(load_u(G, V, mu, x), load_u(G, V, nu, xm));
+        b = m3_mul(load_u(G, V, nu, x), load_u(G, V, mu, xn));
+    } else {
+        a = m3_mul(load_u(G, V, nu, xm), m3_dag(load_u(G, V, mu, xn)));
+        b = m3_mul(m3_dag(load_u(G, V, mu, x)), load_u(G, V, nu, x));
     }
-    store_x(w, V, x, a);
-    store_x(w + (size_t)18 * V, V, x, carry(a, un));
-    a = carry(a, um);
-    store_x(w + (size_t)9 * V, V, x, a);
-    store_x(w + (size_t)27 * V, V, x, carry(a, un_m));
+    store_x(w + (size_t)(blockIdx.z == 0 ? 0 : 9) * V, V, x, anti_of_abdag(a, b));
+    store_x(w + (size_t)(blockIdx.z == 0 ? 27 : 18) * V, V, x, anti_of_abdag(m3_dag(b), m3_dag(a)));
 }
 
 // 8 Fhat of plane (mu, nu) at x from its leaves
@@ -320,7 +293,7 @@ cudaError_t launch_build_clover(wc_lattice lat, double csw, double kappa, cudaSt
     double *ws = reinterpret_cast<double *>(lat->clover.cdf);
     const double f = csw * kappa / 8.0;
     const int4 pair[3] = {make_int4(0, 1, 2, 3), make_int4(1, 2, 0, 3), make_int4(0, 2, 1, 3)};
-    const dim3 gl((g.V + 63) / 64, 2), gg((g.V + 127) / 128), gs((g.V + 127) / 128, 2);
+    const dim3 gl((g.V + 63) / 64, 2, 2), gg((g.V + 127) / 128), gs((g.V + 127) / 128, 2);
     for (int s = 0; s < 3; ++s) {
         k_leaves<<<gl, 64, 0, stream>>>(g, lat->gauge, pair[s], ws);
         if (s == 0) k_gather<0><<<gg, 128, 0, stream>>>(g, lat->clover, pair[s], ws, f);

@@ -69,3 +69,19 @@ def test_clover_block_beside_three_zero_modes_is_inverted():
     fi, fo = lat.field(0).load(psi), lat.field(0)
     lat.apply_schur(fo, fi)
     assert_elementwise(fo.store(np.zeros_like(psi)), EvenOdd(DIMS, -1, kappa, U, op.T).schur(psi), 1e-12 * cond)
+
+
+@pytest.mark.parametrize("dims", [(2, 2, 2, 2), (3, 4, 5, 2), (4, 4, 4, 6)])
+def test_clover_term_of_links_rounded_to_fp32(dims):
+    """Links kept in FP32, as configurations often are: unitary to 1e-7 only.
+    The clover term is the one of these links (two rows as given, the third
+    their cross product, as the library and here the oracle have it), not
+    one that assumes U^+ U = 1: FP64 tolerance."""
+    csw, kappa, tbc = 1.3, 0.12, -1
+    U = synth.haar_links(dims, 341).astype(np.complex64).astype(complex)
+    U[..., 2, :] = np.conj(np.cross(U[..., 0, :], U[..., 1, :]))
+    lat = make_lattice(dims, U, csw, kappa, tbc)
+    psi = synth.gaussian_source(dims, 342)
+    fi, fo = lat.field(0).load(psi), lat.field(0)
+    lat.apply_M(fo, fi)
+    assert_elementwise(fo.store(np.zeros_like(psi)), oracle.apply_M(dims, tbc, kappa, csw, U, psi), 1e-12)
