@@ -869,7 +869,7 @@ struct HalfSite<P32> {
         const float4 *p = static_cast<const float4 *>(d) + (size_t)3 * h * V + x;
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
-            const float4 w = __ldg(p + (size_t)q * V);
+            const float4 w = p[(size_t)q * V];
             s[2 * q] = mkc(w.x, w.y);
             s[2 * q + 1] = mkc(w.z, w.w);
         }
@@ -901,9 +901,9 @@ struct HalfSite<P16> {
     static __device__ __forceinline__ void load(const void *d, const float *nrm, int V, int x, int h, cx<float> s[6])
     {
         const uint4 *p = static_cast<const uint4 *>(d) + x;
-        const float sc = __ldg(nrm + x);
-        const uint4 a = __ldg(p + (h ? (size_t)2 * V : 0));
-        const uint2 b = __ldg(reinterpret_cast<const uint2 *>(p + V) + h);
+        const float sc = nrm[x];
+        const uint4 a = p[h ? (size_t)2 * V : 0];
+        const uint2 b = reinterpret_cast<const uint2 *>(p + V)[h];
         const unsigned w[6] = {h ? b.x : a.x, h ? b.y : a.y, h ? a.x : a.z, h ? a.y : a.w, h ? a.z : b.x, h ? a.w : b.y};
 #pragma unroll
         for (int k = 0; k < 6; ++k) s[k] = sc * h2c(w[k]);
@@ -939,7 +939,7 @@ __global__ void __launch_bounds__(kRedBlock) k_refresh_tail(int V, const double2
             double2 bv[6], rv[6];
 #pragma unroll
             for (int k = 0; k < 6; ++k) {
-                bv[k] = __ldg(b + at + (size_t)k * V);
+                bv[k] = b[at + (size_t)k * V];
                 rv[k] = r[at + (size_t)k * V];
             }
             HalfSite<PL>::load(rhat, rhat_n, V, x, h, hat);

@@ -205,6 +205,11 @@ struct CloverStore {
 // completed and its writes are visible.  launch_dependents lets the next
 // such kernel start once every CTA of this grid is running.  Both are no-ops
 // for kernels launched without the attribute.
+//
+// Vectors are read by ordinary loads: a dependent is on the SMs while the
+// kernel before it writes its input, and the non-coherent path (__ldg) is for
+// data that nothing writes in a kernel's whole lifetime.  Links and clover
+// term, which no kernel of a solve writes, keep it.
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void griddep_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;"); }
 
@@ -293,7 +298,7 @@ struct P64 {
         const double2 *p = static_cast<const double2 *>(d);
 #pragma unroll
         for (int k = 0; k < 12; ++k) {
-            double2 v = __ldg(p + (size_t)k * V + x);
+            double2 v = p[(size_t)k * V + x];
             s[k] = {v.x, v.y};
         }
     }
@@ -351,7 +356,7 @@ struct P32 {
         const float4 *p = static_cast<const float4 *>(d);
 #pragma unroll
         for (int j = 0; j < 6; ++j) {
-            float4 v = __ldg(p + (size_t)j * V + x);
+            float4 v = p[(size_t)j * V + x];
             s[2 * j] = {v.x, v.y};
             s[2 * j + 1] = {v.z, v.w};
         }
@@ -370,9 +375,8 @@ struct P32 {
         for (int j = 0; j < 6; ++j)
             p[(size_t)j * V + x] = make_float4(s[2 * j].re, s[2 * j].im, s[2 * j + 1].re, s[2 * j + 1].im);
     }
-    // s as a store_spinor followed by a load_spinor returns it (computed in
-    // registers: load_spinor reads through the non-coherent path, which need
-    // not see a write of the same kernel)
+    // s as a store_spinor followed by a load_spinor returns it (without the way
+    // through memory)
     static __device__ __forceinline__ void as_stored(cx<float> s[12]) {}
     static __device__ __forceinline__ void load_link(const GaugeStore &g, int V, int mu, int x,
                                                      cx<float> a[6], cx<float> c[3])
@@ -413,7 +417,7 @@ struct PDF {
         const double2 *p = static_cast<const double2 *>(d);
 #pragma unroll
         for (int k = 0; k < 12; ++k) {
-            const double2 v = __ldg(p + (size_t)k * V + x);
+            const double2 v = p[(size_t)k * V + x];
             s[k] = {df_from_double(v.x), df_from_double(v.y)};
         }
     }
@@ -467,22 +471,22 @@ struct P16 {
         const uint4 *p = static_cast<const uint4 *>(d);
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
-            uint4 v = __ldg(p + (size_t)j * V + x);
+            uint4 v = p[(size_t)j * V + x];
             s[4 * j] = h2c(v.x);
             s[4 * j + 1] = h2c(v.y);
             s[4 * j + 2] = h2c(v.z);
             s[4 * j + 3] = h2c(v.w);
         }
-        return __ldg(nrm + x);
+        return nrm[x];
     }
     static __device__ __forceinline__ void load_spinor(const void *d, const float *nrm, int V, int x,
                                                        cx<float> s[12])
     {
         const uint4 *p = static_cast<const uint4 *>(d);
-        const float sc = __ldg(nrm + x);
+        const float sc = nrm[x];
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
-            uint4 v = __ldg(p + (size_t)j * V + x);
+            uint4 v = p[(size_t)j * V + x];
             s[4 * j] = sc * h2c(v.x);
             s[4 * j + 1] = sc * h2c(v.y);
             s[4 * j + 2] = sc * h2c(v.z);

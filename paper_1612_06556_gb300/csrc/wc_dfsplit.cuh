@@ -131,8 +131,8 @@ __device__ __forceinline__ z2 finish(Sum t)
 template <bool SPLIT>
 __device__ __forceinline__ z2 load(const void *f, int V, int k, int y)
 {
-    if (SPLIT) return of4(__ldg(static_cast<const float4 *>(f) + (size_t)k * V + y));
-    return of_double(__ldg(static_cast<const double2 *>(f) + (size_t)k * V + y));
+    if (SPLIT) return of4(static_cast<const float4 *>(f)[(size_t)k * V + y]);
+    return of_double(static_cast<const double2 *>(f)[(size_t)k * V + y]);
 }
 
 // h = two-spinor of (1 + S g_mu) psi; a, b: the spins that give h0 and h1 by

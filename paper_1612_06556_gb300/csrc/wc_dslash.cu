@@ -149,7 +149,7 @@ __global__ void __launch_bounds__(kSplit64 * kSplit64Sites, 3)
         const double2 *p = static_cast<const double2 *>(in) + (size_t)(w >> 1) * 6 * g.V + x;
 #pragma unroll
         for (int k = 0; k < 6; ++k) {
-            const double2 a = __ldg(p + (size_t)k * g.V);
+            const double2 a = p[(size_t)k * g.V];
             v[k] = mkc(a.x, a.y);
         }
         clover_rows64(C, g.V, x, w, v, y);
@@ -188,7 +188,7 @@ __global__ void __launch_bounds__(kSplit64 * kSplit64Sites, 3)
         const double2 *p = static_cast<const double2 *>(in) + (size_t)(w >> 1) * 6 * g.V + x;
 #pragma unroll
         for (int k = 0; k < 6; ++k) {
-            const double2 b = __ldg(p + (size_t)k * g.V);
+            const double2 b = p[(size_t)k * g.V];
             v[k] = mkc(b.x, b.y);
         }
         clover_rows64(C, g.V, x, w, v, y);
@@ -198,7 +198,7 @@ __global__ void __launch_bounds__(kSplit64 * kSplit64Sites, 3)
             const cx<double> h = sum_split64(sm, 3 * w + r, s);
             y[r] = mkc(fma(-kappa, h.re, y[r].re), fma(-kappa, h.im, y[r].im));
             static_cast<double2 *>(out)[k] = make_double2(y[r].re, y[r].im);
-            const double2 b = __ldg(static_cast<const double2 *>(ss.with) + k);
+            const double2 b = static_cast<const double2 *>(ss.with)[k];
             a[r] = mkc(b.x, b.y);
         }
         add_step_sums<OMEGA, 3>(y, a, acc);
@@ -235,7 +235,7 @@ __global__ void __launch_bounds__(kSplit64 * kSplit64Sites, dfs::kCtas)
         const double2 *p = static_cast<const double2 *>(in) + (size_t)(w >> 1) * 6 * g.V + x;
 #pragma unroll
         for (int k = 0; k < 6; ++k) {
-            const double2 a = __ldg(p + (size_t)k * g.V);
+            const double2 a = p[(size_t)k * g.V];
             v[k] = mkc(a.x, a.y);
         }
         clover_rows64(C, g.V, x, w, v, y);

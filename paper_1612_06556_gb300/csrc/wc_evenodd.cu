@@ -428,7 +428,7 @@ __global__ void __launch_bounds__(kSplit64 * kSplit64Sites, 3)
             } else if (MODE == 1) {
                 v[r] = beta * h;
             } else {
-                const double2 a = __ldg(vin + (size_t)k * Vh + i);
+                const double2 a = vin[(size_t)k * Vh + i];
                 v[r] = MODE == 4 ? mkc(a.x, a.y) : mkc(fma(beta, h.re, a.x), fma(beta, h.im, a.y));
             }
         }
@@ -461,7 +461,7 @@ __global__ void __launch_bounds__(kSplit64 * kSplit64Sites, 3)
         const double2 *q = vin + (size_t)(w >> 1) * 6 * Vh + i;
 #pragma unroll
         for (int k = 0; k < 6; ++k) {
-            const double2 a = __ldg(q + (size_t)k * Vh);
+            const double2 a = q[(size_t)k * Vh];
             vb[k] = mkc(a.x, a.y);
         }
         clover_rows64(C, g.V, pos, w, vb, o);
@@ -544,7 +544,7 @@ __global__ void __launch_bounds__(kSplit64 * kSplit64Sites, 3)
         const double2 *q = vin + (size_t)(w >> 1) * 6 * Vh + i;
 #pragma unroll
         for (int k = 0; k < 6; ++k) {
-            const double2 b = __ldg(q + (size_t)k * Vh);
+            const double2 b = q[(size_t)k * Vh];
             vb[k] = mkc(b.x, b.y);
         }
         clover_rows64(C, g.V, wc_idx(p * Vh + i, g.V), w, vb, o);
@@ -553,7 +553,7 @@ __global__ void __launch_bounds__(kSplit64 * kSplit64Sites, 3)
             const size_t k = (size_t)(3 * w + r) * Vh + i;
             o[r] = o[r] + beta * sum_split64(sm, 3 * w + r, s);
             out[k] = make_double2(o[r].re, o[r].im);
-            const double2 b = __ldg(static_cast<const double2 *>(ss.with) + k);
+            const double2 b = static_cast<const double2 *>(ss.with)[k];
             a[r] = mkc(b.x, b.y);
         }
         add_step_sums<OMEGA, 3>(o, a, acc);
@@ -563,15 +563,21 @@ __global__ void __launch_bounds__(kSplit64 * kSplit64Sites, 3)
 
 // An FP64 half field as z2 values (wc_dfsplit.cuh), for the hops of the next
 // pass: each of its spinors is read eight times.
-__global__ void __launch_bounds__(256) k_to_df(long long n, const double2 *__restrict__ in, float4 *__restrict__ out,
-                                               const int *skip)
+__global__ void __launch_bounds__(256) k_to_df(long long n, const double2 *in, float4 *out, const int *skip)
 {
     griddep_wait();
     griddep_launch_dependents();
     if (skip && *skip) return;
-#pragma unroll 4
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        out[i] = dfs::to4(dfs::of_double(in[i]));
+    const long long step = (long long)gridDim.x * blockDim.x;
+    // four reads in flight
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += 4 * step) {
+        double2 v[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[k] = i + k * step < n ? in[i + k * step] : make_double2(0.0, 0.0);
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (i + k * step < n) out[i + k * step] = dfs::to4(dfs::of_double(v[k]));
+    }
 }
 
 // k_eo of FP64 fields in double-FP32 arithmetic, on four warps per 32 sites as
@@ -609,7 +615,7 @@ __global__ void __launch_bounds__(kSplit64 * kSplit64Sites, dfs::kCtas)
                 dfs::Sum t = dfs::first_term(bt, h);
                 v[r] = dfs::finish(t);
             } else {
-                const z2 a = dfs::of_double(__ldg(vin + (size_t)k * Vh + i));
+                const z2 a = dfs::of_double(vin[(size_t)k * Vh + i]);
                 dfs::Sum t = dfs::start(a);
                 if (MODE != 4) dfs::add_term(t, bt, h);
                 v[r] = dfs::finish(t);
@@ -643,7 +649,7 @@ __global__ void __launch_bounds__(kSplit64 * kSplit64Sites, dfs::kCtas)
         if (!valid) return;
         const double2 *q = vin + (size_t)(w >> 1) * 6 * Vh + i;
 #pragma unroll
-        for (int k = 0; k < 6; ++k) vb[k] = dfs::of_double(__ldg(q + (size_t)k * Vh));
+        for (int k = 0; k < 6; ++k) vb[k] = dfs::of_double(q[(size_t)k * Vh]);
         dfs::Sum y[3] = {dfs::start(v[0]), dfs::start(v[1]), dfs::start(v[2])};
         dfs::clover_rows(C, g.V, pos, w, vb, y);
         const z2 o[3] = {dfs::finish(y[0]), dfs::finish(y[1]), dfs::finish(y[2])};

@@ -64,8 +64,15 @@ __device__ __forceinline__ void hop_mrhs(const Stage<S> &st, int s, const float4
     constexpr int lam = FWD ? MU : 4 + MU;
     cx<float> h[6], u[6], r2[3];
     {
+        // never a programmatic dependent, so that the read-only path is open:
+        // 410 us for 12 fields at 24^3x32, 417 by ordinary loads
         cx<float> p[12];
-        P32::load_spinor(in, nullptr, V, y, p);
+#pragma unroll
+        for (int j = 0; j < 6; ++j) {
+            const float4 v = __ldg(in + (size_t)j * V + y);
+            p[2 * j] = mkc(v.x, v.y);
+            p[2 * j + 1] = mkc(v.z, v.w);
+        }
         project<MU, SG>(p, h);
     }
     if (MU == 3 && ph != 1.f) {

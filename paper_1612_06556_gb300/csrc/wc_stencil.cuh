@@ -450,9 +450,9 @@ __device__ __forceinline__ void hop_dir_h16(const Geom &g, const GaugeStore &U, 
         const bool wrap = dir == 0 ? c[MU] == L - 1 : c[MU] == 0;
         const int y = wc_idx(dir == 0 ? (wrap ? x - (L - 1) * st : x + st) : (wrap ? x + (L - 1) * st : x - st), g.V);
         const int z = sidx(y);
-        const uint4 s0 = __ldg(ps + z), s1 = __ldg(ps + (size_t)Vin + z), s2 = __ldg(ps + 2 * (size_t)Vin + z);
+        const uint4 s0 = ps[z], s1 = ps[(size_t)Vin + z], s2 = ps[2 * (size_t)Vin + z];
         const unsigned w[12] = {s0.x, s0.y, s0.z, s0.w, s1.x, s1.y, s1.z, s1.w, s2.x, s2.y, s2.z, s2.w};
-        const float coef = ((MU == 3 && wrap) ? k * (float)g.tbc : k) * __ldg(in_nrm + z);
+        const float coef = ((MU == 3 && wrap) ? k * (float)g.tbc : k) * in_nrm[z];
         cx<float> h[6], u[6], r2[3], wv[6];
         if (dir == 0) {
             project_h16<MU, SF>(w, h);
@@ -698,8 +698,8 @@ __device__ __forceinline__ void apply_site_at(const Geom &g, int x, const GaugeS
         // clover products from the stored halves, the centre scale applied
         // once to the result
         const uint4 *ps = static_cast<const uint4 *>(in);
-        const uint4 s0 = __ldg(ps + x), s1 = __ldg(ps + (size_t)g.V + x), s2 = __ldg(ps + 2 * (size_t)g.V + x);
-        const float sc = __ldg(in_nrm + x);
+        const uint4 s0 = ps[x], s1 = ps[(size_t)g.V + x], s2 = ps[2 * (size_t)g.V + x];
+        const float sc = in_nrm[x];
         const unsigned v0[6] = {s0.x, s0.y, s0.z, s0.w, s1.x, s1.y};
         const unsigned v1[6] = {s1.z, s1.w, s2.x, s2.y, s2.z, s2.w};
         clover_block_h(C, g.V, x, 0, v0, acc);
