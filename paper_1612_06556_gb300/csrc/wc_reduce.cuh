@@ -75,16 +75,18 @@ __device__ __forceinline__ void grid_reduce(T (&acc)[M], const ReduceScratch &rs
     __syncthreads();
     if (wid == 0) {
         const T u = block_sums(sm);
-        if (lane < M * W && lane % W == 0) {
-            rs.partials[(size_t)blockIdx.x * 4 + lane / W] = (double)u;
+        if (lane < M * W && lane % W == 0) rs.partials[(size_t)blockIdx.x * 4 + lane / W] = (double)u;
+        __syncwarp();
+        // the fences stand between the other lanes' partials and this
+        // lane's ticket, and between the ticket and the block's reads
+        if (lane == 0) {
+            __threadfence();
+            last = atomicAdd(rs.ticket, 1u) == gridDim.x - 1;
             __threadfence();
         }
-        __syncwarp();
-        if (lane == 0) last = atomicAdd(rs.ticket, 1u) == gridDim.x - 1;
     }
     __syncthreads();
     if (!last) return;
-    __threadfence();
     if constexpr (W < N) {
         // a single warp: all sums in one loop, so that their loads overlap
         static_assert(W == 1, "one warp, or one for each sum");
