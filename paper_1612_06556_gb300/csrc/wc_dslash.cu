@@ -139,11 +139,16 @@ __global__ void __launch_bounds__(kSplit64 * kSplit64Sites, 3)
     if (valid) {
         int c[4];
         site_coords_fast(g, x, c);
-        hop_split64<KIND == 1 ? +1 : -1>(g, U, in, g.V, x, c, sm, w, s, [](int y) { return y; });
+        hop_split64<KIND == 1 ? +1 : -1, KIND == 2>(g, U, in, g.V, x, c, sm, w, s, [](int y) { return y; });
     }
     __syncthreads();
     if (!valid) return;
     cx<double> y[3];
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+        y[r] = sum_split64(sm, 3 * w + r, s);
+        if (KIND != 2) y[r] = -kappa * y[r];
+    }
     if (KIND != 2) {
         cx<double> v[6];
         const double2 *p = static_cast<const double2 *>(in) + (size_t)(w >> 1) * 6 * g.V + x;
@@ -156,11 +161,7 @@ __global__ void __launch_bounds__(kSplit64 * kSplit64Sites, 3)
     }
     double2 *o = static_cast<double2 *>(out) + (size_t)3 * w * g.V + x;
 #pragma unroll
-    for (int r = 0; r < 3; ++r) {
-        const cx<double> h = sum_split64(sm, 3 * w + r, s);
-        o[(size_t)r * g.V] = KIND == 2 ? make_double2(h.re, h.im)
-                                       : make_double2(fma(-kappa, h.re, y[r].re), fma(-kappa, h.im, y[r].im));
-    }
+    for (int r = 0; r < 3; ++r) o[(size_t)r * g.V] = make_double2(y[r].re, y[r].im);
 }
 
 // k_apply_split64 as the operator of a solver step: the pass also forms the
@@ -191,12 +192,12 @@ __global__ void __launch_bounds__(kSplit64 * kSplit64Sites, 3)
             const double2 b = p[(size_t)k * g.V];
             v[k] = mkc(b.x, b.y);
         }
+#pragma unroll
+        for (int r = 0; r < 3; ++r) y[r] = -kappa * sum_split64(sm, 3 * w + r, s);
         clover_rows64(C, g.V, x, w, v, y);
 #pragma unroll
         for (int r = 0; r < 3; ++r) {
             const size_t k = (size_t)(3 * w + r) * g.V + x;
-            const cx<double> h = sum_split64(sm, 3 * w + r, s);
-            y[r] = mkc(fma(-kappa, h.re, y[r].re), fma(-kappa, h.im, y[r].im));
             static_cast<double2 *>(out)[k] = make_double2(y[r].re, y[r].im);
             const double2 b = static_cast<const double2 *>(ss.with)[k];
             a[r] = mkc(b.x, b.y);
@@ -229,7 +230,7 @@ __global__ void __launch_bounds__(kSplit64 * kSplit64Sites, dfs::kCtas)
     }
     __syncthreads();
     if (!valid) return;
-    cx<double> y[3];
+    cx<double> y[3] = {};
     if (KIND != 2) {
         cx<double> v[6];
         const double2 *p = static_cast<const double2 *>(in) + (size_t)(w >> 1) * 6 * g.V + x;

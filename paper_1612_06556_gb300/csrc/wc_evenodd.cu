@@ -464,14 +464,14 @@ __global__ void __launch_bounds__(kSplit64 * kSplit64Sites, 3)
             const double2 a = q[(size_t)k * Vh];
             vb[k] = mkc(a.x, a.y);
         }
-        clover_rows64(C, g.V, pos, w, vb, o);
-#pragma unroll
-        for (int r = 0; r < 3; ++r) o[r] = o[r] + v[r];
-        store(out, o);
+        clover_rows64(C, g.V, pos, w, vb, v);
+        store(out, v);
         return;
     }
     share(v);
     if (valid) {
+#pragma unroll
+        for (int r = 0; r < 3; ++r) o[r] = mkc(0.0, 0.0);
         clover_rows64(Ci, g.V, pos, w, vb, o);
         store(out, o);
     }
@@ -479,10 +479,10 @@ __global__ void __launch_bounds__(kSplit64 * kSplit64Sites, 3)
         __syncthreads();   // vb is read
         share(o);
         if (valid) {
-            cx<double> y[3];
+            cx<double> y[3] = {times_iq<2>(v[0]), times_iq<2>(v[1]), times_iq<2>(v[2])};   // A x_o - v
             clover_rows64(C, g.V, pos, w, vb, y);
 #pragma unroll
-            for (int r = 0; r < 3; ++r) y[r] = v[r] - y[r];
+            for (int r = 0; r < 3; ++r) y[r] = times_iq<2>(y[r]);
             store(out2, y);
         }
     }
@@ -547,11 +547,12 @@ __global__ void __launch_bounds__(kSplit64 * kSplit64Sites, 3)
             const double2 b = q[(size_t)k * Vh];
             vb[k] = mkc(b.x, b.y);
         }
+#pragma unroll
+        for (int r = 0; r < 3; ++r) o[r] = beta * sum_split64(sm, 3 * w + r, s);
         clover_rows64(C, g.V, wc_idx(p * Vh + i, g.V), w, vb, o);
 #pragma unroll
         for (int r = 0; r < 3; ++r) {
             const size_t k = (size_t)(3 * w + r) * Vh + i;
-            o[r] = o[r] + beta * sum_split64(sm, 3 * w + r, s);
             out[k] = make_double2(o[r].re, o[r].im);
             const double2 b = static_cast<const double2 *>(ss.with)[k];
             a[r] = mkc(b.x, b.y);

@@ -476,7 +476,13 @@ __device__ __forceinline__ void hop_dir_h16(const Geom &g, const GaugeStore &U, 
 // w_b, whose sum runs on through both products, and the upper ones from
 // w_f + w_b = 2 w_f - d: 180 instructions a direction, the hopping
 // coefficient applied once to the sum of all four, against 236 for hops
-// taken one at a time with a coefficient each.
+// taken one at a time with a coefficient each.  The extra rounding of 2 w_f - d
+// is below those of the clover term's rows, once these end with their
+// largest term (clover_rows64_at): error of M against 64 bits 3.6 -> 3.2e-16, of
+// M^ 2.9 -> 2.5e-16.
+// Where the hops are the result (SEP) the two products are kept apart, 192
+// instructions: error of H 6.76e-16, 6.79e-16 with the hops one at a time, 6.80e-16
+// by the difference (H at 16^3x32 197 us, 183 by the difference).
 
 // a with the sign bit flipped by mask (0 or 0x80000000): no FP64 instruction
 __device__ __forceinline__ double flip(double a, unsigned mask)
@@ -499,7 +505,7 @@ __device__ __forceinline__ cx<double> times_iq(cx<double> a)
 // t = the upper, lo = the lower spins (components 0..5 and 6..11) of
 // W_f (1 + SF g_MU) in(x+mu) + W_b (1 - SF g_MU) in(x-mu), the neighbour
 // spinors read at sidx(y) of a field of Vin sites
-template <int MU, int SF, class SiteIdx>
+template <int MU, int SF, bool SEP, class SiteIdx>
 __device__ __forceinline__ void hop_pair64(const Geom &g, const GaugeStore &U, const void *in, int Vin, int x,
                                            const int c[4], cx<double> t[6], cx<double> lo[6], SiteIdx sidx)
 {
@@ -541,13 +547,21 @@ __device__ __forceinline__ void hop_pair64(const Geom &g, const GaugeStore &U, c
         for (int s = 0; s < 2; ++s)
 #pragma unroll
             for (int i = 0; i < 3; ++i) {
-                cx<double> y = cfma_conj(u[i], -h[3 * s], t[3 * s + i]);
-                y = cfma_conj(u[3 + i], -h[3 * s + 1], y);
-                d[3 * s + i] = cfma_conj(r2[i], -h[3 * s + 2], y);
+                cx<double> y = SEP ? cmul_conj(u[i], h[3 * s]) : cfma_conj(u[i], -h[3 * s], t[3 * s + i]);
+                y = cfma_conj(u[3 + i], SEP ? h[3 * s + 1] : -h[3 * s + 1], y);
+                d[3 * s + i] = cfma_conj(r2[i], SEP ? h[3 * s + 2] : -h[3 * s + 2], y);
             }
     }
 #pragma unroll
-    for (int k = 0; k < 6; ++k) t[k] = mkc(fma(2.0, t[k].re, -d[k].re), fma(2.0, t[k].im, -d[k].im));
+    for (int k = 0; k < 6; ++k) {
+        if (SEP) {   // d holds w_b
+            const cx<double> w = d[k];
+            d[k] = t[k] - w;
+            t[k] = t[k] + w;
+        } else {
+            t[k] = mkc(fma(2.0, t[k].re, -d[k].re), fma(2.0, t[k].im, -d[k].im));
+        }
+    }
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
         const cx<double> d0 = d[k], d1 = d[3 + k];
@@ -578,15 +592,15 @@ constexpr int kSplit64 = 4;
 constexpr int kSplit64Sites = 32;
 using Split64Mem = double2[kSplit64][12][kSplit64Sites];
 
-template <int SF, class SiteIdx>
+template <int SF, bool SEP = false, class SiteIdx>
 __device__ __forceinline__ void hop_split64(const Geom &g, const GaugeStore &U, const void *in, int Vin, int x,
                                             const int c[4], Split64Mem &sm, int w, int s, SiteIdx sidx)
 {
     cx<double> t[6], lo[6];
-    if (w == 0) hop_pair64<0, SF>(g, U, in, Vin, x, c, t, lo, sidx);
-    else if (w == 1) hop_pair64<1, SF>(g, U, in, Vin, x, c, t, lo, sidx);
-    else if (w == 2) hop_pair64<2, SF>(g, U, in, Vin, x, c, t, lo, sidx);
-    else hop_pair64<3, SF>(g, U, in, Vin, x, c, t, lo, sidx);
+    if (w == 0) hop_pair64<0, SF, SEP>(g, U, in, Vin, x, c, t, lo, sidx);
+    else if (w == 1) hop_pair64<1, SF, SEP>(g, U, in, Vin, x, c, t, lo, sidx);
+    else if (w == 2) hop_pair64<2, SF, SEP>(g, U, in, Vin, x, c, t, lo, sidx);
+    else hop_pair64<3, SF, SEP>(g, U, in, Vin, x, c, t, lo, sidx);
 #pragma unroll
     for (int k = 0; k < 6; ++k) {
         sm[w][k][s] = make_double2(t[k].re, t[k].im);
@@ -601,8 +615,9 @@ __device__ __forceinline__ cx<double> sum_split64(const Split64Mem &sm, int k, i
     return mkc((a.x + b.x) + (c.x + d.x), (a.y + b.y) + (c.y + d.y));
 }
 
-// rows I0 .. I0 + 2 of y = B v, clover block b of the packed FP64 store at
-// position x
+// rows I0 .. I0 + 2 of y + B v, clover block b of the packed FP64 store at
+// position x.  The diagonal, the largest term, comes last: the roundings of the
+// sum before it are those of its smaller size.
 template <int I0>
 __device__ __forceinline__ void clover_rows64_at(const CloverStore &C, int V, int x, int b, const cx<double> v[6],
                                                  cx<double> y[3])
@@ -617,8 +632,6 @@ __device__ __forceinline__ void clover_rows64_at(const CloverStore &C, int V, in
         d[0] = a.y, d[1] = e.x, d[2] = e.y;
     }
 #pragma unroll
-    for (int r = 0; r < 3; ++r) y[r] = d[r] * v[I0 + r];
-#pragma unroll
     for (int i = 1; i < 6; ++i)
 #pragma unroll
         for (int j = 0; j < i; ++j) {
@@ -629,6 +642,8 @@ __device__ __forceinline__ void clover_rows64_at(const CloverStore &C, int V, in
             if (row) y[i - I0] = cfma(l, v[j], y[i - I0]);
             if (col) y[j - I0] = cfma_conj(l, v[i], y[j - I0]);
         }
+#pragma unroll
+    for (int r = 0; r < 3; ++r) y[r] = mkc(fma(d[r], v[I0 + r].re, y[r].re), fma(d[r], v[I0 + r].im, y[r].im));
 }
 
 // rows 3 w .. 3 w + 2 of the 12 (w uniform in the warp)
