@@ -230,7 +230,7 @@ __global__ void __launch_bounds__(kSplit64 * kSplit64Sites, dfs::kCtas)
     }
     __syncthreads();
     if (!valid) return;
-    cx<double> y[3] = {};
+    cx<double> y[3];
     if (KIND != 2) {
         cx<double> v[6];
         const double2 *p = static_cast<const double2 *>(in) + (size_t)(w >> 1) * 6 * g.V + x;
@@ -239,7 +239,7 @@ __global__ void __launch_bounds__(kSplit64 * kSplit64Sites, dfs::kCtas)
             const double2 a = p[(size_t)k * g.V];
             v[k] = mkc(a.x, a.y);
         }
-        clover_rows64(C, g.V, x, w, v, y);
+        clover_rows64<true>(C, g.V, x, w, v, y);
     }
     double2 *o = static_cast<double2 *>(out) + (size_t)3 * w * g.V + x;
 #pragma unroll
