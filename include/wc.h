@@ -180,7 +180,7 @@ wc_status wc_set_stream(wc_lattice lat, void *cuda_stream);
  * updates, true residuals, even-odd source preparation and
  * reconstruction).  WC_ARITH_F64 (the default): FP64 arithmetic.
  * WC_ARITH_DF32: double-FP32 arithmetic -- each value is carried as the
- * unevaluated sum of two floats (about 47 significant bits) and the
+ * unevaluated sum of two floats (about 48 significant bits) and the
  * operations run on the FP32 pipes, which on GB300 are 64 times faster than
  * its FP64 pipe.  Storage stays FP64.  Results agree with FP64 arithmetic to
  * ~1e-14 relative to the largest input; inputs with |x| < 2^-103 keep only

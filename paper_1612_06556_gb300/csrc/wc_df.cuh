@@ -3,7 +3,7 @@
 // GB300 executes FP64 arithmetic at about 1/64 of its FP32 rate, so the FP64
 // Wilson-Clover operator is bound by the FP64 pipe, not by memory.  A df
 // value is the unevaluated sum hi + lo of two floats with |lo| <= ulp(hi),
-// about 47 significant bits, and every operation runs on the FP32 pipes
+// about 48 significant bits, and every operation runs on the FP32 pipes
 // (roughly 7 instructions per product, 11 per sum, 15 per fused
 // multiply-add).  The building blocks are the classical error-free
 // transformations:
@@ -82,7 +82,10 @@ __device__ __forceinline__ df fma(df a, df b, df c)
 }
 
 // FP64 -> df with integer operations: hi = x truncated to 24 significant
-// bits, lo = the next 23 bits (truncated), both with the sign of x.
+// bits, lo = the other 29 rounded to 24 significant bits, both with the sign
+// of x.  (lo = the next 23 bits, cut off, had been off by up to 2^-46 of x, more
+// than any sum or product that follows: with it the error of H against 64 bits
+// was 1.06e-14 and that of M^ 1.5e-14.)
 __device__ __forceinline__ df df_from_double(double x)
 {
     const unsigned hw = (unsigned)__double2hiint(x), lw = (unsigned)__double2loint(x);
@@ -98,8 +101,7 @@ __device__ __forceinline__ df df_from_double(double x)
     float lo = 0.0f;
     const int se = e - 919;                              // biased FP32 exponent of 2^(e - 1046)
     if (se > 0 && e != 0x7FF && fe < 255) {
-        const unsigned t = (lw & 0x1FFFFFFFu) >> 6;      // top 23 of the 29 remaining bits
-        const float f = __fsub_rn(__uint_as_float(0x3F800000u | t), 1.0f);   // t * 2^-23, exact
+        const float f = __fmul_rn(__uint2float_rn(lw & 0x1FFFFFFFu), 0x1p-29f);
         lo = __fmul_rn(f, __uint_as_float((unsigned)se << 23));
         lo = __uint_as_float(__float_as_uint(lo) | sign);
     }

@@ -11,10 +11,10 @@
 // paired instructions a term and a chain of seven through the running sum,
 // where a multiply-add of double-word numbers that normalises each time takes
 // 16 and a chain of twelve), and the diagonal of a clover block, its largest
-// term, comes last.  Relative errors against FP64, M / M^: 5.1e-15 / 1.5e-14 at
-// kappa 0.12, 5.6e-15 / 1.7e-14 at 0.137, csw 1.9 (a site per thread with
-// double-word multiply-adds: 6.6e-15 / 1.5e-14, 8.5e-15 / 1.7e-14; one
-// normalisation per sum: 2.2e-14 / 2.3e-14, 5 % faster).
+// term, comes last.  Relative errors against 64 bits, M / H / M^: 2.0e-15 /
+// 4.6e-15 / 5.5e-15 at kappa 0.12 (a site per thread with double-word
+// multiply-adds and a split of FP64 values cut off at 47 bits: 6.1e-15 / 9.0e-15
+// / 1.5e-14, though its hops in x were in FP64).
 //
 // One site per thread at 128 registers spilled 1 KB and ran 22 500 warp
 // instructions per 32 sites of an even-odd pass in 38 % of the issue slots;
