@@ -287,7 +287,9 @@ wc_status wc_apply_schur(wc_lattice lat, wc_field out, wc_field in, int dagger);
  * first call blocks; not done while the stream is being captured, where the
  * default shape is used).  force_index >= 0 pins candidate #force_index
  * (0..23; WC_ERR_ARG if its tile does not divide the lattice or it is a
- * register-capped shape with FP64); -1 only reports.  shape_out receives
+ * register-capped shape with FP64), in solves too; -1 only reports; -2 takes
+ * a pin, or what was timed, back, and the next call chooses anew.  shape_out
+ * receives
  * {threads per CTA, tile x, y, z, t (all 0: lexicographic), flags}, flags
  * = register cap (0 none, 1: 64, 2: 85 registers per thread) + 4 if the
  * launch is persistent (grid = resident CTAs, each CTA walking the site
@@ -296,10 +298,10 @@ wc_status wc_apply_schur(wc_lattice lat, wc_field out, wc_field in, int dagger);
  * links and clover into L2, then waits for that kernel; plain launch while
  * the stream is being captured) + 64 if the four directions of a site are
  * on four warps (FP64 with no shape pinned; nothing is timed then); all -1
- * if nothing was chosen yet.  The choice is shared by lattices of equal
- * extent in the process.  With prec = WC_F64 on a lattice in WC_ARITH_DF32
- * mode (wc_set_fp64_arith) the call reports or pins the double-FP32
- * operator's shape, which is chosen separately from the FP64 one. */
+ * if nothing was chosen yet.  The choice is shared by lattices of equal extent in the process.
+ * With prec = WC_F64 on a lattice in WC_ARITH_DF32 mode (wc_set_fp64_arith)
+ * the call reports or pins the double-FP32 operator's shape, which is chosen
+ * separately from the FP64 one. */
 wc_status wc_apply_shape(wc_lattice lat, wc_prec prec, int kind, int force_index, int shape_out[6]);
 
 /* outs[r] (even sites) = M^ ins[r] (even sites), M^ = A_ee - kappa^2 H_eo

@@ -327,7 +327,7 @@ class Lattice:
 
     def apply_shape(self, prec: int, kind: int = 0, force: int = -1):
         """(threads, tile, capped) of the operator launch for prec / kind
-        (0 M, 1 M^+, 2 H); force >= 0 pins candidate #force."""
+        (0 M, 1 M^+, 2 H); force >= 0 pins candidate #force, -2 unpins."""
         out = (ctypes.c_int * 6)()
         _check(_L.wc_apply_shape(self.handle, int(prec), int(kind), int(force), out), self.handle)
         return out[0], tuple(out[1:5]), out[5]

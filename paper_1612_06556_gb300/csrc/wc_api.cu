@@ -855,7 +855,7 @@ wc_status wc_apply_shape(wc_lattice lat, wc_prec prec, int kind, int force_index
     if (!lat || !shape_out) return set_error(lat, WC_ERR_ARG, "lattice and shape_out must not be NULL");
     if (prec != WC_F64 && prec != WC_F32 && prec != WC_F16) return set_error(lat, WC_ERR_ARG, "bad precision");
     if (kind < 0 || kind > 2) return set_error(lat, WC_ERR_ARG, "kind must be 0 (M), 1 (M^+) or 2 (H)");
-    if (force_index < -1 || force_index >= apply_shape_count())
+    if (force_index < -2 || force_index >= apply_shape_count())
         return set_error(lat, WC_ERR_ARG, "force_index out of range");
     if (!apply_shape(lat, prec, kind, force_index, shape_out))
         return set_error(lat, WC_ERR_ARG, "launch shape does not fit this lattice / precision");

@@ -390,7 +390,27 @@ cudaError_t launch_shape(wc_lattice lat, wc_field out, wc_field in, int kind, in
 }
 
 std::mutex g_shape_mutex;
-std::map<std::array<int, 6>, int> g_shape_choice;   // (L, prec, kind) -> shape index
+struct ShapeChoice {
+    int index;
+    bool pinned;   // by a caller (wc_apply_shape)
+};
+std::map<std::array<int, 6>, ShapeChoice> g_shape_choice;   // by (L, prec, kind)
+
+std::array<int, 6> shape_key(const Geom &g, int pcode, int kind)
+{
+    return {g.L[0], g.L[1], g.L[2], g.L[3], pcode, kind};
+}
+
+// the double-FP32 operator has its own entries
+constexpr int kPrecDf = 3;
+
+// whether a caller has pinned a shape (g_shape_mutex held by nobody)
+bool shape_pinned(const Geom &g, int pcode, int kind)
+{
+    std::lock_guard<std::mutex> lk(g_shape_mutex);
+    const auto it = g_shape_choice.find(shape_key(g, pcode, kind));
+    return it != g_shape_choice.end() && it->second.pinned;
+}
 
 // Time every fitting shape (three rounds of 16 launches after one warm-up,
 // best round kept, candidates interleaved so that clock drift affects all
@@ -459,28 +479,27 @@ template <class P>
 cudaError_t launch_apply_p(wc_lattice lat, wc_field out, wc_field in, int kind, cudaStream_t stream,
                            const int *skip, bool pdl)
 {
-    // the double-FP32 operator has its own entry (precision code 3)
-    const int pcode = std::is_same<P, PDF>::value ? 3 : (int)in->prec;
-    const std::array<int, 6> key = {lat->g.L[0], lat->g.L[1], lat->g.L[2], lat->g.L[3], pcode, kind};
+    constexpr bool df = std::is_same<P, PDF>::value;
+    const std::array<int, 6> key = shape_key(lat->g, df ? kPrecDf : (int)in->prec, kind);
     int choice = -1;
     {
         std::lock_guard<std::mutex> lk(g_shape_mutex);
         auto it = g_shape_choice.find(key);
-        if (it != g_shape_choice.end()) choice = it->second;
+        if (it != g_shape_choice.end()) choice = it->second.index;
     }
-    if (choice < 0 && std::is_same<P, P64>::value) {
-        choice = kShapeSplit64;
-        std::lock_guard<std::mutex> lk(g_shape_mutex);
-        g_shape_choice.emplace(key, choice);
-    } else if (choice < 0) {
-        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-        cudaStreamIsCapturing(stream, &cs);
-        if (cs != cudaStreamCaptureStatusNone) {
-            choice = 0;   // no timing inside a capture: default shape, not cached
+    if (choice < 0) {
+        bool keep = true;
+        if (std::is_same<P, P64>::value) {
+            choice = kShapeSplit64;
         } else {
-            choice = tune_shape<P>(lat, out, in, kind, stream);
+            cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+            cudaStreamIsCapturing(stream, &cs);
+            keep = cs == cudaStreamCaptureStatusNone;
+            choice = keep ? tune_shape<P>(lat, out, in, kind, stream) : 0;   // no timing inside a capture
+        }
+        if (keep) {
             std::lock_guard<std::mutex> lk(g_shape_mutex);
-            g_shape_choice[key] = choice;
+            choice = g_shape_choice.emplace(key, ShapeChoice{choice, false}).first->second.index;
         }
     }
     return launch_shape<P>(lat, out, in, kind, choice, stream, skip, pdl);
@@ -536,29 +555,31 @@ cudaError_t launch_copy_s(wc_lattice lat, wc_field dst, wc_field src, double sca
 }  // namespace
 
 // Query or pin the launch shape of (lat extent, prec, kind): force >= 0 pins
-// shape #force (false if it does not fit); out = {threads, tile[4], capped},
-// all -1 when no shape was chosen yet.
+// shape #force (false if it does not fit), -2 forgets what was pinned or
+// timed; out = {threads, tile[4], flags}, all -1 when no shape was chosen yet.
 bool apply_shape(wc_lattice lat, wc_prec prec, int kind, int force, int out[6])
 {
     // FP64 fields on a lattice in double-FP32 mode use that operator's entry
-    const int pcode = (prec == WC_F64 && lat->fp64_arith == WC_ARITH_DF32) ? 3 : (int)prec;
-    const std::array<int, 6> key = {lat->g.L[0], lat->g.L[1], lat->g.L[2], lat->g.L[3], pcode, kind};
+    const int pcode = (prec == WC_F64 && lat->fp64_arith == WC_ARITH_DF32) ? kPrecDf : (int)prec;
+    const std::array<int, 6> key = shape_key(lat->g, pcode, kind);
     for (int i = 0; i < 6; ++i) out[i] = -1;
     std::lock_guard<std::mutex> lk(g_shape_mutex);
     if (force >= 0) {
-        const int caps = prec != WC_F64 ? P32::kCaps : pcode == 3 ? PDF::kCaps : P64::kCaps;
+        const int caps = prec != WC_F64 ? P32::kCaps : pcode == kPrecDf ? PDF::kCaps : P64::kCaps;
         if (force >= kNumShapes || !shape_fits(lat->g, kShapes[force], caps)) return false;
-        g_shape_choice[key] = force;
+        g_shape_choice[key] = ShapeChoice{force, true};
+    } else if (force == -2) {
+        g_shape_choice.erase(key);
     }
     auto it = g_shape_choice.find(key);
     if (it == g_shape_choice.end()) return true;
-    if (it->second == kShapeSplit64) {
+    if (it->second.index == kShapeSplit64) {
         out[0] = kSplit64 * kSplit64Sites;
         for (int m = 0; m < 4; ++m) out[1 + m] = 0;
         out[5] = 64;
         return true;
     }
-    const ApplyShape &s = kShapes[it->second];
+    const ApplyShape &s = kShapes[it->second.index];
     out[0] = s.threads;
     for (int m = 0; m < 4; ++m) out[1 + m] = s.tile[m];
     out[5] = s.capped + 4 * s.persistent + 16 * s.pdl;
@@ -584,13 +605,7 @@ cudaError_t launch_apply64_sum(wc_lattice lat, wc_field out, wc_field in, int ki
                                const StepSum &ss, bool omega, bool pdl)
 {
     const Geom &g = lat->g;
-    {
-        // a launch shape that a caller has pinned stays in use
-        std::lock_guard<std::mutex> lk(g_shape_mutex);
-        if (g_shape_choice.emplace(std::array<int, 6>{g.L[0], g.L[1], g.L[2], g.L[3], (int)WC_F64, kind}, kShapeSplit64)
-                .first->second != kShapeSplit64)
-            return cudaErrorNotSupported;
-    }
+    if (shape_pinned(g, (int)WC_F64, kind)) return cudaErrorNotSupported;   // a pinned launch shape stays in use
     const dim3 grid((g.V + kSplit64Sites - 1) / kSplit64Sites);
     const auto kern = kind == 0 ? (omega ? k_apply_split64_sum<0, true> : k_apply_split64_sum<0, false>)
                                 : (omega ? k_apply_split64_sum<1, true> : k_apply_split64_sum<1, false>);
@@ -601,9 +616,10 @@ cudaError_t launch_apply64_sum(wc_lattice lat, wc_field out, wc_field in, int ki
 cudaError_t launch_apply_df(wc_lattice lat, wc_field out, wc_field in, wc_field split, int kind, cudaStream_t stream,
                             const int *skip, bool pdl)
 {
-    cudaError_t e = launch_to_df(12LL * lat->g.V, in, split, stream, skip, pdl);
-    if (e != cudaSuccess) return e;
     const Geom &g = lat->g;
+    if (shape_pinned(g, kPrecDf, kind)) return launch_apply(lat, out, in, kind, stream, skip, pdl);   // stays in use
+    cudaError_t e = launch_to_df(12LL * g.V, in, split, stream, skip, pdl);
+    if (e != cudaSuccess) return e;
     const dim3 grid((g.V + kSplit64Sites - 1) / kSplit64Sites);
     const auto kern = kind == 0 ? k_apply_splitdf<0, true> : kind == 1 ? k_apply_splitdf<1, true> : k_apply_splitdf<2, true>;
     return launch_step(pdl && pdl_grid(grid.x), kern, grid, kSplit64 * kSplit64Sites, stream, g, lat->gauge, lat->clover,
