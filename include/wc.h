@@ -297,8 +297,10 @@ wc_status wc_apply_schur(wc_lattice lat, wc_field out, wc_field in, int dagger);
  * start while the previous kernel of the stream drains, prefetches its
  * links and clover into L2, then waits for that kernel; plain launch while
  * the stream is being captured) + 64 if the four directions of a site are
- * on four warps (FP64 with no shape pinned; nothing is timed then); all -1
- * if nothing was chosen yet.  The choice is shared by lattices of equal extent in the process.
+ * on four warps (FP64, and double-FP32 up to 2^18 sites, with no shape
+ * pinned; nothing is timed then); all -1 if nothing was chosen yet.  The
+ * candidates of one precision give the same bits, the form on four warps
+ * others.  The choice is shared by lattices of equal extent in the process.
  * With prec = WC_F64 on a lattice in WC_ARITH_DF32 mode (wc_set_fp64_arith)
  * the call reports or pins the double-FP32 operator's shape, which is chosen
  * separately from the FP64 one. */

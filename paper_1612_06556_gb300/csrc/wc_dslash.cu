@@ -277,11 +277,16 @@ constexpr int kNumShapes = sizeof(kShapes) / sizeof(kShapes[0]);
 // against 39 us, 8^4 14 / 39, 12^4 49 / 60, 16^3x32 247 / 266, 24^3x32
 // 828 / 863, 17x19x21x23 299 / 331, 32^3x64 3960-4016 / 4014-4022), so
 // nothing is timed for it.
-// In double-FP32 arithmetic it is one more candidate to time: each hop there
-// splits its spinor anew, which costs more than it gains on large lattices
-// (8^4 17 against 47 us, 16^3x32 181 / 218, 24^3x32 605 / 608, 32^3x64 2924 /
-// 2550); a solve splits its vector once (launch_apply_df).
 constexpr int kShapeSplit64 = kNumShapes;
+// In double-FP32 arithmetic up to this many sites; above, one of the shapes
+// is timed and taken.  Each hop splits its spinor anew, which costs more than it
+// gains on large lattices: 8^4 17 against 47 us, 16^3x32 190 / 209, 17x19x21x23
+// 227 / 250, 20^3x32 367 / 376, 24^3x24 477 / 466, 24^3x32 632 / 596, 28^3x32 1007 /
+// 905.  The line is one of size, not of times measured in a process: the two
+// forms round differently, and a result must not depend on a timing (the
+// shapes all give the same bits).  A solve splits its vector once
+// (launch_apply_df).
+constexpr int kSplitDfSites = 1 << 18;
 
 // caps: bit c-1 set if register cap c is compiled for the operator (P::kCaps)
 bool shape_fits(const Geom &g, const ApplyShape &s, int caps)
@@ -445,12 +450,11 @@ int tune_shape(wc_lattice lat, wc_field out, wc_field in, int kind, cudaStream_t
         npair = k + 1;
     }
     cudaGetLastError();
-    constexpr int n = kNumShapes + std::is_same<P, PDF>::value;   // with kShapeSplit64
-    float best_ms[n];
-    for (int i = 0; i < n; ++i) best_ms[i] = 1e30f;
+    float best_ms[kNumShapes];
+    for (int i = 0; i < kNumShapes; ++i) best_ms[i] = 1e30f;
     for (int round = 0; round < 3; ++round) {
-        for (int i = 0; i < n; ++i) {
-            if (i < kNumShapes && !shape_fits(lat->g, kShapes[i], P::kCaps)) continue;
+        for (int i = 0; i < kNumShapes; ++i) {
+            if (!shape_fits(lat->g, kShapes[i], P::kCaps)) continue;
             if (launch_shape<P>(lat, out, in, kind, i, stream) != cudaSuccess) continue;
             cudaEventRecord(e0, stream);
             for (int r = 0; r < 16; ++r)
@@ -463,7 +467,7 @@ int tune_shape(wc_lattice lat, wc_field out, wc_field in, int kind, cudaStream_t
         }
     }
     int best = 0;
-    for (int i = 1; i < n; ++i)
+    for (int i = 1; i < kNumShapes; ++i)
         if (best_ms[i] < best_ms[best]) best = i;
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
@@ -489,7 +493,7 @@ cudaError_t launch_apply_p(wc_lattice lat, wc_field out, wc_field in, int kind, 
     }
     if (choice < 0) {
         bool keep = true;
-        if (std::is_same<P, P64>::value) {
+        if (std::is_same<P, P64>::value || (df && lat->g.V <= kSplitDfSites)) {
             choice = kShapeSplit64;
         } else {
             cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;

@@ -38,3 +38,11 @@ def test_a_pinned_shape_is_used_in_solves_and_can_be_taken_back(arith):
     with pytest.raises(wc().WCError):
         lat.apply_shape(0, 0, force=-3)
 
+
+@pytest.mark.parametrize("dims,split", [((32, 16, 16, 32), True), ((34, 16, 16, 32), False)])
+def test_double_fp32_form_depends_on_the_size_only(dims, split):
+    """On both sides of the line at 2^18 sites."""
+    lat = make_lattice(dims, synth.unit_links(dims), 1.0, 0.12, -1).set_fp64_arith(1)
+    f, g = lat.field(0), lat.field(0)
+    lat.apply_M(g, f)
+    assert (lat.apply_shape(0, 0)[2] == 64) == split
