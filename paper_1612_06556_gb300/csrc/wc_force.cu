@@ -36,23 +36,24 @@
 // with S2 = L2 L3 and T = L1 S2.
 //
 // The four links of a plaquette see the same insertions, so k_force_plaq
-// forms their sum once per plaquette and carries it from link to link.  Let
-// L0 = U_a(x), L1 = U_b(x+a), V = U_a(x+b), W = U_b(x) be the links of the
-// plaquette of (a, b), a < b, at x, P = L0 L1 V^+ W^+, Z0, Z1, Z2, Z3 = Xh_ab at
-// x, x+a, x+a+b, x+b, G = sum_k W_k the sum for the link L0, and Hm(M) = (M +
-// M^+)/2.  As c is imaginary, F = TA(c M) = c Hm(M) - trace, and of G only H =
-// Hm(G) is needed:
-//   G = (L0 (Z1 L1 + L1 Z2) V^+ + L0 L1 V^+ Z3) W^+ + P Z0.
-// Beginning the loop at another corner moves one insertion from the end of the
-// product to its front, which adds a commutator [Z, P] there, and Hm([Z, P]) =
-// Hm(Z X) with X = P - P^+.  In units of c with sigma = +1 the links get
-//   U_a(x)     H
-//   U_b(x)     -(H + Hm(Z0 X))
-//   U_b(x+a)   H1 - Hm(Z1 X1),      H1 + X1 = L0^+ (H + X) L0
-//   U_a(x+b)   -(H3 + Hm(Z3 X3)),   H3 + X3 = W^+ (H + Hm(Z0 X) + X) W
-// (Hermitian and anti-Hermitian parts of the carried matrix): about 1680 FP64
-// operations per plaquette, 10 000 a site, where the four insertions of each
-// leaf pair taken link by link are 19 000.  k_force_link adds the six
+// forms what they share once per plaquette.  Let L0 = U_a(x), L1 = U_b(x+a), V =
+// U_a(x+b), W = U_b(x) be the links of the plaquette of (a, b), a < b, at x, Z0,
+// Z1, Z2, Z3 = Xh_ab at x, x+a, x+a+b, x+b, and Hm(M) = (M + M^+)/2.  As c is
+// imaginary, F = TA(c M) = c Hm(M) - trace, and Hm(M) = Hm(M^+).  With
+//   D = L1 V^+, r = L1 Z2 V^+, Q = D W^+, C = L0 D, m = L0 (r + Z1 D)
+//   P = L0 Q, P1 = Q L0, P3 = W^+ C          the loop from x, x+a and x+b
+// the links get, in units of c with sigma = +1,
+//   U_a(x)      Hm(G),  G = (m + C Z3) W^+ + P Z0
+//   U_b(x)     -Hm(G + [Z0, P]) = -(Hm(G) + Hm(Z0 X)),  X = P - P^+
+//   U_b(x+a)    Hm(((r + D Z3) W^+ + Q Z0) L0 + P1 Z1)
+//   U_a(x+b)   -Hm(W^+ (m + Z0 C) + Z3 P3)
+// (the two links at a corner begin the same loop in its two directions, which
+// moves one insertion from its end to its front): about 2070 FP64 operations
+// per plaquette, 12 400 a site, where the four insertions of each leaf pair
+// taken link by link are 19 000.  (Carrying Hm(G) and X from corner to corner with
+// U^+ (.) U takes 1680, but U^+ U = 1 only as far as the links are unitary: for
+// links rounded to FP32 the force was off by 1.8e-8, and for exact ones its
+// rounding errors were 1.7 times as large.)  k_force_link adds the six
 // contributions of a link and its hopping part; two planes at a time, the
 // pairs (xy, zt), (xz, yt), (yz, xt) that contain every direction once.
 //
@@ -200,6 +201,17 @@ __device__ __forceinline__ H3 operator+(const H3 &a, const H3 &b)
     return r;
 }
 
+__device__ __forceinline__ H3 operator-(const H3 &a, const H3 &b)
+{
+    H3 r;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        r.d[k] = a.d[k] - b.d[k];
+        r.o[k] = a.o[k] - b.o[k];
+    }
+    return r;
+}
+
 // entry (i, j) of X, i != j
 __device__ __forceinline__ cx<double> xoff(const X3 &x, int i, int j)
 {
@@ -273,40 +285,6 @@ __device__ __forceinline__ H3 herm2_zx(const H3 &z, const X3 &x)
         r.o[q] = at(i, j) + conj(at(j, i));
     }
     return r;
-}
-
-// U^+ (h + x) U as its Hermitian and anti-Hermitian parts, twice each
-__device__ __forceinline__ void carry2(const H3 &h, const X3 &x, const M3 &u, H3 &hc, X3 &xc)
-{
-    M3 m;
-#pragma unroll
-    for (int i = 0; i < 3; ++i) m.m[i][i] = mkc(h.d[i], x.d[i]);
-#pragma unroll
-    for (int q = 0; q < 3; ++q) {
-        const int i = off_row(q), j = off_col(q);
-        m.m[i][j] = h.o[q] + x.o[q];
-        m.m[j][i] = conj(h.o[q] - x.o[q]);
-    }
-    const M3 t = mul(m, u);
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            cx<double> s = cmul_conj(u.m[0][i], t.m[0][j]);
-            s = cfma_conj(u.m[1][i], t.m[1][j], s);
-            m.m[i][j] = cfma_conj(u.m[2][i], t.m[2][j], s);
-        }
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-        hc.d[i] = 2.0 * m.m[i][i].re;
-        xc.d[i] = 2.0 * m.m[i][i].im;
-    }
-#pragma unroll
-    for (int q = 0; q < 3; ++q) {
-        const cx<double> a = m.m[off_row(q)][off_col(q)], b = conj(m.m[off_col(q)][off_row(q)]);
-        hc.o[q] = a + b;
-        xc.o[q] = a - b;
-    }
 }
 
 __device__ __forceinline__ void store_h3(double *p, int V, int x, const H3 &h)
@@ -391,8 +369,8 @@ __global__ void __launch_bounds__(64) k_xi(Geom g, const double2 *X, const doubl
 }
 
 // The contributions of one plaquette to its four links (see above), twice
-// each, in units of c: slot 0 U_a(x), 1 U_b(x), 2 U_b(x+a), 3 U_a(x+b), at the
-// index of x.  Plane (planes.x, planes.y) for blockIdx.y = 0, (planes.z,
+// each, in units of c: slot 0 U_a(x), 1 U_b(x), 2 U_b(x+a), 3 U_a(x+b), the signs of
+// 1 and 3 left to k_force_link, at the index of x.  Plane (planes.x, planes.y) for blockIdx.y = 0, (planes.z,
 // planes.w) for 1; ws: [2 planes][4 slots][9][V].
 __global__ void __launch_bounds__(64) k_force_plaq(Geom g, GaugeStore G, const double *xh, int4 planes, double *ws)
 {
@@ -407,58 +385,43 @@ __global__ void __launch_bounds__(64) k_force_plaq(Geom g, GaugeStore G, const d
     const int xa = wc_idx(c[a] == g.L[a] - 1 ? x - (g.L[a] - 1) * g.stride[a] : x + g.stride[a], V);
     const int xb = wc_idx(c[b] == g.L[b] - 1 ? x - (g.L[b] - 1) * g.stride[b] : x + g.stride[b], V);
     const int xab = wc_idx(c[b] == g.L[b] - 1 ? xa - (g.L[b] - 1) * g.stride[b] : xa + g.stride[b], V);
-    const M3 L0 = link(G, V, a, x), W = link(G, V, b, x);
-    const H3 Z0 = load_h3(xp, V, x);
-    H3 H;
-    X3 X;
+    const auto put = [&](int slot, const H3 &h) { store_h3(w0 + (size_t)(9 * slot) * V, V, x, h); };
+    M3 D, r;
     {
         const M3 L1 = link(G, V, b, xa), Vd = dag(link(G, V, a, xb));
-        M3 t = zero3();
-        fma_hm(load_h3(xp, V, xa), L1, t);
-        fma_mh(L1, load_h3(xp, V, xab), t);
-        M3 E = mul(mul(L0, t), Vd);
-        const M3 C = mul(mul(L0, L1), Vd);
-        fma_mh(C, load_h3(xp, V, xb), E);
-        const M3 P = mul_dag(C, W);
-        H = herm2(E, W, P, Z0);
+        M3 s = zero3();
+        fma_mh(L1, load_h3(xp, V, xab), s);
+        r = mul(s, Vd);
+        D = mul(L1, Vd);
+    }
+    const M3 L0 = link(G, V, a, x), W = link(G, V, b, x);
+    const M3 Q = mul_dag(D, W);
+    {
+        M3 n = r;
+        fma_mh(D, load_h3(xp, V, xb), n);
+        n = mul_dag(n, W);
+        fma_mh(Q, load_h3(xp, V, x), n);
+        put(2, herm2(n, dag(L0), mul(Q, L0), load_h3(xp, V, xa)));
+    }
+    fma_hm(load_h3(xp, V, xa), D, r);
+    const M3 m = mul(L0, r), C = mul(L0, D);
+    {
+        M3 e = m;
+        fma_mh(C, load_h3(xp, V, xb), e);
+        const M3 P = mul(L0, Q);
+        X3 X;
 #pragma unroll
         for (int i = 0; i < 3; ++i) X.d[i] = 2.0 * P.m[i][i].im;
 #pragma unroll
         for (int q = 0; q < 3; ++q) X.o[q] = P.m[off_row(q)][off_col(q)] - conj(P.m[off_col(q)][off_row(q)]);
+        const H3 Z0 = load_h3(xp, V, x), H = herm2(e, W, P, Z0);
+        put(0, H);
+        put(1, H + herm2_zx(Z0, X));
     }
-    // H is 2 Hm(G); below hc, xc are twice the carried H and X
-    store_h3(w0, V, x, H);
-    H3 hc;
-    X3 xc;
-    carry2(H, X, L0, hc, xc);
     {
-        const H3 k = herm2_zx(load_h3(xp, V, xa), xc);   // 4 Hm(Z1 X1)
-        H3 r;
-#pragma unroll
-        for (int q = 0; q < 3; ++q) {
-            r.d[q] = 0.5 * (hc.d[q] - k.d[q]);
-            r.o[q] = 0.5 * (hc.o[q] - k.o[q]);
-        }
-        store_h3(w0 + (size_t)18 * V, V, x, r);
-    }
-    H = H + herm2_zx(Z0, X);
-    H3 n;
-#pragma unroll
-    for (int q = 0; q < 3; ++q) {
-        n.d[q] = -H.d[q];
-        n.o[q] = -H.o[q];
-    }
-    store_h3(w0 + (size_t)9 * V, V, x, n);
-    carry2(H, X, W, hc, xc);
-    {
-        const H3 k = herm2_zx(load_h3(xp, V, xb), xc);
-        H3 r;
-#pragma unroll
-        for (int q = 0; q < 3; ++q) {
-            r.d[q] = -0.5 * (hc.d[q] + k.d[q]);
-            r.o[q] = -0.5 * (hc.o[q] + k.o[q]);
-        }
-        store_h3(w0 + (size_t)27 * V, V, x, r);
+        M3 y = m;
+        fma_hm(load_h3(xp, V, x), C, y);
+        put(3, herm2(dag(y), dag(W), dag(mul(dag(W), C)), load_h3(xp, V, xb)));
     }
 }
 
@@ -520,7 +483,8 @@ __global__ void __launch_bounds__(64) k_force_link(Geom g, GaugeStore G, const d
         const double *w0 = ws + (size_t)second * 36 * V;
         const int nu = mu == a ? b : a;
         const int xd = wc_idx(c[nu] == 0 ? x + (g.L[nu] - 1) * g.stride[nu] : x - g.stride[nu], V);
-        h = load_h3(w0 + (size_t)(mu == a ? 0 : 9) * V, V, x) + load_h3(w0 + (size_t)(mu == a ? 27 : 18) * V, V, xd);
+        h = load_h3(w0 + (size_t)(mu == a ? 0 : 18) * V, V, mu == a ? x : xd) -
+            load_h3(w0 + (size_t)(mu == a ? 27 : 9) * V, V, mu == a ? xd : x);
         if (!FIRST) {
             H3 p;
             const double2 d0 = out[0], d1 = out[1];

@@ -111,3 +111,20 @@ def test_force_times_links_kernel():
     assert np.max(np.abs(out.cpu().numpy() - ref)) <= 1e-13 * np.max(np.abs(ref))
     with pytest.raises(ValueError):
         lat.force_times_links(torch.from_numpy(F), Ut, 1.0, out)
+
+
+@pytest.mark.parametrize("dims,csw", [((2, 2, 2, 2), 1.4), ((3, 2, 5, 4), 1.0), ((4, 4, 4, 6), 1.3)])
+def test_force_of_links_rounded_to_fp32(dims, csw):
+    """Random links unitary to 1e-7 only (two rows as given, the third their
+    cross product): the force formula of these links, not one that assumes
+    U^+ U = 1.  Both solves to 5e-15, amplified by |M^-1| <= 10 each, leave the
+    force within a few 1e-13."""
+    kappa, tbc = 0.11, -1
+    U = synth.haar_links(dims, 72).astype(np.complex64).astype(complex)
+    U[..., 2, :] = np.conj(np.cross(U[..., 0, :], U[..., 1, :]))
+    phi = synth.gaussian_source(dims, 74)
+    lat = make_lattice(dims, U, csw, kappa, tbc)
+    F = np.zeros((synth.volume(dims), 4, 3, 3), complex)
+    lat.action_force(lat.field(0).load(phi), F, tol=5e-15)
+    _, F_ref, _, _ = oracle.action_and_force(oracle.Operator(dims, U, csw, kappa, tbc), phi, tol=1e-15)
+    assert np.linalg.norm(F - F_ref) <= 1e-12 * np.linalg.norm(F_ref)
