@@ -368,24 +368,29 @@ __global__ void __launch_bounds__(64) k_xi(Geom g, const double2 *X, const doubl
     }
 }
 
+// Where the contributions of the plaquettes of two planes go: [9][V] for each
+// plane and each of its four slots.
+struct ForceSlots {
+    double *at[2][4];
+};
+
 // The contributions of one plaquette to its four links (see above), twice
 // each, in units of c: slot 0 U_a(x), 1 U_b(x), 2 U_b(x+a), 3 U_a(x+b), the signs of
 // 1 and 3 left to k_force_link, at the index of x.  Plane (planes.x, planes.y) for blockIdx.y = 0, (planes.z,
-// planes.w) for 1; ws: [2 planes][4 slots][9][V].
-__global__ void __launch_bounds__(64) k_force_plaq(Geom g, GaugeStore G, const double *xh, int4 planes, double *ws)
+// planes.w) for 1.
+__global__ void __launch_bounds__(64) k_force_plaq(Geom g, GaugeStore G, const double *xh, int4 planes, ForceSlots ws)
 {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= g.V) return;
     const int V = g.V;
     const int a = blockIdx.y ? planes.z : planes.x, b = blockIdx.y ? planes.w : planes.y;
     const double *xp = xh + (size_t)plane_of(a, b) * 9 * V;
-    double *w0 = ws + (size_t)blockIdx.y * 36 * V;
     int c[4];
     site_coords(g, x, c);
     const int xa = wc_idx(c[a] == g.L[a] - 1 ? x - (g.L[a] - 1) * g.stride[a] : x + g.stride[a], V);
     const int xb = wc_idx(c[b] == g.L[b] - 1 ? x - (g.L[b] - 1) * g.stride[b] : x + g.stride[b], V);
     const int xab = wc_idx(c[b] == g.L[b] - 1 ? xa - (g.L[b] - 1) * g.stride[b] : xa + g.stride[b], V);
-    const auto put = [&](int slot, const H3 &h) { store_h3(w0 + (size_t)(9 * slot) * V, V, x, h); };
+    const auto put = [&](int slot, const H3 &h) { store_h3(ws.at[blockIdx.y][slot], V, x, h); };
     M3 D, r;
     {
         const M3 L1 = link(G, V, b, xa), Vd = dag(link(G, V, a, xb));
@@ -467,7 +472,7 @@ __device__ __forceinline__ M3 hop_outer(const double2 *X, const double2 *Y, int 
 // part too and F = TA(G) in the canonical layout [V][4][3][3].
 template <bool FIRST, bool LAST>
 __global__ void __launch_bounds__(64) k_force_link(Geom g, GaugeStore G, const double2 *X, const double2 *Y, int4 planes,
-                                                   const double *ws, double kappa, double csw, double2 *F)
+                                                   ForceSlots ws, double kappa, double csw, double2 *F)
 {
     const int x = blockIdx.x * blockDim.x + threadIdx.x, mu = blockIdx.y;
     if (x >= g.V) return;
@@ -480,11 +485,10 @@ __global__ void __launch_bounds__(64) k_force_link(Geom g, GaugeStore G, const d
         // the plane of this step that contains mu: (a, b) with a = mu or b = mu
         const int second = mu == planes.z || mu == planes.w;
         const int a = second ? planes.z : planes.x, b = second ? planes.w : planes.y;
-        const double *w0 = ws + (size_t)second * 36 * V;
         const int nu = mu == a ? b : a;
         const int xd = wc_idx(c[nu] == 0 ? x + (g.L[nu] - 1) * g.stride[nu] : x - g.stride[nu], V);
-        h = load_h3(w0 + (size_t)(mu == a ? 0 : 18) * V, V, mu == a ? x : xd) -
-            load_h3(w0 + (size_t)(mu == a ? 27 : 9) * V, V, mu == a ? xd : x);
+        h = load_h3(ws.at[second][mu == a ? 0 : 2], V, mu == a ? x : xd) -
+            load_h3(ws.at[second][mu == a ? 3 : 1], V, mu == a ? xd : x);
         if (!FIRST) {
             H3 p;
             const double2 d0 = out[0], d1 = out[1];
@@ -543,17 +547,37 @@ bool is_device_ptr(const void *p)
 
 }  // namespace
 
+// Slots in the work vectors of a solver state, which are free between solves:
+// from slot number `have` on, up to eight in all; returns the new number.  The
+// even-odd and FP64 solvers leave all eight, so that a force takes no more
+// memory than Xh (432 B a site; with slots of its own it took 1008).
+static int borrow_slots(const SolverState &S, size_t bytes, double **slot, int have)
+{
+    for (const wc_field_s *f : S.work) {
+        if (!f) continue;
+        char *p = static_cast<char *>(f->data);
+        for (size_t left = spinor_bytes(f->prec, f->lat->g.V); left >= bytes && have < 8; left -= bytes, p += bytes)
+            slot[have++] = reinterpret_cast<double *>(p);
+    }
+    return have;
+}
+
 // F from X, Y (FP64 fields) into the canonical force layout at dst (device).
 wc_status force_from_solutions(wc_lattice lat, wc_field X, wc_field Y, double2 *dst)
 {
     const int V = lat->g.V;
     cudaStream_t s = lat->stream;
     const double2 *x = static_cast<const double2 *>(X->data), *y = static_cast<const double2 *>(Y->data);
-    // Xh of the six planes, then the link contributions of two planes
+    // Xh of the six planes, and the slots that idle solver vectors do not give
+    ForceSlots ws{};
+    const size_t slot_bytes = sizeof(double) * 9 * (size_t)V;
+    int have = borrow_slots(lat->st, slot_bytes, &ws.at[0][0], 0);
+    if (lat->half) have = borrow_slots(lat->half->st, slot_bytes, &ws.at[0][0], have);
     double *xh = nullptr;
-    wc_status st = check_cuda(lat, cudaMalloc(&xh, sizeof(double) * (54 + 72) * (size_t)V), "cudaMalloc(force)");
+    wc_status st = check_cuda(lat, cudaMalloc(&xh, sizeof(double) * 54 * (size_t)V + slot_bytes * (8 - have)),
+                              "cudaMalloc(force)");
     if (st != WC_OK) return st;
-    double *ws = xh + (size_t)54 * V;
+    for (int k = have; k < 8; ++k) (&ws.at[0][0])[k] = xh + (size_t)(54 + 9 * (k - have)) * V;
     const int4 pair[3] = {make_int4(0, 1, 2, 3), make_int4(0, 2, 1, 3), make_int4(1, 2, 0, 3)};
     const unsigned blocks = (V + 63) / 64;
     const bool clover = lat->csw != 0.0;

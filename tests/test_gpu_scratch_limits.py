@@ -47,3 +47,22 @@ def test_even_odd_call_after_one_that_ran_out_of_memory(left):
     torch.cuda.empty_cache()
     lat.apply_schur(g, f)
     assert np.array_equal(g.store(np.zeros_like(src)), ref)
+
+
+@pytest.mark.parametrize("kw", [dict(solver=1, even_odd=True), dict(), dict(solver=1, even_odd=True, krylov_prec=2)])
+def test_force_in_the_memory_of_its_fields_and_xi(kw):
+    """At 16^3x32 a force needs two fields (50 MB) and Xh (57 MB) once its
+    solver's vectors exist: it runs with 140 MB left, and gives the same bits."""
+    import torch
+    dims, kappa, csw, tbc = (16, 16, 16, 32), 0.11, 1.0, -1
+    U = synth.pool_links(dims, 351)
+    phi = synth.gaussian_source(dims, 352)
+    lat = make_lattice(dims, U, csw, kappa, tbc)
+    b = lat.field(0).load(phi)
+    F = [torch.zeros(int(np.prod(dims)), 4, 3, 3, dtype=torch.complex128, device="cuda") for _ in range(2)]
+    S0 = lat.action_force(b, F[0], tol=1e-10, **kw)
+    hog = _leave(140)
+    S1 = lat.action_force(b, F[1], tol=1e-10, **kw)
+    del hog
+    torch.cuda.empty_cache()
+    assert S0 == S1 and torch.equal(F[0], F[1])
