@@ -834,9 +834,9 @@ wc_status wc_apply_schur(wc_lattice lat, wc_field out, wc_field in, int dagger)
     wc_lattice h = nullptr;
     st = half_lattice(lat, &h);
     if (st != WC_OK) return st;
-    // the half fields are kept between calls (creating and freeing three per
-    // call had cost 0.4 ms, the FP64 operator itself takes 0.3 ms at
-    // 16^3x32); the lock is held until the stream has finished
+    // the half fields are kept between calls up to kKeptWorkspace (creating and
+    // freeing three per call had cost 0.4 ms, the FP64 operator itself takes
+    // 0.3 ms at 16^3x32); the lock is held until the stream has finished
     std::lock_guard<std::mutex> lk(lat->eom_mutex);
     wc_field *io = lat->schur_io[in->prec];
     for (int k = 0; k < 2 && st == WC_OK; ++k)
@@ -845,6 +845,11 @@ wc_status wc_apply_schur(wc_lattice lat, wc_field out, wc_field in, int dagger)
     if (st == WC_OK) st = check_cuda(lat, launch_schur(h, io[1], io[0], dagger ? 1 : 0, lat->stream), "schur");
     if (st == WC_OK) st = check_cuda(lat, launch_merge(lat, io[1], nullptr, out, lat->stream), "merge");
     if (st == WC_OK) st = check_cuda(lat, cudaStreamSynchronize(lat->stream), "sync");
+    if (2 * spinor_bytes(in->prec, h->g.V) > kKeptWorkspace)
+        for (int k = 0; k < 2; ++k) {
+            wc_field_destroy(io[k]);
+            io[k] = nullptr;
+        }
     return st;
 }
 wc_status wc_apply_Mdag(wc_lattice lat, wc_field out, wc_field in) { return apply_common(lat, out, in, 1); }

@@ -457,8 +457,9 @@ extern "C" wc_status wc_apply_schur_multi(wc_lattice lat, int n, wc_field *outs,
     const wc_prec pr = ins[0]->prec;
     const int Vh = h->g.V;
     // n odd-site intermediates in the lattice's workspace, kept between
-    // calls (allocating three half fields per right-hand side on every call
-    // cost 2.7 ms of a 2.9 ms call at 12 right-hand sides and 16^3x32); one
+    // calls up to kKeptWorkspace (allocating three half fields per right-hand
+    // side on every call cost 2.7 ms of a 2.9 ms call at 12 right-hand sides and
+    // 16^3x32; a larger workspace goes with a call of milliseconds); one
     // call at a time uses it: the lock is held until the stream has finished
     const size_t data_bytes = (spinor_bytes(pr, Vh) + 255) / 256 * 256;
     const size_t nrm_bytes = pr == WC_F16 ? ((size_t)Vh * sizeof(float) + 255) / 256 * 256 : 0;
@@ -490,5 +491,10 @@ extern "C" wc_status wc_apply_schur_multi(wc_lattice lat, int n, wc_field *outs,
                    : launch_eom<P16, 0, true>(lat, n, outs, ins, tmps, nullptr, 0, nullptr, nullptr, lat->stream);
     st = check_cuda(lat, e, "schur_multi");
     if (st == WC_OK) st = check_cuda(lat, cudaStreamSynchronize(lat->stream), "sync");
+    if (lat->eom_ws_bytes > kKeptWorkspace) {
+        cudaFree(lat->eom_ws);
+        lat->eom_ws = nullptr;
+        lat->eom_ws_bytes = 0;
+    }
     return st;
 }

@@ -120,7 +120,7 @@ struct wc_lattice_s {
     // precision (created on first use)
     wc_field_s *ras_half[3][2] = {};
     // wc_apply_schur_multi: odd-site intermediates of its right-hand sides
-    // (up to kMrhsMax half-lattice spinors), held until wc_destroy_lattice
+    // (half-lattice spinors), held until wc_destroy_lattice
     void *eom_ws = nullptr;
     size_t eom_ws_bytes = 0;
     std::mutex eom_mutex;
@@ -138,6 +138,11 @@ struct wc_field_s {
 };
 
 namespace wc {
+
+// What wc_apply_schur_multi, and wc_apply_schur in each precision, keep of their
+// workspace on a lattice between calls, at most (bytes); a call that needs
+// more frees it at its end.
+constexpr size_t kKeptWorkspace = (size_t)256 << 20;
 
 inline size_t spinor_bytes(wc_prec p, int V)
 {
