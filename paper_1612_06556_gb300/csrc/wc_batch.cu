@@ -322,14 +322,14 @@ wc_status enqueue_group_step(wc_lattice half, const std::vector<int> &idx, Resou
     for (int k = 0; k < m; ++k) rh[k] = R.LW[idx[k]].rhat;
     wc_status st = check_cuda(half, lo_group(LO_STEP_P, half, m, dm, hv, mb, s), "lo_p");
     if (st == WC_OK)
-        st = check_cuda(half, launch_schur_multi(half, m, v.data(), p.data(), tmp.data(), 0, skip.data(), s,
+        st = check_cuda(half, launch_schur_multi(half, m, v.data(), p.data(), tmp.data(), skip.data(), s,
                                                  fused ? 1 : 0, rh.data(), part), "schur_multi");
     if (st == WC_OK)
         st = fused ? check_cuda(half, lo_group_finalize(LO_STEP_ALPHA, m, nblk, part, dm, s), "alpha")
                    : check_cuda(half, lo_group(LO_STEP_ALPHA, half, m, dm, hv, mb, s), "lo_alpha");
     if (st == WC_OK) st = check_cuda(half, lo_group(LO_STEP_S, half, m, dm, hv, mb, s), "lo_s");
     if (st == WC_OK)
-        st = check_cuda(half, launch_schur_multi(half, m, t.data(), sv.data(), tmp.data(), 0, skip.data(), s,
+        st = check_cuda(half, launch_schur_multi(half, m, t.data(), sv.data(), tmp.data(), skip.data(), s,
                                                  fused ? 2 : 0, nullptr, part), "schur_multi");
     if (st == WC_OK)
         st = fused ? check_cuda(half, lo_group_finalize(LO_STEP_OMEGA, m, nblk, part, dm, s), "omega")
@@ -848,10 +848,8 @@ static wc_status batch_even_odd(int n, const wc_lattice *lats, wc_field *xs, wc_
         wc_field t = H[i]->schur_tmp[WC_F64];
         if (st == WC_OK) st = check_cuda(lat, launch_split(lat, bs[i], F(i, 0), F(i, 1), s), "split");
         if (st == WC_OK) st = check_cuda(lat, launch_split(lat, xs[i], F(i, 2), F(i, 3), s), "split");
-        if (st == WC_OK) st = check_cuda(lat, launch_eo(lat, 1, 4, 0, nullptr, F(i, 1), t, 0.0, s, nullptr, nullptr, false,
-                                            eo_split(lat, t) ? kEoOutSplit : 0), "A_oo^-1 b_o");
-        if (st == WC_OK) st = check_cuda(lat, launch_eo(lat, 0, 2, 0, t, F(i, 0), F(i, 4), lat->kappa, s, nullptr, nullptr, false,
-                                            eo_split(lat, t) ? kEoInSplit : 0), "b^_e");
+        if (st == WC_OK) st = check_cuda(lat, launch_eo(lat, 1, 4, 0, nullptr, F(i, 1), t, 0.0, s), "A_oo^-1 b_o");
+        if (st == WC_OK) st = check_cuda(lat, launch_eo(lat, 0, 2, 0, t, F(i, 0), F(i, 4), lat->kappa, s), "b^_e");
         if (st == WC_OK) st = reduce_norm2(lat, bs[i], &bb[i]);
         if (st == WC_OK) st = reduce_norm2(H[i], F(i, 4), &bbh[i]);
         if (st == WC_OK && bb[i] > 0.0 && bbh[i] > 0.0) scale[i] = sqrt(bb[i] / bbh[i]);

@@ -13,10 +13,12 @@
 // (s, r) computes site s of right-hand side r from the staged links and
 // block and the 8 neighbour spinors of field r (through L1/L2).  A CTA takes
 // 32 sites for up to 6 fields and 16 above: more and smaller CTAs on an SM,
-// one of them staging while the others compute (M^ at 24^3x32 in FP32, 16 /
-// 32 sites: 5 fields 314 / 317 us, 6 321 / 333, 8 393 / 410, 12 559 / 585, 16
-// 748 / 978; binary16: 5 258 / 237, 6 252 / 251, 8 311 / 320, 12 440 / 472, 16
-// 583 / 771; at 64 registers 16 sites spill, 696 for 12 FP32 fields).  The third
+// one of them staging while the others compute.  M^ with 16 / 32 sites, FP32 at
+// 16^3x32 4 fields 105 / 103 us, 5 123 / 119, 6 125 / 126, 7 140 / 139, 8 145 /
+// 148, at 24^3x32 5 313 / 312, 6 318 / 327, 8 389 / 403, 12 559 / 585, 16 748 /
+// 978; binary16 at 24^3x32 5 256 / 236, 6 251 / 252, 7 315 / 304, 8 309 / 322, 12
+// 440 / 472, 16 583 / 771 (at 64 registers 16 sites spill, 696 for 12 FP32 fields
+// at 24^3x32).  The third
 // row of each link is rebuilt once per site after staging (into shared
 // memory), not once per right-hand side.  The arithmetic per (site,
 // right-hand side) is otherwise that of the single-field pass (spin
@@ -407,19 +409,15 @@ cudaError_t launch_eom(const wc_lattice_s *full, int n, wc_field_s *const *outs,
 }  // namespace
 
 cudaError_t launch_schur_multi(wc_lattice half, int n, wc_field const *outs, wc_field const *ins,
-                               wc_field const *tmps, int dagger, const int *const *skip, cudaStream_t stream,
-                               int red, wc_field const *dots, double *part)
+                               wc_field const *tmps, const int *const *skip, cudaStream_t stream, int red,
+                               wc_field const *dots, double *part)
 {
     if (n < 1 || n > kMrhsMax || !half->schur_parent) return cudaErrorInvalidValue;
     const wc_lattice_s *full = half->schur_parent;
     const wc_prec pr = ins[0]->prec;
     if (red != 0 && (pr != WC_F32 || !part || (red == 1 && !dots))) return cudaErrorInvalidValue;
-    if (pr == WC_F32)
-        return dagger ? launch_eom<P32, 1, false>(full, n, outs, ins, tmps, skip, red, dots, part, stream)
-                      : launch_eom<P32, 0, false>(full, n, outs, ins, tmps, skip, red, dots, part, stream);
-    if (pr == WC_F16)
-        return dagger ? launch_eom<P16, 1, false>(full, n, outs, ins, tmps, skip, 0, nullptr, nullptr, stream)
-                      : launch_eom<P16, 0, false>(full, n, outs, ins, tmps, skip, 0, nullptr, nullptr, stream);
+    if (pr == WC_F32) return launch_eom<P32, 0, false>(full, n, outs, ins, tmps, skip, red, dots, part, stream);
+    if (pr == WC_F16) return launch_eom<P16, 0, false>(full, n, outs, ins, tmps, skip, 0, nullptr, nullptr, stream);
     return cudaErrorInvalidValue;
 }
 

@@ -285,18 +285,6 @@ __device__ __forceinline__ void clover_eo(const CloverStore &S, int V, int pos, 
     }
 }
 
-// For the sites of parity p (half index i):
-//   HOP: h = sum of hops of `hin` (opposite parity)
-//   C, Ci: clover and inverse in parity order (k_clover_invert)
-//   MODE 0: out = Cinv h
-//        1: out = C vin + beta h
-//        2: out = vin + beta h
-//        3: out = Cinv (vin + beta h)
-//        4: out = Cinv vin
-//        5: out = Cinv w and out2 = w - C out, w = vin + beta h (with
-//           vin = b_o, h = H_oe x_e, beta = k: the reconstructed x_o and
-//           the odd-site residual b_o - (A_oo x_o - k H_oe x_e) of the
-//           x_o as stored, in one pass; FP64 fields only)
 // o = C v + beta h
 template <class P>
 __device__ __forceinline__ void add_clover_eo(const Geom &g, int p, const CloverStore &C, double beta, int Vh, int i,
@@ -310,65 +298,43 @@ __device__ __forceinline__ void add_clover_eo(const Geom &g, int p, const Clover
     for (int k = 0; k < 12; ++k) o[k] = o[k] + bt * h[k];
 }
 
-// The site-local part of k_eo after the hops h: everything but the hops,
-// in the arithmetic of P.
-template <class P, int MODE>
-__device__ __forceinline__ void eo_tail(const Geom &g, int p, const CloverStore &C, const CloverStore &Ci,
-                                        const void *vin, const float *vin_nrm, void *out, float *out_nrm,
-                                        double beta, int Vh, int i, const cx<typename P::real> h[12])
-{
-    using R = typename P::real;
-    cx<R> v[12], o[12];
-    const R bt = R(beta);
-    if (MODE == 0) {
-#pragma unroll
-        for (int k = 0; k < 12; ++k) v[k] = h[k];
-    } else {
-        P::load_spinor(vin, vin_nrm, Vh, i, v);
-        if (MODE == 1) {
-            add_clover_eo<P>(g, p, C, beta, Vh, i, v, h, o);
-            P::store_spinor(out, out_nrm, Vh, i, o);
-            return;
-        }
-        if (MODE == 2 || MODE == 3)
-#pragma unroll
-            for (int k = 0; k < 12; ++k) v[k] = v[k] + bt * h[k];
-        if (MODE == 2) {
-            P::store_spinor(out, out_nrm, Vh, i, v);
-            return;
-        }
-    }
-    clover_eo<P, true>(Ci, g.V, wc_idx(p * Vh + i, g.V), v, o);
-    P::store_spinor(out, out_nrm, Vh, i, o);
-}
-
-// h = the hops of hin (opposite parity) to full-lattice site x; 0 without HOP
-template <class P, int DAG, bool HOP>
+// h = the hops of hin (opposite parity) to full-lattice site x
+template <class P, int DAG>
 __device__ __forceinline__ void eo_hops(const Geom &g, const GaugeStore &U, const void *hin, const float *hin_nrm, int Vh,
                                         int x, const int c[4], cx<typename P::real> h[12])
 {
     using R = typename P::real;
 #pragma unroll
     for (int k = 0; k < 12; ++k) h[k] = mkc(R(0), R(0));
-    if (HOP) {
-        constexpr int SF = DAG ? +1 : -1;
-        constexpr int SB = -SF;
-        if constexpr (std::is_same<P, P16>::value) {
-            const auto half = [](int y) { return y >> 1; };
-            hop_dir_h16<0, SF, SB>(g, U, hin, hin_nrm, Vh, x, c, 1.f, h, half);
-            hop_dir_h16<1, SF, SB>(g, U, hin, hin_nrm, Vh, x, c, 1.f, h, half);
-            hop_dir_h16<2, SF, SB>(g, U, hin, hin_nrm, Vh, x, c, 1.f, h, half);
-            hop_dir_h16<3, SF, SB>(g, U, hin, hin_nrm, Vh, x, c, 1.f, h, half);
-        } else {
-            const R one = R(1);
-            eo_hop_dir<P, 0, SF, SB>(g, U, hin, hin_nrm, Vh, x, c, one, h);
-            eo_hop_dir<P, 1, SF, SB>(g, U, hin, hin_nrm, Vh, x, c, one, h);
-            eo_hop_dir<P, 2, SF, SB>(g, U, hin, hin_nrm, Vh, x, c, one, h);
-            eo_hop_dir<P, 3, SF, SB>(g, U, hin, hin_nrm, Vh, x, c, one, h);
-        }
+    constexpr int SF = DAG ? +1 : -1;
+    constexpr int SB = -SF;
+    if constexpr (std::is_same<P, P16>::value) {
+        const auto half = [](int y) { return y >> 1; };
+        hop_dir_h16<0, SF, SB>(g, U, hin, hin_nrm, Vh, x, c, 1.f, h, half);
+        hop_dir_h16<1, SF, SB>(g, U, hin, hin_nrm, Vh, x, c, 1.f, h, half);
+        hop_dir_h16<2, SF, SB>(g, U, hin, hin_nrm, Vh, x, c, 1.f, h, half);
+        hop_dir_h16<3, SF, SB>(g, U, hin, hin_nrm, Vh, x, c, 1.f, h, half);
+    } else {
+        const R one = R(1);
+        eo_hop_dir<P, 0, SF, SB>(g, U, hin, hin_nrm, Vh, x, c, one, h);
+        eo_hop_dir<P, 1, SF, SB>(g, U, hin, hin_nrm, Vh, x, c, one, h);
+        eo_hop_dir<P, 2, SF, SB>(g, U, hin, hin_nrm, Vh, x, c, one, h);
+        eo_hop_dir<P, 3, SF, SB>(g, U, hin, hin_nrm, Vh, x, c, one, h);
     }
 }
 
+// One pass of the even-odd operators, for the sites of parity p (half index
+// i); h = sum of the hops of `hin` (opposite parity), C, Ci: clover term and
+// inverse in parity order (k_clover_invert):
+//   MODE 0: out = Ci h
+//        1: out = C vin + beta h
+//   and on FP64 fields
+//        2: out = vin + beta h
+//        4: out = Ci vin
+//        5: out = Ci w and out2 = w - C out, w = vin + beta h (with
+//           vin = b_o, h = H_oe x_e, beta = k: the reconstructed x_o and
+//           the odd-site residual b_o - (A_oo x_o - k H_oe x_e) of the
+//           x_o as stored, in one pass)
 // (FP32 and FP16 fields.  One CTA per SM is all that is asked of the register
 // allocation: without that it keeps fewer loads in flight, a solver step at
 // 16^3x32 in binary16 136 instead of 122 us; four CTAs measured the same, five
@@ -384,15 +350,23 @@ __global__ void __launch_bounds__(128, 1) k_eo(Geom g, int p, GaugeStore U, Clov
     griddep_wait();
     griddep_launch_dependents();
     if (skip && *skip) return;
+    static_assert(MODE == 0 || MODE == 1, "the other modes are for FP64 fields");
     using R = typename P::real;
     const int Vh = g.V >> 1;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= Vh) return;
     int c[4];
     const int x = full_site(g, i, p, c);
-    cx<R> h[12];
-    eo_hops<P, DAG, MODE != 4>(g, U, hin, hin_nrm, Vh, x, c, h);
-    eo_tail<P, MODE>(g, p, C, Ci, vin, vin_nrm, out, out_nrm, beta, Vh, i, h);
+    cx<R> h[12], o[12];
+    eo_hops<P, DAG>(g, U, hin, hin_nrm, Vh, x, c, h);
+    if (MODE == 0) {
+        clover_eo<P, true>(Ci, g.V, wc_idx(p * Vh + i, g.V), h, o);
+    } else {
+        cx<R> v[12];
+        P::load_spinor(vin, vin_nrm, Vh, i, v);
+        add_clover_eo<P>(g, p, C, beta, Vh, i, v, h, o);
+    }
+    P::store_spinor(out, out_nrm, Vh, i, o);
 }
 
 // k_eo in FP64 on four warps per 32 sites (hop_split64): warp w finishes
@@ -507,7 +481,7 @@ __global__ void __launch_bounds__(32 * W, 1) k_eo_sum(Geom g, int p, GaugeStore 
         int c[4];
         const int x = full_site(g, i, p, c);
         cx<R> h[12], v[12], o[12];
-        eo_hops<P, DAG, true>(g, U, hin, hin_nrm, Vh, x, c, h);
+        eo_hops<P, DAG>(g, U, hin, hin_nrm, Vh, x, c, h);
         P::load_spinor(vin, vin_nrm, Vh, i, v);
         add_clover_eo<P>(g, p, C, beta, Vh, i, v, h, o);
         P::store_spinor(out, out_nrm, Vh, i, o);
@@ -582,8 +556,9 @@ __global__ void __launch_bounds__(256) k_to_df(long long n, const double2 *in, f
 }
 
 // k_eo of FP64 fields in double-FP32 arithmetic, on four warps per 32 sites as
-// k_eo_split64.  HDF, ODF: hin / out is kept as z2 values.
-template <int DAG, int MODE, bool HDF, bool ODF>
+// k_eo_split64.  hin, and the output of modes 0 and 4, which the next pass takes
+// its hops from, are kept as z2 values.
+template <int DAG, int MODE>
 __global__ void __launch_bounds__(kSplit64 * kSplit64Sites, dfs::kCtas)
     k_eo_splitdf(Geom g, int p, GaugeStore U, CloverStore C, CloverStore Ci, const void *hin, const double2 *vin,
                  void *out, double2 *out2, double beta, const int *skip)
@@ -600,7 +575,7 @@ __global__ void __launch_bounds__(kSplit64 * kSplit64Sites, dfs::kCtas)
     if (MODE != 4 && valid) {
         int c[4];
         const int x = full_site(g, i, p, c);
-        dfs::hops<DAG ? +1 : -1, HDF>(g, U, hin, Vh, x, c, sm, w, s, [](int y) { return y >> 1; });
+        dfs::hops<DAG ? +1 : -1, true>(g, U, hin, Vh, x, c, sm, w, s, [](int y) { return y >> 1; });
     }
     __syncthreads();
     const df bt(beta);
@@ -637,7 +612,7 @@ __global__ void __launch_bounds__(kSplit64 * kSplit64Sites, dfs::kCtas)
 #pragma unroll
         for (int r = 0; r < 3; ++r) {
             const size_t at = (size_t)(3 * w + r) * Vh + i;
-            if (ODF) static_cast<float4 *>(out)[at] = dfs::to4(a[r]);
+            if (MODE == 0 || MODE == 4) static_cast<float4 *>(out)[at] = dfs::to4(a[r]);
             else static_cast<double2 *>(out)[at] = dfs::to_double(a[r]);
         }
     };
@@ -737,9 +712,9 @@ cudaError_t launch_eo_split64(const wc_lattice_s *full, int parity, int mode, co
     case 0: WC_EO(0); break;
     case 1: WC_EO(1); break;
     case 2: WC_EO(2); break;
-    case 3: WC_EO(3); break;
     case 4: WC_EO(4); break;
-    default: WC_EO(5);
+    case 5: WC_EO(5); break;
+    default: return cudaErrorInvalidValue;
     }
 #undef WC_EO
 }
@@ -747,36 +722,25 @@ cudaError_t launch_eo_split64(const wc_lattice_s *full, int parity, int mode, co
 template <int DAG>
 cudaError_t launch_eo_splitdf(const wc_lattice_s *full, int parity, int mode, const wc_field_s *hin,
                               const wc_field_s *vin, wc_field_s *out, double beta, cudaStream_t stream,
-                              wc_field_s *out2, const int *skip, bool pdl, int split)
+                              wc_field_s *out2, const int *skip, bool pdl)
 {
     if (mode == 5 && (!out2 || out2->prec != WC_F64)) return cudaErrorInvalidValue;
-    const bool hdf = split & kEoInSplit, odf = split & kEoOutSplit;
-    if (odf && mode != 0 && mode != 4) return cudaErrorInvalidValue;
     const int Vh = full->g.V >> 1;
     const dim3 grid((Vh + kSplit64Sites - 1) / kSplit64Sites);
     const void *hd = hin ? hin->data : nullptr;
     const double2 *vd = vin ? static_cast<const double2 *>(vin->data) : nullptr;
     double2 *o2 = out2 ? static_cast<double2 *>(out2->data) : nullptr;
-#define WC_EO(M, H, O)                                                                                                \
-    return launch_step(pdl && pdl_grid(grid.x), k_eo_splitdf<DAG, M, H, O>, grid, kSplit64 *kSplit64Sites, stream,    \
-                       full->g, parity, full->gauge, full->ceo, full->cinv, hd, vd, out->data, o2, beta, skip)
-#define WC_EO_H(M) \
-    if (hdf) WC_EO(M, true, false); \
-    WC_EO(M, false, false)
+#define WC_EO(M)                                                                                                    \
+    return launch_step(pdl && pdl_grid(grid.x), k_eo_splitdf<DAG, M>, grid, kSplit64 *kSplit64Sites, stream, full->g, \
+                       parity, full->gauge, full->ceo, full->cinv, hd, vd, out->data, o2, beta, skip)
     switch (mode) {
-    case 0:
-        if (hdf && odf) WC_EO(0, true, true);
-        if (odf) WC_EO(0, false, true);
-        WC_EO_H(0);
-    case 1: WC_EO_H(1);
-    case 2: WC_EO_H(2);
-    case 3: WC_EO_H(3);
-    case 4:
-        if (odf) WC_EO(4, false, true);
-        WC_EO(4, false, false);
-    default: WC_EO_H(5);
+    case 0: WC_EO(0); break;
+    case 1: WC_EO(1); break;
+    case 2: WC_EO(2); break;
+    case 4: WC_EO(4); break;
+    case 5: WC_EO(5); break;
+    default: return cudaErrorInvalidValue;
     }
-#undef WC_EO_H
 #undef WC_EO
 }
 
@@ -801,10 +765,7 @@ cudaError_t launch_eo_p(const wc_lattice_s *full, int parity, int mode, const wc
     switch (mode) {
     case 0: WC_EO(0); break;
     case 1: WC_EO(1); break;
-    case 2: WC_EO(2); break;
-    case 3: WC_EO(3); break;
-    case 4: WC_EO(4); break;
-    default: return cudaErrorInvalidValue;   // mode 5: FP64 fields only
+    default: return cudaErrorInvalidValue;   // the others: FP64 fields only
     }
 #undef WC_EO
 }
@@ -837,13 +798,12 @@ cudaError_t launch_eo_sum64(const wc_lattice_s *full, const wc_field_s *hin, con
 // one parity-stencil step on half fields of the full lattice `full`
 cudaError_t launch_eo(const wc_lattice_s *full, int parity, int mode, int dagger, const wc_field_s *hin,
                       const wc_field_s *vin, wc_field_s *out, double beta, cudaStream_t stream, wc_field_s *out2,
-                      const int *skip, bool pdl, int split)
+                      const int *skip, bool pdl)
 {
     const wc_prec pr = out->prec;
     if (pr == WC_F64 && full->fp64_arith == WC_ARITH_DF32)
-        return dagger ? launch_eo_splitdf<1>(full, parity, mode, hin, vin, out, beta, stream, out2, skip, pdl, split)
-                      : launch_eo_splitdf<0>(full, parity, mode, hin, vin, out, beta, stream, out2, skip, pdl, split);
-    if (split) return cudaErrorInvalidValue;
+        return dagger ? launch_eo_splitdf<1>(full, parity, mode, hin, vin, out, beta, stream, out2, skip, pdl)
+                      : launch_eo_splitdf<0>(full, parity, mode, hin, vin, out, beta, stream, out2, skip, pdl);
     if (pr == WC_F64)
         return dagger ? launch_eo_split64<1>(full, parity, mode, hin, vin, out, beta, stream, out2, skip, pdl)
                       : launch_eo_split64<0>(full, parity, mode, hin, vin, out, beta, stream, out2, skip, pdl);
@@ -913,11 +873,9 @@ cudaError_t launch_schur(wc_lattice half, wc_field out, wc_field in, int dagger,
     const bool df = eo_split(full, out);
     cudaError_t e = df ? launch_to_df(6LL * full->g.V, in, out, stream, skip, pdl) : cudaSuccess;
     if (e == cudaSuccess)
-        e = launch_eo(full, 1, 0, dagger, df ? out : in, nullptr, t, 0.0, stream, nullptr, skip, pdl,
-                      df ? kEoInSplit | kEoOutSplit : 0);
+        e = launch_eo(full, 1, 0, dagger, df ? out : in, nullptr, t, 0.0, stream, nullptr, skip, pdl);
     if (e == cudaSuccess)
-        e = launch_eo(full, 0, 1, dagger, t, in, out, -full->kappa * full->kappa, stream, nullptr, skip, pdl,
-                      df ? kEoInSplit : 0);
+        e = launch_eo(full, 0, 1, dagger, t, in, out, -full->kappa * full->kappa, stream, nullptr, skip, pdl);
     return e;
 }
 

@@ -234,12 +234,12 @@ cudaError_t launch_apply_multi(wc_lattice lat, int n, const wc_field *outs, cons
                                cudaStream_t stream);
 
 // multi-right-hand-side Schur operator (wc_eomulti.cu): outs[r] = M^ ins[r]
-// (M^+ with dagger) for FP32 or FP16 half-lattice fields of the half lattice
-// `half`, tmps[r] its odd-site intermediates; skip (nullable) holds per field
-// a device flag (nullable) whose nonzero value skips it
+// for FP32 or FP16 half-lattice fields of the half lattice `half`, tmps[r] its
+// odd-site intermediates; skip (nullable) holds per field a device flag
+// (nullable) whose nonzero value skips it
 cudaError_t launch_schur_multi(wc_lattice half, int n, wc_field const *outs, wc_field const *ins,
-                               wc_field const *tmps, int dagger, const int *const *skip, cudaStream_t stream,
-                               int red = 0, wc_field const *dots = nullptr, double *part = nullptr);
+                               wc_field const *tmps, const int *const *skip, cudaStream_t stream, int red = 0,
+                               wc_field const *dots = nullptr, double *part = nullptr);
 // CTAs of one multi-RHS Schur pass of n fields on the half lattice `half` (the
 // second dimension of its partial sums)
 int schur_multi_blocks(wc_lattice half, int n);
@@ -252,11 +252,10 @@ cudaError_t launch_schur(wc_lattice half, wc_field out, wc_field in, int dagger,
 // out2: the second output of mode 5 (nullptr for the other modes)
 cudaError_t launch_eo(const wc_lattice_s *full, int parity, int mode, int dagger, const wc_field_s *hin,
                       const wc_field_s *vin, wc_field_s *out, double beta, cudaStream_t stream,
-                      wc_field_s *out2 = nullptr, const int *skip = nullptr, bool pdl = false, int split = 0);
-// In double-FP32 arithmetic hin (kEoInSplit) or the output of modes 0 and 4
-// (kEoOutSplit) may be held as split values (wc_dfsplit.cuh) in an FP64 half
-// field: launch_to_df makes them, eo_split says whether f is of that kind.
-constexpr int kEoInSplit = 1, kEoOutSplit = 2;
+                      wc_field_s *out2 = nullptr, const int *skip = nullptr, bool pdl = false);
+// In double-FP32 arithmetic (eo_split of the fields) hin, and the output of modes
+// 0 and 4, hold split values (wc_dfsplit.cuh) in an FP64 half field; launch_to_df
+// makes them.
 cudaError_t launch_to_df(long long n /*complex values*/, const wc_field_s *in, wc_field_s *out, cudaStream_t stream,
                          const int *skip = nullptr, bool pdl = false);
 // the whole-lattice operator in double-FP32, in split into `split` first

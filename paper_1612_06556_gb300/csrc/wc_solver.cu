@@ -291,16 +291,14 @@ wc_status eo_reconstruct_residual(wc_lattice lat, int kind, wc_field be, wc_fiel
     const bool df = eo_split(lat, xe);
     if (df) st = check_cuda(lat, launch_to_df(6LL * lat->g.V, xe, re, s), "split x_e");
     if (st == WC_OK)
-        st = check_cuda(lat, launch_eo(lat, 1, 5, kind, df ? re : xe, bo, xo, k, s, ro, nullptr, false,
-                                       df ? kEoInSplit : 0), "x_o and r_o");
+        st = check_cuda(lat, launch_eo(lat, 1, 5, kind, df ? re : xe, bo, xo, k, s, ro), "x_o and r_o");
     if (st == WC_OK) st = check_cuda(lat, norm2_to_result(h, R, d2(ro)), "norm2");
     if (st == WC_OK)
         st = check_cuda(lat, cudaMemcpyAsync(R.red.host_result, R.red.result, sizeof(double), cudaMemcpyDeviceToHost, s),
                         "copy");
     if (st == WC_OK && df) st = check_cuda(lat, launch_to_df(6LL * lat->g.V, xo, ro, s), "split x_o");
     if (st == WC_OK)
-        st = check_cuda(lat, launch_eo(lat, 0, 1, kind, df ? ro : xo, xe, re, -k, s, nullptr, nullptr, false,
-                                       df ? kEoInSplit : 0), "(M x)_e");
+        st = check_cuda(lat, launch_eo(lat, 0, 1, kind, df ? ro : xo, xe, re, -k, s), "(M x)_e");
     if (st == WC_OK) st = check_cuda(lat, launch_merge(lat, xe, xo, x, s), "merge");
     if (st == WC_OK) st = check_cuda(lat, residual(h, R, d2(be), d2(re)), "residual");
     if (st == WC_OK) st = read_scalars(h, R);
@@ -396,10 +394,8 @@ static wc_status eo_bicgstab(wc_lattice lat, int kind, wc_field x, wc_field b, c
     const double k = lat->kappa;
     if (st == WC_OK) st = check_cuda(lat, launch_split(lat, b, be, bo, s), "split");
     if (st == WC_OK) st = check_cuda(lat, launch_split(lat, x, xe, xo, s), "split");
-    if (st == WC_OK) st = check_cuda(lat, launch_eo(lat, 1, 4, kind, nullptr, bo, t, 0.0, s, nullptr, nullptr, false,
-                                        eo_split(lat, t) ? kEoOutSplit : 0), "A_oo^-1 b_o");
-    if (st == WC_OK) st = check_cuda(lat, launch_eo(lat, 0, 2, kind, t, be, bh, k, s, nullptr, nullptr, false,
-                                        eo_split(lat, t) ? kEoInSplit : 0), "b^_e");
+    if (st == WC_OK) st = check_cuda(lat, launch_eo(lat, 1, 4, kind, nullptr, bo, t, 0.0, s), "A_oo^-1 b_o");
+    if (st == WC_OK) st = check_cuda(lat, launch_eo(lat, 0, 2, kind, t, be, bh, k, s), "b^_e");
     double bb = 0.0, bbh = 0.0;
     if (st == WC_OK) st = reduce_norm2(lat, b, &bb);
     if (st == WC_OK) st = reduce_norm2(h, bh, &bbh);

@@ -73,3 +73,29 @@ def test_multi_apply_argument_errors():
     with pytest.raises(w.WCError) as e:
         lat.apply_multi([a[0], a[0]], [b[0], b[1]])             # repeated out
     assert e.value.status == 1
+
+
+@pytest.mark.parametrize("n", [4, 6, 7, 12])
+@pytest.mark.parametrize("krylov", [1, 2])
+def test_one_lockstep_step_is_that_of_single_solves(n, krylov, monkeypatch):
+    """The multi-field Schur passes on half-lattice fields, on both sides of
+    the rule for a CTA's sites and on a ragged half volume: x of each source
+    after one step of a lockstep group from zero is that of a single solve's
+    step, whose operator is the single-field pass.  The two form their sums in
+    different orders: x is first order in the step's scalars and vectors, so
+    the tolerance is that of the Krylov vectors."""
+    monkeypatch.setenv("WC_BATCH_LOCKSTEP", "1")
+    dims, kappa, csw, tbc = (6, 2, 10, 6), 0.12, 1.0, -1
+    U = synth.exp_links(dims, 0.3, 361)
+    lat = make_lattice(dims, U, csw, kappa, tbc)
+    srcs = [synth.gaussian_source(dims, 362 + r) for r in range(n)]
+    bs, xs = [lat.field(0).load(s) for s in srcs], [lat.field(0) for _ in srcs]
+    kw = dict(tol=1e-13, max_iter=1, max_restarts=0, check=False, solver=1, even_odd=True, krylov_prec=krylov)
+    infos = wc().solve_batch([lat] * n, xs, bs, **kw)
+    for s, b, x, info in zip(srcs, bs, xs, infos):
+        assert info.iters == 1
+        one = lat.field(0)
+        lat.solve(one, b, **kw)
+        ref = one.store(np.zeros_like(s))
+        out = x.store(np.zeros_like(s))
+        assert np.linalg.norm(out - ref) <= {1: 1e-5, 2: 5e-3}[krylov] * np.linalg.norm(ref)
