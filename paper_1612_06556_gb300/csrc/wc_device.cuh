@@ -162,8 +162,10 @@ __device__ __forceinline__ void site_coords(const Geom &g, int s, int c[4])
 }
 
 // site_coords with the divisions by multiplication.  Measured per operator:
-// the FP16 kernel (bound by instruction issue) gains 3 %, the FP32 kernel
-// (at 80 registers, bandwidth-bound) loses 2 %, so only the FP16 path uses it.
+// the whole-lattice FP16 kernel (bound by instruction issue) gains 3 %, the FP32
+// one (at 80 registers, bandwidth-bound) loses 2 % and keeps the divisions; the
+// four-warp FP64 and double-FP32 kernels, the even-odd passes and the
+// multi-field kernels use it.
 __device__ __forceinline__ void site_coords_fast(const Geom &g, int s, int c[4])
 {
     int q = fast_div(s, g.div[0]);

@@ -273,10 +273,10 @@ constexpr ApplyShape kShapes[] = {
 };
 constexpr int kNumShapes = sizeof(kShapes) / sizeof(kShapes[0]);
 // What the FP64 operator takes unless a caller pins one of the shapes above:
-// it measured as fast as the best of them or faster on every lattice (4^4 13
-// against 39 us, 8^4 14 / 39, 12^4 49 / 60, 16^3x32 247 / 266, 24^3x32
-// 828 / 863, 17x19x21x23 299 / 331, 32^3x64 3960-4016 / 4014-4022), so
-// nothing is timed for it.
+// it measured faster than the best of them on every lattice (4^4 13
+// against 39 us, 8^4 14 / 39, 12^4 49 / 60, 16^3x32 245 / 266, 24^3x32
+// 809 / 863, 17x19x21x23 299 / 331, 32^3x64 3811 / 4014), so nothing is timed
+// for it.
 constexpr int kShapeSplit64 = kNumShapes;
 // In double-FP32 arithmetic up to this many sites; above, one of the shapes
 // is timed and taken.  Each hop splits its spinor anew, which costs more than it
@@ -298,7 +298,8 @@ bool shape_fits(const Geom &g, const ApplyShape &s, int caps)
     return s.tile[0] * s.tile[1] * s.tile[2] * s.tile[3] == s.threads;
 }
 
-// Resident CTAs per SM of one kernel instantiation (cached per function).
+// Resident CTAs per SM of one kernel instantiation, asked of the runtime at
+// every launch of a persistent shape.
 template <class K>
 int resident_ctas(K kernel, int threads)
 {

@@ -123,7 +123,9 @@ __device__ bool invert6(cx<double> a[6][6])
 // over 8192 blocks of Haar links, by this form / by elimination, csw 1 1.23 /
 // 1.28e-16, csw 2 1.26 / 1.31, csw 3 1.34 / 1.37 (88 % of the blocks pass), csw 5
 // 4.6 / 4.6 (13 %); a bound of 1/4 would pass 84 % at csw 5, at 4.8e-16.
-// (By 3x3 blocks and cofactors: 1.65 1.67 1.79 5.4e-16.)
+// (By 3x3 blocks and cofactors: 1.65 1.67 1.79 5.4e-16.)  At 16^3x32 297 us for
+// both blocks of all sites and their copies, FP64 pipe 88 % busy; 1637 with every
+// block eliminated.
 __device__ __forceinline__ bool invert_block(const double r[36], double inv[36])
 {
     double big = 0.0, d[6], e[6];

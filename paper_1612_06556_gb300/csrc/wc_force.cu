@@ -57,8 +57,10 @@
 // contributions of a link and its hopping part; two planes at a time, the
 // pairs (xy, zt), (xz, yt), (yz, xt) that contain every direction once.
 //
-// Everything here is bound by the FP64 pipe.  At 16^3x32 (k_xi + the force):
-// 244 + 4650 us link by link; now the plaquettes 3 x 794, the last link pass 313.
+// Everything here but the first two link passes is bound by the FP64 pipe (97 %
+// busy in the plaquettes, 91 % in the last link pass).  At 16^3x32 (k_xi + the
+// force): 244 + 4650 us link by link; now the plaquettes 3 x 947, the link
+// passes 50 + 50 + 316.
 
 #include <math.h>
 

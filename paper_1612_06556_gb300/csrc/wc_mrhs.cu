@@ -19,9 +19,10 @@
 // per SM count, and CTAs small enough that one stages while others compute:
 // 16 sites and 64 registers (32 warps) above four right-hand sides, 32 sites
 // and 80 registers up to four, where a CTA has few warps anyway.  24^3x32,
-// 16 x 64 / 32 x 80: 297 / 312 us for one field, 201 / 187 for 3, 215 / 201
-// for 4, 230 / 263 for 6, 274 / 320 for 8, 410 / 468 for 12, 527 / 791 for 16;
-// 96 registers 491 / 686 for 12, 8 sites 544.
+// 16 x 64 / 32 x 80: 298 / 313 us for one field (16^3x32 87 / 83), 210 / 206 for
+// 2, 204 / 189 for 3, 219 / 204 for 4, 236 / 258 for 5, 232 / 265 for 6, 277 /
+// 324 for 8, 410 / 468 for 12, 527 / 791 for 16; 96 registers 491 / 686 for 12, 8
+// sites 544.
 #include "wc_internal.cuh"
 #include "wc_stencil.cuh"
 
