@@ -74,14 +74,24 @@ bool is_device_pointer(const void *p)
 // ------------------------------------------------------------------------
 
 // A site's 12 components lie together in the canonical layout (96 or 192
-// bytes) and in 12 planes in the device layouts.  A CTA turns kXferSites
-// sites round in shared memory, so that both sides move 16 contiguous bytes
-// per thread and a warp whole 128-byte lines; one thread per site reading or
-// writing its row left the memory system with 12 partly used sectors per
-// request (export at 24^3x32 FP32 -> complex64 27 us = 3.1 TB/s, 12.4 us now;
+// bytes) and in 12 planes in the device layouts.  On export a CTA turns
+// kXferSites sites round in shared memory, so that both sides move 16
+// contiguous bytes per thread and a warp whole 128-byte lines; one thread per
+// site writing its row left the memory system with 12 partly used sectors per
+// request (24^3x32 FP32 -> complex64 27 us = 3.1 TB/s, 12.4 us now;
 // binary16 -> complex64 at 32^3x64 110 us, 42 now).  A row in shared memory
 // is one 16-byte unit longer than in the canonical layout: the eight lanes
 // of a 16-byte access phase then fall on different banks.
+//
+// On import the rows are read, and the sectors that one load of a warp leaves
+// partly used are in L1 for the next: a thread per site is the faster form but
+// where the rows are short beside what is written of them (complex64 ->
+// binary16), and on lattices of less than a CTA of kXferSites per SM, where its
+// loads wait for one another.  Thread per site / turned round, us: complex128 ->
+// FP32 at 8^4 3.2 / 2.8, 16^4 4.9 / 5.7, 24^3x32 23 / 27, 32^3x64 91 / 109; ->
+// FP64 3.1 / 2.3, 4.9 / 4.5, 28 / 31, 120 / 136; complex64 -> FP32 2.1 / 2.0,
+// 3.0 / 3.2, 15.0 / 16.2, 61 / 68; -> binary16 2.1 / 2.2, 2.8 / 2.8, 12.5 / 12.0,
+// 48.9 / 46.6.
 // T: double2 (canonical complex128) or float2 (canonical complex64)
 constexpr int kXferSites = 128;
 
@@ -133,6 +143,22 @@ __global__ void __launch_bounds__(kXferSites) k_import(int V, const T *src, void
     P::store_spinor(dst, nrm, V, x0 + threadIdx.x, s);
 }
 
+// the same, a thread per site
+template <class P, class T>
+__global__ void __launch_bounds__(256) k_import_rows(int V, const T *src, void *dst, float *nrm)
+{
+    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    if (x >= V) return;
+    using R = typename P::real;
+    cx<R> s[12];
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+        const T v = src[(size_t)x * 12 + k];
+        s[k] = mkc((R)v.x, (R)v.y);
+    }
+    P::store_spinor(dst, nrm, V, x, s);
+}
+
 template <class P, class T>
 __global__ void __launch_bounds__(kXferSites) k_export(int V, const void *src, const float *nrm, T *dst)
 {
@@ -151,13 +177,21 @@ __global__ void __launch_bounds__(kXferSites) k_export(int V, const void *src, c
 }
 
 // queue the conversion of canonical data (device) into f, or of f into it
+template <class P, class T>
+void launch_import_p(wc_field f, const T *src, cudaStream_t stream)
+{
+    const int V = f->lat->g.V;
+    const bool turn = (std::is_same<P, P16>::value && std::is_same<T, float2>::value) || V < kXferSites * sm_count();
+    if (turn) k_import<P, T><<<(V + kXferSites - 1) / kXferSites, kXferSites, 0, stream>>>(V, src, f->data, f->nrm);
+    else k_import_rows<P, T><<<(V + 255) / 256, 256, 0, stream>>>(V, src, f->data, f->nrm);
+}
+
 template <class T>
 void launch_import(wc_field f, const T *src, cudaStream_t stream)
 {
-    const int V = f->lat->g.V, grid = (V + kXferSites - 1) / kXferSites;
-    if (f->prec == WC_F64) k_import<P64, T><<<grid, kXferSites, 0, stream>>>(V, src, f->data, f->nrm);
-    else if (f->prec == WC_F32) k_import<P32, T><<<grid, kXferSites, 0, stream>>>(V, src, f->data, f->nrm);
-    else k_import<P16, T><<<grid, kXferSites, 0, stream>>>(V, src, f->data, f->nrm);
+    if (f->prec == WC_F64) launch_import_p<P64>(f, src, stream);
+    else if (f->prec == WC_F32) launch_import_p<P32>(f, src, stream);
+    else launch_import_p<P16>(f, src, stream);
 }
 
 template <class T>
