@@ -277,7 +277,7 @@ wc_status wc_apply_multi(wc_lattice lat, int n, wc_field *outs, wc_field *ins, i
  * singular).  All four extents must be even (WC_ERR_ARG otherwise: a hop
  * across the boundary of an odd extent would keep the parity).  Fields:
  * distinct, same lattice and precision.  Blocking.  The two half-lattice
- * fields it works in are kept by the lattice between calls, up to 256 MB in
+ * fields it works in are kept by the lattice between calls, up to 512 MB in
  * each precision. */
 wc_status wc_apply_schur(wc_lattice lat, wc_field out, wc_field in, int dagger);
 
@@ -315,7 +315,7 @@ wc_status wc_apply_shape(wc_lattice lat, wc_prec prec, int kind, int force_index
  * right-hand sides of a propagator share them; paper Sec. 2: the solvers
  * act on the even-odd preconditioned matrix).  outs must be distinct from
  * each other and from ins.  Blocking.  Its workspace, n half-lattice fields,
- * is kept by the lattice between calls up to 256 MB and freed after the call
+ * is kept by the lattice between calls up to 512 MB and freed after the call
  * above. */
 wc_status wc_apply_schur_multi(wc_lattice lat, int n, wc_field *outs, wc_field *ins, int dagger);
 

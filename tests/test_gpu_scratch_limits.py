@@ -50,15 +50,15 @@ def test_even_odd_call_after_one_that_ran_out_of_memory(left):
 
 
 def test_schur_workspaces_above_their_bound_are_given_back():
-    """16 half-lattice FP32 fields of 24^3x32 are 340 MB and freed with the
-    call, 8 are 170 MB and kept for the next one."""
+    """16 half-lattice FP32 fields of 32^4 are 805 MB and freed with the call, 8
+    are 403 MB and kept for the next one."""
     import torch
 
     def free():
         torch.cuda.synchronize()
         return torch.cuda.mem_get_info()[0]
 
-    dims = (24, 24, 24, 32)
+    dims = (32, 32, 32, 32)
     lat = make_lattice(dims, synth.unit_links(dims), 1.0, 0.12, -1)
     fields = [lat.field(1) for _ in range(32)]
     lat.apply_schur_multi(fields[:1], fields[16:17])
@@ -67,7 +67,7 @@ def test_schur_workspaces_above_their_bound_are_given_back():
     assert free() >= before
     lat.apply_schur_multi(fields[:8], fields[16:24])
     kept = free()
-    assert before - kept >= 140 * MB
+    assert before - kept >= 7 * 48 * 32 ** 4      # the first call had kept one field
     lat.apply_schur_multi(fields[:8], fields[16:24])
     assert free() == kept
 
